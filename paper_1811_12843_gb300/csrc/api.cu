@@ -106,6 +106,7 @@ struct lipz_grid {
   float* TL = nullptr;
   void *J2 = nullptr, *D1 = nullptr, *A3 = nullptr, *A2 = nullptr, *A1 = nullptr;
   float *gG = nullptr, *gD = nullptr;
+  int* bsync = nullptr;  // the tensor-core backward's tile counters
   int* flag = nullptr;
   // generator-mixture weights [cells][5] (always held: part of the state), and with
   // arch.mixture the score's work buffers: row norms [cells][6B], per-row block sums
@@ -748,6 +749,7 @@ int create_impl(lipz_grid* g) {
       if (!g->tc[p]) return fail(g, LIPZ_ERR_CUDA, "tensor-core plan: %s", msg.c_str());
     }
     g->use_tcb = tcb_supported(z, h, x, B);
+    if (g->use_tcb && (rc = dalloc(g, &g->bsync, tcb_sync_ints(C) * sizeof(int)))) return rc;
     for (int p = 0; p < g->nsnap && g->use_tcb; ++p) {
       TcbShape s{C, B, z, h, x, g->a.leaky_slope, g->nsnap * C};
       TcbBuffers b{};
@@ -765,6 +767,7 @@ int create_impl(lipz_grid* g) {
       b.A1 = g->A1;
       b.gG = g->gG;
       b.gD = g->gD;
+      b.sync = g->bsync;
       b.Gwb = g->G[0].wb;
       b.Dwb = g->D[0].wb;
       b.PGs = g->PGs;
@@ -796,7 +799,7 @@ int create_impl(lipz_grid* g) {
       b.eps = g->a.eps;
       AdamRanges rr[2];
       bias_ranges(g, p, &rr[0], &rr[1]);
-      b.ranges = b.fuse_adam ? rr : nullptr;
+      b.ranges = rr;
       std::string msg;
       g->tcb[p] = tcb_plan_create(s, b, &msg);
       if (!g->tcb[p]) return fail(g, LIPZ_ERR_CUDA, "tensor-core backward plan: %s", msg.c_str());
@@ -1070,11 +1073,11 @@ int train_once(lipz_grid* g) {
   if (g->bf)
     launch_dlogit<bf16>(g->TL, (const bf16*)g->TG2, g->D[0].wb, g->PDs, g->ld.off[4], g->src_d, C,
                         B, h, g->a.leaky_slope, (bf16*)g->J2, g->gD, g->PDs, g->ld.off[4],
-                        g->ld.off[5], g->ld.off[3], g->st);
+                        g->ld.off[5], g->ld.off[3], g->bsync, TCB_SYNC_WORDS, g->st);
   else
     launch_dlogit<float>(g->TL, (const float*)g->TG2, g->D[0].w, g->PDs, g->ld.off[4], g->src_d,
                          C, B, h, g->a.leaky_slope, (float*)g->J2, g->gD, g->PDs, g->ld.off[4],
-                         g->ld.off[5], g->ld.off[3], g->st);
+                         g->ld.off[5], g->ld.off[3], nullptr, 0, g->st);
   CKL(g);
   phase_end(g, LIPZ_PHASE_TRAIN_FWD, n_fwd + 1);
   phase_begin(g, LIPZ_PHASE_TRAIN_BWD);
@@ -1082,7 +1085,7 @@ int train_once(lipz_grid* g) {
     // the nine backward products of every cell in one launch (with Adam on the weight
     // matrices unless the gradients are kept; the bias gradients summed in its epilogue)
     std::string msg;
-    if (tcb_run_cells(g->tcb[p], g->st, &msg)) return fail(g, LIPZ_ERR_CUDA, "%s", msg.c_str());
+    if (tcb_run(g->tcb[p], g->st, &msg)) return fail(g, LIPZ_ERR_CUDA, "%s", msg.c_str());
     CKL(g);
     phase_end(g, LIPZ_PHASE_TRAIN_BWD, 1);
     phase_begin(g, LIPZ_PHASE_ADAM);

@@ -1,20 +1,19 @@
 // Tensor-core backward of the training step (Section 3, step 3: the gradient update of every
 // cell's selected generator and discriminator), bf16 operands and fp32 accumulation in TMEM.
 //
-// One grouped GEMM kernel serves every product of the backward: per cell, a 128 x BN output
-// tile of C = A * B^T over K, where each operand is read by TMA either K-major (rows of K) or
-// MN-major (rows of M or N, K in the outer dimension; used for the transposed products dW =
-// delta^T X and delta W, so no transposed copy is ever written). Epilogues: fp32 store
-// (weight gradients) or bf16 delta times the activation derivative read from the stored
-// forward output. The z coordinate of a weight operand is the cell's selected individual.
-// A weight-gradient tile can instead apply Adam on the spot (EPI_ADAM): the gradient never
-// leaves the accumulator. A loader warp streams the selected individual's old weights and
-// moments by TMA into shared memory, 32 columns at a time, while the epilogue turns the
-// previous chunk into the cell's new weights, moments and bf16 copy.
+// One persistent grouped-GEMM kernel runs every product of the backward of every cell: 128 x BN
+// output tiles of C = A * B over K, A read by TMA K-major (rows of K) or MN-major (K in the outer
+// dimension; used for the transposed products dW = delta^T X), B always MN-major, so no transposed
+// copy is ever written. The z coordinate of a weight operand is the cell's selected individual.
+// Epilogues: bf16 delta times the activation derivative of the stored forward output; Adam on the
+// spot for a weight gradient (it never leaves the accumulator), or its fp32 store. What an
+// epilogue reads besides the accumulator (the old weights and moments, the forward output)
+// streams through shared memory in chunks that one warp loads and another stores by TMA.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
 #include <cstring>
+#include <vector>
 
 #include "bwd_tc.h"
 #include "common.cuh"
@@ -28,38 +27,43 @@ using namespace lipz::tc;
 constexpr int BM = 128;
 constexpr int BK = 64;
 constexpr int A_BYTES = BM * BK * 2;        // 16 KB
-constexpr int B_BYTES = 256 * BK * 2;       // 32 KB (BN <= 256)
-constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
 constexpr int MN_BOX_BYTES = 64 * BK * 2;   // one {64 MN, 64 K} box
 constexpr int NUM_EPI_WARPS = 8;
 constexpr int EPI_THREADS = 32 * NUM_EPI_WARPS;
-// bias-gradient partial sums: [2 tiles][4 TMEM lane quarters][256 columns] fp32
-constexpr int BIAS_PART_BYTES = 2 * 4 * 256 * 4;
-// fused Adam: a chunk is 64 rows (one half of a tile) x 32 fp32 columns of each of w, m, v (one
-// 128-byte row each, 128-byte swizzle), updated in place, plus the new bf16 copy (64-byte rows,
-// no swizzle). Chunks alternate between the two row halves, so each half of the epilogue
-// works through its own two of the four buffers. w, m and v lie a fixed distance apart in
-// memory, so that one TMA box {32, 64, 1, 3} of a 4-D map moves the chunk's three arrays: a
-// tiled TMA operation holds its issuing thread for about 0.2 us whatever its size up to 16 KB,
-// so one box per array made the issuing thread, not the bytes, bound the stream.
+// Chunk stream. A chunk is 64 rows (one half of a tile) of what the epilogue reads besides the
+// accumulator, updated in place in shared memory; chunks alternate between the two row halves, so
+// each half of the epilogue works through its own two of the four buffers (an even number: a half
+// that met the other's buffers could run a phase ahead of their barriers).
+//   Adam: 32 fp32 columns of each of w, m, v (one 128-byte row each, 128-byte swizzle), plus the
+//   new bf16 copy (64-byte rows, no swizzle). w, m and v lie a fixed distance apart in memory, so
+//   that one TMA box {32, 64, 1, 3} of a 4-D map moves the chunk's three arrays: a tiled TMA
+//   operation holds its issuing thread for about 0.2 us whatever its size up to 16 KB, so one box
+//   per array made the issuing thread, not the bytes, bound the stream.
+//   Delta: up to 128 bf16 columns of the stored forward output in boxes {64, 64} (128-byte rows,
+//   128-byte swizzle), replaced by the deltas.
+constexpr int CHUNK_ROWS = 64;
 constexpr int ADAM_COLS = 32;
-constexpr int ADAM_ROWS = 64;
-constexpr int ADAM_ARRAY_BYTES = ADAM_ROWS * ADAM_COLS * 4;            // 8 KB
-constexpr int ADAM_WB_BYTES = ADAM_ROWS * ADAM_COLS * 2;               // 4 KB
-constexpr int ADAM_BUF_BYTES = 3 * ADAM_ARRAY_BYTES + ADAM_WB_BYTES;   // 28 KB
+constexpr int ADAM_ARRAY_BYTES = CHUNK_ROWS * ADAM_COLS * 4;           // 8 KB
+constexpr int ADAM_WB_BYTES = CHUNK_ROWS * ADAM_COLS * 2;              // 4 KB
+constexpr int DELTA_COLS = 128;
+constexpr int DELTA_BOX_BYTES = CHUNK_ROWS * 64 * 2;                   // 8 KB
+constexpr int CHUNK_BYTES = 3 * ADAM_ARRAY_BYTES + ADAM_WB_BYTES;      // 28 KB
+// barriers, the ring of claimed tiles and the TMEM slot
+constexpr int MISC_BYTES = 512;
+// Claimed tiles a CTA holds: the one in its epilogue and the next, whose operands load meanwhile.
+// (Four: the tiles claimed early by busy CTAs lengthen the tail, 386 against 382 us at 12x12.)
+constexpr int RING = 2;
+constexpr int CHUNK_BUFS = 4;
+// Operand ring: 96 KB in stages of 16 KB of A and BN x 128 bytes of B, BN the grid's tile width
+// (128: three stages, 64: four).
+constexpr int RING_BYTES = 3 * (A_BYTES + 128 * BK * 2);
+constexpr int MAX_OPS = 4;
+constexpr int SMEM = 1024 + RING_BYTES + CHUNK_BUFS * CHUNK_BYTES + MISC_BYTES;
+static_assert(SMEM <= 232448, "backward: shared memory");
+// producer, MMA issuer, epilogue, chunk loader, chunk storer
+constexpr int THREADS = 64 + EPI_THREADS + 64;
 
-// Without fused Adam: four operand stages. With it: two operand stages, four Adam chunk
-// buffers and two more warps (the Adam stream's loader and storer). One CTA per SM either way.
-template <bool FUSED>
-struct Cfg {
-  static constexpr int STAGES = FUSED ? 2 : 4;
-  static constexpr int ADAM_BUFS = FUSED ? 4 : 0;
-  static constexpr int THREADS = 64 + EPI_THREADS + (FUSED ? 64 : 0);
-  static constexpr int SMEM =
-      1024 + STAGES * STAGE_BYTES + ADAM_BUFS * ADAM_BUF_BYTES + 256 + BIAS_PART_BYTES;
-};
-
-enum { EPI_F32 = 0, EPI_DACT = 1, EPI_ADAM = 2 };
+enum { EPI_F32 = 0, EPI_DACT = 1, EPI_ADAM = 2 };  // fp32 store; deltas; Adam step
 
 // Adam of one weight tensor fused into the tile that computes its gradient (Section 3, step 3:
 // the selected individual of the cell takes one Adam step and becomes the cell's new centre).
@@ -71,163 +75,121 @@ struct AdamRef {
 };
 
 struct GParams {
-  int cells;
   int M, N, K, BN;
   int mtiles, ntiles, kchunks;
-  int a_mn, b_mn;       // operand layouts (1 = MN-major)
-  int a_row0, b_row0;   // first row of a K-major operand
+  int a_mn;             // A's layout: 1 = MN-major (B always is)
+  int a_row0;           // first row of a K-major A
   const int* a_sel;     // z coordinate of A: a_sel[cell] (weights of the selected individual)
   const int* b_sel;     //   or the cell itself when null
   int epi, act;
   float slope;
-  void* C;
-  int64_t c_cell, scm, scn;  // C[cell * c_cell + m * scm + n * scn]
-  const bf16* aux;
-  int64_t aux_cell, sxm, sxn;
-  int aux_wrap_at, aux_wrap_sub;  // aux row of m: m < wrap_at ? m : m - wrap_sub
-  const int* aux_sel;             // non-null: aux also advances (1 + aux_sel[cell]) * aux_sel_stride
-  int64_t aux_sel_stride;
+  float* C;             // EPI_F32: C[cell * c_cell + m * N + n]
+  int64_t c_cell;
+  // EPI_DACT: the stored forward output of row m is row x_row0 + m of the stage's aux map; with
+  // x_slot (non-null) a 4-D map {n, rows, slots, cells}, slot 1 + x_slot[cell]
+  int x_row0;
+  const int* x_slot;
   // split K (ksplit > 0): chunks [0, ksplit) read K rows kc * 64 of A and of B's slot 0;
   // chunks [ksplit, kchunks) read K rows (kc - ksplit) * 64 of A shifted by a_k_off1 and of B's
   // slot 1 + b_slot_sel[cell]; B is then a 4-D map {n, K rows, slots, cells}
   int ksplit, a_k_off1;
   const int* b_slot_sel;
-  // EPI_DACT: column sums of the fp32 deltas over rows m < bias_rows go to
-  // bias_out[cell * bias_cell + n] (a bias gradient); null = none
-  float* bias_out;
+  // EPI_DACT: column sums of the fp32 deltas over the 32 rows q of row tile i go to
+  // bias_part[cell * bias_cell + (4 i + q) * N + n] (together a bias gradient); null = none
+  float* bias_part;
   int64_t bias_cell;
-  int bias_rows;
   AdamRef adam;
-  int* err;
 };
 
-// OR of pred over the eight epilogue warps (named barrier 1, 256 threads); also orders their
-// earlier global stores before their later loads.
-__device__ __forceinline__ bool epi_any(bool pred) {
-  uint32_t r;
-  asm volatile(
-      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n bar.red.or.pred q, 1, 256, p;\n"
-      " selp.u32 %0, 1, 0, q;\n}"
-      : "=r"(r)
-      : "r"((uint32_t)pred)
-      : "memory");
-  return r != 0;
-}
-
-__device__ __forceinline__ float dact(int act, float y, float slope) {
-  switch (act) {
-    case ACT_RELU: return y > 0.f ? 1.f : 0.f;
-    case ACT_LRELU: return y > 0.f ? 1.f : slope;
-    case ACT_TANH: return 1.f - y * y;
-    default: return 1.f;
-  }
-}
-
 // ---------------------------------------------------------------------------------------------
-// The whole backward of one cell in one CTA: the nine products run as consecutive stages of a
-// single tile stream (double-buffered TMEM, one TMA ring). A stage that reads an earlier
-// stage's output waits until the epilogue has finished that stage's last tile: the epilogue
-// threads fence their global stores into the async proxy, meet on an mbarrier, and one of
-// them advances a tile counter in shared memory that the producer polls before loading.
+// The backward of every cell as one list of tiles. A cell's ten products are stages; a stage's
+// tiles are entries of a list that orders the whole grid's work so that every tile comes after
+// the tiles it reads: level by level along the chain, cell by cell within a level, so that the
+// tiles a tile reads lie a whole level (every cell's Adam tiles of that level among it) earlier.
+// Persistent CTAs claim entries in list order from a counter in global memory: each runs what it
+// claimed in that order, so the oldest unfinished tile never waits for a tile that nobody runs,
+// however few CTAs are resident. A delta tile that others read is counted in global memory once
+// its stores are written; the producer of a tile that reads it acquires the count before its loads.
+//
+// Bound: HBM on large grids (26 B per parameter through the chunk stream; 2.36 GB of DRAM traffic
+// at 12x12, B = 100: 382 us, 0.91 of the measured copy rate), the chain of five dependent tiles
+// on small ones (about 8 us each). One CTA per cell walking its own tiles took 422 us at 12x12
+// (its delta tiles stopped its stream), and left most SMs idle on small grids: 307 us at 1x1
+// (now 41), 421 at 5x5, B = 256 (102). Cells 4 to 40 apart per level instead of all of them (a
+// smaller window of activations) were slower: 400 to 535 us at 12x12.
 // ---------------------------------------------------------------------------------------------
-constexpr int MAX_STAGES = 9;
+constexpr int MAX_STAGES = 10;
+constexpr int RANGES_STAGE = MAX_STAGES;  // + 0, 1: list entries of G's and D's ranges of a cell
+constexpr int SYNC_WORDS = TCB_SYNC_WORDS;  // counters per cell in TcbBuffers::sync
 
 struct Stage {
   GParams p;
-  int dep;      // stage whose output this one reads (-1: none)
-  int tile0;    // tiles of the cell before this stage
-  int publish;  // a later stage reads this one's output: its tiles are published and counted
+  int dep;       // stage whose output this one reads (-1: none)
+  int dep_need;  // tiles of that stage per cell
+};
+
+// A cell's ranges entry of one population: the gradients of its biases from their partial sums,
+// then the Adam step of the ranges (biases, D's output layer), or the gradients stored.
+constexpr int MAX_RANGES = 4;
+constexpr int RANGE_REPS = 6;  // elements per epilogue thread and pass
+struct RangeTask {
+  AdamRanges r;
+  float* grad;                     // gradient vectors (r.grad), written without fused Adam
+  const float* part[MAX_RANGES];   // first cell's partials [4 tiles][len]; null: r.grad holds it
+  int tiles[MAX_RANGES];           // row tiles of the partials
+  int64_t part_cell;
+  int total;                       // elements of all ranges
+  int n_dep, dep[MAX_RANGES], need[MAX_RANGES];  // stages that write the partials
 };
 
 struct CellPlan {
   Stage st[MAX_STAGES];
-  int n_stages, tiles_per_cell, pub_per_cell, cells;
-  int pub_end[MAX_STAGES];  // tiles of the cell published by the end of stage k
+  const int2* list;  // {cell, stage << 16 | tile}
+  int n_list;
+  int n_ops, op_bytes;  // operand ring: stages and bytes per stage
+  // [SYNC_WORDS] per cell: finished tiles by stage; after the last cell's, the claim counter
+  int* sync;
+  int cells;
   int* err;
-  // fused Adam: the biases' and D's output layer's step, applied by the epilogue warps to each
-  // cell once its tiles are done (all of its gradients are then in gG / gD)
-  int has_ranges;
-  AdamRanges rg, rd;
+  RangeTask rt[2];  // G, D
+  int adam;         // the weight matrices' tiles and the ranges take their Adam step
   float beta1, beta2, eps;
 };
 
 struct StageMaps {
   CUtensorMap a[MAX_STAGES];
   CUtensorMap b[MAX_STAGES];
-  CUtensorMap ao[MAX_STAGES];  // old w, m, v (EPI_ADAM stages): {in, out, individual, array}
-  CUtensorMap an[MAX_STAGES];  // new w, m, v: {in, out, cell, array}
-  CUtensorMap nb[MAX_STAGES];  // new bf16 copy
+  // EPI_ADAM: old w, m, v {in, out, individual, array}, new w, m, v {in, out, cell, array}, new
+  // bf16 copy; EPI_DACT: the stored forward output, the deltas (clipped to the stage's rows)
+  CUtensorMap in[MAX_STAGES];
+  CUtensorMap out[MAX_STAGES];
+  CUtensorMap nb[MAX_STAGES];
 };
 
 __device__ __forceinline__ void stage_tile(const GParams& p, int t, int& m0, int& n0, int& n) {
   m0 = (t / p.ntiles) * BM;
   n0 = (t % p.ntiles) * p.BN;
   n = min(p.BN, p.N - n0);
-  n = p.b_mn ? (n + 63) & ~63 : (n + 15) & ~15;
+  n = (n + 63) & ~63;  // B is MN-major: boxes of 64 columns
 }
 
-// 16 accumulator columns of one row: fp32 store, or bf16 delta times the activation
-// derivative (read from the stored forward output). `full` = all 16 columns lie inside N.
-__device__ __forceinline__ void epi16(const GParams& p, const uint32_t (&r)[16], int cell, int m,
-                                      int arow, int col0, bool full, float dlo, bool is_tanh,
-                                      float (&vout)[16], const uint4* xpre = nullptr) {
-  if (p.epi == EPI_F32) {
-    float* C = reinterpret_cast<float*>(p.C) + (int64_t)cell * p.c_cell + (int64_t)m * p.scm;
-    if (p.scn == 1) {
-      if (full) {
-        float4* o = reinterpret_cast<float4*>(C + col0);
+// Weight-gradient tile kept for the caller: fp32 store, a row per thread.
+__device__ __forceinline__ void store_tile(const GParams& p, int cell, int m0, int n0, int n,
+                                           uint32_t tbase, int hf, int row) {
+  const int m = m0 + row, ng = n / 16, half = (ng + 1) / 2;
+  float* C = p.C + (int64_t)cell * p.c_cell + (int64_t)m * p.N + n0;
+  for (int g = hf ? half : 0; g < (hf ? ng : half); ++g) {
+    uint32_t r[16];
+    LIPZ_TMEM_LD16(tbase + g * 16, r);
+    tmem_wait_ld();
+    if (m >= p.M) continue;
+    // (the tensors' rows are multiples of 16 columns: a group lies inside or outside)
+    if (n0 + g * 16 >= p.N) continue;
+    float4* o = reinterpret_cast<float4*>(C + g * 16);
 #pragma unroll
-        for (int u = 0; u < 4; ++u)
-          o[u] = make_float4(__uint_as_float(r[4 * u]), __uint_as_float(r[4 * u + 1]),
-                             __uint_as_float(r[4 * u + 2]), __uint_as_float(r[4 * u + 3]));
-      } else {
-        for (int e = 0; e < 16 && col0 + e < p.N; ++e) C[col0 + e] = __uint_as_float(r[e]);
-      }
-    } else {
-      // transposed output: lanes hold consecutive rows, so each store is one coalesced line
-      const int64_t sc = p.scn;
-      float* o = C + (int64_t)col0 * sc;
-      if (full) {
-#pragma unroll
-        for (int e = 0; e < 16; ++e) o[e * sc] = __uint_as_float(r[e]);
-      } else {
-        for (int e = 0; e < 16 && col0 + e < p.N; ++e) o[e * sc] = __uint_as_float(r[e]);
-      }
-    }
-    return;
-  }
-  bf16* C = reinterpret_cast<bf16*>(p.C) + (int64_t)cell * p.c_cell + (int64_t)m * p.scm;
-  const bf16* X = p.aux + (int64_t)cell * p.aux_cell + (int64_t)arow * p.sxm;
-  if (p.aux_sel) X += (int64_t)(1 + __ldg(&p.aux_sel[cell])) * p.aux_sel_stride;
-  if (p.sxn == 1 && p.scn == 1 && full) {
-    // the caller may have loaded this group's forward output ahead (xpre)
-    const uint4* x4 = xpre ? xpre : reinterpret_cast<const uint4*>(X + col0);
-    const uint4 q0 = x4[0], q1 = x4[1];
-    const uint32_t w[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
-    uint32_t pk[8];
-#pragma unroll
-    for (int e = 0; e < 16; e += 2) {
-      const __nv_bfloat162 y2 = *reinterpret_cast<const __nv_bfloat162*>(&w[e >> 1]);
-      const float y0 = __low2float(y2), y1 = __high2float(y2);
-      const float d0 = is_tanh ? 1.f - y0 * y0 : (y0 > 0.f ? 1.f : dlo);
-      const float d1 = is_tanh ? 1.f - y1 * y1 : (y1 > 0.f ? 1.f : dlo);
-      vout[e] = __uint_as_float(r[e]) * d0;
-      vout[e + 1] = __uint_as_float(r[e + 1]) * d1;
-      __nv_bfloat162 b2 = __floats2bfloat162_rn(vout[e], vout[e + 1]);
-      pk[e >> 1] = *reinterpret_cast<uint32_t*>(&b2);
-    }
-    // rows and column groups are 32-byte aligned here
-    st_global_v8(C + col0, make_uint4(pk[0], pk[1], pk[2], pk[3]),
-                 make_uint4(pk[4], pk[5], pk[6], pk[7]));
-    return;
-  }
-  for (int e = 0; e < 16; ++e) {
-    const int col = col0 + e;
-    if (col >= p.N) break;
-    const float y = __bfloat162float(X[(int64_t)col * p.sxn]);
-    const float d = is_tanh ? 1.f - y * y : (y > 0.f ? 1.f : dlo);
-    vout[e] = __uint_as_float(r[e]) * d;
-    C[(int64_t)col * p.scn] = __float2bfloat16_rn(vout[e]);
+    for (int u = 0; u < 4; ++u)
+      o[u] = make_float4(__uint_as_float(r[4 * u]), __uint_as_float(r[4 * u + 1]),
+                         __uint_as_float(r[4 * u + 2]), __uint_as_float(r[4 * u + 3]));
   }
 }
 
@@ -249,148 +211,105 @@ __device__ __forceinline__ float warp_colsum16(const float (&v)[16], int lane) {
   return a1 + __shfl_xor_sync(0xffffffffu, a1, 1);
 }
 
-// Epilogue of one tile: warp (q, hf) owns TMEM lane quarter q (rows 32q .. 32q + 31) and column
-// half hf. With a bias output, the column sums of the tile's fp32 deltas over the counted rows
-// go through warp_colsum16 and shared memory (one partial per lane quarter, double-buffered by
-// bias tile) and are added in a fixed order into bias_out (stored by the first row tile).
-__device__ __forceinline__ bool epilogue_tile(const GParams& p, int cell, int m0, int n0, int n,
-                                              uint32_t tbase, int hf, int row, int q, int lane,
-                                              float* bpart, int& btile, uint32_t bSum,
-                                              volatile int* abort_flag, int* err) {
-  const int m = m0 + row;
-  const int ng = n / 16;
-  const int half = (ng + 1) / 2;
-  const int g0 = hf ? half : 0, g1 = hf ? ng : half;
-  const bool row_ok = m < p.M;
-  const int arow = m < p.aux_wrap_at ? m : m - p.aux_wrap_sub;
+// Delta epilogue of one tile: warp (q, hf) owns TMEM lane quarter q (rows 32q .. 32q + 31) and
+// column half hf of each chunk. A chunk's stored forward outputs wait in its buffer (chunk number
+// cj of a row half, as in adam_tile) as boxes of 64 columns, 16-byte unit u of box row r at unit
+// u ^ (r & 7); the bf16 deltas go back to the same places and the storer warp writes the boxes
+// out. With a bias output, the column sums of the warp's 32 rows of fp32 deltas go to global
+// memory as partials (before the chunk's arrival, so that the storer's count of the tile covers
+// them). Through per-thread global loads and stores (a row per lane) a 128 x 256 tile took 7 us.
+__device__ __forceinline__ bool delta_tile(const GParams& p, int cell, int m0, int n0, int n,
+                                           uint32_t tbase, int hf, int row, int q, int lane,
+                                           uint32_t sChunk, uint32_t cFull, uint32_t cDone, int& cj,
+                                           volatile int* abort_flag, int* err) {
+  const bool row_ok = m0 + row < p.M;
   const bool is_tanh = p.act == ACT_TANH;
   const float dlo = p.act == ACT_RELU ? 0.f : p.slope;
-  const bool bias = p.epi == EPI_DACT && p.bias_out != nullptr;
-  const bool brow = row_ok && m < p.bias_rows;
-  float* bp = bpart + (btile & 1) * (4 * 256) + q * 256;
-  int gi = g0;
-  // EPI_DACT reads its row's stored forward output: the next pair of groups' values are loaded
-  // while this pair is converted (one memory latency per tile instead of one per pair)
-  const bool pre = p.epi == EPI_DACT && p.sxn == 1 && p.scn == 1 && row_ok;
-  const bf16* X = nullptr;
-  if (pre) {
-    X = p.aux + (int64_t)cell * p.aux_cell + (int64_t)arow * p.sxm;
-    if (p.aux_sel) X += (int64_t)(1 + __ldg(&p.aux_sel[cell])) * p.aux_sel_stride;
-  }
-  // (16 bf16 of a row per 256-bit load: the stored outputs' rows are 32-byte aligned)
-  auto load_pair = [&](int g, uint4(&d)[4]) {
-    const bf16* x = X + n0 + g * 16;
-    if (n0 + g * 16 + 16 <= p.N) {
-      const U8 v = ld_global_v8(x);
-      d[0] = v.a;
-      d[1] = v.b;
-    }
-    if (g + 1 < g1 && n0 + g * 16 + 32 <= p.N) {
-      const U8 v = ld_global_v8(x + 16);
-      d[2] = v.a;
-      d[3] = v.b;
-    }
-  };
-  uint4 xc[4], xn[4];
-  if (pre && gi < g1) load_pair(gi, xc);
-  // two 16-column groups per TMEM load where possible
-  for (; gi + 1 < g1; gi += 2) {
-    if (pre && gi + 2 < g1) load_pair(gi + 2, xn);
-    uint32_t r[32];
-    LIPZ_TMEM_LD32(tbase + gi * 16, r);
-    tmem_wait_ld();
-    const int col0 = n0 + gi * 16;
-    const uint32_t(&ra)[16] = *reinterpret_cast<const uint32_t(*)[16]>(&r[0]);
-    const uint32_t(&rb)[16] = *reinterpret_cast<const uint32_t(*)[16]>(&r[16]);
-    float va[16], vb[16];
+  const int h = row / CHUNK_ROWS, rr = row % CHUNK_ROWS;
+  float* bp = p.bias_part ? p.bias_part + (int64_t)cell * p.bias_cell +
+                                (int64_t)(m0 / BM * 4 + q) * p.N + n0
+                          : nullptr;
+  for (int c0 = 0; c0 < n; c0 += DELTA_COLS, ++cj) {
+    const int bi = (2 * cj + h) % CHUNK_BUFS, use = (2 * cj + h) / CHUNK_BUFS;
+    const int cw = min(DELTA_COLS, n - c0) / 2;  // 64 or 32 columns of this thread
+    if (!mbar_wait_warp(cFull + 8 * bi, (uint32_t)(use & 1), abort_flag, err, 18))
+      return false;
+    const uint32_t rb = sChunk + (uint32_t)(bi * CHUNK_BYTES) + (uint32_t)rr * 128u;
+#pragma unroll 1
+    for (int g = 0; g < cw; g += 32) {
+      const int cl = hf * cw + g;  // first column, within the chunk
+      // the TMEM load is warp-collective: every lane takes part, live row or not
+      uint32_t r[32];
+      LIPZ_TMEM_LD32(tbase + c0 + cl, r);
+      const uint32_t bx = rb + (uint32_t)((cl >> 6) * DELTA_BOX_BYTES);
+      const uint32_t u0 = (uint32_t)(cl & 63) >> 3;
+      uint32_t x[16];
 #pragma unroll
-    for (int e = 0; e < 16; ++e) va[e] = vb[e] = 0.f;
-    if (row_ok) {
-      epi16(p, ra, cell, m, arow, col0, col0 + 16 <= p.N, dlo, is_tanh, va, pre ? &xc[0] : nullptr);
-      if (col0 + 16 < p.N)
-        epi16(p, rb, cell, m, arow, col0 + 16, col0 + 32 <= p.N, dlo, is_tanh, vb,
-              pre ? &xc[2] : nullptr);
-    }
-    if (pre) {
+      for (int u = 0; u < 4; ++u)
+        asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(x[4 * u]), "=r"(x[4 * u + 1]), "=r"(x[4 * u + 2]), "=r"(x[4 * u + 3])
+                     : "r"(bx + (((u0 + u) ^ (uint32_t)(rr & 7)) << 4))
+                     : "memory");
+      tmem_wait_ld();
+      float v[32];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) xc[u] = xn[u];
-    }
-    if (bias) {
-      if (!brow) {
-#pragma unroll
-        for (int e = 0; e < 16; ++e) va[e] = vb[e] = 0.f;
+      for (int e = 0; e < 32; e += 2) {
+        const __nv_bfloat162 y2 = *reinterpret_cast<const __nv_bfloat162*>(&x[e >> 1]);
+        const float y0 = __low2float(y2), y1 = __high2float(y2);
+        const float d0 = is_tanh ? 1.f - y0 * y0 : (y0 > 0.f ? 1.f : dlo);
+        const float d1 = is_tanh ? 1.f - y1 * y1 : (y1 > 0.f ? 1.f : dlo);
+        v[e] = __uint_as_float(r[e]) * d0;
+        v[e + 1] = __uint_as_float(r[e + 1]) * d1;
+        x[e >> 1] = pack_bf16(v[e], v[e + 1]);
       }
-      const float s0 = warp_colsum16(va, lane), s1 = warp_colsum16(vb, lane);
-      if (!(lane & 1)) {
-        bp[gi * 16 + (lane >> 1)] = s0;
-        bp[(gi + 1) * 16 + (lane >> 1)] = s1;
-      }
-    }
-  }
-  if (gi < g1) {
-    uint32_t r[16];
-    LIPZ_TMEM_LD16(tbase + gi * 16, r);
-    tmem_wait_ld();
-    const int col0 = n0 + gi * 16;
-    float va[16];
 #pragma unroll
-    for (int e = 0; e < 16; ++e) va[e] = 0.f;
-    if (row_ok && col0 < p.N)
-      epi16(p, r, cell, m, arow, col0, col0 + 16 <= p.N, dlo, is_tanh, va, pre ? &xc[0] : nullptr);
-    if (bias) {
-      if (!brow) {
+      for (int u = 0; u < 4; ++u)
+        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(
+                         bx + (((u0 + u) ^ (uint32_t)(rr & 7)) << 4)),
+                     "r"(x[4 * u]), "r"(x[4 * u + 1]), "r"(x[4 * u + 2]), "r"(x[4 * u + 3])
+                     : "memory");
+      if (bp) {
+        // rows past the stage's M are not counted
+        const float(&va)[16] = *reinterpret_cast<const float(*)[16]>(&v[0]);
+        const float(&vb)[16] = *reinterpret_cast<const float(*)[16]>(&v[16]);
+        if (!row_ok) {
 #pragma unroll
-        for (int e = 0; e < 16; ++e) va[e] = 0.f;
-      }
-      const float s0 = warp_colsum16(va, lane);
-      if (!(lane & 1)) bp[gi * 16 + (lane >> 1)] = s0;
-    }
-  }
-  if (bias) {
-    // once every epilogue thread has written its partials (mbarrier bSum[btile & 1]), the
-    // lane-quarter-0 warp of each column half adds the four quarters (fixed order) into the
-    // running sum over row tiles. A buffer is rewritten two bias tiles later, which needs the
-    // TMEM region that this tile's readers (those warps included) release after this.
-    const uint32_t bar = bSum + 8 * (btile & 1);
-    mbar_arrive(bar);
-    if (q == 0) {
-      if (!mbar_wait_warp(bar, (uint32_t)((btile >> 1) & 1), abort_flag, err, 20)) return false;
-      const float* b0 = bpart + (btile & 1) * (4 * 256);
-      for (int col = g0 * 16 + lane; col < g1 * 16; col += 32) {
-        const int gc = n0 + col;
-        if (gc < p.N) {
-          const float t = ((b0[col] + b0[256 + col]) + b0[512 + col]) + b0[768 + col];
-          float* o = p.bias_out + (int64_t)cell * p.bias_cell + gc;
-          *o = m0 == 0 ? t : *o + t;
+          for (int e = 0; e < 32; ++e) v[e] = 0.f;
         }
+        const float s0 = warp_colsum16(va, lane), s1 = warp_colsum16(vb, lane);
+        // (even lanes hold the first 16 columns' sums, odd lanes store the others')
+        const int col = c0 + cl + (lane >> 1) + (lane & 1) * 16;
+        if (n0 + col < p.N) bp[col] = lane & 1 ? s1 : s0;
       }
     }
-    ++btile;
+    // make the deltas visible to the TMA store, then hand the chunk to the storer warp
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    mbar_arrive(cDone + 8 * bi);
   }
   return true;
 }
 
 // Adam epilogue of one weight-gradient tile: for each 32-column chunk of the thread's row half
-// h, the warp's 16 columns of its row. Chunk number cj of a half sits in buffer 2 (cj & 1) + h
-// (its (cj >> 1)-th use) as three 64 x 128-byte boxes of old w, m, v in the 128-byte swizzle
+// h, the warp's 16 columns of its row. Chunk number cj of a half, the CTA's chunk 2 cj + h, sits
+// in buffer (2 cj + h) mod CHUNK_BUFS as three 64 x 128-byte boxes of old w, m, v in the 128-byte swizzle
 // (16-byte unit u of box row r at unit u ^ (r & 7)); the new values go back to the same places,
-// the bf16 copy to the buffer's 64-byte-row box, and the loader warp stores the four boxes once
-// the half's 128 threads have arrived on aDone. Returns false on a timeout.
+// the bf16 copy to the buffer's 64-byte-row box, and the storer warp stores the four boxes once
+// the half's 128 threads have arrived on cDone. Returns false on a timeout.
 __device__ __forceinline__ bool adam_tile(const GParams& p, int cell, int m0, int n0,
-                                          uint32_t tbase, int hf, int row, uint32_t sAdam,
-                                          uint32_t aFull, uint32_t aDone, int& cj,
+                                          uint32_t tbase, int hf, int row, uint32_t sChunk,
+                                          uint32_t cFull, uint32_t cDone, int& cj,
                                           volatile int* abort_flag, int* err) {
   const AdamRef& a = p.adam;
   const float4 cf = __ldg(&a.coef[cell]);
   const bool row_ok = m0 + row < p.M;
-  const int h = row / ADAM_ROWS, rr = row % ADAM_ROWS;
+  const int h = row / CHUNK_ROWS, rr = row % CHUNK_ROWS;
   const int nch = (min(p.BN, p.N - n0) + ADAM_COLS - 1) / ADAM_COLS;
   for (int k = 0; k < nch; ++k, ++cj) {
-    const int bi = 2 * (cj & 1) + h;
-    if (!mbar_wait_warp(aFull + 8 * bi, (uint32_t)((cj >> 1) & 1), abort_flag, err, 18))
+    const int bi = (2 * cj + h) % CHUNK_BUFS, use = (2 * cj + h) / CHUNK_BUFS;
+    if (!mbar_wait_warp(cFull + 8 * bi, (uint32_t)(use & 1), abort_flag, err, 18))
       return false;
     const int cl = k * ADAM_COLS + 16 * hf;  // first column of this thread, within the tile
-    const uint32_t bb = sAdam + (uint32_t)(bi * ADAM_BUF_BYTES);
+    const uint32_t bb = sChunk + (uint32_t)(bi * CHUNK_BYTES);
     const uint32_t rb = bb + (uint32_t)rr * 128u;
     // the TMEM load is warp-collective: every lane takes part, live row or not
     uint32_t r[16];
@@ -443,57 +362,153 @@ __device__ __forceinline__ bool adam_tile(const GParams& p, int cell, int m0, in
                    "r"(pack_bf16(w[12], w[13])), "r"(pack_bf16(w[14], w[15]))
                    : "memory");
     }
-    // make the new values visible to the TMA store, then hand the chunk to the loader warp
+    // make the new values visible to the TMA store, then hand the chunk to the storer warp
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    mbar_arrive(aDone + 8 * bi);
+    mbar_arrive(cDone + 8 * bi);
   }
   return true;
 }
 
-template <bool FUSED>
-__global__ void __launch_bounds__(Cfg<FUSED>::THREADS, 1)
-    k_bwd_cells(const __grid_constant__ StageMaps maps, const __grid_constant__ CellPlan cp) {
-  constexpr int STAGES = Cfg<FUSED>::STAGES;
+// Bounded wait until *cnt (counted by other CTAs) reaches `need`.
+__device__ __forceinline__ bool count_wait(const int* cnt, int need, volatile int* abort_flag,
+                                           int* err, int code) {
+  const unsigned long long t0 = globaltimer();
+  for (uint32_t it = 1;; ++it) {
+    int v;
+    asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(cnt) : "memory");
+    if (v >= need) return true;
+    if ((it & 63u) == 0) {
+      if (*abort_flag) return false;
+      if (globaltimer() - t0 > WAIT_NS) {
+        *abort_flag = 1;
+        atomicExch(err, code);
+        return false;
+      }
+    }
+  }
+}
+
+// A cell's ranges entry: epilogue thread et takes elements et, et + 256, ... of the population's
+// ranges laid end to end. A pass's loads are issued before any is used (one memory latency per
+// row tile of partials; element by element, an entry took 14 us). A bias gradient is the sum of
+// its partials: the four lane quarters of a row tile in order, then the row tiles in order.
+__device__ __forceinline__ bool ranges_entry(const CellPlan& cp, const RangeTask& t, int cell,
+                                             int et, int lane, volatile int* abort_flag) {
+  int good = 1;
+  if (lane < t.n_dep)
+    good = count_wait(cp.sync + (int64_t)cell * SYNC_WORDS + t.dep[lane], t.need[lane], abort_flag,
+                      cp.err, 24);
+  if (!__all_sync(0xffffffffu, good)) return false;
+  __syncwarp();
+  const AdamRanges& r = t.r;
+  const int src = __ldg(&r.src[cell]);
+  const float4 cf = __ldg(&r.coef[cell]);
+  if (cp.adam && et == 0) {
+    r.new_p.step[cell] = (int)cf.w;
+    r.new_p.lr[cell] = cf.x;
+  }
+  const int64_t so = (int64_t)src * r.Ps, co = (int64_t)cell * r.Ps;
+  for (int j0 = et; j0 < t.total; j0 += RANGE_REPS * EPI_THREADS) {
+    int64_t k[RANGE_REPS];          // the element's place in the parameter vector
+    const float* part[RANGE_REPS];  // its partials' column, null: none
+    int len[RANGE_REPS], tiles[RANGE_REPS], most = 0;
+    float w[RANGE_REPS], m[RANGE_REPS], v[RANGE_REPS], g[RANGE_REPS];
+#pragma unroll
+    for (int u = 0; u < RANGE_REPS; ++u) {
+      int j = j0 + u * EPI_THREADS;
+      k[u] = -1;
+      part[u] = nullptr;
+      tiles[u] = len[u] = 0;
+      w[u] = m[u] = v[u] = g[u] = 0.f;
+      if (j >= t.total) continue;
+      int q = 0;
+      while (j >= r.len[q]) j -= r.len[q++];
+      k[u] = r.off[q] + j;
+      len[u] = r.len[q];
+      if (t.part[q]) {
+        part[u] = t.part[q] + cell * t.part_cell + j;
+        tiles[u] = t.tiles[q];
+        most = max(most, tiles[u]);
+      } else if (cp.adam) {
+        g[u] = t.grad[co + k[u]];
+      }
+      if (cp.adam) {
+        w[u] = r.old_p.w[so + k[u]];
+        m[u] = r.old_p.m[so + k[u]];
+        v[u] = r.old_p.v[so + k[u]];
+      }
+    }
+    for (int i = 0; i < most; ++i) {
+      float a[RANGE_REPS][4];
+#pragma unroll
+      for (int u = 0; u < RANGE_REPS; ++u)
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          a[u][q] = i < tiles[u] ? __ldcg(part[u] + (int64_t)(4 * i + q) * len[u]) : 0.f;
+#pragma unroll
+      for (int u = 0; u < RANGE_REPS; ++u) {
+        const float s = ((a[u][0] + a[u][1]) + a[u][2]) + a[u][3];
+        if (i < tiles[u]) g[u] = i ? g[u] + s : s;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < RANGE_REPS; ++u) {
+      if (k[u] < 0) continue;
+      if (!cp.adam) {
+        if (part[u]) t.grad[co + k[u]] = g[u];
+        continue;
+      }
+      adam_elem(w[u], m[u], v[u], g[u], cp.beta1, cp.beta2, cf.x, cf.y, cf.z, cp.eps);
+      r.new_p.w[co + k[u]] = w[u];
+      r.new_p.m[co + k[u]] = m[u];
+      r.new_p.v[co + k[u]] = v[u];
+      if (r.new_p.wb) r.new_p.wb[co + k[u]] = __float2bfloat16_rn(w[u]);
+    }
+  }
+  return true;
+}
+
+__global__ void __launch_bounds__(THREADS, 1)
+    k_bwd(const __grid_constant__ StageMaps maps, const __grid_constant__ CellPlan cp) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   uint8_t* gbase = smem_raw + (base - raw);
-  const uint32_t sAdam = base + STAGES * STAGE_BYTES;  // [ADAM_BUFS][w | m | v] chunks
-  uint8_t* misc = gbase + STAGES * STAGE_BYTES + Cfg<FUSED>::ADAM_BUFS * ADAM_BUF_BYTES;
-  const uint32_t bFull = smem_u32(misc), bEmpty = bFull + 8 * STAGES;
-  const uint32_t bAcc = bEmpty + 8 * STAGES, bReg = bAcc + 16, bFinal = bReg + 16;
-  const uint32_t bEpi = bFinal + 8;    // [2], alternating by tile
-  const uint32_t aFull = bEpi + 16;   // [4] Adam chunk buffers: old values landed
-  const uint32_t aDone = aFull + 32;  // [4] new values written back by the epilogue half
-  const uint32_t bSum = aDone + 32;   // [2] bias partial sums written, by bias tile
-  const uint32_t aFree = bSum + 16;   // [4] the stores have read the buffer
-  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(misc + 224);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 228);
-  volatile int* done_tiles = reinterpret_cast<volatile int*>(misc + 232);
-  float* bpart = reinterpret_cast<float*>(misc + 256);  // bias partial sums
+  const uint32_t sChunk = base + RING_BYTES;
+  uint8_t* misc = gbase + RING_BYTES + CHUNK_BUFS * CHUNK_BYTES;
+  const uint32_t bFull = smem_u32(misc), bEmpty = bFull + 8 * MAX_OPS;
+  const uint32_t bAcc = bEmpty + 8 * MAX_OPS, bReg = bAcc + 16, bFinal = bReg + 16;
+  const uint32_t cFull = bFinal + 8;          // [CHUNK_BUFS] the chunk's old values landed
+  const uint32_t cDone = cFull + 8 * CHUNK_BUFS;  // new values written by the epilogue half
+  const uint32_t cFree = cDone + 8 * CHUNK_BUFS;  // the stores have read the buffer
+  const uint32_t tFull = cFree + 8 * CHUNK_BUFS;  // [RING] a claimed tile is in the ring slot
+  const uint32_t tEmpty = tFull + 8 * RING;  // [RING] every role has read the slot
+  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(misc + 384);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 388);
+  volatile int2* ring = reinterpret_cast<volatile int2*>(misc + 400);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) {
+    for (int s = 0; s < MAX_OPS; ++s) {
       mbar_init(bFull + 8 * s, 1);
       mbar_init(bEmpty + 8 * s, 1);
     }
-    mbar_init(bAcc, 1);
-    mbar_init(bAcc + 8, 1);
-    mbar_init(bReg, EPI_THREADS);
-    mbar_init(bReg + 8, EPI_THREADS);
-    mbar_init(bFinal, 1);
-    mbar_init(bEpi, EPI_THREADS);
-    mbar_init(bEpi + 8, EPI_THREADS);
-    for (int b = 0; b < Cfg<FUSED>::ADAM_BUFS; ++b) {
-      mbar_init(aFull + 8 * b, 1);
-      mbar_init(aDone + 8 * b, EPI_THREADS / 2);
-      mbar_init(aFree + 8 * b, 1);
+    for (int r = 0; r < 2; ++r) {
+      mbar_init(bAcc + 8 * r, 1);
+      mbar_init(bReg + 8 * r, EPI_THREADS);
     }
-    mbar_init(bSum, EPI_THREADS);
-    mbar_init(bSum + 8, EPI_THREADS);
+    mbar_init(bFinal, 1);
+    for (int b = 0; b < CHUNK_BUFS; ++b) {
+      mbar_init(cFull + 8 * b, 1);
+      mbar_init(cDone + 8 * b, EPI_THREADS / 2);
+      mbar_init(cFree + 8 * b, 1);
+    }
+    for (int b = 0; b < RING; ++b) {
+      mbar_init(tFull + 8 * b, 1);
+      // readers: the MMA thread, one lane of each epilogue warp, the chunk loader and storer
+      mbar_init(tEmpty + 8 * b, 1 + NUM_EPI_WARPS + 2);
+    }
     *abort_flag = 0;
-    *done_tiles = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -507,91 +522,117 @@ __global__ void __launch_bounds__(Cfg<FUSED>::THREADS, 1)
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   int* err = cp.err;
+  int* const claim = cp.sync + (int64_t)cp.cells * SYNC_WORDS;
+  const int n_ops = cp.n_ops, op_bytes = cp.op_bytes;  // operand ring: stages, bytes of each
   // the set-up above touched no global memory: from here on the previous kernel's results
   // are needed (programmatic dependent launch)
   pdl_wait();
 
+  // The next claimed tile for a role of one thread (the epilogue has its own, warp-wide): waits
+  // for ring slot i, returns its entry {cell, stage << 16 | tile} and releases the slot. False:
+  // the list is done or the CTA gave up.
+  auto next_tile = [&](int i, int2& e) -> bool {
+    const int s = i % RING;
+    if (!mbar_wait(tFull + 8 * s, (uint32_t)((i / RING) & 1), abort_flag, err, 22)) return false;
+    e.x = ring[s].x;
+    e.y = ring[s].y;
+    mbar_arrive(tEmpty + 8 * s);
+    return e.x >= 0;
+  };
+
   if (warp == 0) {
     if (lane == 0) {
-      int issued[STAGES] = {};
+      int issued[MAX_OPS] = {};
       bool ok = true;
       int stage = 0;
       uint32_t phase = 0;
-      int cells_done = 0;
-      for (int cell = blockIdx.x; cell < cp.cells && ok; cell += gridDim.x, ++cells_done) {
-        for (int si = 0; si < cp.n_stages && ok; ++si) {
-          const GParams& p = cp.st[si].p;
-          const int dep = cp.st[si].dep;
-          if (dep >= 0) {
-            // the stage reads the output of stage `dep` of this cell: wait for its last tile
-            const int need = cells_done * cp.pub_per_cell + cp.pub_end[dep];
-            const unsigned long long t0 = globaltimer();
-            uint32_t it = 0;
-            while (*done_tiles < need) {
-              if ((++it & 255u) == 0) {
-                if (*abort_flag) {
-                  ok = false;
-                  break;
-                }
-                if (globaltimer() - t0 > WAIT_NS) {
-                  *abort_flag = 1;
-                  atomicExch(err, 16);
-                  ok = false;
-                  break;
-                }
-              }
-            }
-            if (!ok) break;
-            __threadfence_block();
+      for (int i = 0; ok; ++i) {
+        const int idx = atomicAdd(claim, 1);
+        const int2 e = idx < cp.n_list ? __ldg(&cp.list[idx]) : make_int2(-1, 0);
+        const int s = i % RING;
+        if (i >= RING && !mbar_wait(tEmpty + 8 * s, (uint32_t)((i / RING - 1) & 1), abort_flag,
+                                    err, 23)) {
+          ok = false;
+          break;
+        }
+        ring[s].x = e.x;
+        ring[s].y = e.y;
+        mbar_arrive(tFull + 8 * s);
+        if (e.x < 0) break;
+        const int cell = e.x, si = e.y >> 16, t = e.y & 0xFFFF;
+        if (si >= RANGES_STAGE) continue;
+        const GParams& p = cp.st[si].p;
+        const int dep = cp.st[si].dep;
+        const CUtensorMap* mA = &maps.a[si];
+        const CUtensorMap* mB = &maps.b[si];
+        const int za = p.a_sel ? __ldg(&p.a_sel[cell]) : cell;
+        const int zb = p.b_sel ? __ldg(&p.b_sel[cell]) : cell;
+        const int fake_slot = p.ksplit > 0 ? 1 + __ldg(&p.b_slot_sel[cell]) : 0;
+        const uint32_t bytes = (uint32_t)(A_BYTES + p.BN * 128);
+        int m0, n0, n;
+        stage_tile(p, t, m0, n0, n);
+        auto load_a = [&](int kc, int st) {
+          const bool part1 = p.ksplit > 0 && kc >= p.ksplit;
+          const int ka = (part1 ? kc - p.ksplit : kc) * BK + (part1 ? p.a_k_off1 : 0);
+          const uint32_t sA = base + st * op_bytes, full = bFull + 8 * st;
+          if (p.a_mn) {
+            tma_load_3d(sA, mA, full, m0, ka, za);
+            tma_load_3d(sA + MN_BOX_BYTES, mA, full, m0 + 64, ka, za);
+          } else {
+            tma_load_3d(sA, mA, full, ka, p.a_row0 + m0, za);
           }
-          const CUtensorMap* mA = &maps.a[si];
-          const CUtensorMap* mB = &maps.b[si];
-          const int za = p.a_sel ? __ldg(&p.a_sel[cell]) : cell;
-          const int zb = p.b_sel ? __ldg(&p.b_sel[cell]) : cell;
-          const uint32_t b_bytes =
-              p.b_mn ? (uint32_t)((p.BN / 64) * MN_BOX_BYTES) : (uint32_t)(p.BN * 128);
-          const int nt = p.mtiles * p.ntiles;
-          for (int t = 0; t < nt && ok; ++t) {
-            int m0, n0, n;
-            stage_tile(p, t, m0, n0, n);
-            for (int kc = 0; kc < p.kchunks; ++kc) {
-              if (!mbar_wait(bEmpty + 8 * stage, phase ^ 1u, abort_flag, err, 11)) {
-                ok = false;
-                break;
-              }
-              const uint32_t full = bFull + 8 * stage;
-              mbar_expect_tx(full, (uint32_t)A_BYTES + b_bytes);
-              const uint32_t sA = base + stage * STAGE_BYTES, sB = sA + A_BYTES;
-              const bool part1 = p.ksplit > 0 && kc >= p.ksplit;
-              const int kk = part1 ? kc - p.ksplit : kc;
-              const int ka = kk * BK + (part1 ? p.a_k_off1 : 0);
-              if (p.a_mn) {
-                tma_load_3d(sA, mA, full, m0, ka, za);
-                tma_load_3d(sA + MN_BOX_BYTES, mA, full, m0 + 64, ka, za);
-              } else {
-                tma_load_3d(sA, mA, full, ka, p.a_row0 + m0, za);
-              }
-              if (p.ksplit > 0) {
-                const int slot = part1 ? 1 + __ldg(&p.b_slot_sel[cell]) : 0;
-                for (int i = 0; i < p.BN / 64; ++i)
-                  tma_load_4d(sB + i * MN_BOX_BYTES, mB, full, n0 + 64 * i, kk * BK, slot, cell);
-              } else if (p.b_mn) {
-                for (int i = 0; i < p.BN / 64; ++i)
-                  tma_load_3d(sB + i * MN_BOX_BYTES, mB, full, n0 + 64 * i, kc * BK, zb);
-              } else {
-                tma_load_3d(sB, mB, full, kc * BK, p.b_row0 + n0, zb);
-              }
-              issued[stage]++;
-              if (++stage == STAGES) {
-                stage = 0;
-                phase ^= 1u;
-              }
-            }
+        };
+        auto load_b = [&](int kc, int st) {
+          const uint32_t sB = base + st * op_bytes + A_BYTES, full = bFull + 8 * st;
+          mbar_expect_tx(full, bytes);
+          if (p.ksplit > 0) {
+            const bool part1 = kc >= p.ksplit;
+            const int kb = (part1 ? kc - p.ksplit : kc) * BK, slot = part1 ? fake_slot : 0;
+            for (int u = 0; u < p.BN / 64; ++u)
+              tma_load_4d(sB + u * MN_BOX_BYTES, mB, full, n0 + 64 * u, kb, slot, cell);
+          } else {
+            for (int u = 0; u < p.BN / 64; ++u)
+              tma_load_3d(sB + u * MN_BOX_BYTES, mB, full, n0 + 64 * u, kc * BK, zb);
           }
+          issued[st]++;
+        };
+        // a tile that reads the output of the cell's stage `dep` (its A, written by any CTA)
+        // loads its first chunks' B, which does not depend on it, before it waits
+        const int ahead = dep >= 0 ? min(p.kchunks, n_ops) : 0;
+        const int stage0 = stage;
+        for (int kc = 0; kc < p.kchunks && ok; ++kc) {
+          if (kc == ahead && ahead > 0) {
+            if (!count_wait(cp.sync + (int64_t)cell * SYNC_WORDS + dep, cp.st[si].dep_need,
+                            abort_flag, err, 16)) {
+              ok = false;
+              break;
+            }
+            asm volatile("fence.proxy.async;" ::: "memory");
+            for (int u = 0; u < ahead; ++u) load_a(u, (stage0 + u) % n_ops);
+          }
+          if (!mbar_wait(bEmpty + 8 * stage, phase ^ 1u, abort_flag, err, 11)) {
+            ok = false;
+            break;
+          }
+          load_b(kc, stage);
+          if (kc >= ahead) load_a(kc, stage);
+          if (++stage == n_ops) {
+            stage = 0;
+            phase ^= 1u;
+          }
+        }
+        if (ok && ahead == p.kchunks) {
+          if (!count_wait(cp.sync + (int64_t)cell * SYNC_WORDS + dep, cp.st[si].dep_need,
+                          abort_flag, err, 16)) {
+            ok = false;
+            break;
+          }
+          asm volatile("fence.proxy.async;" ::: "memory");
+          for (int u = 0; u < ahead; ++u) load_a(u, (stage0 + u) % n_ops);
         }
       }
       if (!ok) {
-        for (int s = 0; s < STAGES; ++s)
+        for (int s = 0; s < MAX_OPS; ++s)
           if (issued[s] > 0) {
             volatile int never = 0;
             mbar_wait(bFull + 8 * s, (uint32_t)((issued[s] - 1) & 1), &never, err, 11);
@@ -604,214 +645,178 @@ __global__ void __launch_bounds__(Cfg<FUSED>::THREADS, 1)
       uint32_t phase = 0;
       bool ok = true;
       int lt = 0;
-      for (int cell = blockIdx.x; cell < cp.cells && ok; cell += gridDim.x) {
-        for (int si = 0; si < cp.n_stages && ok; ++si) {
-          const GParams& p = cp.st[si].p;
-          const int nt = p.mtiles * p.ntiles;
-          for (int t = 0; t < nt && ok; ++t, ++lt) {
-            int m0, n0, n;
-            stage_tile(p, t, m0, n0, n);
-            const int R = lt & 1, use = lt >> 1;
-            if (use > 0 &&
-                !mbar_wait(bReg + 8 * R, (uint32_t)((use - 1) & 1), abort_flag, err, 15)) {
-              ok = false;
-              break;
-            }
-            tc_fence_after();
-            const uint32_t d = tmem + (uint32_t)(R * 256);
-            const uint32_t idesc = idesc_bf16_major(BM, n, p.a_mn, p.b_mn);
-            for (int kc = 0; kc < p.kchunks; ++kc) {
-              if (!mbar_wait(bFull + 8 * stage, phase, abort_flag, err, 12)) {
-                ok = false;
-                break;
-              }
-              tc_fence_after();
-              const uint32_t sA = base + stage * STAGE_BYTES, sB = sA + A_BYTES;
+      int2 e;
+      for (int i = 0; ok && next_tile(i, e); ++i) {
+        const int si = e.y >> 16;
+        if (si >= RANGES_STAGE) continue;
+        const GParams& p = cp.st[si].p;
+        int m0, n0, n;
+        stage_tile(p, e.y & 0xFFFF, m0, n0, n);
+        const int R = lt & 1, use = lt >> 1;
+        if (use > 0 && !mbar_wait(bReg + 8 * R, (uint32_t)((use - 1) & 1), abort_flag, err, 15)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        const uint32_t d = tmem + (uint32_t)(R * 256);
+        const uint32_t idesc = idesc_bf16_major(BM, n, p.a_mn, 1);
+        for (int kc = 0; kc < p.kchunks; ++kc) {
+          if (!mbar_wait(bFull + 8 * stage, phase, abort_flag, err, 12)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint32_t sA = base + stage * op_bytes, sB = sA + A_BYTES;
 #pragma unroll
-              for (int kk = 0; kk < BK / 16; ++kk) {
-                const uint64_t ad = p.a_mn ? sw128_mn_desc(sA + kk * 2048, MN_BOX_BYTES)
-                                           : sw128_desc(sA + kk * 32);
-                const uint64_t bd = p.b_mn ? sw128_mn_desc(sB + kk * 2048, MN_BOX_BYTES)
-                                           : sw128_desc(sB + kk * 32);
-                tc_mma(d, ad, bd, idesc, (kc | kk) != 0 ? 1u : 0u);
-              }
-              tc_commit(bEmpty + 8 * stage);
-              if (++stage == STAGES) {
-                stage = 0;
-                phase ^= 1u;
-              }
-            }
-            if (!ok) break;
-            tc_commit(bAcc + 8 * R);
+          for (int kk = 0; kk < BK / 16; ++kk) {
+            const uint64_t ad = p.a_mn ? sw128_mn_desc(sA + kk * 2048, MN_BOX_BYTES)
+                                       : sw128_desc(sA + kk * 32);
+            const uint64_t bd = sw128_mn_desc(sB + kk * 2048, MN_BOX_BYTES);
+            tc_mma(d, ad, bd, idesc, (kc | kk) != 0 ? 1u : 0u);
+          }
+          tc_commit(bEmpty + 8 * stage);
+          if (++stage == n_ops) {
+            stage = 0;
+            phase ^= 1u;
           }
         }
+        if (!ok) break;
+        tc_commit(bAcc + 8 * R);
+        ++lt;
       }
       tc_commit(bFinal);
       volatile int never = 0;
       mbar_wait(bFinal, 0u, &never, err, 14);
     }
-  } else if (FUSED && warp >= 2 + NUM_EPI_WARPS) {
-    // ===== Adam stream: the old w, m, v of every chunk of every EPI_ADAM tile, in tile order,
-    // into the four buffers in turn, and the new w, m, v and bf16 copy back out. A tiled TMA
+  } else if (warp >= 2 + NUM_EPI_WARPS) {
+    // ===== chunk stream: the epilogue's inputs of every chunk of every EPI_ADAM and EPI_DACT
+    // tile, in tile order, into the four buffers in turn, and its results back out. A tiled TMA
     // operation holds its issuing thread for about 0.2 us, so two warps share the work:
     //   loader: a chunk's load, once the storer has released the chunk's buffer;
-    //   storer: a chunk's two stores once its epilogue half is done, then, when the stores
-    //           have read the buffer, its release to the loader (releasing it one chunk later,
-    //           to keep a store group in flight, was slower: the stream is bound by the
-    //           latency of each buffer's round trip). =====
+    //   storer: a chunk's stores once its epilogue half is done, then, when the stores have read
+    //           the buffer, its release to the loader (releasing it one chunk later, to keep a
+    //           store group in flight, was slower: the stream is bound by the latency of each
+    //           buffer's round trip); after a delta tile's last chunk, once its stores are
+    //           written, it counts the tile for the tiles that read it. =====
     const bool storer = warp == 3 + NUM_EPI_WARPS;
     if (lane == 0) {
-      constexpr int NB = Cfg<FUSED>::ADAM_BUFS > 0 ? Cfg<FUSED>::ADAM_BUFS : 1;
-      int buf = 0, uses[NB] = {};
+      int buf = 0, uses[CHUNK_BUFS] = {};
       bool ok = true;
-      for (int cell = blockIdx.x; cell < cp.cells && ok; cell += gridDim.x) {
-        for (int si = 0; si < cp.n_stages && ok; ++si) {
-          const GParams& p = cp.st[si].p;
-          if (p.epi != EPI_ADAM) continue;
-          const int zi = __ldg(&p.adam.src[cell]);
-          const int nt = p.mtiles * p.ntiles;
-          for (int t = 0; t < nt && ok; ++t) {
-            const int m0 = (t / p.ntiles) * BM, n0 = (t % p.ntiles) * p.BN;
-            const int nch = (min(p.BN, p.N - n0) + ADAM_COLS - 1) / ADAM_COLS;
-            for (int k = 0; k < 2 * nch; ++k) {
-              const int x0 = n0 + (k >> 1) * ADAM_COLS, y0 = m0 + (k & 1) * ADAM_ROWS;
-              const uint32_t bb = sAdam + (uint32_t)(buf * ADAM_BUF_BYTES);
-              if (storer) {
-                // the (uses[buf] + 1)-th chunk of this buffer is written back
-                if (!mbar_wait(aDone + 8 * buf, (uint32_t)(uses[buf] & 1), abort_flag, err, 19)) {
-                  ok = false;
-                  break;
-                }
-                tma_store_4d(&maps.an[si], bb, x0, y0, cell, 0);
-                tma_store_3d(&maps.nb[si], bb + 3 * ADAM_ARRAY_BYTES, x0, y0, cell);
-                bulk_commit();
-                bulk_wait_read<0>();  // the stores have read the buffer: it may be refilled
-                mbar_arrive(aFree + 8 * buf);
-              } else {
-                if (uses[buf] > 0 && !mbar_wait(aFree + 8 * buf, (uint32_t)((uses[buf] - 1) & 1),
-                                                abort_flag, err, 21)) {
-                  ok = false;
-                  break;
-                }
-                const uint32_t full = aFull + 8 * buf;
-                mbar_expect_tx(full, (uint32_t)(3 * ADAM_ARRAY_BYTES));
-                tma_load_4d(bb, &maps.ao[si], full, x0, y0, zi, 0);
+      int2 e;
+      for (int i = 0; ok && next_tile(i, e); ++i) {
+        const int cell = e.x, si = e.y >> 16;
+        if (si >= RANGES_STAGE) continue;
+        const GParams& p = cp.st[si].p;
+        if (p.epi == EPI_F32) continue;
+        const bool adam = p.epi == EPI_ADAM;
+        int m0, n0, n;
+        stage_tile(p, e.y & 0xFFFF, m0, n0, n);
+        const int cols = adam ? ADAM_COLS : DELTA_COLS;
+        const int nch = ((adam ? min(p.BN, p.N - n0) : n) + cols - 1) / cols;
+        const int zi = adam ? __ldg(&p.adam.src[cell]) : cell;
+        const int slot = !adam && p.x_slot ? 1 + __ldg(&p.x_slot[cell]) : -1;
+        for (int k = 0; k < 2 * nch; ++k) {
+          const int x0 = n0 + (k >> 1) * cols, y0 = m0 + (k & 1) * CHUNK_ROWS;
+          const int boxes = adam ? 1 : min(2, (n - (k >> 1) * cols) / 64);
+          const uint32_t bb = sChunk + (uint32_t)(buf * CHUNK_BYTES);
+          if (storer) {
+            // the (uses[buf] + 1)-th chunk of this buffer is written back
+            if (!mbar_wait(cDone + 8 * buf, (uint32_t)(uses[buf] & 1), abort_flag, err, 19)) {
+              ok = false;
+              break;
+            }
+            if (adam) {
+              tma_store_4d(&maps.out[si], bb, x0, y0, cell, 0);
+              tma_store_3d(&maps.nb[si], bb + 3 * ADAM_ARRAY_BYTES, x0, y0, cell);
+            } else {
+              for (int u = 0; u < boxes; ++u)
+                tma_store_3d(&maps.out[si], bb + u * DELTA_BOX_BYTES, x0 + 64 * u, y0, cell);
+            }
+            bulk_commit();
+            bulk_wait_read<0>();  // the stores have read the buffer: it may be refilled
+            mbar_arrive(cFree + 8 * buf);
+          } else {
+            if (uses[buf] > 0 && !mbar_wait(cFree + 8 * buf, (uint32_t)((uses[buf] - 1) & 1),
+                                            abort_flag, err, 21)) {
+              ok = false;
+              break;
+            }
+            const uint32_t full = cFull + 8 * buf;
+            if (adam) {
+              mbar_expect_tx(full, (uint32_t)(3 * ADAM_ARRAY_BYTES));
+              tma_load_4d(bb, &maps.in[si], full, x0, y0, zi, 0);
+            } else {
+              mbar_expect_tx(full, (uint32_t)(boxes * DELTA_BOX_BYTES));
+              for (int u = 0; u < boxes; ++u) {
+                const uint32_t d = bb + u * DELTA_BOX_BYTES;
+                if (slot >= 0)
+                  tma_load_4d(d, &maps.in[si], full, x0 + 64 * u, p.x_row0 + y0, slot, cell);
+                else
+                  tma_load_3d(d, &maps.in[si], full, x0 + 64 * u, p.x_row0 + y0, cell);
               }
-              uses[buf]++;
-              if (++buf == NB) buf = 0;
             }
           }
+          uses[buf]++;
+          if (++buf == CHUNK_BUFS) buf = 0;
+        }
+        if (storer && !adam && ok) {
+          bulk_wait_all();
+          __threadfence();
+          asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(
+                           cp.sync + (int64_t)cell * SYNC_WORDS + si)
+                       : "memory");
         }
       }
       if (storer) {
         bulk_wait_all();
-      } else if (!ok) {
+      } else if (*abort_flag) {
         // loads issued here land on this CTA's barriers: wait for them before it leaves
-        for (int b = 0; b < NB; ++b)
+        for (int b = 0; b < CHUNK_BUFS; ++b)
           if (uses[b] > 0) {
             volatile int never = 0;
-            mbar_wait(aFull + 8 * b, (uint32_t)((uses[b] - 1) & 1), &never, err, 19);
+            mbar_wait(cFull + 8 * b, (uint32_t)((uses[b] - 1) & 1), &never, err, 19);
           }
       }
     }
   } else {
     const int ew = warp - 2, q = warp & 3, hf = ew >> 2;
     const int row = q * 32 + lane;
-    bool ok = true;
-    int lt = 0, pub = 0;
-    int cj = 0;  // Adam chunks of this thread's row half so far
-    int btile = 0;  // bias-summing tiles so far
-    for (int cell = blockIdx.x; cell < cp.cells; cell += gridDim.x) {
-      for (int si = 0; si < cp.n_stages && ok; ++si) {
-        const GParams& p = cp.st[si].p;
-        const bool publish = cp.st[si].publish != 0;
-        const int nt = p.mtiles * p.ntiles;
-        for (int t = 0; t < nt; ++t, ++lt) {
-          int m0, n0, n;
-          stage_tile(p, t, m0, n0, n);
-          const int R = lt & 1, use = lt >> 1;
-          if (!mbar_wait_warp(bAcc + 8 * R, (uint32_t)(use & 1), abort_flag, err, 13)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(R * 256);
-          if constexpr (FUSED) {
-            if (p.epi == EPI_ADAM) {
-              if (!adam_tile(p, cell, m0, n0, tbase, hf, row, sAdam, aFull, aDone, cj,
-                             abort_flag, err)) {
-                ok = false;
-                break;
-              }
-            } else if (!epilogue_tile(p, cell, m0, n0, n, tbase, hf, row, q, lane, bpart, btile,
-                                      bSum, abort_flag, err)) {
-              ok = false;
-              break;
-            }
-          } else if (!epilogue_tile(p, cell, m0, n0, n, tbase, hf, row, q, lane, bpart, btile,
-                                    bSum, abort_flag, err)) {
-            ok = false;
-            break;
-          }
-          if (publish) {
-            // publish the tile's global stores to the async proxy (a later stage loads them by
-            // TMA). The arrival on bEpi[pub & 1] comes before the arrival on bReg, so no thread
-            // can reach the next-but-one published tile (same barrier) before every thread
-            // has arrived here.
-            asm volatile("fence.proxy.async;" ::: "memory");
-            mbar_arrive(bEpi + 8 * (pub & 1));
-          }
-          tc_fence_before();
-          mbar_arrive(bReg + 8 * R);
-          if (publish) {
-            if (warp == 2) {
-              // one warp counts the tile once all epilogue threads have published their stores
-              if (!mbar_wait_warp(bEpi + 8 * (pub & 1), (uint32_t)((pub >> 1) & 1), abort_flag,
-                                  err, 17)) {
-                ok = false;
-                break;
-              }
-              if (lane == 0) {
-                __threadfence_block();
-                *done_tiles = pub + 1;
-              }
-              __syncwarp();
-            }
-            ++pub;
-          }
-        }
-      }
-      if (FUSED && cp.has_ranges) {
-        // the cell's last tile is done by every epilogue thread (its bias sums are in gG / gD):
-        // the remaining Adam ranges of the cell, the eight warps together (they leave
-        // together when any of them gave up)
-        if (epi_any(!ok)) {
-          ok = false;
+    int lt = 0;
+    int cj = 0;  // chunks of this thread's row half so far
+    for (int i = 0;; ++i) {
+      const int s = i % RING;
+      if (!mbar_wait_warp(tFull + 8 * s, (uint32_t)((i / RING) & 1), abort_flag, err, 22)) break;
+      __syncwarp();
+      const int cell = ring[s].x, w = ring[s].y;
+      __syncwarp();
+      if (lane == 0) mbar_arrive(tEmpty + 8 * s);
+      if (cell < 0) break;
+      const int si = w >> 16;
+      if (si >= RANGES_STAGE) {
+        if (!ranges_entry(cp, cp.rt[si - RANGES_STAGE], cell, threadIdx.x - 64, lane, abort_flag))
           break;
-        }
-        const int et = threadIdx.x - 64;
-        for (int pp = 0; pp < 2; ++pp) {
-          const AdamRanges& r = pp ? cp.rd : cp.rg;
-          const int s = __ldg(&r.src[cell]);
-          const float4 cf = __ldg(&r.coef[cell]);
-          if (et == 0) {
-            r.new_p.step[cell] = (int)cf.w;
-            r.new_p.lr[cell] = cf.x;
-          }
-          const int64_t so = (int64_t)s * r.Ps, co = (int64_t)cell * r.Ps;
-          for (int q = 0; q < r.n; ++q)
-            for (int i = et; i < r.len[q]; i += EPI_THREADS) {
-              const int64_t k = r.off[q] + i;
-              float w = r.old_p.w[so + k], m = r.old_p.m[so + k], v = r.old_p.v[so + k];
-              adam_elem(w, m, v, r.grad[co + k], cp.beta1, cp.beta2, cf.x, cf.y, cf.z, cp.eps);
-              r.new_p.w[co + k] = w;
-              r.new_p.m[co + k] = m;
-              r.new_p.v[co + k] = v;
-              if (r.new_p.wb) r.new_p.wb[co + k] = __float2bfloat16_rn(w);
-            }
-        }
+        continue;
       }
-      if (!ok) break;
+      const GParams& p = cp.st[si].p;
+      int m0, n0, n;
+      stage_tile(p, w & 0xFFFF, m0, n0, n);
+      const int R = lt & 1, use = lt >> 1;
+      if (!mbar_wait_warp(bAcc + 8 * R, (uint32_t)(use & 1), abort_flag, err, 13)) break;
+      tc_fence_after();
+      const uint32_t tbase = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(R * 256);
+      if (p.epi == EPI_ADAM) {
+        if (!adam_tile(p, cell, m0, n0, tbase, hf, row, sChunk, cFull, cDone, cj, abort_flag, err))
+          break;
+      } else if (p.epi == EPI_DACT) {
+        if (!delta_tile(p, cell, m0, n0, n, tbase, hf, row, q, lane, sChunk, cFull, cDone, cj,
+                        abort_flag, err))
+          break;
+      } else {
+        store_tile(p, cell, m0, n0, n, tbase, hf, row);
+      }
+      tc_fence_before();
+      mbar_arrive(bReg + 8 * R);
+      ++lt;
     }
   }
   __syncwarp();
@@ -869,7 +874,7 @@ bool map4f(CUtensorMap* m, const float* base, uint64_t inner, uint64_t rows, uin
            uint64_t depth_elems, uint64_t part, std::string* msg) {
   cuuint64_t dims[4] = {inner, rows, depth, 3};
   cuuint64_t strides[3] = {inner * 4, depth_elems * 4, part * 4};
-  cuuint32_t box[4] = {(cuuint32_t)tcb::ADAM_COLS, (cuuint32_t)tcb::ADAM_ROWS, 1, 3};
+  cuuint32_t box[4] = {(cuuint32_t)tcb::ADAM_COLS, (cuuint32_t)tcb::CHUNK_ROWS, 1, 3};
   cuuint32_t es[4] = {1, 1, 1, 1};
   CUresult r = g_enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<float*>(base), dims,
                      strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
@@ -887,7 +892,7 @@ bool map3b_rows(CUtensorMap* m, const bf16* base, uint64_t inner, uint64_t rows,
                 uint64_t depth_elems, std::string* msg) {
   cuuint64_t dims[3] = {inner, rows, depth};
   cuuint64_t strides[2] = {inner * 2, depth_elems * 2};
-  cuuint32_t box[3] = {(cuuint32_t)tcb::ADAM_COLS, (cuuint32_t)tcb::ADAM_ROWS, 1};
+  cuuint32_t box[3] = {(cuuint32_t)tcb::ADAM_COLS, (cuuint32_t)tcb::CHUNK_ROWS, 1};
   cuuint32_t es[3] = {1, 1, 1};
   CUresult r = g_enc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<bf16*>(base), dims,
                      strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
@@ -917,26 +922,47 @@ bool map4(CUtensorMap* m, const void* base, uint64_t inner, uint64_t rows, uint6
   return true;
 }
 
-struct Gemm {
-  CUtensorMap a, b;
-  CUtensorMap ao;      // old w, m, v of the tensor (fused Adam), by individual and array
-  CUtensorMap an, nb;  // new w, m, v by cell and array; new bf16 copy by cell
-  tcb::GParams p;
-  int grid;
-};
-
 }  // namespace
 
 struct TcbPlan {
-  // order of execution: D1, dW2d, A3, dW1d, A2, dW3g, A1, dW2g, dW1g
-  Gemm g[9];
-  int n;
   int* err;
-  tcb::StageMaps maps;  // the same nine products as one per-cell kernel
+  int2* list;     // the grid's tiles in claim order
+  float* bpart;   // bias-gradient partial sums per cell, stage and row tile
+  tcb::StageMaps maps;
   tcb::CellPlan cells;
-  int grid_cells;
-  bool fused;  // weight tensors take their Adam step in the backward's epilogue
+  int grid;
 };
+
+namespace {
+void free_plan(TcbPlan* P) {
+  if (P->err) cudaFree(P->err);
+  if (P->list) cudaFree(P->list);
+  if (P->bpart) cudaFree(P->bpart);
+  delete P;
+}
+
+// Stages: the chain D1 (rows of G's loss, then of D's) -> A3 -> A2 -> A1, then the weight
+// gradients. S_DEP: the stage whose output a stage reads; S_LEVEL: its place along the chain.
+enum { S_D1G = 0, S_D1D, S_A3, S_A2, S_A1, S_DW2D, S_DW1D, S_DW3G, S_DW2G, S_DW1G };
+constexpr int S_DEP[tcb::MAX_STAGES] = {-1, -1, S_D1G, S_A3, S_A2, -1, S_D1D, S_A3, S_A2, S_A1};
+constexpr int S_LEVEL[tcb::MAX_STAGES + 2] = {0, 0, 1, 2, 3, 0, 1, 2, 3, 4, 4, 1};  // + ranges
+
+// The grid's tiles in claim order (CellPlan::list): by level, then by cell; a cell's chain tiles
+// first. `tiles`: tiles per cell of each stage.
+std::vector<int2> tile_list(int cells, const int* tiles) {
+  static const int order[] = {S_A1, S_A2, S_A3, S_D1G, S_D1D, S_DW1G, S_DW2G, S_DW3G, S_DW1D,
+                              S_DW2D, tcb::RANGES_STAGE, tcb::RANGES_STAGE + 1};
+  std::vector<int2> out;
+  for (int level = 0; level < 5; ++level)
+    for (int c = 0; c < cells; ++c)
+      for (int k : order) {
+        if (S_LEVEL[k] != level) continue;
+        const int n = k >= tcb::RANGES_STAGE ? 1 : tiles[k];
+        for (int t = 0; t < n; ++t) out.push_back(int2{c, k << 16 | t});
+      }
+  return out;
+}
+}  // namespace
 
 bool tcb_supported(int z, int h, int x, int B) {
   return h == 256 && z == 64 && x % 16 == 0 && x >= 64 && B >= 1 && B <= 256;
@@ -956,16 +982,45 @@ TcbPlan* tcb_plan_create(const TcbShape& s, const TcbBuffers& b, std::string* ms
   if (cudaMalloc(&P->err, 4) != cudaSuccess || cudaMemset(P->err, 0, 4) != cudaSuccess) {
     cudaGetLastError();
     if (msg) *msg = "cudaMalloc for the error flag failed";
-    delete P;
+    free_plan(P);
     return nullptr;
   }
   const int C = s.cells, B = s.B, h = s.h, x = s.x, z = s.z;
   const uint64_t NI = s.n_indiv;
   const bf16* Gw = b.Gwb;
   const bf16* Dw = b.Dwb;
-  auto base_params = [&](int M, int N, int K, int BN) {
-    tcb::GParams q;
-    memset(&q, 0, sizeof q);
+  // Tiles of 128 columns: their operands leave three ring stages (256: two, and coarser tiles at
+  // the end of the list; 382 against 387 us at 12x12, 87 against 93 at 5x5). Where a cell's 42 or
+  // so weight tiles of 128 columns would leave SMs idle, 64 (41 against 45 us at 1x1; 447 against
+  // 382 at 12x12, four loads of A's 128 rows where 128 columns need two).
+  const int bn = C * ((h / 128) * (2 * (h / 128) + (x + 127) / 128 + 1) + (x + 127) / 128 * 2) < sms
+                     ? 64
+                     : 128;
+  bool ok = true;
+  // bias-gradient partials [4 x row tiles][column] of D1's D-loss rows and of A3, A2, A1
+  const int mt2 = (2 * B + 127) / 128, mt = (B + 127) / 128;
+  const int64_t bp_cell = 4 * ((int64_t)mt2 * h + (int64_t)mt * (x + 2 * h));
+  if (cudaMalloc(&P->bpart, (size_t)C * bp_cell * 4) != cudaSuccess) {
+    cudaGetLastError();
+    if (msg) *msg = "cudaMalloc for the bias partial sums failed";
+    free_plan(P);
+    return nullptr;
+  }
+  int64_t bp_off = 0;
+  P->cells.adam = b.fuse_adam;
+  P->cells.beta1 = b.beta1;
+  P->cells.beta2 = b.beta2;
+  P->cells.eps = b.eps;
+  for (int pop = 0; pop < 2; ++pop) {
+    tcb::RangeTask& t = P->cells.rt[pop];
+    t.r = b.ranges[pop];
+    t.grad = pop ? b.gD : b.gG;
+    t.part_cell = bp_cell;
+    for (int q = 0; q < t.r.n; ++q) t.total += t.r.len[q];
+  }
+  // C = A * B^T: M rows, N columns in tiles of BN, over K
+  auto stage = [&](int si, int M, int N, int K, int BN) -> tcb::GParams& {
+    tcb::GParams& q = P->cells.st[si].p;
     q.M = M;
     q.N = N;
     q.K = K;
@@ -974,301 +1029,171 @@ TcbPlan* tcb_plan_create(const TcbShape& s, const TcbBuffers& b, std::string* ms
     q.ntiles = (N + BN - 1) / BN;
     q.kchunks = (K + 63) / 64;
     q.slope = s.slope;
-    q.aux_wrap_at = 1 << 30;
-    q.err = P->err;
-    q.cells = C;
     return q;
   };
-  bool ok = true;
-  int i = 0;
-  auto finish = [&](Gemm& G) {
-    const int tiles = C * G.p.mtiles * G.p.ntiles;
-    G.grid = tiles < sms ? tiles : sms;
+  // delta product: A's rows from a_row0 of `amap` {k, rows}, B the selected individual's weight
+  // tensor [k][n]; times act' of the stored output (aux map), into `out` [cells][rows][N] at
+  // out_cell elements per cell. bias_pop >= 0: the column sums are the gradient of that
+  // population's range at bias_off
+  auto delta = [&](int si, int act, const void* A, int a_rows, int64_t a_cell, int a_row0,
+                   const bf16* W, int64_t Ps, const int* sel, void* out, int64_t out_cell,
+                   int bias_pop, int64_t bias_off) {
+    tcb::GParams& q = P->cells.st[si].p;
+    q.epi = tcb::EPI_DACT;
+    q.act = act;
+    q.a_row0 = a_row0;
+    q.b_sel = sel;
+    ok = ok && map3(&P->maps.a[si], A, q.K, a_rows, C, a_cell, 128, msg) &&
+         map3(&P->maps.b[si], W, q.N, q.K, NI, Ps, 64, msg) &&
+         map3(&P->maps.out[si], out, q.N, q.M, C, out_cell, 64, msg);
+    if (bias_pop < 0) return;
+    q.bias_part = P->bpart + bp_off;
+    q.bias_cell = bp_cell;
+    bp_off += 4 * (int64_t)q.mtiles * q.N;
+    tcb::RangeTask& t = P->cells.rt[bias_pop];
+    for (int k = 0; k < t.r.n; ++k)
+      if (t.r.off[k] == bias_off && t.r.len[k] == q.N) {
+        t.part[k] = q.bias_part;
+        t.tiles[k] = q.mtiles;
+        t.dep[t.n_dep] = si;
+        t.need[t.n_dep++] = q.mtiles * q.ntiles;
+      }
   };
-  // weight-gradient stage of tensor `off` of a population: Adam in the epilogue when fused
-  // weight-gradient stage of the tensor at `off` of a population, whose gradient tile is
-  // [out = M][in = N] row-major (scm = N, scn = 1): Adam in the epilogue when fused
-  auto fuse = [&](Gemm& G, const TcbBuffers::AdamPop& a, const int* src, int64_t off,
-                  int64_t Ps) {
+  auto aux3 = [&](int si, const void* X, int rows, int64_t cell, int row0) {
+    P->cells.st[si].p.x_row0 = row0;
+    ok = ok && map3(&P->maps.in[si], X, P->cells.st[si].p.N, rows, C, cell, 64, msg);
+  };
+  // weight gradient dW[o][i] = sum_r A[r][o] Bm[r][i] (both read MN-major) of the tensor at `off`
+  // of a population: the Adam step in the epilogue, or the gradient stored
+  auto weight = [&](int si, const void* A, int a_rows, int64_t a_cell, const TcbBuffers::AdamPop& ap,
+                    const int* src, int64_t off, int64_t Ps, float* grad) {
+    tcb::GParams& q = P->cells.st[si].p;
+    q.a_mn = 1;
+    q.epi = tcb::EPI_F32;
+    q.C = grad + off;
+    q.c_cell = Ps;
+    ok = ok && map3(&P->maps.a[si], A, q.M, a_rows, C, a_cell, 64, msg);
     if (!b.fuse_adam) return;
-    if (G.p.scn != 1 || G.p.scm != G.p.N || G.p.N % 16 != 0 || off % 8 != 0 || Ps % 8 != 0) {
-      if (msg) *msg = "fused Adam needs 16-column tensors at 8-element offsets";
-      ok = false;
-      return;
-    }
-    G.p.epi = tcb::EPI_ADAM;
-    G.p.adam.src = src;
-    G.p.adam.coef = a.coef;
-    G.p.adam.beta1 = b.beta1;
-    G.p.adam.beta2 = b.beta2;
-    G.p.adam.eps = b.eps;
     // w, m, v are one allocation in three equal parts: the part size is the 4th dimension's
     // stride, the same for the old and the new snapshot
-    const int64_t part = a.m - a.w;
-    if (part <= 0 || a.v - a.m != part || a.m_new - a.w_new != part ||
-        a.v_new - a.m_new != part) {
-      if (msg) *msg = "fused Adam needs w, m, v at equal distances";
+    const int64_t part = ap.m - ap.w;
+    if (q.N % 16 != 0 || off % 8 != 0 || Ps % 8 != 0 || part <= 0 || ap.v - ap.m != part ||
+        ap.m_new - ap.w_new != part || ap.v_new - ap.m_new != part) {
+      if (msg) *msg = "fused Adam needs 16-column tensors at 8-element offsets and w, m, v at "
+                      "equal distances";
       ok = false;
       return;
     }
-    ok = ok && map4f(&G.ao, a.w + off, G.p.N, G.p.M, NI, Ps, part, msg) &&
-         map4f(&G.an, a.w_new + off, G.p.N, G.p.M, C, Ps, part, msg) &&
-         map3b_rows(&G.nb, a.wb_new + off, G.p.N, G.p.M, C, Ps, msg);
+    q.epi = tcb::EPI_ADAM;
+    q.adam.src = src;
+    q.adam.coef = ap.coef;
+    q.adam.beta1 = b.beta1;
+    q.adam.beta2 = b.beta2;
+    q.adam.eps = b.eps;
+    ok = ok && map4f(&P->maps.in[si], ap.w + off, q.N, q.M, NI, Ps, part, msg) &&
+         map4f(&P->maps.out[si], ap.w_new + off, q.N, q.M, C, Ps, part, msg) &&
+         map3b_rows(&P->maps.nb[si], ap.wb_new + off, q.N, q.M, C, Ps, msg);
   };
-
-  // 1. D1 = (J2 @ W2d) * lrelu'(TG1 rows r or r - B): M = 3B rows, N = 256, K = 256
+  auto act3 = [&](int si, const void* X, int rows, int64_t cell) {
+    ok = ok && map3(&P->maps.b[si], X, P->cells.st[si].p.N, rows, C, cell, 64, msg);
+  };
+  const int64_t Bh = (int64_t)B * h, Bx = (int64_t)B * x;
+  // D1 = (J2 @ W2d) * lrelu'(TG1): J2's rows [0, 2B) (D's loss; with D's b1) and [2B, 3B) (G's
+  // loss, on TG1's fake rows)
+  stage(S_D1G, B, h, h, bn);
+  delta(S_D1G, ACT_LRELU, b.J2, 3 * B, 3 * Bh, 2 * B, Dw + b.doff[2], b.PDs, b.src_d,
+        (bf16*)b.D1 + 2 * Bh, 3 * Bh, -1, 0);
+  aux3(S_D1G, b.TG1, 2 * B, 2 * Bh, B);
+  stage(S_D1D, 2 * B, h, h, bn);
+  delta(S_D1D, ACT_LRELU, b.J2, 3 * B, 3 * Bh, 0, Dw + b.doff[2], b.PDs, b.src_d, b.D1, 3 * Bh,
+        1, b.doff[1]);
+  aux3(S_D1D, b.TG1, 2 * B, 2 * Bh, 0);
+  // A3 = (D1[2B + r] @ W1d) * (1 - F^2), F the selected generator's fakes: E[c] slot 1 + sel_g[c]
+  // (with G's b3)
+  stage(S_A3, B, x, h, bn).x_slot = b.sel_g;
+  delta(S_A3, ACT_TANH, b.D1, 3 * B, 3 * Bh, 2 * B, Dw + b.doff[0], b.PDs, b.src_d, b.A3, Bx, 0,
+        b.goff[5]);
+  ok = ok && map4(&P->maps.in[S_A3], b.E, x, B, 6, C, Bx, b.e_cell, msg);
+  // A2 = (A3 @ W3g) * relu'(TH2) (with G's b2), A1 = (A2 @ W2g) * relu'(TH1) (with G's b1)
+  stage(S_A2, B, h, x, bn);
+  delta(S_A2, ACT_RELU, b.A3, B, Bx, 0, Gw + b.goff[4], b.PGs, b.src_g, b.A2, Bh, 0,
+        b.goff[3]);
+  aux3(S_A2, b.TH2, B, Bh, 0);
+  stage(S_A1, B, h, h, bn);
+  delta(S_A1, ACT_RELU, b.A2, B, Bh, 0, Gw + b.goff[2], b.PGs, b.src_g, b.A1, Bh, 0,
+        b.goff[1]);
+  aux3(S_A1, b.TH1, B, Bh, 0);
+  // dW2d = J2^T TG1 and dW1d = D1^T X over the 2B D-loss rows. X = [E[c] rows 0..B-1 (real); E[c]
+  // fake rows of slot sel_g[c]] is read in place: K splits into the two B-row parts (rows past B
+  // in a part read as zero), D1 rows shifted by B in the second part
+  stage(S_DW2D, h, h, 2 * B, bn);
+  weight(S_DW2D, b.J2, 3 * B, 3 * Bh, b.adam_d, b.src_d, b.doff[2], b.PDs, b.gD);
+  act3(S_DW2D, b.TG1, 2 * B, 2 * Bh);
   {
-    Gemm& G = P->g[i++];
-    G.p = base_params(3 * B, h, h, 256);
-    G.p.b_mn = 1;
-    G.p.b_sel = b.src_d;
-    G.p.epi = tcb::EPI_DACT;
-    G.p.act = ACT_LRELU;
-    G.p.C = b.D1;
-    G.p.c_cell = (int64_t)3 * B * h;
-    G.p.scm = h;
-    G.p.scn = 1;
-    G.p.aux = (const bf16*)b.TG1;
-    G.p.aux_cell = (int64_t)2 * B * h;
-    G.p.sxm = h;
-    G.p.sxn = 1;
-    G.p.aux_wrap_at = 2 * B;
-    G.p.aux_wrap_sub = B;
-    G.p.bias_out = b.gD + b.doff[1];  // D's b1: rows of the D loss
-    G.p.bias_cell = b.PDs;
-    G.p.bias_rows = 2 * B;
-    ok = ok && map3(&G.a, b.J2, h, 3 * B, C, (uint64_t)3 * B * h, 128, msg) &&
-         map3(&G.b, Dw + b.doff[2], h, h, NI, b.PDs, 64, msg);
-    finish(G);
+    tcb::GParams& q = stage(S_DW1D, h, x, 2 * B, bn);
+    q.ksplit = (B + 63) / 64;
+    q.kchunks = 2 * q.ksplit;
+    q.a_k_off1 = B;
+    q.b_slot_sel = b.sel_g;
   }
-  // 2. dW2d[o][i] = sum_{r < 2B} J2[r][o] TG1[r][i]: M = o, N = i, K = 2B (TG1 ends at 2B).
-  //    An epilogue thread owns one output row o: 16 consecutive parameters per group.
-  {
-    Gemm& G = P->g[i++];
-    G.p = base_params(h, h, 2 * B, 256);
-    G.p.a_mn = 1;
-    G.p.b_mn = 1;
-    G.p.epi = tcb::EPI_F32;
-    G.p.C = b.gD + b.doff[2];
-    G.p.c_cell = b.PDs;
-    G.p.scm = h;
-    G.p.scn = 1;
-    fuse(G, b.adam_d, b.src_d, b.doff[2], b.PDs);
-    ok = ok && map3(&G.a, b.J2, h, 3 * B, C, (uint64_t)3 * B * h, 64, msg) &&
-         map3(&G.b, b.TG1, h, 2 * B, C, (uint64_t)2 * B * h, 64, msg);
-    finish(G);
-  }
-  // 3. A3 = (D1[2B + r] @ W1d) * (1 - F^2): M = B, N = x (tiles of 256), K = 256
-  {
-    Gemm& G = P->g[i++];
-    G.p = base_params(B, x, h, 256);
-    G.p.a_row0 = 2 * B;
-    G.p.b_mn = 1;
-    G.p.b_sel = b.src_d;
-    G.p.epi = tcb::EPI_DACT;
-    G.p.act = ACT_TANH;
-    G.p.C = b.A3;
-    G.p.c_cell = (int64_t)B * x;
-    G.p.scm = x;
-    G.p.scn = 1;
-    G.p.aux = (const bf16*)b.E;  // the selected generator's fakes: E[c] slot 1 + sel_g[c]
-    G.p.aux_cell = b.e_cell;
-    G.p.aux_sel = b.sel_g;
-    G.p.aux_sel_stride = (int64_t)B * x;
-    G.p.bias_out = b.gG + b.goff[5];  // G's b3
-    G.p.bias_cell = b.PGs;
-    G.p.bias_rows = B;
-    G.p.sxm = x;
-    G.p.sxn = 1;
-    ok = ok && map3(&G.a, b.D1, h, 3 * B, C, (uint64_t)3 * B * h, 128, msg) &&
-         map3(&G.b, Dw + b.doff[0], x, h, NI, b.PDs, 64, msg);
-    finish(G);
-  }
-  // 4. dW1d[o][i] = sum_{r < 2B} D1[r][o] X[r][i]: M = o = 256, N = i = x, K = 2B, where X =
-  //    [E[c] rows 0..B-1 (real); E[c] fake rows of slot sel_g[c]] read in place: K splits into
-  //    the two B-row parts (rows past B in a part read as zero), D1 rows shifted by B in the
-  //    second part
-  {
-    Gemm& G = P->g[i++];
-    G.p = base_params(h, x, 2 * B, 256);
-    G.p.kchunks = 2 * ((B + 63) / 64);
-    G.p.ksplit = (B + 63) / 64;
-    G.p.a_k_off1 = B;
-    G.p.b_slot_sel = b.sel_g;
-    G.p.a_mn = 1;
-    G.p.b_mn = 1;
-    G.p.epi = tcb::EPI_F32;
-    G.p.C = b.gD + b.doff[0];
-    G.p.c_cell = b.PDs;
-    G.p.scm = x;
-    G.p.scn = 1;
-    fuse(G, b.adam_d, b.src_d, b.doff[0], b.PDs);
-    ok = ok && map3(&G.a, b.D1, h, 3 * B, C, (uint64_t)3 * B * h, 64, msg) &&
-         map4(&G.b, b.E, x, B, 6, C, (uint64_t)B * x, (uint64_t)b.e_cell, msg);
-    finish(G);
-  }
-  // 5. A2 = (A3 @ W3g) * relu'(TH2): M = B, N = 256, K = x
-  {
-    Gemm& G = P->g[i++];
-    G.p = base_params(B, h, x, 256);
-    G.p.b_mn = 1;
-    G.p.b_sel = b.src_g;
-    G.p.epi = tcb::EPI_DACT;
-    G.p.act = ACT_RELU;
-    G.p.C = b.A2;
-    G.p.c_cell = (int64_t)B * h;
-    G.p.scm = h;
-    G.p.scn = 1;
-    G.p.aux = (const bf16*)b.TH2;
-    G.p.aux_cell = (int64_t)B * h;
-    G.p.bias_out = b.gG + b.goff[3];  // G's b2
-    G.p.bias_cell = b.PGs;
-    G.p.bias_rows = B;
-    G.p.sxm = h;
-    G.p.sxn = 1;
-    ok = ok && map3(&G.a, b.A3, x, B, C, (uint64_t)B * x, 128, msg) &&
-         map3(&G.b, Gw + b.goff[4], h, x, NI, b.PGs, 64, msg);
-    finish(G);
-  }
-  // 6. dW3g[o][i] = sum_r A3[r][o] TH2[r][i]: M = o = x, N = i = 256, K = B
-  {
-    Gemm& G = P->g[i++];
-    G.p = base_params(x, h, B, 256);
-    G.p.a_mn = 1;
-    G.p.b_mn = 1;
-    G.p.epi = tcb::EPI_F32;
-    G.p.C = b.gG + b.goff[4];
-    G.p.c_cell = b.PGs;
-    G.p.scm = h;
-    G.p.scn = 1;
-    fuse(G, b.adam_g, b.src_g, b.goff[4], b.PGs);
-    ok = ok && map3(&G.a, b.A3, x, B, C, (uint64_t)B * x, 64, msg) &&
-         map3(&G.b, b.TH2, h, B, C, (uint64_t)B * h, 64, msg);
-    finish(G);
-  }
-  // 7. A1 = (A2 @ W2g) * relu'(TH1): M = B, N = 256, K = 256
-  {
-    Gemm& G = P->g[i++];
-    G.p = base_params(B, h, h, 256);
-    G.p.b_mn = 1;
-    G.p.b_sel = b.src_g;
-    G.p.epi = tcb::EPI_DACT;
-    G.p.act = ACT_RELU;
-    G.p.C = b.A1;
-    G.p.c_cell = (int64_t)B * h;
-    G.p.scm = h;
-    G.p.scn = 1;
-    G.p.aux = (const bf16*)b.TH1;
-    G.p.aux_cell = (int64_t)B * h;
-    G.p.bias_out = b.gG + b.goff[1];  // G's b1
-    G.p.bias_cell = b.PGs;
-    G.p.bias_rows = B;
-    G.p.sxm = h;
-    G.p.sxn = 1;
-    ok = ok && map3(&G.a, b.A2, h, B, C, (uint64_t)B * h, 128, msg) &&
-         map3(&G.b, Gw + b.goff[2], h, h, NI, b.PGs, 64, msg);
-    finish(G);
-  }
-  // 8. dW2g[o][i] = sum_r A2[r][o] TH1[r][i]: M = o = 256, N = i = 256, K = B
-  {
-    Gemm& G = P->g[i++];
-    G.p = base_params(h, h, B, 256);
-    G.p.a_mn = 1;
-    G.p.b_mn = 1;
-    G.p.epi = tcb::EPI_F32;
-    G.p.C = b.gG + b.goff[2];
-    G.p.c_cell = b.PGs;
-    G.p.scm = h;
-    G.p.scn = 1;
-    fuse(G, b.adam_g, b.src_g, b.goff[2], b.PGs);
-    ok = ok && map3(&G.a, b.A2, h, B, C, (uint64_t)B * h, 64, msg) &&
-         map3(&G.b, b.TH1, h, B, C, (uint64_t)B * h, 64, msg);
-    finish(G);
-  }
-  // 9. dW1g[o][i] = sum_r A1[r][o] Z[r][i]: M = 256 (o), N = z (i), K = B
-  {
-    Gemm& G = P->g[i++];
-    G.p = base_params(h, z, B, z);
-    G.p.a_mn = 1;
-    G.p.b_mn = 1;
-    G.p.epi = tcb::EPI_F32;
-    G.p.C = b.gG + b.goff[0];
-    G.p.c_cell = b.PGs;
-    G.p.scm = z;
-    G.p.scn = 1;
-    fuse(G, b.adam_g, b.src_g, b.goff[0], b.PGs);
-    ok = ok && map3(&G.a, b.A1, h, B, C, (uint64_t)B * h, 64, msg) &&
-         map3(&G.b, b.Z, z, B, C, (uint64_t)B * z, 64, msg);
-    finish(G);
-  }
-  P->n = i;
+  weight(S_DW1D, b.D1, 3 * B, 3 * Bh, b.adam_d, b.src_d, b.doff[0], b.PDs, b.gD);
+  ok = ok && map4(&P->maps.b[S_DW1D], b.E, x, B, 6, C, Bx, b.e_cell, msg);
+  // dW3g = A3^T TH2, dW2g = A2^T TH1, dW1g = A1^T Z
+  stage(S_DW3G, x, h, B, bn);
+  weight(S_DW3G, b.A3, B, Bx, b.adam_g, b.src_g, b.goff[4], b.PGs, b.gG);
+  act3(S_DW3G, b.TH2, B, Bh);
+  stage(S_DW2G, h, h, B, bn);
+  weight(S_DW2G, b.A2, B, Bh, b.adam_g, b.src_g, b.goff[2], b.PGs, b.gG);
+  act3(S_DW2G, b.TH1, B, Bh);
+  stage(S_DW1G, h, z, B, z);
+  weight(S_DW1G, b.A1, B, Bh, b.adam_g, b.src_g, b.goff[0], b.PGs, b.gG);
+  act3(S_DW1G, b.Z, B, (int64_t)B * z);
   if (ok) {
-    // per-cell megakernel: stage order as above; each stage's dependency on an earlier output
-    const int deps[9] = {-1, -1, 0, 0, 2, 2, 4, 4, 6};
-    int tile0 = 0, pub = 0;
-    for (int k = 0; k < i; ++k) {
-      int publish = 0;
-      for (int j = k + 1; j < i; ++j) publish |= deps[j] == k;
-      const int nt = P->g[k].p.mtiles * P->g[k].p.ntiles;
-      P->maps.a[k] = P->g[k].a;
-      P->maps.b[k] = P->g[k].b;
-      P->maps.ao[k] = P->g[k].ao;
-      P->maps.an[k] = P->g[k].an;
-      P->maps.nb[k] = P->g[k].nb;
-      P->cells.st[k].p = P->g[k].p;
-      P->cells.st[k].dep = deps[k];
-      P->cells.st[k].tile0 = tile0;
-      P->cells.st[k].publish = publish;
-      tile0 += nt;
-      if (publish) pub += nt;
-      P->cells.pub_end[k] = pub;
+    int tiles[tcb::MAX_STAGES];
+    for (int k = 0; k < tcb::MAX_STAGES; ++k) {
+      const tcb::GParams& q = P->cells.st[k].p;
+      tiles[k] = q.mtiles * q.ntiles;
     }
-    P->cells.n_stages = i;
-    P->cells.tiles_per_cell = tile0;
-    P->cells.pub_per_cell = pub;
+    for (int k = 0; k < tcb::MAX_STAGES; ++k) {
+      P->cells.st[k].dep = S_DEP[k];
+      P->cells.st[k].dep_need = S_DEP[k] >= 0 ? tiles[S_DEP[k]] : 0;
+    }
+    P->cells.op_bytes = tcb::A_BYTES + bn * tcb::BK * 2;
+    P->cells.n_ops = tcb::RING_BYTES / P->cells.op_bytes;
+    if (P->cells.n_ops > tcb::MAX_OPS) P->cells.n_ops = tcb::MAX_OPS;
+    const std::vector<int2> list = tile_list(C, tiles);
+    P->cells.n_list = (int)list.size();
+    if (cudaMalloc(&P->list, list.size() * sizeof(int2)) != cudaSuccess ||
+        cudaMemcpy(P->list, list.data(), list.size() * sizeof(int2), cudaMemcpyHostToDevice) !=
+            cudaSuccess) {
+      cudaGetLastError();
+      if (msg) *msg = "cudaMalloc for the backward's tile list failed";
+      ok = false;
+    }
+    P->cells.list = P->list;
+    P->cells.sync = b.sync;
     P->cells.cells = C;
     P->cells.err = P->err;
-    P->grid_cells = C < sms ? C : sms;
-    P->fused = b.fuse_adam != 0;
-    P->cells.has_ranges = P->fused && b.ranges ? 1 : 0;
-    if (P->cells.has_ranges) {
-      P->cells.rg = b.ranges[0];
-      P->cells.rd = b.ranges[1];
-      P->cells.beta1 = b.beta1;
-      P->cells.beta2 = b.beta2;
-      P->cells.eps = b.eps;
-    }
-    const cudaError_t e =
-        P->fused ? cudaFuncSetAttribute(tcb::k_bwd_cells<true>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        tcb::Cfg<true>::SMEM)
-                 : cudaFuncSetAttribute(tcb::k_bwd_cells<false>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        tcb::Cfg<false>::SMEM);
-    if (e != cudaSuccess) {
+    P->grid = P->cells.n_list < sms ? P->cells.n_list : sms;
+    if (cudaFuncSetAttribute(tcb::k_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, tcb::SMEM) !=
+        cudaSuccess) {
       cudaGetLastError();
-      if (msg) *msg = "cannot reserve shared memory for the per-cell backward";
+      if (msg) *msg = "cannot reserve shared memory for the backward";
       ok = false;
     }
   }
   if (!ok) {
-    cudaFree(P->err);
-    delete P;
+    free_plan(P);
     return nullptr;
   }
   return P;
 }
 
-int tcb_run_cells(TcbPlan* P, cudaStream_t st, std::string* msg) {
-  if (P->fused)
-    launch_pdl(tcb::k_bwd_cells<true>, dim3(P->grid_cells), dim3(tcb::Cfg<true>::THREADS),
-               tcb::Cfg<true>::SMEM, st, P->maps, P->cells);
-  else
-    launch_pdl(tcb::k_bwd_cells<false>, dim3(P->grid_cells), dim3(tcb::Cfg<false>::THREADS),
-               tcb::Cfg<false>::SMEM, st, P->maps, P->cells);
+int tcb_run(TcbPlan* P, cudaStream_t st, std::string* msg) {
+  launch_pdl(tcb::k_bwd, dim3(P->grid), dim3(tcb::THREADS), tcb::SMEM, st, P->maps, P->cells);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
-    if (msg) *msg = std::string("per-cell backward launch: ") + cudaGetErrorString(e);
+    if (msg) *msg = std::string("backward launch: ") + cudaGetErrorString(e);
     return 1;
   }
   return 0;
@@ -1277,9 +1202,7 @@ int tcb_run_cells(TcbPlan* P, cudaStream_t st, std::string* msg) {
 int* tcb_error_flag(TcbPlan* P) { return P ? P->err : nullptr; }
 
 void tcb_plan_destroy(TcbPlan* P) {
-  if (!P) return;
-  if (P->err) cudaFree(P->err);
-  delete P;
+  if (P) free_plan(P);
 }
 
 }  // namespace lipz

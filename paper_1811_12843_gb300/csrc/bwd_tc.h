@@ -13,6 +13,9 @@
 
 namespace lipz {
 
+enum { TCB_SYNC_WORDS = 16 };
+inline int64_t tcb_sync_ints(int cells) { return (int64_t)cells * TCB_SYNC_WORDS + 16; }
+
 struct TcbShape {
   int cells, B, z, h, x;
   float slope;
@@ -50,9 +53,12 @@ struct TcbBuffers {
     const float4* coef;
   } adam_g, adam_d;
   float beta1, beta2, eps;
-  // with fuse_adam: the remaining ranges (biases, D's output layer) of G and D, [2]; each CTA
-  // applies them to its cell after the cell's last tile
+  // the remaining ranges (biases, D's output layer) of G and D, [2]: the backward sums the
+  // biases' gradients, and with fuse_adam steps every range
   const AdamRanges* ranges;
+  // counters of finished tiles ([cells][TCB_SYNC_WORDS]) and, after them, the claim counter: all
+  // zero when the backward starts (k_dlogit, which runs before it, clears them)
+  int* sync;
 };
 
 struct TcbPlan;
@@ -60,9 +66,9 @@ struct TcbPlan;
 // hidden == 256, z == 64, x a multiple of 16, 1 <= batch <= 256.
 bool tcb_supported(int z, int h, int x, int B);
 TcbPlan* tcb_plan_create(const TcbShape& s, const TcbBuffers& b, std::string* msg);
-// All nine products of every cell in one launch (one CTA per cell), as stages in the order
-// 0 D1, 1 dW2(D), 2 A3, 3 dW1(D), 4 A2, 5 dW3(G), 6 A1, 7 dW2(G), 8 dW1(G).
-int tcb_run_cells(TcbPlan* p, cudaStream_t st, std::string* msg);
+// All nine products of every cell in one launch, as the tiles of the stages 0 D1, 1 dW2(D), 2 A3,
+// 3 dW1(D), 4 A2, 5 dW3(G), 6 A1, 7 dW2(G), 8 dW1(G), claimed by persistent CTAs.
+int tcb_run(TcbPlan* p, cudaStream_t st, std::string* msg);
 int* tcb_error_flag(TcbPlan* p);
 void tcb_plan_destroy(TcbPlan* p);
 

@@ -180,11 +180,13 @@ void launch_fitness_select(const float* logits, int cells, int B, float* LG, flo
 template <typename T>
 void launch_train_prep(const T* E, int64_t e_cell, const int* sel_g, T* TX, int cells, int B,
                        int x_dim, cudaStream_t st);
+// sync (null: none): the tensor-core backward's counters, [cells][sync_words] and sync_words more,
+// which this kernel clears (the backward is the next launch)
 template <typename T>
 void launch_dlogit(const float* TL, const T* TG2, const T* wD, int64_t wD_stride, int64_t off_w3,
                    const int* src_d, int cells, int B, int H, float slope, T* J2, float* gD,
-                   int64_t gD_stride, int64_t off_gw3, int64_t off_gb3, int64_t off_gb2,
-                   cudaStream_t st);
+                   int64_t gD_stride, int64_t off_gw3, int64_t off_gb3, int64_t off_gb2, int* sync,
+                   int sync_words, cudaStream_t st);
 void launch_adam(const PopView& old_p, const PopView& new_p, const float* grad, const int* src,
                  const float4* coef, int cells, int64_t P, int64_t Ps, float beta1, float beta2,
                  float eps, cudaStream_t st);

@@ -648,13 +648,19 @@ __global__ void __launch_bounds__(512) k_dlogit(
     const float* __restrict__ TL, const T* __restrict__ TG2, const T* __restrict__ wD,
     int64_t wD_stride, int64_t off_w3, const int* __restrict__ src_d, int B, int H, float slope,
     T* __restrict__ J2, float* __restrict__ gD, int64_t gD_stride, int64_t off_gw3,
-    int64_t off_gb3, int64_t off_gb2) {
+    int64_t off_gb3, int64_t off_gb2, int* __restrict__ sync, int sync_words) {
   pdl_wait();
   // Lanes own column groups of 8 (threads of the block: H / 8 groups x RG row groups); the RG
   // partial sums of dW3 and of db2 (the column sums of J2 over the D-loss rows) are added in a
   // fixed order.
   extern __shared__ float dl[];  // [3B] deltas, then [RG][H] and [RG][H] partial sums
   const int c = blockIdx.x;
+  if (sync) {
+    // the cell's counters of the backward that follows (block 0 also its claim counter)
+    if ((int)threadIdx.x < sync_words) sync[c * (int64_t)sync_words + threadIdx.x] = 0;
+    if (c == 0 && (int)threadIdx.x < sync_words)
+      sync[gridDim.x * (int64_t)sync_words + threadIdx.x] = 0;
+  }
   const int ng = (H + 7) / 8;
   const int RG = blockDim.x / ng;
   float* part = dl + 3 * B;
@@ -763,8 +769,8 @@ __global__ void __launch_bounds__(512) k_dlogit(
 template <typename T>
 void launch_dlogit(const float* TL, const T* TG2, const T* wD, int64_t wD_stride, int64_t off_w3,
                    const int* src_d, int cells, int B, int H, float slope, T* J2, float* gD,
-                   int64_t gD_stride, int64_t off_gw3, int64_t off_gb3, int64_t off_gb2,
-                   cudaStream_t st) {
+                   int64_t gD_stride, int64_t off_gw3, int64_t off_gb3, int64_t off_gb2, int* sync,
+                   int sync_words, cudaStream_t st) {
   const int ng = (H + 7) / 8;
   int rg = 512 / ng;
   if (rg < 1) rg = 1;
@@ -772,14 +778,14 @@ void launch_dlogit(const float* TL, const T* TG2, const T* wD, int64_t wD_stride
   const int threads = ((rg * ng + 31) / 32) * 32;
   const size_t smem = (3 * (size_t)B + 2 * (size_t)(threads / ng) * H) * sizeof(float);
   launch_pdl(k_dlogit<T>, dim3(cells), dim3(threads), smem, st, TL, TG2, wD, wD_stride, off_w3,
-             src_d, B, H, slope, J2, gD, gD_stride, off_gw3, off_gb3, off_gb2);
+             src_d, B, H, slope, J2, gD, gD_stride, off_gw3, off_gb3, off_gb2, sync, sync_words);
 }
 template void launch_dlogit<float>(const float*, const float*, const float*, int64_t, int64_t,
                                    const int*, int, int, int, float, float*, float*, int64_t,
-                                   int64_t, int64_t, int64_t, cudaStream_t);
+                                   int64_t, int64_t, int64_t, int*, int, cudaStream_t);
 template void launch_dlogit<bf16>(const float*, const bf16*, const bf16*, int64_t, int64_t,
                                   const int*, int, int, int, float, bf16*, float*, int64_t,
-                                  int64_t, int64_t, int64_t, cudaStream_t);
+                                  int64_t, int64_t, int64_t, int*, int, cudaStream_t);
 
 // ------------------------------------------------------------------------------------------
 // Adam (Kingma & Ba 2015, Algorithm 1) fused with the replacement copy: the new centre of
