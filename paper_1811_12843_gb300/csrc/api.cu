@@ -6,6 +6,7 @@
 // one CUDA stream, the kernels with programmatic dependent launch (each kernel's set-up
 // overlaps the previous kernel's tail; its first global access waits for that kernel); the
 // host waits only when the caller asks for host-side results.
+#include <algorithm>
 #include <climits>
 #include <cmath>
 #include <cstdarg>
@@ -29,15 +30,23 @@ enum Phase { PH_IDLE = 0, PH_EVALUATED = 1, PH_SELECTED = 2 };
 
 thread_local std::string t_create_err;
 
+// One launch of the grouped GEMM: problems and their output tiles.
+struct GemmSet {
+  GemmDesc* d = nullptr;
+  int2* t = nullptr;
+  int n = 0, shape = 0;
+};
+
 struct Descs {
   // evaluation (per parity of the snapshot): generator layers over (cell, slot i),
   // discriminator layers over (cell, slot j)
-  GemmDesc *g1, *g2, *g3, *d1, *d2;
+  GemmSet g1, g2, g3, d1, d2;
   GemvDesc* d3;
-  // training (per parity): forward of the selected pair and its backward
-  GemmDesc *tg1, *tg2, *td1, *td2, *bw2d, *bd1, *bw1d, *ba3, *bw3g, *ba2, *bw2g, *ba1, *bw1g;
+  // training (per parity): the discriminator's forward of later minibatch steps, and the backward
+  // in launches of independent products: {dW2d, D1}, {dW1d, A3}, {dW3g, A2}, {dW2g, A1}, {dW1g}
+  GemmSet td1, td2, bw[5];
   GemvDesc* tgv;
-  ColSumDesc *cb1d, *cb3g, *cb2g, *cb1g;  // bias gradients (D's b2 comes from k_dlogit)
+  ColSumDesc* cb;  // bias gradients of every cell (D's b2 comes from k_dlogit)
 };
 
 }  // namespace
@@ -114,7 +123,7 @@ struct lipz_grid {
   // stores the Gram matrices [cells][6B][6B] first
   float *mix = nullptr, *rnorm = nullptr, *mixP = nullptr, *mixS = nullptr, *mixScore = nullptr;
   float* gram = nullptr;
-  GemmDesc* dgram = nullptr;
+  GemmSet dgram;
   int mix_nh = 1;
   bool mix_tc = false;
   Descs dsc[3]{}, dsc_stale[3]{};
@@ -256,7 +265,8 @@ char* eoff(const void* base, int64_t elems, size_t esz) {
 }
 
 GemmDesc gd(const void* A, int64_t sam, int64_t sak, const void* B, int64_t sbk, int64_t sbn,
-            void* C, int64_t scm, int64_t scn, int M, int N, int K) {
+            void* C, int64_t scm, int64_t scn, int M, int N, int K, int epi = EPI_STORE,
+            int act = ACT_NONE) {
   GemmDesc d;
   memset(&d, 0, sizeof d);
   d.A = A;
@@ -271,6 +281,8 @@ GemmDesc gd(const void* A, int64_t sam, int64_t sak, const void* B, int64_t sbk,
   d.M = M;
   d.N = N;
   d.K = K;
+  d.epi = epi;
+  d.act = act;
   return d;
 }
 
@@ -291,6 +303,58 @@ int upload(lipz_grid* g, T** dst, const std::vector<T>& v) {
   int rc = dalloc(g, dst, v.size() * sizeof(T));
   if (rc) return rc;
   return h2d(g, *dst, v.data(), v.size() * sizeof(T));
+}
+
+// One grouped-GEMM launch of the problems v (the longest sums first, so that the last blocks to
+// start are short ones).
+int make_set(lipz_grid* g, GemmSet* S, std::vector<GemmDesc> v) {
+  const int es = (int)g->esz;
+  auto vec = [&](const void* p, int64_t unit, int64_t other, int n_unit, const GemmDesc& d, int op) {
+    return unit == 1 && other % 4 == 0 && n_unit % 4 == 0 && (uintptr_t)p % (4 * es) == 0 &&
+           (!d.wsel || d.wsel_op != op || d.wsel_stride % 4 == 0);
+  };
+  for (GemmDesc& d : v) {
+    d.vec = 0;
+    if (d.sak == 1 ? vec(d.A, 1, d.sam, d.K, d, 1) : vec(d.A, d.sam, d.sak, d.M, d, 1))
+      d.vec |= GEMM_VEC_A;
+    if (d.sbk == 1 ? vec(d.B, 1, d.sbn, d.K, d, 2) : vec(d.B, d.sbn, d.sbk, d.N, d, 2))
+      d.vec |= GEMM_VEC_B;
+  }
+  std::stable_sort(v.begin(), v.end(),
+                   [](const GemmDesc& a, const GemmDesc& b) { return a.K > b.K; });
+  // The tile shape with the least estimated time, in multiply-adds of one SM: the padded tiles'
+  // work over 152 SMs, a multiply-add weighted by what it costs in the shape (outputs per value
+  // read from shared memory), and a quarter of the longest tile's time, which has an SM's `share`th
+  // part. Measured, fp32: 128 x 64 against 32 x 32 takes 367 against 525 us for the
+  // discriminators of a 3x3 grid (900 against 6840 tiles), 215 against 173 for its backward (36 to
+  // 252 tiles of 128 x 64 per launch); for 222 x 200 outputs (padded 1.48 and 1.13 times) 266
+  // against 210.
+  static const double weight[GEMM_N_TILES] = {1.0, 1.2, 1.3};
+  static const double share[GEMM_N_TILES] = {2.5, 4, 6};
+  double best = 0;
+  for (int s = 0; s < GEMM_N_TILES; ++s) {
+    const GemmTile t = GEMM_TILES[s];
+    double work = 0, last = 0;
+    for (const GemmDesc& d : v) {
+      const double tile = (double)t.bm * t.bn * d.K * weight[s];
+      work += tile * ((d.M + t.bm - 1) / t.bm) * ((d.N + t.bn - 1) / t.bn);
+      last = std::max(last, tile * share[s]);
+    }
+    const double cost = work / 152 + 0.25 * last;
+    if (s == 0 || cost < best) {
+      best = cost;
+      S->shape = s;
+    }
+  }
+  const GemmTile t = GEMM_TILES[S->shape];
+  std::vector<int2> tiles;
+  for (size_t i = 0; i < v.size(); ++i)
+    for (int m = 0; m * t.bm < v[i].M; ++m)
+      for (int n = 0; n * t.bn < v[i].N; ++n) tiles.push_back(int2{(int)i, m << 16 | n});
+  S->n = (int)tiles.size();
+  int rc;
+  if ((rc = upload(g, &S->d, v)) || (rc = upload(g, &S->t, tiles))) return rc;
+  return LIPZ_OK;
 }
 
 // Snapshot written by an iteration that reads snapshot p, and the one it read before p.
@@ -325,7 +389,7 @@ int build_descs(lipz_grid* g, int p) {
       return rc;
     return LIPZ_OK;
   }
-  // pair lists of both tables for the tensor-core evaluation
+  // pair lists of both tables for the tensor-core evaluation, or the CUDA-core launches
   auto pair_lists = [&](const std::vector<int>& tab, TcPairs& P) -> int {
     std::vector<int4> gp, dp;
     std::vector<int2> pl;
@@ -338,7 +402,7 @@ int build_descs(lipz_grid* g, int p) {
     P = TcPairs{dg, (int)gp.size(), dd, (int)dp.size(), dl};
     return LIPZ_OK;
   };
-  {
+  if (g->use_tc) {
     int rc;
     if ((rc = pair_lists(cur, g->pairs_cur[p])) ||
         (g->a.stale_neighbors && (rc = pair_lists(stale, g->pairs_stale[p]))))
@@ -354,24 +418,25 @@ int build_descs(lipz_grid* g, int p) {
         const int64_t pg = (int64_t)k * g->PGs, pd = (int64_t)k * g->PDs;
         const int64_t cs = (int64_t)c * 5 + s;
         GemmDesc a = gd(eoff(g->Z, (int64_t)c * B * z, es), z, 1, eoff(Gw, pg + L.off[0], es), 1, z,
-                        eoff(g->H1g, cs * B * h, es), h, 1, B, h, z);
+                        eoff(g->H1g, cs * B * h, es), h, 1, B, h, z, EPI_BIAS_ACT, ACT_RELU);
         a.bias = Gp.w + pg + L.off[1];
         g1.push_back(a);
         GemmDesc b = gd(eoff(g->H1g, cs * B * h, es), h, 1, eoff(Gw, pg + L.off[2], es), 1, h,
-                        eoff(g->H2g, cs * B * h, es), h, 1, B, h, h);
+                        eoff(g->H2g, cs * B * h, es), h, 1, B, h, h, EPI_BIAS_ACT, ACT_RELU);
         b.bias = Gp.w + pg + L.off[3];
         g2.push_back(b);
         GemmDesc e = gd(eoff(g->H2g, cs * B * h, es), h, 1, eoff(Gw, pg + L.off[4], es), 1, h,
                         eoff(g->E, (int64_t)c * g->e_cell + (int64_t)(1 + s) * B * x, es), x, 1, B,
-                        x, h);
+                        x, h, EPI_BIAS_ACT, ACT_TANH);
         e.bias = Gp.w + pg + L.off[5];
         g3.push_back(e);
         GemmDesc f = gd(eoff(g->E, (int64_t)c * g->e_cell, es), x, 1, eoff(Dw, pd + M.off[0], es), 1,
-                        x, eoff(g->H1d, cs * 6 * B * h, es), h, 1, 6 * B, h, x);
+                        x, eoff(g->H1d, cs * 6 * B * h, es), h, 1, 6 * B, h, x, EPI_BIAS_ACT,
+                        ACT_LRELU);
         f.bias = Dp.w + pd + M.off[1];
         d1.push_back(f);
         GemmDesc q2 = gd(eoff(g->H1d, cs * 6 * B * h, es), h, 1, eoff(Dw, pd + M.off[2], es), 1, h,
-                         eoff(g->H2d, cs * 6 * B * h, es), h, 1, 6 * B, h, h);
+                         eoff(g->H2d, cs * 6 * B * h, es), h, 1, 6 * B, h, h, EPI_BIAS_ACT, ACT_LRELU);
         q2.bias = Dp.w + pd + M.off[3];
         d2.push_back(q2);
         GemvDesc v;
@@ -386,26 +451,29 @@ int build_descs(lipz_grid* g, int p) {
         d3.push_back(v);
       }
     int rc;
-    if ((rc = upload(g, &D.g1, g1)) || (rc = upload(g, &D.g2, g2)) ||
-        (rc = upload(g, &D.g3, g3)) || (rc = upload(g, &D.d1, d1)) ||
-        (rc = upload(g, &D.d2, d2)) || (rc = upload(g, &D.d3, d3)))
+    if ((rc = make_set(g, &D.g1, g1)) || (rc = make_set(g, &D.g2, g2)) ||
+        (rc = make_set(g, &D.g3, g3)) || (rc = make_set(g, &D.d1, d1)) ||
+        (rc = make_set(g, &D.d2, d2)) || (rc = upload(g, &D.d3, d3)))
       return rc;
     return LIPZ_OK;
   };
   {
     int rc;
-    if ((rc = upload(g, &g->nbr_cur[p], cur)) || (rc = upload(g, &g->nbr_stale[p], stale)) ||
-        (rc = eval_descs(cur, g->dsc[p])) ||
-        (g->a.stale_neighbors && (rc = eval_descs(stale, g->dsc_stale[p]))))
+    if ((rc = upload(g, &g->nbr_cur[p], cur)) || (rc = upload(g, &g->nbr_stale[p], stale)))
       return rc;
+    if (!g->use_tc &&
+        ((rc = eval_descs(cur, g->dsc[p])) ||
+         (g->a.stale_neighbors && (rc = eval_descs(stale, g->dsc_stale[p])))))
+      return rc;
+    if (g->use_tc && g->use_tcb) return LIPZ_OK;
   }
   Descs& D = g->dsc[p];
   int rc;
 
   // ---- training descriptors: weights of the selected individual (wsel = src_g / src_d)
-  std::vector<GemmDesc> tg1, tg2, td1, td2, bw2d, bd1, bw1d, ba3, bw3g, ba2, bw2g, ba1, bw1g;
+  std::vector<GemmDesc> td1, td2, bw[5];
   std::vector<GemvDesc> tgv;
-  std::vector<ColSumDesc> cb1d, cb3g, cb2g, cb1g;
+  std::vector<ColSumDesc> cb;
   auto selg = [&](GemmDesc d, int c) {
     d.wsel = g->src_g;
     d.wsel_stride = g->PGs;
@@ -444,16 +512,12 @@ int build_descs(lipz_grid* g, int p) {
     float* gGc = g->gG + (int64_t)c * g->PGs;
     float* gDc = g->gD + (int64_t)c * g->PDs;
 
-    GemmDesc a = selg(gd(Zc, z, 1, eoff(Gw, L.off[0], es), 1, z, TH1c, h, 1, B, h, z), c);
-    a.bias = Gp.w + L.off[1];
-    tg1.push_back(a);
-    a = selg(gd(TH1c, h, 1, eoff(Gw, L.off[2], es), 1, h, TH2c, h, 1, B, h, h), c);
-    a.bias = Gp.w + L.off[3];
-    tg2.push_back(a);
-    a = seld(gd(TXc, x, 1, eoff(Dw, M.off[0], es), 1, x, TG1c, h, 1, 2 * B, h, x), c);
+    GemmDesc a = seld(gd(TXc, x, 1, eoff(Dw, M.off[0], es), 1, x, TG1c, h, 1, 2 * B, h, x,
+                         EPI_BIAS_ACT, ACT_LRELU), c);
     a.bias = Dp.w + M.off[1];
     td1.push_back(a);
-    a = seld(gd(TG1c, h, 1, eoff(Dw, M.off[2], es), 1, h, TG2c, h, 1, 2 * B, h, h), c);
+    a = seld(gd(TG1c, h, 1, eoff(Dw, M.off[2], es), 1, h, TG2c, h, 1, 2 * B, h, h, EPI_BIAS_ACT,
+                ACT_LRELU), c);
     a.bias = Dp.w + M.off[3];
     td2.push_back(a);
     GemvDesc v;
@@ -470,70 +534,61 @@ int build_descs(lipz_grid* g, int p) {
     v.K = h;
     tgv.push_back(v);
     // discriminator backward
-    bw2d.push_back(gd(J2c, 1, h, TG1c, h, 1, gDc + M.off[2], h, 1, h, h, 2 * B));
-    a = seld(gd(J2c, h, 1, eoff(Dw, M.off[2], es), h, 1, D1c, h, 1, 2 * B, h, h), c);
+    bw[0].push_back(gd(J2c, 1, h, TG1c, h, 1, gDc + M.off[2], h, 1, h, h, 2 * B));
+    a = seld(gd(J2c, h, 1, eoff(Dw, M.off[2], es), h, 1, D1c, h, 1, 2 * B, h, h,
+                EPI_DACT, ACT_LRELU), c);
     a.aux = TG1c;
     a.sxm = h;
     a.sxn = 1;
-    bd1.push_back(a);
+    bw[0].push_back(a);
     a = seld(gd(eoff(J2c, 2 * (int64_t)B * h, es), h, 1, eoff(Dw, M.off[2], es), h, 1,
-                eoff(D1c, 2 * (int64_t)B * h, es), h, 1, B, h, h), c);
+                eoff(D1c, 2 * (int64_t)B * h, es), h, 1, B, h, h, EPI_DACT, ACT_LRELU), c);
     a.aux = eoff(TG1c, (int64_t)B * h, es);
     a.sxm = h;
     a.sxn = 1;
-    bd1.push_back(a);
-    bw1d.push_back(gd(D1c, 1, h, TXc, x, 1, gDc + M.off[0], x, 1, h, x, 2 * B));
-    cb1d.push_back(cs(D1c, gDc + M.off[1], h, 2 * B, h));
+    bw[0].push_back(a);
+    bw[1].push_back(gd(D1c, 1, h, TXc, x, 1, gDc + M.off[0], x, 1, h, x, 2 * B));
+    cb.push_back(cs(D1c, gDc + M.off[1], h, 2 * B, h));
     // generator backward: into the fakes through D's first layer, then through G
     a = seld(gd(eoff(D1c, 2 * (int64_t)B * h, es), h, 1, eoff(Dw, M.off[0], es), x, 1, A3c, x, 1,
-                B, x, h), c);
+                B, x, h, EPI_DACT, ACT_TANH), c);
     a.aux = eoff(TXc, (int64_t)B * x, es);
     a.sxm = x;
     a.sxn = 1;
-    ba3.push_back(a);
-    bw3g.push_back(gd(A3c, 1, x, TH2c, h, 1, gGc + L.off[4], h, 1, x, h, B));
-    cb3g.push_back(cs(A3c, gGc + L.off[5], x, B, x));
-    a = selg(gd(A3c, x, 1, eoff(Gw, L.off[4], es), h, 1, A2c, h, 1, B, h, x), c);
+    bw[1].push_back(a);
+    bw[2].push_back(gd(A3c, 1, x, TH2c, h, 1, gGc + L.off[4], h, 1, x, h, B));
+    cb.push_back(cs(A3c, gGc + L.off[5], x, B, x));
+    a = selg(gd(A3c, x, 1, eoff(Gw, L.off[4], es), h, 1, A2c, h, 1, B, h, x, EPI_DACT,
+                ACT_RELU), c);
     a.aux = TH2c;
     a.sxm = h;
     a.sxn = 1;
-    ba2.push_back(a);
-    bw2g.push_back(gd(A2c, 1, h, TH1c, h, 1, gGc + L.off[2], h, 1, h, h, B));
-    cb2g.push_back(cs(A2c, gGc + L.off[3], h, B, h));
-    a = selg(gd(A2c, h, 1, eoff(Gw, L.off[2], es), h, 1, A1c, h, 1, B, h, h), c);
+    bw[2].push_back(a);
+    bw[3].push_back(gd(A2c, 1, h, TH1c, h, 1, gGc + L.off[2], h, 1, h, h, B));
+    cb.push_back(cs(A2c, gGc + L.off[3], h, B, h));
+    a = selg(gd(A2c, h, 1, eoff(Gw, L.off[2], es), h, 1, A1c, h, 1, B, h, h, EPI_DACT,
+                ACT_RELU), c);
     a.aux = TH1c;
     a.sxm = h;
     a.sxn = 1;
-    ba1.push_back(a);
-    bw1g.push_back(gd(A1c, 1, h, Zc, z, 1, gGc + L.off[0], z, 1, h, z, B));
-    cb1g.push_back(cs(A1c, gGc + L.off[1], h, B, h));
+    bw[3].push_back(a);
+    bw[4].push_back(gd(A1c, 1, h, Zc, z, 1, gGc + L.off[0], z, 1, h, z, B));
+    cb.push_back(cs(A1c, gGc + L.off[1], h, B, h));
   }
-  if ((rc = upload(g, &D.tg1, tg1)) || (rc = upload(g, &D.tg2, tg2)) ||
-      (rc = upload(g, &D.td1, td1)) || (rc = upload(g, &D.td2, td2)) ||
-      (rc = upload(g, &D.tgv, tgv)) || (rc = upload(g, &D.bw2d, bw2d)) ||
-      (rc = upload(g, &D.bd1, bd1)) || (rc = upload(g, &D.bw1d, bw1d)) ||
-      (rc = upload(g, &D.ba3, ba3)) || (rc = upload(g, &D.bw3g, bw3g)) ||
-      (rc = upload(g, &D.ba2, ba2)) || (rc = upload(g, &D.bw2g, bw2g)) ||
-      (rc = upload(g, &D.ba1, ba1)) || (rc = upload(g, &D.bw1g, bw1g)) ||
-      (rc = upload(g, &D.cb1d, cb1d)) ||
-      (rc = upload(g, &D.cb3g, cb3g)) || (rc = upload(g, &D.cb2g, cb2g)) ||
-      (rc = upload(g, &D.cb1g, cb1g)))
+  // the discriminator's training forward runs for the later minibatch steps only: step 0 takes
+  // the evaluation's activations
+  if (!g->use_tc && g->a.train_steps > 1 &&
+      ((rc = make_set(g, &D.td1, td1)) || (rc = make_set(g, &D.td2, td2)) ||
+       (rc = upload(g, &D.tgv, tgv))))
     return rc;
-  return LIPZ_OK;
+  for (int k = 0; k < 5; ++k)
+    if ((rc = make_set(g, &D.bw[k], bw[k]))) return rc;
+  return upload(g, &D.cb, cb);
 }
 
-// Grouped GEMM in the grid's precision; out_f32 selects an fp32 output (gradients).
-void gemm(lipz_grid* g, const GemmDesc* d, int n, int M, int N, int epi, int act, bool out_f32) {
-  const float sl = g->a.leaky_slope;
-  if (g->bf) {
-    if (out_f32) launch_gemm<bf16, float, EPI_STORE>(d, n, M, N, act, sl, g->st);
-    else if (epi == EPI_BIAS_ACT) launch_gemm<bf16, bf16, EPI_BIAS_ACT>(d, n, M, N, act, sl, g->st);
-    else launch_gemm<bf16, bf16, EPI_DACT>(d, n, M, N, act, sl, g->st);
-  } else {
-    if (out_f32 && epi == EPI_STORE) launch_gemm<float, float, EPI_STORE>(d, n, M, N, act, sl, g->st);
-    else if (epi == EPI_BIAS_ACT) launch_gemm<float, float, EPI_BIAS_ACT>(d, n, M, N, act, sl, g->st);
-    else launch_gemm<float, float, EPI_DACT>(d, n, M, N, act, sl, g->st);
-  }
+void gemm(lipz_grid* g, const GemmSet& S) {
+  if (g->bf) launch_gemm<bf16>(S.d, S.t, S.n, S.shape, g->a.leaky_slope, g->st);
+  else launch_gemm<float>(S.d, S.t, S.n, S.shape, g->a.leaky_slope, g->st);
 }
 
 void gemv(lipz_grid* g, const GemvDesc* d, int n, int rows) {
@@ -541,12 +596,10 @@ void gemv(lipz_grid* g, const GemvDesc* d, int n, int rows) {
   else launch_gemv<float>(d, n, rows, g->st);
 }
 
-void colsum_on(lipz_grid* g, const ColSumDesc* d, int n, int cols, cudaStream_t st) {
-  if (g->bf) launch_colsum<bf16>(d, n, cols, st);
-  else launch_colsum<float>(d, n, cols, st);
+void colsum(lipz_grid* g, const ColSumDesc* d, int n, int cols) {
+  if (g->bf) launch_colsum<bf16>(d, n, cols, g->st);
+  else launch_colsum<float>(d, n, cols, g->st);
 }
-
-void colsum(lipz_grid* g, const ColSumDesc* d, int n, int cols) { colsum_on(g, d, n, cols, g->st); }
 
 int check_arch(const lipz_arch* a) {
   if (!a) return fail(nullptr, LIPZ_ERR_INVALID, "arch is null");
@@ -635,9 +688,18 @@ int create_impl(lipz_grid* g) {
   g->nsnap = g->a.stale_neighbors ? 3 : 2;
   if ((rc = alloc_pops(g, g->G, g->PGs)) || (rc = alloc_pops(g, g->D, g->PDs))) return rc;
   const size_t CB = (size_t)C * B;
+  g->use_tc = !g->dcgan && g->bf && !g->a.force_simt && tc_supported(z, h, x, B);
+  g->use_tcb = g->use_tc && tcb_supported(z, h, x, B);
+  // every slot's hidden activations (CUDA-core evaluation) and the training input in one array
+  // (CUDA-core backward)
+  const bool simt = !g->dcgan && !g->use_tc;
+  if ((simt && ((rc = dalloc(g, &g->H1g, CB * 5 * h * es)) ||
+                (rc = dalloc(g, &g->H2g, CB * 5 * h * es)) ||
+                (rc = dalloc(g, &g->H1d, CB * 30 * h * es)) ||
+                (rc = dalloc(g, &g->H2d, CB * 30 * h * es)))) ||
+      (!g->dcgan && !g->use_tcb && (rc = dalloc(g, &g->TX, CB * 2 * x * es))))
+    return rc;
   if ((rc = dalloc(g, &g->Z, CB * z * es)) || (rc = dalloc(g, &g->E, (size_t)C * g->e_cell * es)) ||
-      (rc = dalloc(g, &g->H1g, CB * 5 * h * es)) || (rc = dalloc(g, &g->H2g, CB * 5 * h * es)) ||
-      (rc = dalloc(g, &g->H1d, CB * 30 * h * es)) || (rc = dalloc(g, &g->H2d, CB * 30 * h * es)) ||
       (rc = dalloc(g, &g->logits, CB * 30 * 4)) || (rc = dalloc(g, &g->LG, C * 25 * 4)) ||
       (rc = dalloc(g, &g->LD, C * 25 * 4)) || (rc = dalloc(g, &g->fG, C * 5 * 4)) ||
       (rc = dalloc(g, &g->fD, C * 5 * 4)) || (rc = dalloc(g, &g->sel_g, C * 4)) ||
@@ -645,7 +707,7 @@ int create_impl(lipz_grid* g) {
       (rc = dalloc(g, &g->src_d, C * 4)) || (rc = dalloc(g, &g->lrn_g, C * 4)) ||
       (rc = dalloc(g, &g->lrn_d, C * 4)) || (rc = dalloc(g, &g->coef_g, C * 16)) ||
       (rc = dalloc(g, &g->coef_d, C * 16)) || (rc = dalloc(g, &g->TH1, CB * h * es)) ||
-      (rc = dalloc(g, &g->TH2, CB * h * es)) || (rc = dalloc(g, &g->TX, CB * 2 * x * es)) ||
+      (rc = dalloc(g, &g->TH2, CB * h * es)) ||
       (rc = dalloc(g, &g->TG1, CB * 2 * h * es)) || (rc = dalloc(g, &g->TG2, CB * 2 * h * es)) ||
       (rc = dalloc(g, &g->TL, CB * 2 * 4)) || (rc = dalloc(g, &g->J2, CB * 3 * h * es)) ||
       (rc = dalloc(g, &g->D1, CB * 3 * h * es)) || (rc = dalloc(g, &g->A3, CB * x * es)) ||
@@ -674,7 +736,7 @@ int create_impl(lipz_grid* g) {
         dg.push_back(gd(eoff(g->E, (int64_t)c * g->e_cell, es), x, 1,
                         eoff(g->E, (int64_t)c * g->e_cell, es), 1, x,
                         g->gram + (int64_t)c * R * R, (int64_t)R, 1, (int)R, (int)R, x));
-      if ((rc = upload(g, &g->dgram, dg))) return rc;
+      if ((rc = make_set(g, &g->dgram, dg))) return rc;
     }
   }
   const int big = INT_MAX;
@@ -692,7 +754,6 @@ int create_impl(lipz_grid* g) {
     if ((rc = h2d(g, g->G[p].lr, lr.data(), C * 4)) || (rc = h2d(g, g->D[p].lr, lr.data(), C * 4)) ||
         (rc = build_descs(g, p)))
       return rc;
-  g->use_tc = !g->dcgan && g->bf && !g->a.force_simt && tc_supported(z, h, x, B);
   if (g->dcgan) {
     DcShape s{C, B, z, g->a.ngf, g->a.ndf, g->bf, g->a.leaky_slope, g->nsnap * C};
     DcBuffers b{};
@@ -748,7 +809,6 @@ int create_impl(lipz_grid* g) {
       g->tc[p] = tc_plan_create(s, b, &msg);
       if (!g->tc[p]) return fail(g, LIPZ_ERR_CUDA, "tensor-core plan: %s", msg.c_str());
     }
-    g->use_tcb = tcb_supported(z, h, x, B);
     if (g->use_tcb && (rc = dalloc(g, &g->bsync, tcb_sync_ints(C) * sizeof(int)))) return rc;
     for (int p = 0; p < g->nsnap && g->use_tcb; ++p) {
       TcbShape s{C, B, z, h, x, g->a.leaky_slope, g->nsnap * C};
@@ -851,7 +911,7 @@ int mixture_impl(lipz_grid* g) {
     std::string msg;
     if (tc_run_gram(g->tc[g->cur], g->st, &msg)) return fail(g, LIPZ_ERR_CUDA, "%s", msg.c_str());
   } else {
-    gemm(g, g->dgram, C, R, R, EPI_STORE, ACT_NONE, true);
+    gemm(g, g->dgram);
     launch_mix_partials(g->gram, g->rnorm, C, R, B, x, g->mixP, g->st);
   }
   CKL(g);
@@ -912,9 +972,9 @@ int eval_impl(lipz_grid* g, const float* xin_dev, bool then_select,
   } else {
     const Descs& D = g->a.stale_neighbors && g->prev_valid ? g->dsc_stale[p] : g->dsc[p];
     phase_begin(g, LIPZ_PHASE_G_FWD);
-    gemm(g, D.g1, C * 5, B, h, EPI_BIAS_ACT, ACT_RELU, false);
-    gemm(g, D.g2, C * 5, B, h, EPI_BIAS_ACT, ACT_RELU, false);
-    gemm(g, D.g3, C * 5, B, x, EPI_BIAS_ACT, ACT_TANH, false);
+    gemm(g, D.g1);
+    gemm(g, D.g2);
+    gemm(g, D.g3);
     phase_end(g, LIPZ_PHASE_G_FWD, 3);
     if (x_ready) {
       CK(g, cudaStreamWaitEvent(g->st, x_ready, 0));
@@ -922,8 +982,8 @@ int eval_impl(lipz_grid* g, const float* xin_dev, bool then_select,
       CKL(g);
     }
     phase_begin(g, LIPZ_PHASE_D_FWD);
-    gemm(g, D.d1, C * 5, 6 * B, h, EPI_BIAS_ACT, ACT_LRELU, false);
-    gemm(g, D.d2, C * 5, 6 * B, h, EPI_BIAS_ACT, ACT_LRELU, false);
+    gemm(g, D.d1);
+    gemm(g, D.d2);
     gemv(g, D.d3, C * 5, 6 * B);
     phase_end(g, LIPZ_PHASE_D_FWD, 3);
   }
@@ -1017,10 +1077,17 @@ void bias_ranges(lipz_grid* g, int p, AdamRanges* rg, AdamRanges* rd) {
 }
 
 // One Adam step of every cell's chosen pair (sel/src/coef) from snapshot cur into the other
-// snapshot, which becomes cur.
-int train_once(lipz_grid* g) {
-  const int C = g->cells, B = g->a.batch, h = g->a.hidden, x = g->a.x_dim, z = g->a.z_dim;
+// snapshot, which becomes cur. `evaluated`: the pair's rows and parameters are those of the
+// evaluation before (minibatch step 0).
+int train_once(lipz_grid* g, bool evaluated) {
+  const int C = g->cells, B = g->a.batch, h = g->a.hidden, x = g->a.x_dim;
   const int p = g->cur;
+  auto adam = [&] {
+    const int q = snap_next(g, p);
+    launch_adam({g->G[0], g->G[q], g->gG, g->src_g, g->coef_g, g->PG, g->PGs},
+                {g->D[0], g->D[q], g->gD, g->src_d, g->coef_d, g->PD, g->PDs}, C, g->a.beta1,
+                g->a.beta2, g->a.eps, g->st);
+  };
   if (g->dcgan) {
     // forward and backward of the selected pairs (gradients into gG, gD), then Adam +
     // replacement into the next snapshot
@@ -1032,27 +1099,40 @@ int train_once(lipz_grid* g) {
     if (dc_train(g->dc, g->st, &msg)) return fail(g, LIPZ_ERR_CUDA, "%s", msg.c_str());
     phase_end(g, LIPZ_PHASE_TRAIN_BWD, dc_train_launches(g->dc));
     phase_begin(g, LIPZ_PHASE_ADAM);
-    launch_adam(g->G[0], g->G[snap_next(g, p)], g->gG, g->src_g, g->coef_g, C, g->PG, g->PGs,
-                g->a.beta1, g->a.beta2, g->a.eps, g->st);
-    launch_adam(g->D[0], g->D[snap_next(g, p)], g->gD, g->src_d, g->coef_d, C, g->PD, g->PDs,
-                g->a.beta1, g->a.beta2, g->a.eps, g->st);
+    adam();
     CKL(g);
-    phase_end(g, LIPZ_PHASE_ADAM, 2);
+    phase_end(g, LIPZ_PHASE_ADAM, 1);
     g->cur = snap_next(g, p);
     return LIPZ_OK;
   }
   const Descs& D = g->dsc[p];
   phase_begin(g, LIPZ_PHASE_TRAIN_FWD);
-  // the CUDA-core kernels read the discriminator's training input as one array TX; the
-  // tensor-core kernels read it from E in place
   int n_fwd = 0;
-  if (!(g->use_tc && g->use_tcb)) {
-    if (g->bf)
-      launch_train_prep<bf16>((const bf16*)g->E, g->e_cell, g->sel_g, (bf16*)g->TX, C, B, x,
-                              g->st);
-    else
-      launch_train_prep<float>((const float*)g->E, g->e_cell, g->sel_g, (float*)g->TX, C, B, x,
-                               g->st);
+  if (!g->use_tcb) {
+    // the CUDA-core kernels read the discriminator's training input as one array TX; the
+    // tensor-core kernels read it from E in place. The CUDA-core evaluation keeps every slot's
+    // activations: the selected pair's are gathered, not computed again (the generator's always:
+    // a later minibatch step has run its forward too)
+    TrainGather t{};
+    t.E = g->E;
+    t.e_cell = g->e_cell;
+    t.sel_g = g->sel_g;
+    t.sel_d = g->sel_d;
+    t.TX = g->TX;
+    t.H1g = g->H1g;
+    t.H2g = g->H2g;
+    t.TH1 = g->TH1;
+    t.TH2 = g->TH2;
+    if (evaluated) {
+      t.H1d = g->H1d;
+      t.H2d = g->H2d;
+      t.logits = g->logits;
+      t.TG1 = g->TG1;
+      t.TG2 = g->TG2;
+      t.TL = g->TL;
+    }
+    if (g->bf) launch_train_gather<bf16>(t, C, B, x, h, g->st);
+    else launch_train_gather<float>(t, C, B, x, h, g->st);
     n_fwd = 1;
   }
   // forward of the selected pair
@@ -1061,13 +1141,11 @@ int train_once(lipz_grid* g) {
     if (tc_run_train_g(g->tc[p], g->st, &msg) || tc_run_train_d(g->tc[p], g->st, &msg))
       return fail(g, LIPZ_ERR_CUDA, "%s", msg.c_str());
     n_fwd += 2;
-  } else {
-    gemm(g, D.tg1, C, B, h, EPI_BIAS_ACT, ACT_RELU, false);
-    gemm(g, D.tg2, C, B, h, EPI_BIAS_ACT, ACT_RELU, false);
-    gemm(g, D.td1, C, 2 * B, h, EPI_BIAS_ACT, ACT_LRELU, false);
-    gemm(g, D.td2, C, 2 * B, h, EPI_BIAS_ACT, ACT_LRELU, false);
+  } else if (!evaluated) {
+    gemm(g, D.td1);
+    gemm(g, D.td2);
     gemv(g, D.tgv, C, 2 * B);
-    n_fwd += 5;
+    n_fwd += 3;
   }
   // logit deltas (and D's output-layer gradient)
   if (g->bf)
@@ -1096,31 +1174,16 @@ int train_once(lipz_grid* g) {
       return LIPZ_OK;
     }
   } else {
-    gemm(g, D.bw2d, C, h, h, EPI_STORE, ACT_NONE, true);
-    gemm(g, D.bd1, 2 * C, 2 * B, h, EPI_DACT, ACT_LRELU, false);
-    gemm(g, D.bw1d, C, h, x, EPI_STORE, ACT_NONE, true);
-    colsum(g, D.cb1d, C, h);
-    // generator's backward through D
-    gemm(g, D.ba3, C, B, x, EPI_DACT, ACT_TANH, false);
-    gemm(g, D.bw3g, C, x, h, EPI_STORE, ACT_NONE, true);
-    colsum(g, D.cb3g, C, x);
-    gemm(g, D.ba2, C, B, h, EPI_DACT, ACT_RELU, false);
-    gemm(g, D.bw2g, C, h, h, EPI_STORE, ACT_NONE, true);
-    colsum(g, D.cb2g, C, h);
-    gemm(g, D.ba1, C, B, h, EPI_DACT, ACT_RELU, false);
-    gemm(g, D.bw1g, C, h, z, EPI_STORE, ACT_NONE, true);
-    colsum(g, D.cb1g, C, h);
+    for (const GemmSet& S : D.bw) gemm(g, S);
+    colsum(g, D.cb, 4 * C, h > x ? h : x);
     CKL(g);
-    phase_end(g, LIPZ_PHASE_TRAIN_BWD, 15);
+    phase_end(g, LIPZ_PHASE_TRAIN_BWD, 6);
     phase_begin(g, LIPZ_PHASE_ADAM);
   }
   // Adam + replacement into the other snapshot (after the bias sums on the tensor-core path)
-  launch_adam(g->G[0], g->G[snap_next(g, p)], g->gG, g->src_g, g->coef_g, C, g->PG, g->PGs, g->a.beta1,
-              g->a.beta2, g->a.eps, g->st);
-  launch_adam(g->D[0], g->D[snap_next(g, p)], g->gD, g->src_d, g->coef_d, C, g->PD, g->PDs, g->a.beta1,
-              g->a.beta2, g->a.eps, g->st);
+  adam();
   CKL(g);
-  phase_end(g, LIPZ_PHASE_ADAM, 2);
+  phase_end(g, LIPZ_PHASE_ADAM, 1);
   g->cur = snap_next(g, p);
   return LIPZ_OK;
 }
@@ -1146,13 +1209,13 @@ int train_again(lipz_grid* g, uint32_t k) {
   } else {
     // the CUDA-core kernels run the generators of all five slots (slot 0 is the one used)
     const Descs& D = g->dsc[g->cur];
-    gemm(g, D.g1, C * 5, B, h, EPI_BIAS_ACT, ACT_RELU, false);
-    gemm(g, D.g2, C * 5, B, h, EPI_BIAS_ACT, ACT_RELU, false);
-    gemm(g, D.g3, C * 5, B, x, EPI_BIAS_ACT, ACT_TANH, false);
+    gemm(g, D.g1);
+    gemm(g, D.g2);
+    gemm(g, D.g3);
     phase_end(g, LIPZ_PHASE_G_FWD, 3);
   }
   CKL(g);
-  return train_once(g);
+  return train_once(g, false);
 }
 
 int train_impl(lipz_grid* g) {
@@ -1162,7 +1225,7 @@ int train_impl(lipz_grid* g) {
   if (K > 1 && g->pool_n <= 0)
     return fail(g, LIPZ_ERR_STATE, "train_steps > 1 draws its minibatches from the pool: call "
                                    "lipz_set_data first");
-  int rc = train_once(g);
+  int rc = train_once(g, true);
   for (int k = 1; k < K && !rc; ++k) rc = train_again(g, (uint32_t)k);
   if (rc) return rc;
   g->t += 1;

@@ -146,8 +146,13 @@ __device__ __forceinline__ void adam_elem(float& w, float& m, float& v, float g,
 
 // ---- grouped GEMM problem: C[m, n] = epi( sum_k A[m*sam + k*sak] * B[k*sbk + n*sbn] )
 // Epilogues: EPI_BIAS_ACT: act(acc + bias[n]);  EPI_DACT: acc * act_bwd(aux[m*sxm + n*sxn]);
-// EPI_STORE: acc. Element strides; pointers typed by the launch.
+// EPI_STORE: acc, in fp32. Element strides; operands (and C, but for EPI_STORE) typed by the
+// launch.
 enum Epi : int { EPI_STORE = 0, EPI_BIAS_ACT = 1, EPI_DACT = 2 };
+
+// GEMM_VEC_A / _B: the operand's unit-stride rows start on a boundary of four elements and hold a
+// multiple of four (four elements in one load).
+enum { GEMM_VEC_A = 1, GEMM_VEC_B = 2 };
 
 // A problem whose weight operand belongs to a selected individual sets wsel: the operand
 // (wsel_op 1 = A, 2 = B) and the bias move by wsel[cell] * wsel_stride elements.
@@ -161,8 +166,16 @@ struct GemmDesc {
   int64_t sam, sak, sbk, sbn, scm, scn, sxm, sxn;
   int64_t wsel_stride;
   int M, N, K;
-  int wsel_op, cell, pad;
+  int wsel_op, cell;
+  int epi, act, vec;
 };
+
+// Output tile shapes of the grouped GEMM (8 x 8, 4 x 8 and 4 x 4 outputs per thread).
+struct GemmTile {
+  int bm, bn;
+};
+constexpr GemmTile GEMM_TILES[] = {{128, 64}, {32, 64}, {32, 32}};
+constexpr int GEMM_N_TILES = 3;
 
 // Column sums: out[n] = sum_{r < rows} X[r * ld + n], n < cols (bias gradients).
 struct ColSumDesc {

@@ -68,9 +68,11 @@ void launch_draw_batch(const T* pool, int64_t n_pool, const float* xin, T* E, in
                        T* Z, int cells, int B, int x_dim, int z_dim, uint64_t seed, uint32_t t,
                        uint32_t step, int parts, bool pdl, cudaStream_t st);
 
-template <typename TI, typename TO, int EPI>
-void launch_gemm(const GemmDesc* descs, int n_problems, int max_m, int max_n, int act,
-                 float slope, cudaStream_t st);
+// tiles [n]: {problem, row tile << 16 | column tile} for output tile shape `shape` (an index into
+// GEMM_TILES).
+template <typename TI>
+void launch_gemm(const GemmDesc* descs, const int2* tiles, int n, int shape, float slope,
+                 cudaStream_t st);
 template <typename T>
 void launch_gemv(const GemvDesc* descs, int n_problems, int max_rows, cudaStream_t st);
 template <typename T>
@@ -177,9 +179,24 @@ void launch_centre_select(int cells, int off, const SelectParams& p, const Selec
 void launch_fitness_select(const float* logits, int cells, int B, float* LG, float* LD,
                            float* fG, float* fD, int* flag, const int* nbr,
                            const SelectParams& p, const SelectIO& io, cudaStream_t st);
+// Training inputs of every cell's selected pair from the evaluation: TX (real rows, the selected
+// generator's fakes) and, where H1g .. are given (the CUDA-core evaluation stores every slot's
+// activations), the generator's TH1, TH2 and the discriminator's TG1, TG2, TL.
+struct TrainGather {
+  const void* E;
+  int64_t e_cell;
+  const int *sel_g, *sel_d;
+  void* TX;
+  const void *H1g, *H2g;  // [cells][5][B][h]; null: TH1, TH2 stay
+  void *TH1, *TH2;
+  const void *H1d, *H2d;  // [cells][5][6B][h]; null: TG1, TG2, TL stay
+  const float* logits;
+  void *TG1, *TG2;
+  float* TL;
+};
 template <typename T>
-void launch_train_prep(const T* E, int64_t e_cell, const int* sel_g, T* TX, int cells, int B,
-                       int x_dim, cudaStream_t st);
+void launch_train_gather(const TrainGather& t, int cells, int B, int x_dim, int hidden,
+                         cudaStream_t st);
 // sync (null: none): the tensor-core backward's counters, [cells][sync_words] and sync_words more,
 // which this kernel clears (the backward is the next launch)
 template <typename T>
@@ -187,8 +204,15 @@ void launch_dlogit(const float* TL, const T* TG2, const T* wD, int64_t wD_stride
                    const int* src_d, int cells, int B, int H, float slope, T* J2, float* gD,
                    int64_t gD_stride, int64_t off_gw3, int64_t off_gb3, int64_t off_gb2, int* sync,
                    int sync_words, cudaStream_t st);
-void launch_adam(const PopView& old_p, const PopView& new_p, const float* grad, const int* src,
-                 const float4* coef, int cells, int64_t P, int64_t Ps, float beta1, float beta2,
+// One population's Adam step + replacement (launch_adam runs both populations in one launch).
+struct AdamPopArgs {
+  PopView old_p, new_p;
+  const float* grad;
+  const int* src;
+  const float4* coef;
+  int64_t P, Ps;
+};
+void launch_adam(const AdamPopArgs& g, const AdamPopArgs& d, int cells, float beta1, float beta2,
                  float eps, cudaStream_t st);
 
 // Adam + replacement restricted to n parameter ranges [off[q], off[q] + len[q]) of every cell

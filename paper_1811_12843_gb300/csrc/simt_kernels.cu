@@ -220,16 +220,95 @@ template void launch_draw_batch<bf16>(const bf16*, int64_t, const float*, bf16*,
                                       cudaStream_t);
 
 // ------------------------------------------------------------------------------------------
-// Grouped GEMM on CUDA cores: 64x64 output tile per block, k-slices of 16 staged in shared
-// memory as fp32, 4x4 outputs per thread, fp32 accumulation in k order.
+// Grouped GEMM on CUDA cores: one output tile of one problem per block, k-slices of 16 staged in
+// shared memory as fp32 (double-buffered; the next slice's global loads are in flight while this
+// one is multiplied), TM x TN outputs per thread as packed pairs along n, fp32 accumulation in k
+// order. Bound: shared-memory reads and FMA pipes alike (an 8 x 8 thread reads 16 values for 64
+// multiply-adds: ncu 68 % and 66 %): 43 TFLOP/s on the 45 discriminator layers 600 x 256 x 784 of a
+// 3x3 grid (18 before, with 64 x 64 tiles, 4 x 4 outputs per thread and scalar loads between two
+// barriers per slice). Scalar FMA was 10-18 % slower, 8 x 16 outputs per thread spill.
 // ------------------------------------------------------------------------------------------
-template <typename TI, typename TO, int EPI>
-__global__ void __launch_bounds__(256) k_gemm(const GemmDesc* __restrict__ descs, int act,
-                                              float slope) {
+constexpr int GEMM_BK = 16;
+
+// d.x = a.x * b.x + d.x, d.y = a.y * b.y + d.y, each rounded once, as fmaf: half the instructions
+__device__ __forceinline__ void fma2(unsigned long long& d, unsigned long long a,
+                                     unsigned long long b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ unsigned long long dup2(float a) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(a));
+  return r;
+}
+
+template <typename T>
+__device__ __forceinline__ float4 load4(const T* p);
+template <>
+__device__ __forceinline__ float4 load4<float>(const float* p) {
+  return __ldg(reinterpret_cast<const float4*>(p));
+}
+template <>
+__device__ __forceinline__ float4 load4<bf16>(const bf16* p) {
+  const uint2 q = __ldg(reinterpret_cast<const uint2*>(p));
+  const float2 lo = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&q.x));
+  const float2 hi = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&q.y));
+  return make_float4(lo.x, lo.y, hi.x, hi.y);
+}
+
+// One operand's k-slice [R rows][16 k] in registers: V groups of four elements per thread, along
+// k (kfast) or along the rows.
+template <typename T, int R, int NT>
+struct GemmSlice {
+  static constexpr int V = R * GEMM_BK / 4 / NT;
+  static_assert(V * NT * 4 == R * GEMM_BK, "slice");
+  float4 v[V];
+  __device__ __forceinline__ void fetch(const T* p, int64_t sr, int64_t sk, bool kfast, bool vec,
+                                        int r0, int rows, int k0, int K) {
+#pragma unroll
+    for (int u = 0; u < V; ++u) {
+      const int id = threadIdx.x + u * NT;
+      const int r = r0 + (kfast ? id / 4 : id % (R / 4) * 4);
+      const int k = k0 + (kfast ? id % 4 * 4 : id / (R / 4));
+      const T* q = p + r * sr + k * sk;
+      v[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (r >= rows || k >= K) continue;
+      if (vec) {
+        v[u] = load4<T>(q);
+      } else {
+        const int n = kfast ? K - k : rows - r;
+        const int64_t st = kfast ? sk : sr;
+        v[u].x = to_f<T>(q[0]);
+        if (n > 1) v[u].y = to_f<T>(q[st]);
+        if (n > 2) v[u].z = to_f<T>(q[2 * st]);
+        if (n > 3) v[u].w = to_f<T>(q[3 * st]);
+      }
+    }
+  }
+  __device__ __forceinline__ void stash(float (*s)[R + 4], bool kfast) const {
+#pragma unroll
+    for (int u = 0; u < V; ++u) {
+      const int id = threadIdx.x + u * NT;
+      if (kfast) {
+        const int r = id / 4, k = id % 4 * 4;
+        s[k][r] = v[u].x;
+        s[k + 1][r] = v[u].y;
+        s[k + 2][r] = v[u].z;
+        s[k + 3][r] = v[u].w;
+      } else {
+        *reinterpret_cast<float4*>(&s[id / (R / 4)][id % (R / 4) * 4]) = v[u];
+      }
+    }
+  }
+};
+
+template <typename TI, int BM, int BN, int TM, int TN>
+__global__ void __launch_bounds__(BM / TM * (BN / TN))
+    k_gemm(const GemmDesc* __restrict__ descs, const int2* __restrict__ tiles, float slope) {
+  constexpr int NT = BM / TM * (BN / TN);
   pdl_wait();
-  const GemmDesc d = descs[blockIdx.z];
-  const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
-  if (m0 >= d.M || n0 >= d.N) return;
+  const int2 tl = __ldg(&tiles[blockIdx.x]);
+  const GemmDesc d = descs[tl.x];
+  const int m0 = (tl.y >> 16) * BM, n0 = (tl.y & 0xFFFF) * BN;
   const TI* A = (const TI*)d.A;
   const TI* Bm = (const TI*)d.B;
   const float* bias = d.bias;
@@ -238,84 +317,98 @@ __global__ void __launch_bounds__(256) k_gemm(const GemmDesc* __restrict__ descs
     if (d.wsel_op == 1) A += off; else Bm += off;
     if (bias) bias += off;
   }
-  __shared__ float As[16][64 + 4];
-  __shared__ float Bs[16][64 + 4];
-  const int tid = threadIdx.x;
-  const int tm = (tid >> 4) * 4, tn = (tid & 15) * 4;
-  float acc[4][4];
+  __shared__ __align__(16) float As[2][GEMM_BK][BM + 4];
+  __shared__ __align__(16) float Bs[2][GEMM_BK][BN + 4];
+  // a thread's rows: groups of four, 4 BM / TM apart, from ty * 4; columns likewise, so that the
+  // lanes of a warp read consecutive 16-byte units
+  const int tx = threadIdx.x % (BN / TN), ty = threadIdx.x / (BN / TN);
+  unsigned long long acc[TM][TN / 2];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < TM; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-  const bool a_kfast = d.sak == 1, b_nfast = d.sbn == 1;
-  for (int k0 = 0; k0 < d.K; k0 += 16) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int idx = tid + 256 * i;
-      int m, k;
-      if (a_kfast) { m = idx >> 4; k = idx & 15; } else { m = idx & 63; k = idx >> 6; }
-      float v = 0.f;
-      if (m0 + m < d.M && k0 + k < d.K)
-        v = to_f<TI>(A[(int64_t)(m0 + m) * d.sam + (int64_t)(k0 + k) * d.sak]);
-      As[k][m] = v;
-      int n, kk;
-      if (b_nfast) { n = idx & 63; kk = idx >> 6; } else { n = idx >> 4; kk = idx & 15; }
-      float w = 0.f;
-      if (n0 + n < d.N && k0 + kk < d.K)
-        w = to_f<TI>(Bm[(int64_t)(k0 + kk) * d.sbk + (int64_t)(n0 + n) * d.sbn]);
-      Bs[kk][n] = w;
+    for (int j = 0; j < TN / 2; ++j) acc[i][j] = 0ull;
+  const bool akf = d.sak == 1, bkf = d.sbk == 1;
+  const bool av = d.vec & GEMM_VEC_A, bv = d.vec & GEMM_VEC_B;
+  GemmSlice<TI, BM, NT> fa;
+  GemmSlice<TI, BN, NT> fb;
+  fa.fetch(A, d.sam, d.sak, akf, av, m0, d.M, 0, d.K);
+  fb.fetch(Bm, d.sbn, d.sbk, bkf, bv, n0, d.N, 0, d.K);
+  fa.stash(As[0], akf);
+  fb.stash(Bs[0], bkf);
+  __syncthreads();
+  int cur = 0;
+  for (int k0 = 0; k0 < d.K; k0 += GEMM_BK, cur ^= 1) {
+    const bool more = k0 + GEMM_BK < d.K;
+    if (more) {
+      fa.fetch(A, d.sam, d.sak, akf, av, m0, d.M, k0 + GEMM_BK, d.K);
+      fb.fetch(Bm, d.sbn, d.sbk, bkf, bv, n0, d.N, k0 + GEMM_BK, d.K);
     }
-    __syncthreads();
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-      float a[4], b[4];
+    for (int k = 0; k < GEMM_BK; ++k) {
+      float a[TM];
+      unsigned long long b[TN / 2];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[k][tm + i];
+      for (int i = 0; i < TM; i += 4)
+        *reinterpret_cast<float4*>(&a[i]) =
+            *reinterpret_cast<const float4*>(&As[cur][k][i * BM / TM + ty * 4]);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[k][tn + j];
+      for (int j = 0; j < TN; j += 4)
+        *reinterpret_cast<ulonglong2*>(&b[j / 2]) =
+            *reinterpret_cast<const ulonglong2*>(&Bs[cur][k][j * BN / TN + tx * 4]);
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < TM; ++i) {
+        const unsigned long long aa = dup2(a[i]);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+        for (int j = 0; j < TN / 2; ++j) fma2(acc[i][j], aa, b[j]);
+      }
+    }
+    if (more) {
+      fa.stash(As[cur ^ 1], akf);
+      fb.stash(Bs[cur ^ 1], bkf);
     }
     __syncthreads();
   }
-  TO* C = (TO*)d.C;
   const TI* aux = (const TI*)d.aux;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int m = m0 + tm + i;
+  for (int i = 0; i < TM; ++i) {
+    const int m = m0 + i / 4 * (4 * BM / TM) + ty * 4 + i % 4;
     if (m >= d.M) continue;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int n = n0 + tn + j;
+    for (int j = 0; j < TN; ++j) {
+      const int n = n0 + j / 4 * (4 * BN / TN) + tx * 4 + j % 4;
       if (n >= d.N) continue;
-      float v = acc[i][j];
-      if (EPI == EPI_BIAS_ACT) {
-        v = act_fwd(act, v + (bias ? bias[n] : 0.f), slope);
-      } else if (EPI == EPI_DACT) {
-        v *= act_bwd(act, to_f<TI>(aux[(int64_t)m * d.sxm + (int64_t)n * d.sxn]), slope);
+      float v = __uint_as_float((uint32_t)(acc[i][j / 2] >> (j % 2 * 32)));
+      const int64_t at = (int64_t)m * d.scm + (int64_t)n * d.scn;
+      if (d.epi == EPI_STORE) {
+        ((float*)d.C)[at] = v;
+        continue;
       }
-      C[(int64_t)m * d.scm + (int64_t)n * d.scn] = from_f<TO>(v);
+      if (d.epi == EPI_BIAS_ACT)
+        v = act_fwd(d.act, v + (bias ? bias[n] : 0.f), slope);
+      else
+        v *= act_bwd(d.act, to_f<TI>(aux[(int64_t)m * d.sxm + (int64_t)n * d.sxn]), slope);
+      ((TI*)d.C)[at] = from_f<TI>(v);
     }
   }
 }
 
-template <typename TI, typename TO, int EPI>
-void launch_gemm(const GemmDesc* descs, int n_problems, int max_m, int max_n, int act,
-                 float slope, cudaStream_t st) {
-  if (n_problems <= 0 || max_m <= 0 || max_n <= 0) return;
-  dim3 grid((max_n + 63) / 64, (max_m + 63) / 64, n_problems);
-  launch_pdl(k_gemm<TI, TO, EPI>, grid, dim3(256), 0, st, descs, act, slope);
+template <typename TI>
+void launch_gemm(const GemmDesc* descs, const int2* tiles, int n, int shape, float slope,
+                 cudaStream_t st) {
+  if (n <= 0) return;
+  switch (shape) {
+    case 0:
+      launch_pdl(k_gemm<TI, 128, 64, 8, 8>, dim3(n), dim3(128), 0, st, descs, tiles, slope);
+      break;
+    case 1:
+      launch_pdl(k_gemm<TI, 32, 64, 4, 8>, dim3(n), dim3(64), 0, st, descs, tiles, slope);
+      break;
+    default:
+      launch_pdl(k_gemm<TI, 32, 32, 4, 4>, dim3(n), dim3(64), 0, st, descs, tiles, slope);
+  }
 }
-#define LIPZ_INST_GEMM(TI, TO, EPI) \
-  template void launch_gemm<TI, TO, EPI>(const GemmDesc*, int, int, int, int, float, cudaStream_t);
-LIPZ_INST_GEMM(float, float, EPI_STORE)
-LIPZ_INST_GEMM(float, float, EPI_BIAS_ACT)
-LIPZ_INST_GEMM(float, float, EPI_DACT)
-LIPZ_INST_GEMM(bf16, float, EPI_STORE)
-LIPZ_INST_GEMM(bf16, bf16, EPI_BIAS_ACT)
-LIPZ_INST_GEMM(bf16, bf16, EPI_DACT)
+template void launch_gemm<float>(const GemmDesc*, const int2*, int, int, float, cudaStream_t);
+template void launch_gemm<bf16>(const GemmDesc*, const int2*, int, int, float, cudaStream_t);
 
 // ------------------------------------------------------------------------------------------
 // Discriminator output layer: one warp per row, lanes stride over k, fixed shuffle tree.
@@ -603,38 +696,55 @@ void launch_centre_select(int cells, int off, const SelectParams& p, const Selec
 }
 
 // ------------------------------------------------------------------------------------------
-// Training input of cell c: TX[c] = [E[c] rows [0, B); E[c] rows of generator slot sel_g[c]].
+// Training inputs of cell c's selected pair (TrainGather), a warp per row r of [real rows, fakes]:
+// the row of E, and what the evaluation stored for it in the selected slots.
 // ------------------------------------------------------------------------------------------
 template <typename T>
-__global__ void k_train_prep(const T* __restrict__ E, int64_t e_cell, const int* __restrict__ sel_g,
-                             T* __restrict__ TX, int B, int x_dim) {
-  pdl_wait();
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int r = blockIdx.x * (blockDim.x >> 5) + warp, c = blockIdx.y;
-  if (r >= 2 * B) return;
-  const int src_row = r < B ? r : B * (1 + sel_g[c]) + (r - B);
-  const T* s = E + (int64_t)c * e_cell + (int64_t)src_row * x_dim;
-  T* d = TX + ((int64_t)c * 2 * B + r) * x_dim;
-  const int bytes = x_dim * (int)sizeof(T);
+__device__ __forceinline__ void copy_row(const void* src, int64_t so, void* dst, int64_t d_o, int n,
+                                         int lane) {
+  const T* s = (const T*)src + so;
+  T* d = (T*)dst + d_o;
+  const int bytes = n * (int)sizeof(T);
   if ((bytes & 15) == 0 && (((uintptr_t)s | (uintptr_t)d) & 15) == 0) {
     const uint4* s4 = reinterpret_cast<const uint4*>(s);
     uint4* d4 = reinterpret_cast<uint4*>(d);
-    for (int k = lane; k < bytes / 16; k += 32) d4[k] = s4[k];
+    for (int k = lane; k < bytes / 16; k += 32) d4[k] = __ldg(s4 + k);
   } else {
-    for (int k = lane; k < x_dim; k += 32) d[k] = s[k];
+    for (int k = lane; k < n; k += 32) d[k] = s[k];
   }
 }
 
 template <typename T>
-void launch_train_prep(const T* E, int64_t e_cell, const int* sel_g, T* TX, int cells, int B,
-                       int x_dim, cudaStream_t st) {
-  launch_pdl(k_train_prep<T>, dim3((2 * B + 7) / 8, cells), dim3(256), 0, st, E, e_cell, sel_g,
-             TX, B, x_dim);
+__global__ void k_train_gather(TrainGather t, int B, int x_dim, int h) {
+  pdl_wait();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int r = blockIdx.x * (blockDim.x >> 5) + warp, c = blockIdx.y;
+  if (r >= 2 * B) return;
+  const int sg = t.sel_g[c];
+  const int row = r < B ? r : B * (1 + sg) + (r - B);  // among the cell's 6B evaluation rows
+  copy_row<T>(t.E, (int64_t)c * t.e_cell + (int64_t)row * x_dim, t.TX,
+              ((int64_t)c * 2 * B + r) * x_dim, x_dim, lane);
+  if (t.H1g && r < B) {
+    const int64_t s = (((int64_t)c * 5 + sg) * B + r) * h, d = ((int64_t)c * B + r) * h;
+    copy_row<T>(t.H1g, s, t.TH1, d, h, lane);
+    copy_row<T>(t.H2g, s, t.TH2, d, h, lane);
+  }
+  if (t.H1d) {
+    const int64_t s = ((int64_t)c * 5 + t.sel_d[c]) * 6 * B + row, d = (int64_t)c * 2 * B + r;
+    copy_row<T>(t.H1d, s * h, t.TG1, d * h, h, lane);
+    copy_row<T>(t.H2d, s * h, t.TG2, d * h, h, lane);
+    if (lane == 0) t.TL[d] = t.logits[s];
+  }
 }
-template void launch_train_prep<float>(const float*, int64_t, const int*, float*, int, int, int,
-                                       cudaStream_t);
-template void launch_train_prep<bf16>(const bf16*, int64_t, const int*, bf16*, int, int, int,
-                                      cudaStream_t);
+
+template <typename T>
+void launch_train_gather(const TrainGather& t, int cells, int B, int x_dim, int hidden,
+                         cudaStream_t st) {
+  launch_pdl(k_train_gather<T>, dim3((2 * B + 7) / 8, cells), dim3(256), 0, st, t, B, x_dim,
+             hidden);
+}
+template void launch_train_gather<float>(const TrainGather&, int, int, int, int, cudaStream_t);
+template void launch_train_gather<bf16>(const TrainGather&, int, int, int, int, cudaStream_t);
 
 // ------------------------------------------------------------------------------------------
 // Logit deltas of the selected pair of cell c, rows [real, fake (D loss), fake (G loss)]:
@@ -685,43 +795,51 @@ __global__ void __launch_bounds__(512) k_dlogit(
     acc2[e] = 0.f;
   }
   if (rg < RG) {
-    const bool vec = sizeof(T) == 2 && (H & 7) == 0;
-    // the rows of this thread in groups of eight, the eight loads issued before any is used (one
-    // memory latency per group); rows are still taken in increasing order
-    constexpr int U = 8;
+    const bool vec = (H & 7) == 0;
+    // the rows of this thread in groups of U, the groups' loads (16 bytes each, eight in flight)
+    // issued before any is used (one memory latency per group); rows are still taken in
+    // increasing order
+    constexpr int Q = (int)sizeof(T) / 2;  // 16-byte vectors per eight columns
+    constexpr int U = 8 / Q;
     for (int r0 = rg; vec && r0 < 3 * B; r0 += U * RG) {
-      uint4 qv[U];
+      uint4 qv[U][Q];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int r = r0 + u * RG;
         const int rr = r < 2 * B ? r : r - B;
-        if (r < 3 * B) qv[u] = *reinterpret_cast<const uint4*>(g2 + (int64_t)rr * H + k0);
+        if (r < 3 * B)
+#pragma unroll
+          for (int i = 0; i < Q; ++i)
+            qv[u][i] = reinterpret_cast<const uint4*>(g2 + (int64_t)rr * H + k0)[i];
       }
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int r = r0 + u * RG;
         if (r >= 3 * B) break;
         const float dr = dl[r];
-        // eight bf16 columns in one 16-byte load and store
-        const uint4 q = qv[u];
-        const uint32_t w[4] = {q.x, q.y, q.z, q.w};
-        uint32_t o[4];
+        float g[8], y[8];
+        if constexpr (Q == 1) {
+          const uint32_t w[4] = {qv[u][0].x, qv[u][0].y, qv[u][0].z, qv[u][0].w};
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const __nv_bfloat162 v = *reinterpret_cast<const __nv_bfloat162*>(&w[e]);
-          const float g0 = __low2float(v), g1 = __high2float(v);
-          const float y0 = dr * wk[2 * e] * (g0 > 0.f ? 1.f : slope);
-          const float y1 = dr * wk[2 * e + 1] * (g1 > 0.f ? 1.f : slope);
-          __nv_bfloat162 y = __floats2bfloat162_rn(y0, y1);
-          o[e] = *reinterpret_cast<uint32_t*>(&y);
+          for (int e = 0; e < 4; ++e) {
+            const __nv_bfloat162 v = *reinterpret_cast<const __nv_bfloat162*>(&w[e]);
+            g[2 * e] = __low2float(v);
+            g[2 * e + 1] = __high2float(v);
+          }
+        } else {
+          *reinterpret_cast<uint4*>(&g[0]) = qv[u][0];
+          *reinterpret_cast<uint4*>(&g[4]) = qv[u][Q - 1];
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          y[e] = dr * wk[e] * (g[e] > 0.f ? 1.f : slope);
           if (r < 2 * B) {
-            acc[2 * e] = fmaf(dr, g0, acc[2 * e]);
-            acc[2 * e + 1] = fmaf(dr, g1, acc[2 * e + 1]);
-            acc2[2 * e] += y0;
-            acc2[2 * e + 1] += y1;
+            acc[e] = fmaf(dr, g[e], acc[e]);
+            acc2[e] += y[e];
           }
         }
-        *reinterpret_cast<uint4*>(j2 + (int64_t)r * H + k0) = make_uint4(o[0], o[1], o[2], o[3]);
+        store4<T>(j2 + (int64_t)r * H + k0, make_float4(y[0], y[1], y[2], y[3]));
+        store4<T>(j2 + (int64_t)r * H + k0 + 4, make_float4(y[4], y[5], y[6], y[7]));
       }
     }
     for (int r = rg; !vec && r < 3 * B; r += RG) {
@@ -801,15 +919,16 @@ __device__ __forceinline__ void adam4(float4& w, float4& m, float4& v, const flo
   adam_elem(w.w, m.w, v.w, g.w, b1, b2, lr, ib1, ib2, eps);
 }
 
-__global__ void __launch_bounds__(256) k_adam(PopView old_p, PopView new_p,
-                                              const float* __restrict__ grad,
-                                              const int* __restrict__ src,
-                                              const float4* __restrict__ coef, int64_t P,
-                                              int64_t Ps, float beta1, float beta2, float eps) {
+__global__ void __launch_bounds__(256) k_adam(AdamPopArgs pg, AdamPopArgs pd, float beta1,
+                                              float beta2, float eps) {
   pdl_wait();
   const int c = blockIdx.y;
-  const int s = src[c];
-  const float4 cf = coef[c];
+  const AdamPopArgs& a = blockIdx.z ? pd : pg;
+  const PopView &old_p = a.old_p, &new_p = a.new_p;
+  const float* __restrict__ grad = a.grad;
+  const int64_t P = a.P, Ps = a.Ps;
+  const int s = a.src[c];
+  const float4 cf = a.coef[c];
   const float lr = cf.x, ib1 = cf.y, ib2 = cf.z;
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     new_p.step[c] = (int)cf.w;
@@ -854,17 +973,15 @@ __global__ void __launch_bounds__(256) k_adam(PopView old_p, PopView new_p,
   }
 }
 
-void launch_adam(const PopView& old_p, const PopView& new_p, const float* grad, const int* src,
-                 const float4* coef, int cells, int64_t P, int64_t Ps, float beta1, float beta2,
+void launch_adam(const AdamPopArgs& g, const AdamPopArgs& d, int cells, float beta1, float beta2,
                  float eps, cudaStream_t st) {
-  // about 8 resident 256-thread blocks per SM over the whole population
+  // about 8 resident 256-thread blocks per SM over each whole population
+  const int64_t P = g.P > d.P ? g.P : d.P;
   int per_cell = (int)((P / 4 + 255) / 256);
   const int target = (152 * 8 + cells - 1) / cells;
   if (per_cell > target * 4) per_cell = target * 4;
   if (per_cell < 1) per_cell = 1;
-  dim3 grid(per_cell, cells);
-  launch_pdl(k_adam, grid, dim3(256), 0, st, old_p, new_p, grad, src, coef, P, Ps, beta1, beta2,
-             eps);
+  launch_pdl(k_adam, dim3(per_cell, cells, 2), dim3(256), 0, st, g, d, beta1, beta2, eps);
 }
 
 // ------------------------------------------------------------------------------------------
