@@ -118,9 +118,10 @@ struct lipz_grid {
   int* bsync = nullptr;  // the tensor-core backward's tile counters
   int* flag = nullptr;
   // generator-mixture weights [cells][5] (always held: part of the state), and with
-  // arch.mixture the score's work buffers: row norms [cells][6B], per-row block sums
-  // [cells][6B][mix_nh][6], block means [cells][6][6], scores [cells]; the CUDA-core path
-  // stores the Gram matrices [cells][6B][6B] first
+  // arch.mixture the score's work buffers: row norms [cells][6B], block sums (per 32 rows, 128
+  // columns and block from the tensor-core Gram kernel, else [cells][6B][6]), block means
+  // [cells][6][6], scores [cells]; the CUDA-core path stores the Gram matrices [cells][6B][6B]
+  // first
   float *mix = nullptr, *rnorm = nullptr, *mixP = nullptr, *mixS = nullptr, *mixScore = nullptr;
   float* gram = nullptr;
   GemmSet dgram;
@@ -725,7 +726,7 @@ int create_impl(lipz_grid* g) {
     g->mix_tc = g->bf && !g->a.force_simt && tc_supported(z, h, x, B) && tc_gram_supported(B);
     g->mix_nh = g->mix_tc ? tc_gram_halves(B) : 1;
     if ((rc = dalloc(g, &g->rnorm, C * R * 4)) ||
-        (rc = dalloc(g, &g->mixP, C * R * g->mix_nh * 6 * 4)) ||
+        (rc = dalloc(g, &g->mixP, (g->mix_tc ? C * tc_gram_floats(B) : C * R * 6) * 4)) ||
         (rc = dalloc(g, &g->mixS, C * 36 * 4)) || (rc = dalloc(g, &g->mixScore, C * 4)) ||
         (rc = dset(g, g->mixS, 0, C * 36 * 4)) || (rc = dset(g, g->mixScore, 0, C * 4)))
       return rc;
@@ -915,7 +916,7 @@ int mixture_impl(lipz_grid* g) {
     launch_mix_partials(g->gram, g->rnorm, C, R, B, x, g->mixP, g->st);
   }
   CKL(g);
-  launch_mix_es(g->mixP, g->mix_nh, C, R, B, g->mix, g->mixS, g->mixScore, g->seed,
+  launch_mix_es(g->mixP, g->mix_nh, g->mix_tc, C, R, B, g->mix, g->mixS, g->mixScore, g->seed,
                 (uint32_t)g->t, g->a.mix_sigma, g->st);
   CKL(g);
   phase_end(g, LIPZ_PHASE_MIXTURE, g->mix_tc ? 3 : 4);

@@ -48,6 +48,9 @@ constexpr int THREADS = 64 + 32 * NUM_EPI_WARPS;
 constexpr int MISC_BYTES = 2048;
 constexpr int BIAS_MAX = 256 + 256 + 1024;  // floats per tile: b1, b2, then b3 (G) or w3, b3 (D)
 constexpr int BIAS_BYTES = 2 * BIAS_MAX * 4;  // double-buffered by tile
+// floats of one buffer of row norms (Gram kind, which has no on-chip activation: its region holds
+// two)
+constexpr int GRAM_NORMS = H_BYTES / 8;
 constexpr int SMEM_BYTES = 1024 + STAGES * STAGE_BYTES + H_BYTES + MISC_BYTES + BIAS_BYTES;
 
 enum { KIND_G = 0, KIND_D = 1, KIND_GRAM = 2 };
@@ -85,10 +88,12 @@ struct KParams {
   // written to E[c] as the fakes of slot 0
   int centre;
   int indiv_off;  // centre-only mode: individual index of cell 0's centre (snapshot * cells)
-  // Gram kind (mixture score): problem c is the Gram matrix of E[c]'s rows with themselves,
-  // reduced in the epilogue to per-row sums of exp(-||e_r - e_s||^2 / x) over the columns s of
-  // each block of B rows. rnorm [cells][rows] holds ||e_r||^2; the sums go to
-  // gram_out[cell][row][half][6], half = 2 * column block + column half of the tile.
+  // Gram kind (mixture score): problem c is the Gram matrix of E[c]'s rows with themselves, its
+  // upper triangle only (the column blocks from the row tile's on; elements left of the diagonal
+  // count zero, those on it a half), reduced in the epilogue to sums of exp(-||e_r - e_s||^2 / x)
+  // over the 32 rows r of a warp in each of the (at most two) blocks of B rows they meet and the
+  // columns s of each block. rnorm [cells][rows] holds ||e_r||^2; the sums go to
+  // gram_out[cell][row tile][row quarter][half][2][6], half = 2 * column block + column half.
   const float* rnorm;
   float* gram_out;
 };
@@ -130,6 +135,31 @@ template <int KND>
 __device__ __forceinline__ int n_jobs(const KParams& p) {
   if (KND == KIND_GRAM) return (p.rows + HID - 1) / HID;
   return (KND == KIND_D || p.train) ? 2 : 2 + p.n3;
+}
+
+// First job of a tile: the Gram kind starts at the column block that holds its diagonal.
+template <int KND>
+__device__ __forceinline__ int first_job(int m0) {
+  return KND == KIND_GRAM ? m0 / HID : 0;
+}
+
+// A tile's problem and first row. The Gram kind's tiles go from the longest (row tile 0 of every
+// cell) to the shortest, every other round of the CTAs backwards, so that their sums balance.
+template <int KND>
+__device__ __forceinline__ void tile_place(const KParams& p, int tile, int& prob, int& m0) {
+  if (KND == KIND_GRAM) {
+    const int g = (int)gridDim.x, round = tile / g;
+    if (round & 1) {
+      const int last = min(g, p.n_tiles - round * g) - 1;
+      // (a partial round: the CTAs without a tile are those that had the shortest before)
+      tile = round * g + last - (tile - round * g);
+    }
+    prob = tile % p.cells;
+    m0 = tile / p.cells * BM;
+  } else {
+    prob = tile / p.mtiles;
+    m0 = tile % p.mtiles * BM;
+  }
 }
 
 // Problem -> (cell whose activations are the A operand, individual whose weights are B).
@@ -230,10 +260,11 @@ __global__ void __launch_bounds__(THREADS, 1)
       int issued[STAGES] = {0, 0, 0};
       bool ok = true;
       for (int tile = blockIdx.x; tile < p.n_tiles && ok; tile += gridDim.x) {
-        const int prob = tile / p.mtiles, m0 = (tile % p.mtiles) * BM;
+        int prob, m0;
+        tile_place<KND>(p, tile, prob, m0);
         const int c = prob_cell<KND>(p, prob);
         const int k = prob_individual<KND>(p, prob);
-        for (int j = 0; j < nj && ok; ++j) {
+        for (int j = first_job<KND>(m0); j < nj && ok; ++j) {
           const Job J = get_job<KND>(p, j);
           const CUtensorMap* mb = J.bmap == 0 ? &mB1 : (J.bmap == 1 ? &mB2 : &mB3);
           for (int kc = 0; kc < J.kchunks; ++kc) {
@@ -282,7 +313,9 @@ __global__ void __launch_bounds__(THREADS, 1)
       bool ok = true;
       int jobs_done = 0;
       for (int tile = blockIdx.x; tile < p.n_tiles && ok; tile += gridDim.x) {
-        for (int j = 0; j < nj && ok; ++j, ++jobs_done) {
+        int prob, m0;
+        tile_place<KND>(p, tile, prob, m0);
+        for (int j = first_job<KND>(m0); j < nj && ok; ++j, ++jobs_done) {
           const Job J = get_job<KND>(p, j);
           // the Gram kind alternates the two accumulators over all its jobs (3 per tile)
           const int R = KND == KIND_GRAM ? (jobs_done & 1) : J.region;
@@ -342,7 +375,8 @@ __global__ void __launch_bounds__(THREADS, 1)
     int ltile = 0, jobs_done = 0;
     const int et = threadIdx.x - 64;  // epilogue thread 0..255
     for (int tile = blockIdx.x; tile < p.n_tiles && ok; tile += gridDim.x, ++ltile) {
-      const int prob = tile / p.mtiles, m0 = (tile % p.mtiles) * BM;
+      int prob, m0;
+      tile_place<KND>(p, tile, prob, m0);
       const int c = prob_cell<KND>(p, prob), slot = p.centre ? 0 : prob % 5;
       const int k = prob_individual<KND>(p, prob);
       const float* wm = p.wmaster ? p.wmaster + (int64_t)k * p.pstride : nullptr;
@@ -352,7 +386,9 @@ __global__ void __launch_bounds__(THREADS, 1)
       // The tile's biases (and D's output weights) go to shared memory once, while the MMAs
       // run, so that no epilogue waits on a global load. Buffer ltile & 1; a thread cannot
       // reach tile ltile + 2 before every thread has passed this tile's arrival.
-      float* sb = s_bias + (ltile & 1) * BIAS_MAX;
+      float* sb = KND == KIND_GRAM ? reinterpret_cast<float*>(gbase + STAGES * STAGE_BYTES) +
+                                         (ltile & 1) * GRAM_NORMS
+                                   : s_bias + (ltile & 1) * BIAS_MAX;
       if (KND == KIND_GRAM) {
         // the squared norms of the cell's rows (the Gram tile's row and column terms)
         // -|e_s|^2 / x for the cell's rows s, zero for the 32 entries past the last row
@@ -395,7 +431,7 @@ __global__ void __launch_bounds__(THREADS, 1)
           break;
         }
       }
-      for (int j = 0; j < nj && ok; ++j, ++jobs_done) {
+      for (int j = first_job<KND>(m0); j < nj && ok; ++j, ++jobs_done) {
         const Job J = get_job<KND>(p, j);
         const int R = KND == KIND_GRAM ? (jobs_done & 1) : J.region;
         if (!mbar_wait_warp(bAcc + 8 * R, (uint32_t)(reg_uses[R] & 1), abort_flag, p.err, 6)) {
@@ -529,10 +565,12 @@ __global__ void __launch_bounds__(THREADS, 1)
           }
         } else if (J.epi == EPI_GRAM) {
           // Gaussian kernel exp((2 e_r.e_s - |e_r|^2 - |e_s|^2) / x) of this thread's row r
-          // against the warp's 128 columns s, summed per column block of B >= 32 rows: a group
+          // against the warp's 128 columns s >= r, summed per column block of B >= 32 rows: a group
           // of 32 columns meets at most one block boundary (at column sp of the group, the same
           // for every lane), columns past the last row count zero; two interleaved partial sums
-          // per side, combined in a fixed order
+          // per side, combined in a fixed order. (Bound: the exponentials beside the MMAs. Mixture
+          // phase at 5x5, B = 256: 74 us, 5025 with the stored Gram matrix of the CUDA-core path,
+          // which batches above 250 took; the triangle halves the work of the full square.)
           const float nr = row_ok ? sb[rr] : 0.f;
           const float two_ix = 2.f / (float)p.x;
           float acc[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
@@ -540,12 +578,15 @@ __global__ void __launch_bounds__(THREADS, 1)
           for (int cg = hf * 4; cg < hf * 4 + 4; ++cg) {
             const int col0 = J.brow0 + cg * 32;
             if (col0 >= p.rows) break;
+            if (col0 + 32 <= m0) continue;  // left of the tile's first row
             uint32_t r[32];
             LIPZ_TMEM_LD32(tbase + cg * 32, r);
             tmem_wait_ld();
             const int blk = col0 / p.B;
             const int sp = (blk + 1) * p.B - col0;
             const int nv = p.rows - col0;
+            const bool diag = col0 < m0 + BM;  // the tile's diagonal may cross the group
+            const int dg = rr - col0;          // this row's diagonal column in the group
             const float4* s4 = reinterpret_cast<const float4*>(sb + col0);
             float lo0 = 0.f, lo1 = 0.f, hi0 = 0.f, hi1 = 0.f;
 #pragma unroll
@@ -557,6 +598,7 @@ __global__ void __launch_bounds__(THREADS, 1)
                 const int e = 4 * q + u;
                 float v = __expf(fmaf(__uint_as_float(r[e]), two_ix, nr + nsv[u]));
                 v = e < nv ? v : 0.f;
+                if (diag) v = e > dg ? v : (e == dg ? 0.5f * v : 0.f);
                 const float vl = e < sp ? v : 0.f, vh = e < sp ? 0.f : v;
                 if (e & 1) {
                   lo1 += vl;
@@ -573,11 +615,24 @@ __global__ void __launch_bounds__(THREADS, 1)
           }
           tc_fence_before();
           mbar_arrive(bReg + 8 * R);
-          if (row_ok) {
-            float* o = p.gram_out + (((int64_t)c * p.rows + rr) * (2 * nj) + 2 * j + hf) * 6;
+          // the warp's rows in the block of its first row, and those in the next one
+          const int w0 = m0 + q * 32;
+          const bool first = rr < (w0 / p.B + 1) * p.B;
+          float out = 0.f;
 #pragma unroll
-            for (int t = 0; t < 6; ++t) o[t] = acc[t];
+          for (int t = 0; t < 6; ++t) {
+            float a0 = row_ok && first ? acc[t] : 0.f, a1 = row_ok && !first ? acc[t] : 0.f;
+#pragma unroll
+            for (int o = 16; o; o >>= 1) {
+              a0 += __shfl_xor_sync(0xffffffffu, a0, o);
+              a1 += __shfl_xor_sync(0xffffffffu, a1, o);
+            }
+            if (lane == t) out = a0;
+            if (lane == 6 + t) out = a1;
           }
+          if (lane < 12 && w0 < p.rows)
+            p.gram_out[((((int64_t)c * p.mtiles + m0 / BM) * 4 + q) * (2 * nj) + 2 * j + hf) * 12 +
+                       lane] = out;
         } else {
           // generator output block: bias + tanh, bf16, into the fake rows of E[c]
           const float* bias = sb + 512;
@@ -1635,7 +1690,7 @@ int tc_run_g_centre(TcPlan* p, cudaStream_t st, std::string* msg) {
 
 int tc_run_gram(TcPlan* p, cudaStream_t st, std::string* msg) {
   if (!p->pgram.rnorm || !p->pgram.gram_out || !tc_gram_supported(p->s.B)) {
-    if (msg) *msg = "tensor-core Gram kernel: no buffers, or batch outside 32..250";
+    if (msg) *msg = "tensor-core Gram kernel: no buffers, or batch outside 32..1360";
     return 1;
   }
   return launch(p->grid_gram, p->mE, p->mEB, p->mEB, p->mEB, p->pgram, st, "mixture Gram", msg);
@@ -1643,9 +1698,13 @@ int tc_run_gram(TcPlan* p, cudaStream_t st, std::string* msg) {
 
 int tc_gram_halves(int B) { return 2 * ((6 * B + tc::HID - 1) / tc::HID); }
 
+int64_t tc_gram_floats(int B) {
+  return (int64_t)((6 * B + tc::BM - 1) / tc::BM) * 4 * tc_gram_halves(B) * 12;
+}
+
 // B >= 32: a 32-column group meets at most one block boundary; the norms and 32 zero entries
-// past them fit one bias buffer
-bool tc_gram_supported(int B) { return B >= 32 && 6 * B + 32 <= tc::BIAS_MAX; }
+// past them fit one norm buffer (B <= 1360)
+bool tc_gram_supported(int B) { return B >= 32 && 6 * B + 32 <= tc::GRAM_NORMS; }
 
 int tc_run_d(TcPlan* p, cudaStream_t st, std::string* msg) {
   if (p->ncl_d > 0 && p->ppd.pairs)

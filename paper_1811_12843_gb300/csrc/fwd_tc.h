@@ -47,7 +47,7 @@ struct TcBuffers {
   int64_t PDs;
   const int64_t* doff;
   // mixture score: squared norms of E's rows [cells][6B] fp32 (input) and the Gram kernel's
-  // per-row block sums [cells][6B][tc_gram_halves(B)][6] fp32 (output); null without mixture
+  // block sums [cells][tc_gram_floats(B)] fp32 (output); null without mixture
   const float* rnorm;
   float* gram_out;
   int indiv_off;     // individual index of this snapshot's cell 0 (snapshot * cells)
@@ -87,11 +87,15 @@ void tc_set_nbr(TcPlan* p, const int* nbr, const TcPairs* pairs);
 // Generator forward of every cell's own centre on its z, into E's slot-0 fakes.
 int tc_run_g_centre(TcPlan* p, cudaStream_t st, std::string* msg);
 int tc_run_d(TcPlan* p, cudaStream_t st, std::string* msg);
-// Mixture score: for every cell c and row r of E[c], the sums over each block b of B columns
-// s of exp(-||E[c][r] - E[c][s]||^2 / x), into gram_out[c][r][h][b] split over the
-// tc_gram_halves(B) column ranges h (32 <= B <= 250, i.e. tc_gram_supported).
+// Mixture score: for every cell c and each 32 rows of E[c], the sums of
+// exp(-||E[c][r] - E[c][s]||^2 / x) over its rows r in the block of the first and in the next block
+// of B rows, and over the columns s > r (s = r counting a half) of each block, into
+// gram_out[c][row tile of 128][4][h][2][6], split over the tc_gram_halves(B) column ranges h of
+// 128 (ranges before the 256 columns that hold the tile's diagonal are not written).
+// 32 <= B <= 1360, i.e. tc_gram_supported.
 int tc_run_gram(TcPlan* p, cudaStream_t st, std::string* msg);
 int tc_gram_halves(int B);
+int64_t tc_gram_floats(int B);  // of gram_out, per cell
 bool tc_gram_supported(int B);
 // Training forward of every cell's selected generator (hidden activations into TH1, TH2) and
 // selected discriminator (TG1, TG2 and the logits TL).

@@ -1056,11 +1056,15 @@ __device__ __forceinline__ float mix_mmd2(const float* w, const float* S) {
   return q - 2.f * l + S[0];
 }
 
-// One block per cell: the 6x6 block means S[a][b] = (sum over the rows r of block a and the
-// column ranges h of part[c][r][h][b]) / B^2, then the ES-(1+1) step of the cell's weights w:
+// One block per cell: the 6x6 block means, then the ES-(1+1) step of the cell's weights w:
 // w' = max(w + sigma n, 0) / sum (n: the first five normals of stream MIX at iteration t; w kept
-// if the sum is 0), kept iff its squared MMD is lower. Warp a sums block a's rows: lane l takes
-// rows l, l + 32, ... (all h), then a fixed shuffle tree.
+// if the sum is 0), kept iff its squared MMD is lower. Warp a sums block a's rows, lane by lane in
+// a fixed order, then a fixed shuffle tree.
+//   TRI = false: S[a][b] = (sum over the rows r of block a of part[c][r][b]) / B^2;
+//   TRI = true (tensor-core Gram kernel): part[c][row tile][quarter][h][2][6] holds the upper
+//   triangle's sums, so S[a][b] = S[b][a] for a < b, and S[a][a] counts each element twice (the
+//   diagonal was counted half). nh = column ranges h of 128.
+template <bool TRI>
 __global__ void __launch_bounds__(192) k_mix_es(const float* __restrict__ part, int nh, int rows,
                                                 int B, float* mix, float* __restrict__ S_out,
                                                 float* __restrict__ score_out, uint64_t seed,
@@ -1070,11 +1074,23 @@ __global__ void __launch_bounds__(192) k_mix_es(const float* __restrict__ part, 
   __shared__ float S[36];
   const int a = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float acc[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-  for (int r = a * B + lane; r < (a + 1) * B; r += 32) {
-    const float* q = part + ((int64_t)c * rows + r) * nh * 6;
-    for (int h = 0; h < nh; ++h) {
+  if constexpr (TRI) {
+    const int groups = (rows + 31) / 32;  // of 32 rows; block a's rows lie in [first, last]
+    const int first = a * B / 32, last = ((a + 1) * B - 1) / 32;
+    const float* p = part + (int64_t)c * ((rows + 127) / 128 * 4) * nh * 12;
+    for (int i = lane; i < (last - first + 1) * nh; i += 32) {
+      const int g = first + i / nh, h = i % nh;
+      if (g >= groups || h / 2 < g * 32 / 128 * 128 / 256) continue;
+      const int slot = a - g * 32 / B;  // the group's first block, or the next
+      const float* q = p + ((int64_t)g * nh + h) * 12 + slot * 6;
 #pragma unroll
-      for (int b = 0; b < 6; ++b) acc[b] += q[h * 6 + b];
+      for (int b = 0; b < 6; ++b) acc[b] += q[b];
+    }
+  } else {
+    for (int r = a * B + lane; r < (a + 1) * B; r += 32) {
+      const float* q = part + ((int64_t)c * rows + r) * 6;
+#pragma unroll
+      for (int b = 0; b < 6; ++b) acc[b] += q[b];
     }
   }
 #pragma unroll
@@ -1082,9 +1098,14 @@ __global__ void __launch_bounds__(192) k_mix_es(const float* __restrict__ part, 
     float v = acc[b];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if (lane == 0) {
-      S[a * 6 + b] = v / ((float)B * (float)B);
-      S_out[(int64_t)c * 36 + a * 6 + b] = S[a * 6 + b];
+    if (lane == 0 && (!TRI || b >= a)) {
+      const float s = (TRI && b == a ? 2.f * v : v) / ((float)B * (float)B);
+      S[a * 6 + b] = s;
+      S_out[(int64_t)c * 36 + a * 6 + b] = s;
+      if (TRI && b > a) {
+        S[b * 6 + a] = s;
+        S_out[(int64_t)c * 36 + b * 6 + a] = s;
+      }
     }
   }
   __syncthreads();
@@ -1116,10 +1137,11 @@ __global__ void __launch_bounds__(192) k_mix_es(const float* __restrict__ part, 
   score_out[c] = acc_new ? nw : old;
 }
 
-void launch_mix_es(const float* part, int nh, int cells, int rows, int B, float* mix, float* S,
-                   float* score, uint64_t seed, uint32_t t, float sigma, cudaStream_t st) {
-  launch_pdl(k_mix_es, dim3(cells), dim3(192), 0, st, part, nh, rows, B, mix, S, score, seed, t,
-             sigma);
+void launch_mix_es(const float* part, int nh, bool tri, int cells, int rows, int B, float* mix,
+                   float* S, float* score, uint64_t seed, uint32_t t, float sigma,
+                   cudaStream_t st) {
+  launch_pdl(tri ? k_mix_es<true> : k_mix_es<false>, dim3(cells), dim3(192), 0, st, part, nh, rows,
+             B, mix, S, score, seed, t, sigma);
 }
 
 // The iteration's results for one host copy: out[0, n) = fG, out[n, 2n) = fD (n = cells * 5),
