@@ -20,6 +20,7 @@
 
 #include <algorithm>
 #include <string>
+#include <type_traits>
 
 #include "common.cuh"
 #include "conv_tc.h"
@@ -81,13 +82,44 @@ __device__ __forceinline__ bool gather_bar_or(bool pred) {
 enum { AK_CONV = 0, AK_TRANS = 1, AK_SCATTER = 2, AK_NCHW = 3, AK_GATHER = 4,
        AK_NCHW_WIDE = 5, AK_TRANS_C = 6 };
 
-// dynamic shared memory of a variant: the compact first layer (three 24 KB stages) and the
-// compact parity classes (256-row tiles of weight tiles of at most 64 rows: two 40 KB stages,
-// no patch buffers) fit two CTAs per SM
+// Variants that run on CTA pairs (clusters of two, tcgen05 .cta_group::2): A by TMA and channel-last
+// outputs or logits. Each CTA holds its own 128 rows of A (256 with m2) and half of the weight
+// tile's rows; rank 0 issues MMAs of 256 rows (two per chunk with m2) that read both halves, so
+// that a CTA's tensor core gets a 128 x 256 (m2: 256 x 128) chunk product from 32 (40) KB of
+// operands instead of 48. Bound: the tensor cores at nbox 256 (a 256 x 256 x 64 chunk in 640 to
+// 690 clocks, cuBLAS's rate; 850 before the MMA thread looked at the next stage early), shared
+// memory at nbox 128 (1,046: each MMA reads as many bytes of B as of A). Discriminator
+// evaluation of the 3x3 configuration 7.17 -> 6.55 ms; without pairs 6.65.
+constexpr bool conv_pair(int ak, int om) {
+  return ak == AK_CONV ||
+         (ak == AK_TRANS && (om == CTC_F32_HWC || om == CTC_DLRELU_HWC));
+}
+constexpr int PAIR_STAGES = 6;  // at most: six of 32 KB (nbox 256), four of 40 KB (m2, nbox 128)
+
+// scatter mode: one tap's products of the tile's 128 input pixels (float4 each: three outputs), and
+// four more, so that neighbouring lanes, which read two taps, meet different banks
+constexpr int SC_PLANE = 132;
+
+// dynamic shared memory of a variant: the compact first layer (three 24 KB stages), the compact
+// parity classes (256-row tiles of weight tiles of at most 64 rows: two 40 KB stages, no patch
+// buffers) and the scatter mode (three 24 KB stages, the 16 taps' products) fit two CTAs per SM
+constexpr bool conv_compact(int ak) {
+  return ak == AK_NCHW || ak == AK_TRANS_C || ak == AK_SCATTER;
+}
+// first-layer input patches: buffers, and tiles they are copied ahead (the compact variant's
+// copies come from DRAM: one tile ahead, a tile waited for them)
+constexpr int patch_bufs(int ak) { return ak == AK_NCHW ? 4 : 3; }
+constexpr int patch_ahead(int ak) { return patch_bufs(ak) - 2; }
+// their bytes, up to the next 1024-byte boundary after the 256 of the barriers (the epilogue's
+// staging tile follows)
+constexpr int patch_area(int ak) {
+  return ak == AK_TRANS_C ? 0 : (256 + patch_bufs(ak) * PATCH_BYTES + 1023) / 1024 * 1024 - 256;
+}
 constexpr int conv_smem(int ak) {
-  return ak == AK_NCHW
-             ? 1024 + 3 * (A_BYTES + 64 * BK * 2) + 256 + 3 * PATCH_BYTES + 4 * STG_WORDS * 4
+  return ak == AK_NCHW ? 1024 + 3 * (A_BYTES + 64 * BK * 2) + 256 + patch_area(ak) +
+                             4 * STG_WORDS * 4
          : ak == AK_TRANS_C ? 1024 + 2 * (2 * A_BYTES + 64 * BK * 2) + 256 + 4 * STG_WORDS * 4
+         : ak == AK_SCATTER ? 1024 + 3 * (A_BYTES + 64 * BK * 2) + 256 + 16 * SC_PLANE * 16
                             : SMEM_BYTES;
 }
 
@@ -98,7 +130,7 @@ constexpr int conv_smem(int ak) {
 // parity classes as p.transposed says). OM: the out_mode. Each launch runs the instantiation
 // its parameters name, so that a kernel holds only its own code paths.
 template <int AK, int OM>
-__global__ void __launch_bounds__(THREADS, AK == AK_NCHW || AK == AK_TRANS_C ? 2 : 1)
+__global__ void __launch_bounds__(THREADS, conv_compact(AK) ? 2 : 1)
     k_conv_tc(const __grid_constant__ CUtensorMap mW, const __grid_constant__ CUtensorMap mA,
               const __grid_constant__ CtcParams p) {
   extern __shared__ uint8_t smem_raw[];
@@ -106,19 +138,32 @@ __global__ void __launch_bounds__(THREADS, AK == AK_NCHW || AK == AK_TRANS_C ? 2
   constexpr bool kScatter = AK == AK_SCATTER, kNchw = AK == AK_NCHW || AK == AK_NCHW_WIDE;
   // AK_NCHW (weight tiles of at most 64 rows): three 24 KB stages and 256 TMEM columns, so
   // that two CTAs share an SM
-  constexpr bool kCompact = AK == AK_NCHW || AK == AK_TRANS_C;
-  constexpr int STAGES = AK == AK_NCHW ? 3 : AK == AK_TRANS_C ? 2 : ctc::STAGES;
-  constexpr uint32_t STAGE_BYTES = AK == AK_NCHW     ? A_BYTES + 64 * BK * 2
+  constexpr bool kCompact = conv_compact(AK);
+  // CTA pairs (see conv_pair): n_st stages of st_bytes each in the same ring
+  constexpr bool kPair = conv_pair(AK, OM);
+  constexpr int STAGES = AK == AK_NCHW || kScatter ? 3
+                         : AK == AK_TRANS_C         ? 2
+                         : kPair                    ? PAIR_STAGES
+                                                    : ctc::STAGES;
+  constexpr uint32_t STAGE_BYTES = AK == AK_NCHW || kScatter ? A_BYTES + 64 * BK * 2
                                    : AK == AK_TRANS_C ? 2 * A_BYTES + 64 * BK * 2
                                                       : ctc::STAGE_BYTES;
   // the first layer's patch buffers sit between the barriers and the epilogue staging
-  constexpr int kPatchArea = AK == AK_TRANS_C ? 0 : 3 * PATCH_BYTES;
+  constexpr int kPatchBufs = patch_bufs(AK), kPatchAhead = patch_ahead(AK);
+  constexpr int kPatchArea = patch_area(AK);
   constexpr uint32_t kTmemCols = kCompact ? 256 : 512, kAccStride = kCompact ? 128 : 256;
   const bool transposed = AK == AK_TRANS || AK == AK_TRANS_C || (AK == AK_GATHER && p.transposed);
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   uint8_t* gbase = smem_raw + (base - raw);
-  uint8_t* misc = gbase + STAGES * STAGE_BYTES;
+  uint8_t* misc = gbase + (kPair ? ctc::STAGES : STAGES) * STAGE_BYTES;
+  const int nA = p.m2 ? 2 : 1;  // 128-row A tiles of a CTA
+  const uint32_t st_bytes =
+      kPair ? (uint32_t)(nA * A_BYTES + p.nbox * BK) : (uint32_t)STAGE_BYTES;
+  const int n_st = kPair ? min(PAIR_STAGES, (int)(ctc::STAGES * STAGE_BYTES / st_bytes)) : STAGES;
+  const uint32_t rank = kPair ? cluster_ctarank() : 0u;
+  const int cta = kPair ? (int)cluster_id_x() : (int)blockIdx.x;   // tiles cta, cta + n_cta, ...
+  const int n_cta = kPair ? (int)nclusters_x() : (int)gridDim.x;
   const uint32_t bars = smem_u32(misc);
   const uint32_t bFullA = bars, bFullB = bars + 8 * STAGES, bEmpty = bars + 16 * STAGES;
   const uint32_t bAccF = bars + 24 * STAGES, bAccE = bAccF + 16, bFinal = bAccE + 16;
@@ -133,56 +178,78 @@ __global__ void __launch_bounds__(THREADS, AK == AK_NCHW || AK == AK_TRANS_C ? 2
     }
     mbar_init(bAccF, 1);
     mbar_init(bAccF + 8, 1);
-    mbar_init(bAccE, 128);
-    mbar_init(bAccE + 8, 128);
+    // (a pair: a lane of each epilogue warp of both CTAs, on rank 0's barrier)
+    mbar_init(bAccE, kPair ? 8 : 128);
+    mbar_init(bAccE + 8, kPair ? 8 : 128);
     mbar_init(bFinal, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                     smem_u32((const void*)tmem_slot)),
-                 "r"(kTmemCols));
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    if constexpr (kPair) {
+      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                       smem_u32((const void*)tmem_slot)),
+                   "r"(kTmemCols));
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;");
+    } else {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                       smem_u32((const void*)tmem_slot)),
+                   "r"(kTmemCols));
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
   }
   tc_fence_before();
-  __syncthreads();
+  if constexpr (kPair) cluster_sync_all();  // no remote arrival before the peer's barriers exist
+  else __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  const uint32_t lFullB = kPair ? mapa_shared(bFullB, 0) : bFullB;
+  const uint32_t lAccE = kPair ? mapa_shared(bAccE, 0) : bAccE;
   pdl_wait();
   // output pixels per problem (per parity class when transposed)
   // rows of a problem: output pixels (class pixels when transposed; input pixels in scatter)
   const int lq = kScatter ? p.lhi : p.lho - (transposed ? 1 : 0);
   const int M = p.rows << (2 * lq);
   const int nbox = p.nbox;
+  // first row of this CTA's part of a tile
+  auto tile_row = [&](int tile) {
+    const int i = tile % p.mtiles;
+    return (kPair ? 2 * i + (int)rank : i) * nA * BM;
+  };
 
-  if (warp == 0) {
-    // ---- weights by TMA
-    if (lane == 0) {
+  if (warp == 0 || (kTma && (warp == 2 || warp == 3))) {
+    // ---- TMA: the weights (warp 0, which also announces the stage's bytes) and, where A comes
+    // by TMA, its first (warp 2) and second (m2: warp 3) 128 rows. A tiled TMA operation holds its
+    // issuing thread for 0.2 us and more, most of a chunk's time on the tensor cores, so each
+    // thread issues one per chunk.
+    if (lane == 0 && (warp < 3 || p.m2)) {
       int stage = 0, issued[STAGES] = {};
       uint32_t phase = 0;
       bool ok = true;
-      for (int tile = blockIdx.x; tile < p.n_tiles && ok; tile += gridDim.x) {
+      for (int tile = cta; tile < p.n_tiles && ok; tile += n_cta) {
         const int pc = tile / p.mtiles;  // problem (x 4 parity classes when transposed)
         const ConvTcDesc d = p.descs[transposed ? pc >> 2 : pc];
         const int cls = transposed ? (pc & 3) : 0;
         const int indiv = __ldg(&p.wsel[d.wsel_idx]);
         // channel-last A rows by TMA (a_tma): the tile is 128 consecutive output pixels (class
         // pixels when transposed) of whole rows; its origin is image n0, row y0
-        const int m0 = (tile % p.mtiles) * (p.m2 ? 2 * BM : BM);
+        const int m0 = tile_row(tile) + (warp == 3 ? BM : 0);
         const int n0 = m0 >> (2 * lq), y0 = (m0 >> lq) & ((1 << lq) - 1);
-        // m2: the second 128 rows of a 256-row tile
-        const int n1 = (m0 + BM) >> (2 * lq), y1 = ((m0 + BM) >> lq) & ((1 << lq) - 1);
         for (int j = 0; j < p.nj && ok; ++j)
           for (int kc = 0; kc < p.kchunks; ++kc) {
             if (!mbar_wait(bEmpty + 8 * stage, phase ^ 1u, abort_flag, p.err, 21)) {
               ok = false;
               break;
             }
-            mbar_expect_tx(bFullB + 8 * stage,
-                           (uint32_t)(nbox * BK * 2 + (kTma ? (p.m2 ? 2 : 1) * A_BYTES : 0)));
-            if constexpr (kTma) {
+            // (loads may land before their bytes are announced; a pair: rank 0 expects both
+            // CTAs' bytes)
+            if (warp == 0 && rank == 0)
+              mbar_expect_tx(bFullB + 8 * stage,
+                             kPair ? 2 * st_bytes
+                                   : (uint32_t)(nbox * BK * 2 + (kTma ? nA * A_BYTES : 0)));
+            const uint32_t sS = base + stage * st_bytes, full = lFullB + 8 * stage;
+            if (kTma && warp != 0) {
               // Convolution: tap (ky, kx), input rows 2 y - 1 + ky, columns 2 x - 1 + kx (the
               // map's traversal stride 2). Transposed, class (a, b), tap (u, v): ky = (a + 1)
               // mod 2 + 2u, input row y + (a + 1 - ky) / 2, column x + (b + 1 - kx) / 2.
@@ -206,22 +273,29 @@ __global__ void __launch_bounds__(THREADS, AK == AK_NCHW || AK == AK_TRANS_C ? 2
                 x = (tap & 3) - 1;
               }
               const int prob = transposed ? pc >> 2 : pc;
-              tma_load_5d(base + stage * STAGE_BYTES, &mA, bFullB + 8 * stage, c0, x,
-                          ym * y0 + ya, n0, prob);
-              if (p.m2)
-                tma_load_5d(base + stage * STAGE_BYTES + A_BYTES, &mA, bFullB + 8 * stage, c0, x,
-                            ym * y1 + ya, n1, prob);
+              const uint32_t dst = sS + (warp - 2) * A_BYTES;
+              if constexpr (kPair) tma_load_5d_cg2(dst, &mA, full, c0, x, ym * y0 + ya, n0, prob);
+              else tma_load_5d(dst, &mA, full, c0, x, ym * y0 + ya, n0, prob);
+            } else if constexpr (kPair) {
+              tma_load_3d_cg2(sS + nA * A_BYTES, &mW, full, kc * BK,
+                              cls * p.cls_rows + j * 256 + (int)rank * (nbox / 2), indiv);
+            } else {
+              tma_load_3d(sS + nA * A_BYTES, &mW, full, kc * BK, cls * p.cls_rows + j * 256, indiv);
             }
-            tma_load_3d(base + stage * STAGE_BYTES + (p.m2 ? 2 : 1) * A_BYTES, &mW,
-                        bFullB + 8 * stage, kc * BK, cls * p.cls_rows + j * 256, indiv);
             issued[stage]++;
-            if (++stage == STAGES) {
+            if (++stage == n_st) {
               stage = 0;
               phase ^= 1u;
             }
           }
       }
-      if (!ok) {
+      if (kPair && !ok) {
+        // loads issued here complete on rank 0's barriers: give them time to land before the
+        // CTA leaves
+        const unsigned long long t0 = globaltimer();
+        while (globaltimer() - t0 < 200000ull) {
+        }
+      } else if (!ok) {
         for (int s = 0; s < STAGES; ++s)
           if (issued[s] > 0) {
             volatile int never = 0;
@@ -230,13 +304,13 @@ __global__ void __launch_bounds__(THREADS, AK == AK_NCHW || AK == AK_TRANS_C ? 2
       }
     }
   } else if (warp == 1) {
-    // ---- MMA issue
-    if (lane == 0) {
+    // ---- MMA issue (a pair: rank 0, 256-row MMAs over both CTAs' tiles)
+    if (lane == 0 && rank == 0) {
       int stage = 0, uses[2] = {0, 0}, jobs = 0;
       uint32_t phase = 0;
-      bool ok = true;
-      const uint32_t idesc = idesc_bf16(BM, nbox);
-      for (int tile = blockIdx.x; tile < p.n_tiles && ok; tile += gridDim.x)
+      bool ok = true, ready = false;
+      const uint32_t idesc = idesc_bf16(kPair ? 2 * BM : BM, nbox);
+      for (int tile = cta; tile < p.n_tiles && ok; tile += n_cta)
         for (int j = 0; j < p.nj && ok; ++j, ++jobs) {
           const int R = jobs & 1;
           if (uses[R] > 0 &&
@@ -246,34 +320,58 @@ __global__ void __launch_bounds__(THREADS, AK == AK_NCHW || AK == AK_TRANS_C ? 2
           }
           tc_fence_after();
           const uint32_t dt = tmem + (uint32_t)(R * kAccStride);
+          // one chunk: its MMAs (a 16-element K step is 32 bytes: 2 in the descriptors' address
+          // field), with `look` run before the last pair of them
+          auto chunk = [&](auto m2, bool first, auto look) {
+            const uint32_t sA = base + stage * st_bytes;
+            const uint64_t dA = sw128_desc(sA), dA1 = sw128_desc(sA + A_BYTES);
+            const uint64_t dB = sw128_desc(sA + (decltype(m2)::value ? 2 : 1) * A_BYTES);
+#pragma unroll
+            for (int kk = 0; kk < BK / 16; ++kk) {
+              if (kk == BK / 16 - 1) look();
+              if constexpr (kPair) {
+                if (kk) tc_mma_cg2_acc(dt, dA + 2 * kk, dB + 2 * kk, idesc);
+                else tc_mma_cg2(dt, dA, dB, idesc, first ? 0u : 1u);
+                if constexpr (decltype(m2)::value) {
+                  if (kk) tc_mma_cg2_acc(dt + (uint32_t)nbox, dA1 + 2 * kk, dB + 2 * kk, idesc);
+                  else tc_mma_cg2(dt + (uint32_t)nbox, dA1, dB, idesc, first ? 0u : 1u);
+                }
+              } else {
+                if (kk) tc_mma_acc(dt, dA + 2 * kk, dB + 2 * kk, idesc);
+                else tc_mma(dt, dA, dB, idesc, first ? 0u : 1u);
+                if constexpr (decltype(m2)::value) {
+                  if (kk) tc_mma_acc(dt + (uint32_t)nbox, dA1 + 2 * kk, dB + 2 * kk, idesc);
+                  else tc_mma(dt + (uint32_t)nbox, dA1, dB, idesc, first ? 0u : 1u);
+                }
+              }
+            }
+          };
           for (int kc = 0; kc < p.kchunks; ++kc) {
             if ((!kTma && !mbar_wait(bFullA + 8 * stage, phase, abort_flag, p.err, 24)) ||
-                !mbar_wait(bFullB + 8 * stage, phase, abort_flag, p.err, 25)) {
+                (!ready && !mbar_wait(bFullB + 8 * stage, phase, abort_flag, p.err, 25))) {
               ok = false;
               break;
             }
             tc_fence_after();
-            const uint32_t sA = base + stage * STAGE_BYTES;
-            const uint32_t sB = sA + (p.m2 ? 2 : 1) * A_BYTES;
-#pragma unroll
-            for (int kk = 0; kk < BK / 16; ++kk) {
-              tc_mma(dt, sw128_desc(sA + kk * 32), sw128_desc(sB + kk * 32), idesc,
-                     (kc | kk) != 0 ? 1u : 0u);
-              if (p.m2)
-                tc_mma(dt + (uint32_t)nbox, sw128_desc(sA + A_BYTES + kk * 32),
-                       sw128_desc(sB + kk * 32), idesc, (kc | kk) != 0 ? 1u : 0u);
-            }
-            tc_commit(bEmpty + 8 * stage);
-            if (++stage == STAGES) {
-              stage = 0;
-              phase ^= 1u;
-            }
+            // the next stage is looked at while this chunk's MMAs run: the tensor core takes few
+            // MMAs ahead, so what this thread does between two chunks is time without any
+            const int next = stage + 1 == n_st ? 0 : stage + 1;
+            const uint32_t next_phase = next ? phase : phase ^ 1u;
+            auto look = [&] { ready = mbar_test(bFullB + 8 * next, next_phase); };
+            if (p.m2) chunk(std::true_type{}, kc == 0, look);
+            else chunk(std::false_type{}, kc == 0, look);
+            if constexpr (kPair) tc_commit_cg2(bEmpty + 8 * stage, 3);
+            else tc_commit(bEmpty + 8 * stage);
+            stage = next;
+            phase = next_phase;
           }
           if (!ok) break;
-          tc_commit(bAccF + 8 * R);
+          if constexpr (kPair) tc_commit_cg2(bAccF + 8 * R, 3);
+          else tc_commit(bAccF + 8 * R);
           uses[R]++;
         }
-      tc_commit(bFinal);
+      if constexpr (kPair) tc_commit_cg2(bFinal, 3);
+      else tc_commit(bFinal);
       volatile int never = 0;
       mbar_wait(bFinal, 0u, &never, p.err, 26);
     }
@@ -290,11 +388,11 @@ __global__ void __launch_bounds__(THREADS, AK == AK_NCHW || AK == AK_TRANS_C ? 2
       // first layer (3 channels, 64 x 64 CHW images, 32 x 32 outputs, one k chunk of
       // k = c * 16 + ky * 4 + kx over 48 values, the weights' own [out][c][ky][kx] order): a
       // tile's 128 rows are 4 output rows, fed by
-      // a 3 x 10 x 64 input patch that the gather threads copy one tile ahead by 8-byte
-      // cp.async into one of three shared buffers whose halo columns stay zero
+      // a 3 x 10 x 64 input patch that the gather threads copy kPatchAhead tiles ahead by
+      // 8-byte cp.async into one of kPatchBufs shared buffers whose halo columns stay zero
       uint8_t* patches = misc + 256;
       const uint32_t patch0 = smem_u32(patches);
-      for (int i = r; i < 3 * PATCH_BYTES / 16; i += 128)
+      for (int i = r; i < kPatchBufs * PATCH_BYTES / 16; i += 128)
         *reinterpret_cast<uint4*>(patches + 16 * i) = make_uint4(0u, 0u, 0u, 0u);
       gather_bar_or(false);
       auto prefetch = [&](int tile, int buf) {
@@ -313,12 +411,12 @@ __global__ void __launch_bounds__(THREADS, AK == AK_NCHW || AK == AK_TRANS_C ? 2
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
       };
-      prefetch(blockIdx.x, 0);
+      for (int i = 0; i < kPatchAhead; ++i) prefetch(blockIdx.x + i * gridDim.x, i);
       int buf = 0;
       const int ox = r & 31, oyl = r >> 5;
       for (int tile = blockIdx.x; tile < p.n_tiles; tile += gridDim.x) {
-        prefetch(tile + gridDim.x, buf == 2 ? 0 : buf + 1);
-        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        prefetch(tile + kPatchAhead * gridDim.x, (buf + kPatchAhead) % kPatchBufs);
+        asm volatile("cp.async.wait_group %0;" ::"n"(kPatchAhead) : "memory");
         const bool okw = mbar_wait_warp(bEmpty + 8 * stage, phase ^ 1u, abort_flag, p.err, 27);
         if (gather_bar_or(!okw)) {
           ok = false;
@@ -356,7 +454,7 @@ __global__ void __launch_bounds__(THREADS, AK == AK_NCHW || AK == AK_TRANS_C ? 2
           stage = 0;
           phase ^= 1u;
         }
-        buf = buf == 2 ? 0 : buf + 1;
+        buf = buf + 1 == kPatchBufs ? 0 : buf + 1;
       }
     } else
     for (int tile = blockIdx.x; tile < p.n_tiles && ok; tile += gridDim.x) {
@@ -439,11 +537,11 @@ __global__ void __launch_bounds__(THREADS, AK == AK_NCHW || AK == AK_TRANS_C ? 2
     const uint32_t tileb = smem_u32(misc + 256 + kPatchArea);
     int uses[2] = {0, 0}, jobs = 0;
     bool ok = true;
-    for (int tile = blockIdx.x; tile < p.n_tiles && ok; tile += gridDim.x) {
+    for (int tile = cta; tile < p.n_tiles && ok; tile += n_cta) {
       const int pc = tile / p.mtiles;
       const ConvTcDesc d = p.descs[transposed ? pc >> 2 : pc];
       const int cls = transposed ? (pc & 3) : 0;
-      const int m = (tile % p.mtiles) * (p.m2 ? 2 * BM : BM) + row;
+      const int m = tile_row(tile) + row;
       const bool valid = m < M;
       const int nb = m >> (2 * lq);
       int oy = (m >> lq) & ((1 << lq) - 1), ox = m & ((1 << lq) - 1);
@@ -469,14 +567,16 @@ __global__ void __launch_bounds__(THREADS, AK == AK_NCHW || AK == AK_TRANS_C ? 2
         }
         tc_fence_after();
         if constexpr (kScatter) {
-          // input pixel (y0 + q, lane) holds Y[tap * 4 + o] (16 taps, 3 channels); the taps are
-          // added one after the other into the tile's 10 x 66 output window in shared memory
-          // (output row 2 y - 1 + ky, column 2 x - 1 + kx; window origin (2 y0 - 1, -1))
-          float* acc = reinterpret_cast<float*>(stg - (warp - 6) * STG_WORDS);
+          // input pixel (y0 + q, lane) holds Y[tap * 4 + o] (16 taps, 3 channels), tap (ky, kx)
+          // belonging to output row 2 y - 1 + ky, column 2 x - 1 + kx. The products go to shared
+          // memory by tap, and each output of the tile's window (10 rows from 8 blk - 1, 64
+          // columns) gathers its own, at most four, in tap order (adding tap after tap into the
+          // window in shared memory took 4,000 clocks a tile: 620 us for the 3x3 configuration's
+          // evaluation). Bound: instructions and shared-memory reads of this epilogue.
+          float4* yp = reinterpret_cast<float4*>(misc + 256);
           const int et = threadIdx.x - 192;
           const int m0t = m - row;  // the tile's first input pixel: image img, rows 4 blk ..
           const int img = m0t >> 10, blk = (m0t >> 7) & 7;
-          for (int i = et; i < 1980; i += 128) acc[i] = 0.f;
           uint32_t v[32], w[32];  // columns 0..31 (taps 0..7) and 32..63 (taps 8..15)
           LIPZ_TMEM_LD32(tmem + lane_base + (uint32_t)(R * kAccStride), v);
           LIPZ_TMEM_LD32(tmem + lane_base + (uint32_t)(R * kAccStride + 32), w);
@@ -484,46 +584,65 @@ __global__ void __launch_bounds__(THREADS, AK == AK_NCHW || AK == AK_TRANS_C ? 2
           tc_fence_before();
           mbar_arrive(bAccE + 8 * R);
           uses[R]++;
-          epi_bar();
-          // taps with ky < 2 first (warp q writes window rows 2q, 2q + 1: no two warps share a
-          // row), then ky >= 2 (rows 2q + 2, 2q + 3); inside a warp the taps go in order
+          // (the vote above came after every thread's reads of the previous tile's products)
 #pragma unroll
           for (int tap = 0; tap < 16; ++tap) {
-            float* a = acc + ((2 * q + (tap >> 2)) * 66 + 2 * lane + (tap & 3)) * 3;
             const uint32_t* y = tap < 8 ? v + tap * 4 : w + (tap - 8) * 4;
-            if (valid) {
-              a[0] += __uint_as_float(y[0]);
-              a[1] += __uint_as_float(y[1]);
-              a[2] += __uint_as_float(y[2]);
-            }
-            if (tap == 7 || tap == 15)
-              epi_bar();
-            else
-              __syncwarp();
-          }
-          // window rows 2..7 (output rows 8 blk + 1 .. 8 blk + 6) are complete; rows 0, 1, 8, 9
-          // are shared with the blocks above and below and go to the halo buffer
-          const bool tv = m0t < M;
-          if (tv) {
-            for (int i = et; i < 6 * 64 * 3; i += 128) {
-              const int o = i / 384, rem = i - o * 384, lr = 2 + (rem >> 6), gx = rem & 63;
-              const int64_t oi = (((int64_t)img * 3 + o) << 12) + ((8 * blk - 1 + lr) << 6) + gx;
-              float x = acc[(lr * 66 + gx + 1) * 3 + o];
-              if (OM == CTC_TANH_CHW) {
-                x = tanhf(x);
-              } else {
-                const float f = __bfloat162float(d.aux[oi]);
-                x = x * (1.f - f * f);
-              }
-              d.out[oi] = __float2bfloat16_rn(x);
-            }
-            float* h = p.halo + (((int64_t)pc * p.rows + img) * 8 + blk) * 768;
-            for (int i = et; i < 768; i += 128) {
-              const int pr = i / 192, rem = i - pr * 192, gx = rem / 3, o = rem - gx * 3;
-              h[i] = acc[((pr < 2 ? pr : pr + 6) * 66 + gx + 1) * 3 + o];
-            }
+            yp[tap * SC_PLANE + row] =
+                make_float4(__uint_as_float(y[0]), __uint_as_float(y[1]), __uint_as_float(y[2]), 0.f);
           }
           epi_bar();
+          if (m0t >= M) continue;
+          // two neighbouring columns per thread: column c of the window (gx + 1) takes pixel c / 2
+          // with kx = c mod 2, then pixel c / 2 - 1 with kx + 2; rows likewise
+          for (int i = et; i < 10 * 32; i += 128) {
+            const int lr = i >> 5, gx = 2 * (i & 31);
+            float x[2][3];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+              const int c = gx + e + 1;
+              float s0 = 0.f, s1 = 0.f, s2 = 0.f;
+#pragma unroll
+              for (int t = 0; t < 4; ++t) {
+                const int yl = (lr >> 1) - (t >> 1), xl = (c >> 1) - (t & 1);
+                if (yl < 0 || yl > 3 || xl < 0 || xl > 31) continue;
+                const int tap = ((lr & 1) + (t & 2)) * 4 + (c & 1) + 2 * (t & 1);
+                const float4 a = yp[tap * SC_PLANE + yl * 32 + xl];
+                s0 += a.x;
+                s1 += a.y;
+                s2 += a.z;
+              }
+              x[e][0] = s0;
+              x[e][1] = s1;
+              x[e][2] = s2;
+            }
+            // window rows 2..7 (output rows 8 blk + 1 .. 8 blk + 6) are complete; rows 0, 1, 8, 9
+            // are shared with the blocks above and below and go to the halo buffer
+            if (lr >= 2 && lr < 8) {
+#pragma unroll
+              for (int o = 0; o < 3; ++o) {
+                const int64_t oi = (((int64_t)img * 3 + o) << 12) + ((8 * blk - 1 + lr) << 6) + gx;
+                float x0 = x[0][o], x1 = x[1][o];
+                if (OM == CTC_TANH_CHW) {
+                  x0 = tanhf(x0);
+                  x1 = tanhf(x1);
+                } else {
+                  const __nv_bfloat162 f2 = *reinterpret_cast<const __nv_bfloat162*>(d.aux + oi);
+                  const float f0 = __low2float(f2), f1 = __high2float(f2);
+                  x0 = x0 * (1.f - f0 * f0);
+                  x1 = x1 * (1.f - f1 * f1);
+                }
+                *reinterpret_cast<__nv_bfloat162*>(d.out + oi) = __floats2bfloat162_rn(x0, x1);
+              }
+            } else {
+              float* h = p.halo + (((int64_t)pc * p.rows + img) * 8 + blk) * 768 +
+                         (lr < 2 ? lr : lr - 6) * 192 + gx * 3;
+#pragma unroll
+              for (int e = 0; e < 2; ++e)
+#pragma unroll
+                for (int o = 0; o < 3; ++o) h[e * 3 + o] = x[e][o];
+            }
+          }
           continue;
         }
         if (OM == CTC_TANH_CHW || OM == CTC_DTANH_CHW) {
@@ -655,8 +774,11 @@ __global__ void __launch_bounds__(THREADS, AK == AK_NCHW || AK == AK_TRANS_C ? 2
                   bq = fmaf(x, x, bq);
                 }
               }
-              const int64_t slot = ((int64_t)tile * (p.m2 ? 2 : 1) + h) * 4 + q;
-              p.bn_part[slot * p.co + j * 256 + g * 32 + lane] = make_float2(bs, bq);
+              // (the last pair tile's second CTA may lie past the problem's mt1 parts)
+              const int i1 = kPair ? 2 * (tile % p.mtiles) + (int)rank : tile % p.mtiles;
+              const int64_t slot = (((int64_t)pc * p.mt1 + i1) * nA + h) * 4 + q;
+              if (i1 < p.mt1)
+                p.bn_part[slot * p.co + j * 256 + g * 32 + lane] = make_float2(bs, bq);
             }
             const int lpr = f32 ? 8 : 4, rpi = 32 / lpr;
             const int part = lane % lpr;
@@ -687,7 +809,12 @@ __global__ void __launch_bounds__(THREADS, AK == AK_NCHW || AK == AK_TRANS_C ? 2
           }
         }
         tc_fence_before();
-        mbar_arrive(bAccE + 8 * R);
+        if constexpr (kPair) {
+          __syncwarp();
+          if (lane == 0) mbar_arrive_remote(lAccE + 8 * R);
+        } else {
+          mbar_arrive(bAccE + 8 * R);
+        }
         uses[R]++;
       }
       if constexpr (OM == CTC_LRELU_LOGIT) {
@@ -703,10 +830,16 @@ __global__ void __launch_bounds__(THREADS, AK == AK_NCHW || AK == AK_TRANS_C ? 2
   __syncwarp();
   tc_fence_before();
   __syncthreads();
+  if constexpr (kPair) cluster_sync_all();  // the peer may still arrive on this CTA's barriers
   tc_fence_after();
-  if (warp == 1)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
-                 "r"(kTmemCols));
+  if (warp == 1) {
+    if constexpr (kPair)
+      asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                   "r"(kTmemCols));
+    else
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                   "r"(kTmemCols));
+  }
 }
 
 // ---- weight gradients on tcgen05 -----------------------------------------------------------
@@ -838,7 +971,7 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
     if (lane == 0) {
       int stage = 0, uses[2] = {0, 0}, jobs = 0;
       uint32_t phase = 0;
-      bool ok = true;
+      bool ok = true, ready = false;
       const uint32_t idesc = idesc_bf16_major(128, BCHW ? 64 : 256, 1, 1);
       for (int tile = blockIdx.x; tile < p.n_tiles && ok; tile += gridDim.x, ++jobs) {
         const int split = (tile / per_split) % p.splits;
@@ -854,23 +987,26 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
         const uint32_t dt = tmem + (uint32_t)(R * 256);
         bool first = true;
         for (int64_t kb = k0; kb < k1; kb += 64) {
-          if (!mbar_wait(bFull + 8 * stage, phase, abort_flag, p.err, 32)) {
+          if (!ready && !mbar_wait(bFull + 8 * stage, phase, abort_flag, p.err, 32)) {
             ok = false;
             break;
           }
           tc_fence_after();
           const uint32_t sA = base + stage * STAGE_BYTES, sB = sA + A_BYTES;
-#pragma unroll
-          for (int kk = 0; kk < 4; ++kk) {
-            tc_mma(dt, sw128_mn_desc(sA + kk * 2048, 8192), sw128_mn_desc(sB + kk * 2048, 8192),
-                   idesc, first ? 0u : 1u);
-            first = false;
-          }
+          // a 16-pixel K step is 2048 bytes: 128 in the descriptors' address field
+          const uint64_t dA = sw128_mn_desc(sA, 8192), dB = sw128_mn_desc(sB, 8192);
+          tc_mma(dt, dA, dB, idesc, first ? 0u : 1u);
+          first = false;
+          tc_mma_acc(dt, dA + 128, dB + 128, idesc);
+          tc_mma_acc(dt, dA + 256, dB + 256, idesc);
+          // the next stage is looked at while the MMAs run (see k_conv_tc)
+          const int next = stage + 1 == WG_STAGES ? 0 : stage + 1;
+          const uint32_t next_phase = next ? phase : phase ^ 1u;
+          ready = mbar_test(bFull + 8 * next, next_phase);
+          tc_mma_acc(dt, dA + 384, dB + 384, idesc);
           tc_commit(bEmpty + 8 * stage);
-          if (++stage == WG_STAGES) {
-            stage = 0;
-            phase ^= 1u;
-          }
+          stage = next;
+          phase = next_phase;
         }
         if (!ok) break;
         tc_commit(bAccF + 8 * R);
@@ -2189,6 +2325,12 @@ bool ctc_make_map(CUtensorMap* m, const void* base, uint64_t K, uint64_t rows, u
   return true;
 }
 
+bool ctc_make_weight_maps(ConvWeightMaps* m, const void* base, uint64_t K, uint64_t rows,
+                          uint64_t depth, uint64_t depth_elems, uint32_t nbox, std::string* msg) {
+  return ctc_make_map(&m->full, base, K, rows, depth, depth_elems, nbox, msg) &&
+         ctc_make_map(&m->half, base, K, rows, depth, depth_elems, nbox / 2, msg);
+}
+
 bool ctc_make_out_map(CUtensorMap* m, CtcParams* q, const ConvTcDesc* descs, int n_probs,
                       std::string* msg) {
   q->tma_out = 0;
@@ -2217,53 +2359,6 @@ bool ctc_make_out_map(CUtensorMap* m, CtcParams* q, const ConvTcDesc* descs, int
     return false;
   }
   q->tma_out = 1;
-  return true;
-}
-
-bool ctc_make_act_map(CUtensorMap* m, CtcParams* q, const ConvTcDesc* descs, int n_probs,
-                      std::string* msg, bool use_tma) {
-  q->a_tma = 0;
-  q->m2 = 0;
-  if (!use_tma || q->nchw_in || q->ci % 64 != 0 || n_probs < 1) return true;
-  const int lq = q->scatter ? q->lhi : q->lho - q->transposed;
-  if (lq > 7) return true;
-  const int64_t Wi = (int64_t)1 << q->lhi;
-  const int64_t per = (int64_t)q->rows * Wi * Wi * q->ci;  // elements of one problem's input
-  int64_t pstride = per;
-  if (n_probs > 1) pstride = (int64_t)(descs[1].in - descs[0].in);
-  if (pstride < per || pstride % 8 != 0) return true;
-  for (int k = 1; k < n_probs; ++k)
-    if (descs[k].in != descs[0].in + (int64_t)k * pstride) return true;
-  if (!ensure_encode(msg)) return false;
-  const int stride = q->transposed || q->scatter ? 1 : 2;
-  const int tw = 1 << lq, th = std::min(1 << lq, 128 / tw), tn = std::max(1, 128 / (tw * th));
-  cuuint64_t dims[5] = {(cuuint64_t)q->ci, (cuuint64_t)Wi, (cuuint64_t)Wi, (cuuint64_t)q->rows,
-                        (cuuint64_t)n_probs};
-  cuuint64_t strides[4] = {(cuuint64_t)q->ci * 2, (cuuint64_t)(Wi * q->ci * 2),
-                           (cuuint64_t)(Wi * Wi * q->ci * 2), (cuuint64_t)(pstride * 2)};
-  cuuint32_t box[5] = {64, (cuuint32_t)(tw * stride), (cuuint32_t)(th * stride), (cuuint32_t)tn, 1};
-  cuuint32_t es[5] = {1, (cuuint32_t)stride, (cuuint32_t)stride, 1, 1};
-  CUresult r = g_encode_ctc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5,
-                            const_cast<bf16*>(descs[0].in), dims, strides, box, es,
-                            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  if (r != CUDA_SUCCESS) {
-    if (msg)
-      *msg = "cuTensorMapEncodeTiled (convolution activations) failed: " +
-             std::to_string((int)r);
-    return false;
-  }
-  q->a_tma = 1;
-  // 256-row tiles (two accumulators sharing each weight chunk) for narrow weight tiles
-  if (!q->scatter && q->nbox <= 128 &&
-      (q->out_mode == CTC_LRELU_HWC || q->out_mode == CTC_F32_HWC ||
-       q->out_mode == CTC_DLRELU_HWC)) {
-    const int M = q->rows << (2 * lq);
-    const int mt2 = (M + 255) / 256;
-    q->n_tiles = q->n_tiles / q->mtiles * mt2;
-    q->mtiles = mt2;
-    q->m2 = 1;
-  }
   return true;
 }
 
@@ -2313,6 +2408,83 @@ ConvKernel conv_kernel(const CtcParams& p) {
   return nullptr;
 }
 }  // namespace
+
+bool ctc_make_act_map(CUtensorMap* m, CtcParams* q, const ConvTcDesc* descs, int n_probs,
+                      std::string* msg, bool use_tma) {
+  q->a_tma = 0;
+  q->m2 = 0;
+  q->mt1 = q->mtiles;
+  if (!use_tma || q->nchw_in || q->ci % 64 != 0 || n_probs < 1) return true;
+  const int lq = q->scatter ? q->lhi : q->lho - q->transposed;
+  if (lq > 7) return true;
+  const int64_t Wi = (int64_t)1 << q->lhi;
+  const int64_t per = (int64_t)q->rows * Wi * Wi * q->ci;  // elements of one problem's input
+  int64_t pstride = per;
+  if (n_probs > 1) pstride = (int64_t)(descs[1].in - descs[0].in);
+  if (pstride < per || pstride % 8 != 0) return true;
+  for (int k = 1; k < n_probs; ++k)
+    if (descs[k].in != descs[0].in + (int64_t)k * pstride) return true;
+  if (!ensure_encode(msg)) return false;
+  const int stride = q->transposed || q->scatter ? 1 : 2;
+  const int tw = 1 << lq, th = std::min(1 << lq, 128 / tw), tn = std::max(1, 128 / (tw * th));
+  cuuint64_t dims[5] = {(cuuint64_t)q->ci, (cuuint64_t)Wi, (cuuint64_t)Wi, (cuuint64_t)q->rows,
+                        (cuuint64_t)n_probs};
+  cuuint64_t strides[4] = {(cuuint64_t)q->ci * 2, (cuuint64_t)(Wi * q->ci * 2),
+                           (cuuint64_t)(Wi * Wi * q->ci * 2), (cuuint64_t)(pstride * 2)};
+  cuuint32_t box[5] = {64, (cuuint32_t)(tw * stride), (cuuint32_t)(th * stride), (cuuint32_t)tn, 1};
+  cuuint32_t es[5] = {1, (cuuint32_t)stride, (cuuint32_t)stride, 1, 1};
+  CUresult r = g_encode_ctc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5,
+                            const_cast<bf16*>(descs[0].in), dims, strides, box, es,
+                            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
+                            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) {
+    if (msg)
+      *msg = "cuTensorMapEncodeTiled (convolution activations) failed: " +
+             std::to_string((int)r);
+    return false;
+  }
+  q->a_tma = 1;
+  // 256-row tiles (two accumulators sharing each weight chunk) for narrow weight tiles
+  if (!q->scatter && q->nbox <= 128 &&
+      (q->out_mode == CTC_LRELU_HWC || q->out_mode == CTC_F32_HWC ||
+       q->out_mode == CTC_DLRELU_HWC)) {
+    const int M = q->rows << (2 * lq);
+    const int mt2 = (M + 255) / 256;
+    q->n_tiles = q->n_tiles / q->mtiles * mt2;
+    q->mtiles = mt2;
+    q->m2 = 1;
+  }
+  q->mt1 = q->mtiles;
+  if (ctc::conv_pair(conv_ak(*q), q->out_mode)) {
+    // clusters of two that can be resident at once (one CTA per SM)
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2);
+    cfg.blockDim = dim3(ctc::THREADS);
+    cfg.dynamicSmemBytes = ctc::conv_smem(conv_ak(*q));
+    cudaLaunchAttribute a;
+    a.id = cudaLaunchAttributeClusterDimension;
+    a.val.clusterDim.x = 2;
+    a.val.clusterDim.y = 1;
+    a.val.clusterDim.z = 1;
+    cfg.attrs = &a;
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&q->clusters, (const void*)conv_kernel(*q), &cfg) !=
+            cudaSuccess ||
+        q->clusters < 1) {
+      cudaGetLastError();
+      if (msg) *msg = "no CTA pair of the tensor-core convolution can be resident";
+      return false;
+    }
+    const int mtp = (q->mt1 + 1) / 2;
+    q->n_tiles = q->n_tiles / q->mtiles * mtp;
+    q->mtiles = mtp;
+  }
+  return true;
+}
+
+int ctc_bn_slots(const CtcParams& q, int n_probs) {
+  return q.n_tiles / q.mtiles / n_probs * q.mt1 * (q.m2 ? 2 : 1) * 4;
+}
 
 bool wgtc_make_maps(CUtensorMap* mA, CUtensorMap* mB, WgtcParams* q, const WgtcDesc* descs,
                     int n_probs, std::string* msg) {
@@ -2438,15 +2610,34 @@ void launch_relayout_g1(const bf16* src, int64_t src_ps, int64_t src_off, bf16* 
              dst_ps, ca, co, n_indiv);
 }
 
-bool launch_conv_tc(const CUtensorMap& mW, const CUtensorMap& mA, const CtcParams& p, int sms,
+bool launch_conv_tc(const ConvWeightMaps& mW, const CUtensorMap& mA, const CtcParams& p, int sms,
                     cudaStream_t st) {
   const ConvKernel k = conv_kernel(p);
   if (!k) return false;
   const int ak = conv_ak(p);
+  if (ctc::conv_pair(ak, p.out_mode)) {
+    const int clusters = p.n_tiles < p.clusters ? p.n_tiles : p.clusters;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2 * clusters);
+    cfg.blockDim = dim3(ctc::THREADS);
+    cfg.dynamicSmemBytes = ctc::conv_smem(ak);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    const bool shared = st == nullptr || st == cudaStreamLegacy || st == cudaStreamPerThread;
+    cfg.attrs = attr;
+    cfg.numAttrs = shared ? 1 : 2;
+    return cudaLaunchKernelEx(&cfg, k, mW.half, mA, p) == cudaSuccess;
+  }
   // the compact variants: two CTAs per SM
-  const int ctas = ak == ctc::AK_NCHW || ak == ctc::AK_TRANS_C ? 2 * sms : sms;
+  const int ctas = ctc::conv_compact(ak) ? 2 * sms : sms;
   const int grid = p.n_tiles < ctas ? p.n_tiles : ctas;
-  launch_pdl(k, dim3(grid), dim3(ctc::THREADS), ctc::conv_smem(ak), st, mW, mA, p);
+  launch_pdl(k, dim3(grid), dim3(ctc::THREADS), ctc::conv_smem(ak), st, mW.full, mA, p);
   return true;
 }
 

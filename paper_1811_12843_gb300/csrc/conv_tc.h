@@ -57,6 +57,10 @@ struct CtcParams {
   // m2: 256-row tiles (set by ctc_make_act_map for channel-last outputs with nbox <= 128): two
   // 128-row A boxes and two accumulators (columns h * nbox) share each weight chunk
   int m2;
+  // parts of nA 128-row tiles (nA = m2 ? 2 : 1) per problem (and class): mtiles, or on CTA pairs,
+  // whose tiles hold two, before the pairing; clusters = CTA pairs resident at once (both set by
+  // ctc_make_act_map)
+  int mt1, clusters;
   const bf16* logit_w;  // CTC_LRELU_LOGIT
   int64_t logit_ws;
   // first layer, CTC_LRELU_HWC, 64 output channels: the output tiles go out by TMA through
@@ -65,10 +69,10 @@ struct CtcParams {
   const int* wsel;
   float slope;
   int* err;
-  // CTC_F32_HWC: non-null = also the batch-norm statistics of the output: per (tile, 128-row
+  // CTC_F32_HWC: non-null = also the batch-norm statistics of the output: per (part, 128-row
   // half, TMEM lane quarter) slot the per-channel sum and sum of squares over its valid rows,
-  // bn_part[slot][co] (slot = (tile * (m2 ? 2 : 1) + half) * 4 + quarter), for
-  // launch_bn_relu_hwc_part
+  // bn_part[slot][co] (slot = (part * (m2 ? 2 : 1) + half) * 4 + quarter; ctc_bn_slots of them per
+  // problem), for launch_bn_relu_hwc_part
   float2* bn_part;
 };
 
@@ -124,11 +128,20 @@ void launch_wgrad_tc(const CUtensorMap& mA, const CUtensorMap& mB, const WgtcPar
 
 bool ctc_make_map(CUtensorMap* m, const void* base, uint64_t K, uint64_t rows, uint64_t depth,
                   uint64_t depth_elems, uint32_t box_rows, std::string* msg);
+// A convolution's weight maps: boxes of nbox rows, and of nbox / 2 (a CTA pair's halves).
+struct ConvWeightMaps {
+  CUtensorMap full, half;
+};
+bool ctc_make_weight_maps(ConvWeightMaps* m, const void* base, uint64_t K, uint64_t rows,
+                          uint64_t depth, uint64_t depth_elems, uint32_t nbox, std::string* msg);
+// Batch-norm slots per problem of a launch of n_probs problems.
+int ctc_bn_slots(const CtcParams& q, int n_probs);
 // Activation map of a launch whose problems' channel-last inputs (ci a multiple of 64) sit at
 // a uniform stride from descs[0].in: dims (ci, W, W, rows, problems), a box of 64 channels by
 // the input pixels of 128 output pixels (traversal stride 2 for the convolution, 1 for the
 // parity classes). Sets q->a_tma = 1 when it applies (else 0, and the gather warps load A;
-// use_tma = false forces that), and then q->m2 and the 256-row tile count where they apply;
+// use_tma = false forces that), and then q->m2, the 256-row tile and CTA pair counts where they
+// apply (ctc_prepare comes first);
 // q->mtiles and q->n_tiles must count 128-row tiles on entry. False only when the driver
 // refuses the map.
 bool ctc_make_act_map(CUtensorMap* m, CtcParams* q, const ConvTcDesc* descs, int n_probs,
@@ -146,8 +159,9 @@ void launch_scatter_fix(const ConvTcDesc* descs, const float* halo, int n_proble
 // rows tap * 4 + output][64], the scatter mode's weights.
 void launch_relayout_s(const bf16* src, int64_t src_ps, int64_t src_off, bf16* dst, int n_indiv,
                        cudaStream_t st);
-// False (and nothing launched) when no kernel variant serves p's A kind and out mode.
-bool launch_conv_tc(const CUtensorMap& mW, const CUtensorMap& mA, const CtcParams& p, int sms,
+// False (and nothing launched) when no kernel variant serves p's A kind and out mode, or the
+// launch is refused.
+bool launch_conv_tc(const ConvWeightMaps& mW, const CUtensorMap& mA, const CtcParams& p, int sms,
                     cudaStream_t st);
 void launch_relayout_d(const bf16* src, bf16* dst, int n_indiv, int64_t Ps, const RelayoutD& r,
                        cudaStream_t st);

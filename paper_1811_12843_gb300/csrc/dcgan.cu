@@ -91,11 +91,12 @@ struct DcPlan {
   int splits_dw[4], splits_gw[5];
   int64_t pstride_dw[4], pstride_gw[5];
   int eval_launches, train_launches;
+  int ecells = 1;  // cells per launch of the tensor-core discriminator evaluation
   // tensor-core discriminator evaluation (bf16, ndf a multiple of 64): weights re-laid out as
   // [out][ky][kx][in] for every individual, a TMA map per layer, channel-last activations
   bool tc = false;
   bf16* Dwt = nullptr;
-  CUtensorMap mW[4];
+  ConvWeightMaps mW[4];
   CtcParams cp[4];
   ConvTcDesc* tcd[4];
   RelayoutD rel;
@@ -115,7 +116,7 @@ struct DcPlan {
   int64_t ddt_ps = 0, gct_ps = 0;
   RelayoutG reld;
   RelayoutC relc;
-  CUtensorMap mDd[4], mGc[4];
+  ConvWeightMaps mDd[4], mGc[4];
   CtcParams ddp[3], gdp[4], gcp[4];
   ConvTcDesc *ddd[3], *gdd[4], *gcd[4];
   LogitDesc *tdl_tc, *tdl_back_d_tc, *tdl_back_g_tc;
@@ -138,7 +139,7 @@ struct DcPlan {
   float2* bnp = nullptr;
   int bn_slots_e[3] = {0, 0, 0}, bn_slots_t[3] = {0, 0, 0};
   RelayoutG relg;
-  CUtensorMap mG[4];
+  ConvWeightMaps mG[4];
   CtcParams gp[4];
   ConvTcDesc* gtd[4];
   // activation maps of the channel-last tensor-core launches (A rows by TMA): evaluation D
@@ -149,7 +150,8 @@ struct DcPlan {
   // G-loss input gradient of discriminator layer 1 (gds)
   bool scg = false, scd = false;
   bf16 *Gs = nullptr, *Ds = nullptr;
-  CUtensorMap mGs, mDs, aEgs, aTgs, aGds;
+  ConvWeightMaps mGs, mDs;
+  CUtensorMap aEgs, aTgs, aGds;
   CtcParams egs, tgs, gds;
   float* halo = nullptr;
   std::vector<ConvTcDesc> h_gtd5, h_tgd5, h_gdd1;
@@ -260,12 +262,27 @@ DcPlan* dc_plan_create(const DcShape& s, const DcBuffers& b, std::string* msg) {
   float *ec, *emean, *einv, *tc, *tmean, *tinv, *dh;
   void *eh, *ex, *ey, *th, *ta, *P, *Q, *P2, *Q2, *dcb, *d5;
   int64_t stats = 15 * (int64_t)g;  // channels of the four batch-normalised layers
+  // The discriminator evaluation's activations, for the cells that share a launch: the
+  // tensor-core path takes as many as 8 GB hold (one cell per launch leaves the last wave of 480
+  // tiles on 152 SMs a sixth full: 5.1 against 4.6 ms for the 3x3 configuration's layers 2-4),
+  // and one where that much is not free
+  const int64_t per_cell = (int64_t)5 * 6 * B * (dmax + dsz[2]) * es;
+  p->ecells = tcd ? (int)std::min<int64_t>(C, std::max<int64_t>(1, (int64_t)8000000000 / per_cell))
+                  : 1;
+  auto alloc_chunk = [&]() -> int {
+    for (;;) {
+      if (!dev_alloc(p, &ex, (size_t)p->ecells * 5 * 6 * B * dmax * es, msg) &&
+          !dev_alloc(p, &ey, (size_t)p->ecells * 5 * 6 * B * dsz[2] * es, msg))
+        return 0;
+      if (p->ecells == 1) return 1;
+      p->ecells = 1;
+    }
+  };
   if (dev_alloc(p, &ec, (size_t)PE * B * gmax * 4, msg) ||
       dev_alloc(p, &eh, (size_t)PE * B * gmax * es, msg) ||
       dev_alloc(p, &emean, (size_t)PE * stats * 4, msg) ||
       dev_alloc(p, &einv, (size_t)PE * stats * 4, msg) ||
-      dev_alloc(p, &ex, (size_t)5 * 6 * B * dmax * es, msg) ||
-      dev_alloc(p, &ey, (size_t)5 * 6 * B * dsz[2] * es, msg) ||
+      alloc_chunk() ||
       dev_alloc(p, &tc, (size_t)C * B * gall * 4, msg) ||
       dev_alloc(p, &th, (size_t)C * B * gall * es, msg) ||
       dev_alloc(p, &tmean, (size_t)C * stats * 4, msg) ||
@@ -558,7 +575,7 @@ DcPlan* dc_plan_create(const DcShape& s, const DcBuffers& b, std::string* msg) {
       const int nbox = co < 256 ? co : 256;
       // the first layer's weights in their own [out][c][ky][kx] order, from the population
       const bf16* wbase = l == 1 ? (const bf16*)b.Dop + dof[0] : p->Dwt + dof[l - 1];
-      ok = ctc_make_map(&p->mW[l - 1], wbase, (uint64_t)ci * 16, co, s.n_indiv, b.PDs, nbox, msg);
+      ok = ctc_make_weight_maps(&p->mW[l - 1], wbase, (uint64_t)ci * 16, co, s.n_indiv, b.PDs, nbox, msg);
       CtcParams q;
       memset(&q, 0, sizeof q);
       q.rows = 6 * B;
@@ -571,7 +588,7 @@ DcPlan* dc_plan_create(const DcShape& s, const DcBuffers& b, std::string* msg) {
       q.nj = (co + 255) / 256;
       q.nbox = nbox;
       q.mtiles = ((6 * B << (2 * q.lho)) + 127) / 128;
-      q.n_tiles = 5 * q.mtiles;
+      q.n_tiles = 5 * p->ecells * q.mtiles;
       q.slope = s.slope;
       q.err = p->err;
       if (l == 4) {
@@ -584,8 +601,9 @@ DcPlan* dc_plan_create(const DcShape& s, const DcBuffers& b, std::string* msg) {
       std::vector<ConvTcDesc> vt;
       for (int c = 0; c < C; ++c)
         for (int sl = 0; sl < 5; ++sl) {
-          void* bx = elw(ex, (int64_t)sl * 6 * B * dmax);
-          void* by = elw(ey, (int64_t)sl * 6 * B * dsz[2]);
+          const int k = c % p->ecells * 5 + sl;  // place in the launch's buffers
+          void* bx = elw(ex, (int64_t)k * 6 * B * dmax);
+          void* by = elw(ey, (int64_t)k * 6 * B * dsz[2]);
           ConvTcDesc t;
           memset(&t, 0, sizeof t);
           t.in = (const bf16*)(l == 1 ? el(b.E, (int64_t)c * b.e_cell) : (l % 2 == 0 ? bx : by));
@@ -595,13 +613,14 @@ DcPlan* dc_plan_create(const DcShape& s, const DcBuffers& b, std::string* msg) {
           vt.push_back(t);
         }
       ok = ok && !upload(p, &p->tcd[l - 1], vt, msg);
-      // one map serves every cell: the chunk buffers are shared
-      ok = ok && act_map(&p->aEd[l - 1], &p->cp[l - 1], vt.data(), 5);
+      // one map serves every launch: the buffers are shared
+      const int n = 5 * p->ecells;
+      ok = ok && act_map(&p->aEd[l - 1], &p->cp[l - 1], vt.data(), n);
       // the first layer stores its output by TMA (its gather needs no activation map)
-      if (l == 1) ok = ok && ctc_make_out_map(&p->aEd[0], &p->cp[0], vt.data(), 5, msg);
-      for (size_t k = 5; k < vt.size() && ok && l >= 2; ++k)
-        if (vt[k].in != vt[k % 5].in) {
-          if (msg) *msg = "DCGAN evaluation buffers differ between cells";
+      if (l == 1) ok = ok && ctc_make_out_map(&p->aEd[0], &p->cp[0], vt.data(), n, msg);
+      for (size_t k = n; k < vt.size() && ok && l >= 2; ++k)
+        if (vt[k].in != vt[k % n].in) {
+          if (msg) *msg = "DCGAN evaluation buffers differ between launches";
           ok = false;
         }
     }
@@ -646,7 +665,7 @@ DcPlan* dc_plan_create(const DcShape& s, const DcBuffers& b, std::string* msg) {
       const int l = i + 2;
       const int ci = gc[l - 1], co = gc[l];
       const int nbox = l == 5 ? 16 : (co < 256 ? co : 256);
-      ok = ctc_make_map(&p->mG[i], p->Gwt + r.dst_off[i], (uint64_t)4 * ci, 4 * r.cls_rows[i],
+      ok = ctc_make_weight_maps(&p->mG[i], p->Gwt + r.dst_off[i], (uint64_t)4 * ci, 4 * r.cls_rows[i],
                         s.n_indiv, p->gwt_ps, nbox, msg);
       CtcParams q;
       memset(&q, 0, sizeof q);
@@ -687,13 +706,13 @@ DcPlan* dc_plan_create(const DcShape& s, const DcBuffers& b, std::string* msg) {
     int64_t bnmax = p->g1tc ? (int64_t)PE * 16 * gc[1] : 0;  // layer 1: a slot per tap
     for (int i = 0; i < 3; ++i) {
       const CtcParams& q = p->gp[i];
-      bnmax = std::max(bnmax, (int64_t)q.n_tiles * (q.m2 ? 2 : 1) * 4 * q.co);
+      bnmax = std::max(bnmax, (int64_t)ctc_bn_slots(q, PE) * PE * q.co);
     }
     ok = ok && !dev_alloc(p, &p->bnp, (size_t)bnmax * sizeof(float2), msg);
     for (int i = 0; i < 3 && ok; ++i) {
       CtcParams& q = p->gp[i];
       q.bn_part = p->bnp;
-      p->bn_slots_e[i] = q.n_tiles / PE * (q.m2 ? 2 : 1) * 4;
+      p->bn_slots_e[i] = ctc_bn_slots(q, PE);
     }
   }
   // ---- tensor-core training forward (channel-last), and the output layer's descriptors in
@@ -718,7 +737,7 @@ DcPlan* dc_plan_create(const DcShape& s, const DcBuffers& b, std::string* msg) {
       if (l == 5) p->h_tgd5 = vt;
       ok = ok && act_map(&p->aTg[i], &p->tgp[i], vt.data(), C);
       if (i < 3)
-        p->bn_slots_t[i] = p->tgp[i].n_tiles / C * (p->tgp[i].m2 ? 2 : 1) * 4;
+        p->bn_slots_t[i] = ctc_bn_slots(p->tgp[i], C);
     }
     for (int l = 1; l <= 4 && ok; ++l) {
       CtcParams q = p->cp[l - 1];
@@ -792,7 +811,7 @@ DcPlan* dc_plan_create(const DcShape& s, const DcBuffers& b, std::string* msg) {
     for (int i = 0; i < 4 && ok; ++i) {
       const int l = 4 - i;
       const int nbox = l == 1 ? 16 : (dc[l - 1] < 256 ? dc[l - 1] : 256);
-      ok = ctc_make_map(&p->mDd[l - 1], p->Ddt + r.dst_off[i], (uint64_t)4 * dc[l],
+      ok = ctc_make_weight_maps(&p->mDd[l - 1], p->Ddt + r.dst_off[i], (uint64_t)4 * dc[l],
                         4 * r.cls_rows[i], s.n_indiv, p->ddt_ps, nbox, msg);
       for (int chain = 0; chain < 2 && ok; ++chain) {
         if (chain == 0 && l == 1) continue;  // the D loss needs no input gradient of layer 1
@@ -865,9 +884,9 @@ DcPlan* dc_plan_create(const DcShape& s, const DcBuffers& b, std::string* msg) {
       // the output layer's input gradient reads 3-channel images: its weights in their own
       // [out][c][ky][kx] order, from the population (launch_relayout_c leaves them out)
       ok = gc[l] == 3
-               ? ctc_make_map(&p->mGc[i], (const bf16*)b.Gop + go[3 * (l - 1)], 48, co,
+               ? ctc_make_weight_maps(&p->mGc[i], (const bf16*)b.Gop + go[3 * (l - 1)], 48, co,
                               s.n_indiv, b.PGs, nbox, msg)
-               : ctc_make_map(&p->mGc[i], p->Gct + rc.dst_off[i], (uint64_t)16 * gc[l], co,
+               : ctc_make_weight_maps(&p->mGc[i], p->Gct + rc.dst_off[i], (uint64_t)16 * gc[l], co,
                               s.n_indiv, p->gct_ps, nbox, msg);
       CtcParams q;
       memset(&q, 0, sizeof q);
@@ -1022,7 +1041,7 @@ DcPlan* dc_plan_create(const DcShape& s, const DcBuffers& b, std::string* msg) {
     ok = !dev_alloc(p, &p->halo, (size_t)std::max(PE, C) * B * 8 * 768 * 4, msg);
     if (ok && p->scg) {
       ok = !dev_alloc(p, &p->Gs, (size_t)s.n_indiv * 4096 * 2, msg) &&
-           ctc_make_map(&p->mGs, p->Gs, 64, 64, s.n_indiv, 4096, 64, msg);
+           ctc_make_weight_maps(&p->mGs, p->Gs, 64, 64, s.n_indiv, 4096, 64, msg);
       p->egs = scatter_params(B, PE, CTC_TANH_CHW);
       p->egs.halo = p->halo;
       ok = ok && ctc_make_act_map(&p->aEgs, &p->egs, p->h_gtd5.data(), PE, msg);
@@ -1035,7 +1054,7 @@ DcPlan* dc_plan_create(const DcShape& s, const DcBuffers& b, std::string* msg) {
     }
     if (ok && p->scd) {
       ok = !dev_alloc(p, &p->Ds, (size_t)s.n_indiv * 4096 * 2, msg) &&
-           ctc_make_map(&p->mDs, p->Ds, 64, 64, s.n_indiv, 4096, 64, msg);
+           ctc_make_weight_maps(&p->mDs, p->Ds, 64, 64, s.n_indiv, 4096, 64, msg);
       p->gds = scatter_params(B, C, CTC_DTANH_CHW);
       p->gds.halo = p->halo;
       ok = ok && ctc_make_act_map(&p->aGds, &p->gds, p->h_gdd1.data(), C, msg);
@@ -1144,9 +1163,10 @@ int dc_eval_d(DcPlan* p, const int* nbr, cudaStream_t st, std::string* msg) {
     const int nI = p->rl_n > 0 ? p->rl_n : s.n_indiv;
     launch_relayout_d((const bf16*)p->b.Dop + lo * p->b.PDs, p->Dwt + lo * p->b.PDs, nI,
                       p->b.PDs, p->rel, st);
-    for (int c = 0; c < C; ++c) {
+    for (int c = 0; c < C; c += p->ecells) {
       for (int l = 1; l <= 4; ++l) {
         CtcParams q = p->cp[l - 1];
+        q.n_tiles = q.n_tiles / p->ecells * std::min(p->ecells, C - c);
         q.descs = p->tcd[l - 1] + c * 5;
         q.wsel = nbr;
         if (!launch_conv_tc(p->mW[l - 1], p->aEd[l - 1], q, p->sms, st)) return no_variant(msg);
@@ -1327,7 +1347,8 @@ int dc_train(DcPlan* p, cudaStream_t st, std::string* msg) {
 
 int dc_eval_launches(const DcPlan* p, int part) {
   if (part == 0) return p->tcg ? 14 + (p->scg ? 2 : 0) : 9;
-  return p->eval_launches - 9 + (p->tc ? 1 - p->s.cells : 0);
+  if (p->tc) return 1 + 4 * ((p->s.cells + p->ecells - 1) / p->ecells);
+  return p->eval_launches - 9;
 }
 
 int* dc_error_flag(DcPlan* p) { return p && (p->tc || p->tcg) ? p->err : nullptr; }
