@@ -80,7 +80,7 @@ __device__ __forceinline__ bool gather_bar_or(bool pred) {
 }
 
 enum { AK_CONV = 0, AK_TRANS = 1, AK_SCATTER = 2, AK_NCHW = 3, AK_GATHER = 4,
-       AK_NCHW_WIDE = 5, AK_TRANS_C = 6 };
+       AK_NCHW_WIDE = 5, AK_TRANS_C = 6, AK_FIRST = 7 };
 
 // Variants that run on CTA pairs (clusters of two, tcgen05 .cta_group::2): A by TMA and channel-last
 // outputs or logits. Each CTA holds its own 128 rows of A (256 with m2) and half of the weight
@@ -104,7 +104,7 @@ constexpr int SC_PLANE = 132;
 // parity classes (256-row tiles of weight tiles of at most 64 rows: two 40 KB stages, no patch
 // buffers) and the scatter mode (three 24 KB stages, the 16 taps' products) fit two CTAs per SM
 constexpr bool conv_compact(int ak) {
-  return ak == AK_NCHW || ak == AK_TRANS_C || ak == AK_SCATTER;
+  return ak == AK_NCHW || ak == AK_TRANS_C || ak == AK_SCATTER || ak == AK_FIRST;
 }
 // first-layer input patches: buffers, and tiles they are copied ahead (the compact variant's
 // copies come from DRAM: one tile ahead, a tile waited for them)
@@ -115,8 +115,14 @@ constexpr int patch_ahead(int ak) { return patch_bufs(ak) - 2; }
 constexpr int patch_area(int ak) {
   return ak == AK_TRANS_C ? 0 : (256 + patch_bufs(ak) * PATCH_BYTES + 1023) / 1024 * 1024 - 256;
 }
+// first layer of the discriminator (k_conv_first): two A tiles, three weight tiles, two 4 KB output
+// tiles per epilogue warp, the barriers and the patches
+constexpr int F_A = 2, F_B = 3, F_PATCHES = 4;
+constexpr int F_B_BYTES = 64 * BK * 2, F_OUT_BYTES = 32 * 128;
+constexpr int F_RING = F_A * A_BYTES + F_B * F_B_BYTES + 8 * F_OUT_BYTES;
 constexpr int conv_smem(int ak) {
-  return ak == AK_NCHW ? 1024 + 3 * (A_BYTES + 64 * BK * 2) + 256 + patch_area(ak) +
+  return ak == AK_FIRST ? 1024 + F_RING + 256 + F_PATCHES * PATCH_BYTES
+         : ak == AK_NCHW ? 1024 + 3 * (A_BYTES + 64 * BK * 2) + 256 + patch_area(ak) +
                              4 * STG_WORDS * 4
          : ak == AK_TRANS_C ? 1024 + 2 * (2 * A_BYTES + 64 * BK * 2) + 256 + 4 * STG_WORDS * 4
          : ak == AK_SCATTER ? 1024 + 3 * (A_BYTES + 64 * BK * 2) + 256 + 16 * SC_PLANE * 16
@@ -530,11 +536,6 @@ __global__ void __launch_bounds__(THREADS, conv_compact(AK) ? 2 : 1)
     const int row = q * 32 + lane;
     const uint32_t lane_base = (uint32_t)(q * 32) << 16;
     uint32_t* stg = reinterpret_cast<uint32_t*>(misc + 256 + kPatchArea) + (warp - 6) * STG_WORDS;
-    // tma_out (first layer, 64 channels): the tile's 128 rows x 128 bytes go to the staging area
-    // (1024-byte aligned) in the 128-byte swizzle, and one thread stores them by TMA through the
-    // output map (passed as mA, which the first layer's gather does not use)
-    const bool kTmaOut = AK == AK_NCHW && OM == CTC_LRELU_HWC && p.tma_out;
-    const uint32_t tileb = smem_u32(misc + 256 + kPatchArea);
     int uses[2] = {0, 0}, jobs = 0;
     bool ok = true;
     for (int tile = cta; tile < p.n_tiles && ok; tile += n_cta) {
@@ -561,7 +562,7 @@ __global__ void __launch_bounds__(THREADS, conv_compact(AK) ? 2 : 1)
         // the scatter epilogue synchronises the four warps: they leave together
         const bool okw =
             mbar_wait_warp(bAccF + 8 * R, (uint32_t)(uses[R] & 1), abort_flag, p.err, 28);
-        if ((kScatter || kTmaOut) ? epi_bar_or(!okw) : !okw) {
+        if (kScatter ? epi_bar_or(!okw) : !okw) {
           ok = false;
           break;
         }
@@ -676,11 +677,6 @@ __global__ void __launch_bounds__(THREADS, conv_compact(AK) ? 2 : 1)
             oxh = 2 * oxh + (cls & 1);
           }
           const int64_t pix = ((int64_t)(mh >> (2 * lq)) << (2 * p.lho)) + (oyh << p.lho) + oxh;
-          if (kTmaOut) {
-            // the previous tile's store has read the staging area before anyone rewrites it
-            if (threadIdx.x == 192) bulk_wait_read<0>();
-            epi_bar();
-          }
           for (int g = 0; g < nbox / 32; ++g) {
             uint32_t v[32];
             LIPZ_TMEM_LD32(tmem + lane_base + (uint32_t)(R * kAccStride + h * nbox + g * 32), v);
@@ -722,18 +718,6 @@ __global__ void __launch_bounds__(THREADS, conv_compact(AK) ? 2 : 1)
                 b = b > 0.f ? b : p.slope * b;
                 pk[e >> 1] = pack_bf16(a, b);
               }
-            }
-            if (kTmaOut) {
-              // row `row`, 16-byte units 4 g + u of its 128 bytes, in the 128-byte swizzle
-              const uint32_t rb = tileb + (uint32_t)row * 128u;
-#pragma unroll
-              for (int u = 0; u < 4; ++u)
-                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(
-                                 rb + ((uint32_t)((4 * g + u) ^ (row & 7)) << 4)),
-                             "r"(pk[4 * u]), "r"(pk[4 * u + 1]), "r"(pk[4 * u + 2]),
-                             "r"(pk[4 * u + 3])
-                             : "memory");
-              continue;
             }
             if constexpr (OM == CTC_LRELU_LOGIT) {
               // the output layer instead of storing the activations
@@ -797,15 +781,6 @@ __global__ void __launch_bounds__(THREADS, conv_compact(AK) ? 2 : 1)
             }
             __syncwarp();
           }
-          if (kTmaOut) {
-            // the four warps' rows are written: one thread stores the tile
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            epi_bar();
-            if (threadIdx.x == 192) {
-              tma_store_3d(&mA, tileb, j * 256, mh - row, pc);
-              bulk_commit();
-            }
-          }
           }
         }
         tc_fence_before();
@@ -825,8 +800,6 @@ __global__ void __launch_bounds__(THREADS, conv_compact(AK) ? 2 : 1)
       }
     }
   }
-  // the last TMA stores of the output have finished before the CTA leaves
-  if (AK == AK_NCHW && OM == CTC_LRELU_HWC && p.tma_out && threadIdx.x == 192) bulk_wait_all();
   __syncwarp();
   tc_fence_before();
   __syncthreads();
@@ -840,6 +813,255 @@ __global__ void __launch_bounds__(THREADS, conv_compact(AK) ? 2 : 1)
       asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
                    "r"(kTmemCols));
   }
+}
+
+// ---- the discriminator's first layer --------------------------------------------------------
+// 3 x 64 x 64 channel-major images to 64 x 32 x 32, LeakyReLU, bf16 channel-last: K = 48 values
+// (channel, ky, kx), 64 outputs, 128 output pixels (4 rows) per tile, M a multiple of 128. The
+// p.share problems of a group (a cell's discriminators in the evaluation) read the same images: a
+// tile's A operand is built once, by four gather warps from input patches copied ahead, and
+// multiplied with every problem's weights. Each epilogue warp stages its 32 rows x 128 bytes in the
+// 128-byte swizzle and stores them by TMA itself. Two CTAs per SM.
+// Bound: HBM (the outputs' store: 4.5 GB for the 3x3 configuration's evaluation).
+__global__ void __launch_bounds__(THREADS, 2)
+    k_conv_first(const __grid_constant__ CUtensorMap mW, const __grid_constant__ CUtensorMap mO,
+                 const __grid_constant__ CtcParams p) {
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t raw = smem_u32(smem_raw);
+  const uint32_t base = (raw + 1023u) & ~1023u;
+  uint8_t* misc = smem_raw + (base - raw) + F_RING;
+  const uint32_t sB = base + F_A * A_BYTES, sO = sB + F_B * F_B_BYTES;
+  const uint32_t fullA = smem_u32(misc), emptyA = fullA + 8 * F_A;
+  const uint32_t fullB = emptyA + 8 * F_A, emptyB = fullB + 8 * F_B;
+  const uint32_t accF = emptyB + 8 * F_B, accE = accF + 32, bFinal = accE + 32;  // [4] each
+  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(misc + 240);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 244);
+  uint8_t* patches = misc + 256;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < F_A; ++s) {
+      mbar_init(fullA + 8 * s, 128);
+      mbar_init(emptyA + 8 * s, 1);
+    }
+    for (int s = 0; s < F_B; ++s) {
+      mbar_init(fullB + 8 * s, 1);
+      mbar_init(emptyB + 8 * s, 1);
+    }
+    for (int r = 0; r < 4; ++r) {
+      mbar_init(accF + 8 * r, 1);
+      mbar_init(accE + 8 * r, 4);
+    }
+    mbar_init(bFinal, 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 256;" ::"r"(
+        smem_u32((const void*)tmem_slot)));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  pdl_wait();
+
+  if (warp == 0) {
+    // ---- weights by TMA, one tile of 64 rows per (tile, problem)
+    if (lane == 0) {
+      int st = 0, issued[F_B] = {};
+      uint32_t phase = 0;
+      bool ok = true;
+      for (int tile = blockIdx.x; tile < p.n_tiles && ok; tile += gridDim.x)
+        for (int j = 0; j < p.share; ++j) {
+          const int prob = tile / p.mtiles * p.share + j;
+          const int indiv = __ldg(&p.wsel[__ldg(&p.descs[prob].wsel_idx)]);
+          if (!mbar_wait(emptyB + 8 * st, phase ^ 1u, abort_flag, p.err, 21)) {
+            ok = false;
+            break;
+          }
+          mbar_expect_tx(fullB + 8 * st, (uint32_t)F_B_BYTES);
+          tma_load_3d(sB + st * F_B_BYTES, &mW, fullB + 8 * st, 0, 0, indiv);
+          issued[st]++;
+          if (++st == F_B) {
+            st = 0;
+            phase ^= 1u;
+          }
+        }
+      if (!ok)
+        for (int s = 0; s < F_B; ++s)
+          if (issued[s] > 0) {
+            volatile int never = 0;
+            mbar_wait(fullB + 8 * s, (uint32_t)((issued[s] - 1) & 1), &never, p.err, 22);
+          }
+    }
+  } else if (warp == 1) {
+    // ---- MMA issue: three K steps of 16 (the 49th value on is zero)
+    if (lane == 0) {
+      int sa = 0, sb = 0, job = 0;
+      uint32_t pa = 0, pb = 0;
+      bool ok = true;
+      const uint32_t idesc = idesc_bf16(BM, 64);
+      for (int tile = blockIdx.x; tile < p.n_tiles && ok; tile += gridDim.x) {
+        if (!mbar_wait(fullA + 8 * sa, pa, abort_flag, p.err, 24)) break;
+        for (int j = 0; j < p.share; ++j, ++job) {
+          const int R = job & 3, use = job >> 2;
+          if (!mbar_wait(fullB + 8 * sb, pb, abort_flag, p.err, 25) ||
+              (use > 0 &&
+               !mbar_wait(accE + 8 * R, (uint32_t)((use - 1) & 1), abort_flag, p.err, 23))) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint64_t dA = sw128_desc(base + sa * A_BYTES), dB = sw128_desc(sB + sb * F_B_BYTES);
+          const uint32_t dt = tmem + (uint32_t)(R * 64);
+          tc_mma(dt, dA, dB, idesc, 0u);
+          tc_mma_acc(dt, dA + 2, dB + 2, idesc);
+          tc_mma_acc(dt, dA + 4, dB + 4, idesc);
+          tc_commit(emptyB + 8 * sb);
+          tc_commit(accF + 8 * R);
+          if (++sb == F_B) {
+            sb = 0;
+            pb ^= 1u;
+          }
+        }
+        if (!ok) break;
+        tc_commit(emptyA + 8 * sa);
+        if (++sa == F_A) {
+          sa = 0;
+          pa ^= 1u;
+        }
+      }
+      tc_commit(bFinal);
+      volatile int never = 0;
+      mbar_wait(bFinal, 0u, &never, p.err, 26);
+    }
+  } else if (warp < 6) {
+    // ---- A operand: thread r builds row r of a tile from its 3 x 10 x 64 input patch, which the
+    // gather threads copy two tiles ahead by 8-byte cp.async into one of four buffers whose halo
+    // columns stay zero
+    const int r = threadIdx.x - 64;
+    const uint32_t patch0 = smem_u32(patches);
+    for (int i = r; i < F_PATCHES * PATCH_BYTES / 16; i += 128)
+      *reinterpret_cast<uint4*>(patches + 16 * i) = make_uint4(0u, 0u, 0u, 0u);
+    gather_bar_or(false);
+    auto prefetch = [&](int tile, int buf) {
+      if (tile < p.n_tiles) {
+        const bf16* in = p.descs[tile / p.mtiles * p.share].in;
+        const int m0 = (tile % p.mtiles) * BM;
+        const int nb = m0 >> 10, oy0 = (m0 >> 5) & 31;
+        for (int u = r; u < 480; u += 128) {
+          const int c = u / 160, rem = u - c * 160, pr = rem >> 4, q = rem & 15;
+          const int iy = 2 * oy0 - 1 + pr;
+          const bool ok = iy >= 0 && iy < 64;
+          const bf16* src = ok ? in + ((int64_t)(nb * 3 + c) << 12) + (iy << 6) + 4 * q : in;
+          cp_async8(patch0 + (uint32_t)(buf * PATCH_BYTES + ((c * 10 + pr) * 72 + 4 + 4 * q) * 2),
+                    src, ok ? 8 : 0);
+        }
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    prefetch(blockIdx.x, 0);
+    prefetch(blockIdx.x + gridDim.x, 1);
+    int buf = 0, sa = 0;
+    uint32_t phase = 0;
+    const int ox = r & 31, oyl = r >> 5;
+    for (int tile = blockIdx.x; tile < p.n_tiles; tile += gridDim.x) {
+      prefetch(tile + 2 * gridDim.x, (buf + 2) % F_PATCHES);
+      asm volatile("cp.async.wait_group 2;" ::: "memory");
+      const bool okw = mbar_wait_warp(emptyA + 8 * sa, phase ^ 1u, abort_flag, p.err, 27);
+      if (gather_bar_or(!okw)) break;
+      const uint32_t row = base + sa * A_BYTES + (uint32_t)r * 128u;
+      // group (c, ky) = k / 4: the four kx values are patch columns 2 ox + 3 .. 2 ox + 6 of
+      // patch row c * 10 + 2 oyl + ky, taken from the three aligned words at 2 ox + 2
+      const uint32_t* pw = reinterpret_cast<const uint32_t*>(patches + buf * PATCH_BYTES);
+#pragma unroll
+      for (int u = 0; u < 6; ++u) {
+        uint32_t w[4];
+#pragma unroll
+        for (int hh = 0; hh < 2; ++hh) {
+          const int gidx = 2 * u + hh;  // c * 4 + ky
+          const int c = gidx >> 2, ky = gidx & 3;
+          const int e0 = (c * 10 + 2 * oyl + ky) * 72 + 2 * ox + 2;
+          const uint32_t w0 = pw[e0 >> 1], w1 = pw[(e0 >> 1) + 1], w2 = pw[(e0 >> 1) + 2];
+          w[2 * hh] = __byte_perm(w0, w1, 0x5432);
+          w[2 * hh + 1] = __byte_perm(w1, w2, 0x5432);
+        }
+        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(
+                         row + ((uint32_t)(u ^ (r & 7)) << 4)),
+                     "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3])
+                     : "memory");
+      }
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      mbar_arrive(fullA + 8 * sa);
+      if (++sa == F_A) {
+        sa = 0;
+        phase ^= 1u;
+      }
+      buf = (buf + 1) % F_PATCHES;
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+  } else {
+    // ---- epilogue: LeakyReLU, bf16, this warp's 32 rows out by TMA
+    const int q = warp & 3;
+    const uint32_t lane_base = (uint32_t)(q * 32) << 16;
+    const uint32_t out0 = sO + (uint32_t)(q * 2 * F_OUT_BYTES);
+    int job = 0;
+    bool ok = true;
+    for (int tile = blockIdx.x; tile < p.n_tiles && ok; tile += gridDim.x)
+      for (int j = 0; j < p.share; ++j, ++job) {
+        const int R = job & 3, use = job >> 2;
+        if (!mbar_wait_warp(accF + 8 * R, (uint32_t)(use & 1), abort_flag, p.err, 28)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        uint32_t v[2][32];
+        LIPZ_TMEM_LD32(tmem + lane_base + (uint32_t)(R * 64), v[0]);
+        LIPZ_TMEM_LD32(tmem + lane_base + (uint32_t)(R * 64 + 32), v[1]);
+        tmem_wait_ld();
+        tc_fence_before();
+        __syncwarp();
+        // (the store of two jobs ago, from the same buffer, has read it)
+        if (lane == 0) {
+          mbar_arrive(accE + 8 * R);
+          bulk_wait_read<1>();
+        }
+        __syncwarp();
+        const uint32_t ob = out0 + (uint32_t)((job & 1) * F_OUT_BYTES), rb = ob + lane * 128u;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          uint32_t pk[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            float a = __uint_as_float(v[u >> 2][(u & 3) * 8 + 2 * e]);
+            float b = __uint_as_float(v[u >> 2][(u & 3) * 8 + 2 * e + 1]);
+            a = a > 0.f ? a : p.slope * a;
+            b = b > 0.f ? b : p.slope * b;
+            pk[e] = pack_bf16(a, b);
+          }
+          asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(
+                           rb + ((uint32_t)(u ^ (lane & 7)) << 4)),
+                       "r"(pk[0]), "r"(pk[1]), "r"(pk[2]), "r"(pk[3])
+                       : "memory");
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) {
+          tma_store_3d(&mO, ob, 0, (tile % p.mtiles) * BM + q * 32,
+                       tile / p.mtiles * p.share + j);
+          bulk_commit();
+        }
+      }
+    if (lane == 0) bulk_wait_all();
+  }
+  __syncwarp();
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == 1)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(tmem));
 }
 
 // ---- weight gradients on tcgen05 -----------------------------------------------------------
@@ -2334,21 +2556,24 @@ bool ctc_make_weight_maps(ConvWeightMaps* m, const void* base, uint64_t K, uint6
 bool ctc_make_out_map(CUtensorMap* m, CtcParams* q, const ConvTcDesc* descs, int n_probs,
                       std::string* msg) {
   q->tma_out = 0;
-  if (!q->nchw_in || q->out_mode != CTC_LRELU_HWC || q->co != 64 || q->nj != 1 || q->m2 ||
-      n_probs < 1)
-    return true;
+  if (!q->nchw_in || q->out_mode != CTC_LRELU_HWC || q->co != 64) return true;
   const int64_t M = (int64_t)q->rows << (2 * q->lho);  // output pixels of a problem
-  if (M % ctc::BM != 0) return true;
   const int64_t per = M * q->co;
   int64_t pstride = per;
   if (n_probs > 1) pstride = (int64_t)(descs[1].out - descs[0].out);
-  if (pstride < per || pstride % 8 != 0 || ((uintptr_t)descs[0].out & 15) != 0) return true;
-  for (int i = 2; i < n_probs; ++i)
-    if ((int64_t)(descs[i].out - descs[0].out) != i * pstride) return true;
+  bool fits = pstride >= per && pstride % 8 == 0 && ((uintptr_t)descs[0].out & 15) == 0 &&
+              q->share >= 1 && n_probs % q->share == 0;
+  for (int i = 1; i < n_probs && fits; ++i)
+    fits = (int64_t)(descs[i].out - descs[0].out) == i * pstride &&
+           descs[i].in == descs[i - i % q->share].in;
+  if (!fits) {
+    if (msg) *msg = "first convolution: outputs not at one stride, or a group's inputs differ";
+    return false;
+  }
   if (!ensure_encode(msg)) return false;
   cuuint64_t dims[3] = {(cuuint64_t)q->co, (cuuint64_t)M, (cuuint64_t)n_probs};
   cuuint64_t strides[2] = {(cuuint64_t)q->co * 2, (cuuint64_t)(pstride * 2)};
-  cuuint32_t box[3] = {64, (cuuint32_t)ctc::BM, 1};
+  cuuint32_t box[3] = {64, 32, 1};  // an epilogue warp's rows
   cuuint32_t es[3] = {1, 1, 1};
   CUresult r = g_encode_ctc(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, (void*)descs[0].out, dims,
                             strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -2381,7 +2606,7 @@ const ConvVariant kConvVariants[] = {
     {ctc::AK_TRANS_C, CTC_DLRELU_HWC, ctc::k_conv_tc<ctc::AK_TRANS_C, CTC_DLRELU_HWC>},
     {ctc::AK_SCATTER, CTC_TANH_CHW, ctc::k_conv_tc<ctc::AK_SCATTER, CTC_TANH_CHW>},
     {ctc::AK_SCATTER, CTC_DTANH_CHW, ctc::k_conv_tc<ctc::AK_SCATTER, CTC_DTANH_CHW>},
-    {ctc::AK_NCHW, CTC_LRELU_HWC, ctc::k_conv_tc<ctc::AK_NCHW, CTC_LRELU_HWC>},
+    {ctc::AK_FIRST, CTC_LRELU_HWC, ctc::k_conv_first},
     {ctc::AK_NCHW, CTC_F32_HWC, ctc::k_conv_tc<ctc::AK_NCHW, CTC_F32_HWC>},
     {ctc::AK_NCHW_WIDE, CTC_LRELU_HWC, ctc::k_conv_tc<ctc::AK_NCHW_WIDE, CTC_LRELU_HWC>},
     {ctc::AK_NCHW_WIDE, CTC_F32_HWC, ctc::k_conv_tc<ctc::AK_NCHW_WIDE, CTC_F32_HWC>},
@@ -2395,6 +2620,7 @@ const ConvVariant kConvVariants[] = {
 
 int conv_ak(const CtcParams& p) {
   return p.scatter   ? ctc::AK_SCATTER
+         : p.tma_out ? ctc::AK_FIRST
          : p.nchw_in ? (p.nbox <= 64 ? ctc::AK_NCHW : ctc::AK_NCHW_WIDE)
          : p.a_tma   ? (p.transposed ? (p.m2 && p.nbox <= 64 ? ctc::AK_TRANS_C : ctc::AK_TRANS)
                                      : ctc::AK_CONV)

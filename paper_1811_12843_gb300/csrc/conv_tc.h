@@ -63,9 +63,11 @@ struct CtcParams {
   int mt1, clusters;
   const bf16* logit_w;  // CTC_LRELU_LOGIT
   int64_t logit_ws;
-  // first layer, CTC_LRELU_HWC, 64 output channels: the output tiles go out by TMA through
-  // the map that ctc_make_out_map builds (passed in place of the activation map)
-  int tma_out;
+  // first layer, CTC_LRELU_HWC, 64 output channels: runs on k_conv_first, whose outputs go out by
+  // TMA through the map that ctc_make_out_map builds (passed in place of the activation map; it
+  // sets tma_out); `share` consecutive problems read the same images (n_tiles counts each group's
+  // tiles once)
+  int tma_out, share;
   const int* wsel;
   float slope;
   int* err;
@@ -146,10 +148,10 @@ int ctc_bn_slots(const CtcParams& q, int n_probs);
 // refuses the map.
 bool ctc_make_act_map(CUtensorMap* m, CtcParams* q, const ConvTcDesc* descs, int n_probs,
                       std::string* msg, bool use_tma = true);
-// Output map of a first-layer launch (nchw_in, CTC_LRELU_HWC, co 64) whose problems' outputs
-// sit at a uniform stride from descs[0].out: dims (64 channels, output pixels, problems), boxes
-// of 128 pixels in the 128-byte swizzle. Sets q->tma_out = 1 when it applies (else 0); false
-// only when the driver refuses the map.
+// Output map of a first-layer launch (nchw_in, CTC_LRELU_HWC, co 64; else nothing is done) whose
+// problems' outputs sit at a uniform stride from descs[0].out: dims (64 channels, output pixels,
+// problems), boxes of 32 pixels in the 128-byte swizzle. Sets q->tma_out = 1; false when the
+// outputs or the groups' shared inputs do not fit, or the driver refuses the map.
 bool ctc_make_out_map(CUtensorMap* m, CtcParams* q, const ConvTcDesc* descs, int n_probs,
                       std::string* msg);
 bool ctc_prepare(std::string* msg);

@@ -588,7 +588,9 @@ DcPlan* dc_plan_create(const DcShape& s, const DcBuffers& b, std::string* msg) {
       q.nj = (co + 255) / 256;
       q.nbox = nbox;
       q.mtiles = ((6 * B << (2 * q.lho)) + 127) / 128;
-      q.n_tiles = 5 * p->ecells * q.mtiles;
+      // the first layer builds a tile once for the cell's five discriminators
+      q.share = l == 1 && co == 64 ? 5 : 1;
+      q.n_tiles = 5 / q.share * p->ecells * q.mtiles;
       q.slope = s.slope;
       q.err = p->err;
       if (l == 4) {
@@ -742,6 +744,7 @@ DcPlan* dc_plan_create(const DcShape& s, const DcBuffers& b, std::string* msg) {
     for (int l = 1; l <= 4 && ok; ++l) {
       CtcParams q = p->cp[l - 1];
       q.rows = 2 * B;
+      q.share = 1;
       q.mtiles = ((2 * B << (2 * q.lho)) + 127) / 128;
       q.n_tiles = C * q.mtiles;
       q.out_mode = CTC_LRELU_HWC;  // training keeps the activations (the backward reads them)

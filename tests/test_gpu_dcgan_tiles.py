@@ -1,0 +1,39 @@
+"""The tensor-core convolutions' tiles: batches whose output pixels end inside a 128-row tile, a
+CTA pair or a 256-row tile, one and several cells per launch, and widths with 128- and 256-column
+weight tiles. One iteration through the TMA kernels (CTA pairs, 256-row tiles, the shared first
+layer) must end in the state of the one-CTA kernels that gather their A rows, bit for bit, and the
+evaluation must meet the oracle."""
+
+import numpy as np
+import pytest
+
+from oracle import lipz_oracle as O
+
+from helpers import max_rel
+from test_gpu_dcgan import L, _field_pool, _grid, _state  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("rows,cols,batch,ngf,ndf", [
+    (1, 1, 1, 64, 64), (1, 2, 3, 64, 64), (1, 1, 7, 64, 64), (2, 2, 20, 64, 64), (1, 2, 35, 64, 64),
+    (1, 1, 8, 128, 64)])
+def test_tma_pairs_equal_gathered_tiles(L, monkeypatch, rows, cols, batch, ngf, ndf):  # noqa: F811
+    pool = _field_pool(6, 64)
+    out = []
+    for gather in ("0", "1"):
+        monkeypatch.setenv("LIPZ_CONV_GATHER", gather)
+        g = _grid(L, rows, cols, 3, pool, precision="bf16", batch=batch, ngf=ngf, ndf=ndf)
+        g.iterate(2)
+        out.append(np.frombuffer(g.export_state(), np.uint8))
+    assert np.array_equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("batch", [1, 9])
+def test_evaluation_against_the_oracle(L, batch):  # noqa: F811
+    pool = _field_pool(5, 30)
+    g = _grid(L, 1, 1, 9, pool, precision="bf16", batch=batch, ngf=64, ndf=64)
+    s = _state(g)
+    ref = O.eval_neighborhoods(s, O.batches(s, pool))
+    g.eval()
+    assert max_rel(g.logits(), ref["logits"]) < 2e-2
