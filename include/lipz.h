@@ -313,21 +313,16 @@ LIPZ_API int lipz_profile_read(lipz_grid* g, double* ms, int64_t* count, int64_t
  * cudaMalloc when they need the fitness: a serving loop whose device memory is fully reserved
  * by another allocator (a new allocation would fail), or a latency-critical path that cannot
  * afford the implicit synchronisation of cudaMalloc / cudaFree. The per-pair losses that the
- * computation needs go to one file-scope device array of about 800 KB, which every GPU that
- * loads this library holds until the process exits.
+ * computation needs stay on chip.
  *   logits: device, [cells][5 (j)][6 * batch] fp32, laid out as lipz_get_logits returns it;
  *   fit_g, fit_d: device outputs [cells][5] fp32 (as lipz_eval_neighborhoods computes them);
  *   stream: the cudaStream_t to run on (0 = legacy default). The call is asynchronous.
  * The library cannot check device buffers: they must hold the sizes above.
  * Limits: 1 <= cells <= LIPZ_NOALLOC_MAX_CELLS and batch >= 1, else LIPZ_ERR_INVALID with
  * nothing launched; a null pointer also gives LIPZ_ERR_INVALID. LIPZ_ERR_CUDA if a CUDA call
- * fails. The first call on a device looks up the array's device address (once per device,
- * with that device current) and keeps it for the life of the process: make that first call
- * before any stream capture, and do not use the call across a cudaDeviceReset (the array
- * moves with the device's primary context). All calls share the array, and each call
- * overwrites what it uses, so two calls whose work overlaps on the GPU (different streams,
- * no ordering) race. Non-finite losses are reported only through NaN/Inf fitness values
- * (lipz_eval_neighborhoods returns LIPZ_ERR_NONFINITE for them; this call has no channel).
+ * fails. Calls share nothing: they may overlap on several streams, and be captured. Non-finite
+ * losses are reported only through NaN/Inf fitness values (lipz_eval_neighborhoods returns
+ * LIPZ_ERR_NONFINITE for them; this call has no channel).
  */
 #define LIPZ_NOALLOC_MAX_CELLS 4096
 LIPZ_API int lipz_fitness_from_logits_noalloc(const float* logits, int32_t cells, int32_t batch,

@@ -85,6 +85,7 @@ struct StatusFlags {
 };
 void launch_gather_status(const float* fG, const float* fD, int n, const StatusFlags& fl,
                           float* out, bool pdl, cudaStream_t st);
+// LG, LD and flag may be null together.
 void launch_fitness(const float* logits, int cells, int B, float* LG, float* LD, float* fG,
                     float* fD, int* flag, cudaStream_t st);
 // Also writes, per cell and population, the Adam coefficients of the new centre's next step:

@@ -82,135 +82,117 @@ __device__ __forceinline__ void store4<bf16>(bf16* dst, float4 v) {
   *reinterpret_cast<uint2*>(dst) = pk;
 }
 
-// Four minibatch rows per warp: one Philox block gives the four rows' pool indices, and the
-// rows' 16-byte-vector copies are issued together (every load, then every store), so a warp
-// waits for memory once; then each row's normals, one Philox block (four normals) per lane at
-// a time. The pool is held in the population's precision, so a drawn row is a plain copy;
-// rows given by the caller (xin, fp32) are rounded here.
+// Blocks [0, nr) of a cell copy its real rows: four per warp from the pool (one Philox block gives
+// their indices; their vectors' loads are issued eight at a time, then stored), or one per warp
+// from the caller's fp32 batch xin, rounded here. The other blocks draw the noise, a Philox block
+// (four normals, consecutive in Z) per thread. The pool is held in the population's precision, so a
+// drawn row is a plain copy in vectors of the widest size that its length allows.
+// Bound: the launch and two memory latencies on small grids, then the rows' copies. Measured as a
+// phase, before (a warp's noise behind its rows, half of the lanes idle, rows of no 16-byte multiple
+// element by element) and now: 12x12 cells, B = 100, bf16 20 -> 15.5 us; 3x4 cells with rows of 500
+// bf16 28 -> 8.7 us; 3x3 cells, fp32 15 -> 11 us.
 constexpr int DRAW_RPW = 4;
 
+template <typename V>
+__device__ __forceinline__ void copy_rows(const char* pool, const uint32_t (&idx)[DRAW_RPW],
+                                          char* dst, int nb, int64_t bytes, int lane) {
+  const int nv = (int)(bytes / sizeof(V));
+  for (int v0 = lane; v0 < nb * nv; v0 += 8 * 32) {
+    V t[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int v = v0 + 32 * u;
+      if (v >= nb * nv) continue;
+      const int r = (v >= nv) + (v >= 2 * nv) + (v >= 3 * nv);
+      const uint32_t i = r == 0 ? idx[0] : r == 1 ? idx[1] : r == 2 ? idx[2] : idx[3];
+      t[u] = __ldg(reinterpret_cast<const V*>(pool + i * bytes) + (v - r * nv));
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (v0 + 32 * u < nb * nv) reinterpret_cast<V*>(dst)[v0 + 32 * u] = t[u];
+  }
+}
+
 template <typename T>
-__global__ void k_draw_batch(const T* __restrict__ pool, int64_t n_pool,
-                             const float* __restrict__ xin, T* __restrict__ E, int64_t e_cell,
-                             T* __restrict__ Z, int B, int x_dim, int z_dim, uint64_t seed,
-                             uint32_t t, uint32_t step, int parts) {
-  pdl_wait();
+__global__ void __launch_bounds__(256) k_draw_batch(
+    const T* __restrict__ pool, int64_t n_pool, const float* __restrict__ xin, T* __restrict__ E,
+    int64_t e_cell, T* __restrict__ Z, int B, int x_dim, int z_dim, uint64_t seed, uint32_t t,
+    uint32_t step, int nr) {
   const uint32_t s_batch = 3u + (step << 8), s_noise = 4u + (step << 8);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int q = blockIdx.x * (blockDim.x >> 5) + warp, c = blockIdx.y;
-  const int b0 = q * DRAW_RPW;
+  const int c = blockIdx.y, bx = blockIdx.x;
+  if (bx >= nr) {
+    const int64_t n = (int64_t)B * z_dim;
+    const int64_t blk = (int64_t)(bx - nr) * blockDim.x + threadIdx.x;
+    if (4 * blk >= n) {
+      pdl_wait();
+      return;
+    }
+    const U4 rn = philox_block(seed, s_noise, t, (uint32_t)c, (uint32_t)blk);
+    const float2 g01 = box_muller(rn.x, rn.y), g23 = box_muller(rn.z, rn.w);
+    pdl_wait();
+    T* z = Z + c * n + 4 * blk;
+    if ((n & 3) == 0) {
+      store4<T>(z, make_float4(g01.x, g01.y, g23.x, g23.y));
+    } else {
+      const float v[4] = {g01.x, g01.y, g23.x, g23.y};
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (4 * blk + q < n) z[q] = from_f<T>(v[q]);
+    }
+    return;
+  }
+  if (xin) {
+    pdl_wait();
+    const int b = bx * 8 + warp;
+    if (b >= B) return;
+    T* dst = E + (int64_t)c * e_cell + (int64_t)b * x_dim;
+    const float* src = xin + ((int64_t)c * B + b) * x_dim;
+    const bool vec = (x_dim & 3) == 0 && ((reinterpret_cast<uintptr_t>(src) & 15) == 0) &&
+                     ((reinterpret_cast<uintptr_t>(dst) & (4 * sizeof(T) - 1)) == 0);
+    if (!vec) {
+      for (int k = lane; k < x_dim; k += 32) dst[k] = from_f<T>(src[k]);
+      return;
+    }
+    for (int k0 = lane * 4; k0 < x_dim; k0 += 8 * 128) {
+      float4 v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (k0 + 128 * u < x_dim) v[u] = __ldg(reinterpret_cast<const float4*>(src + k0 + 128 * u));
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (k0 + 128 * u < x_dim) store4<T>(dst + k0 + 128 * u, v[u]);
+    }
+    return;
+  }
+  // rows 4q .. 4q + 3 take the four words of Philox block q
+  const int q = bx * 8 + warp, b0 = q * DRAW_RPW;
+  const U4 r = philox_block(seed, s_batch, t, (uint32_t)c, (uint32_t)q);
+  const uint32_t idx[DRAW_RPW] = {mulhi_u32(r.x, (uint32_t)n_pool), mulhi_u32(r.y, (uint32_t)n_pool),
+                                  mulhi_u32(r.z, (uint32_t)n_pool), mulhi_u32(r.w, (uint32_t)n_pool)};
+  pdl_wait();
   if (b0 >= B) return;
   const int nb = min(DRAW_RPW, B - b0);
-  T* const dst0 = E + (int64_t)c * e_cell + (int64_t)b0 * x_dim;
-  if (!(parts & DRAW_REAL)) {
-  } else if (xin) {
-    for (int i = 0; i < nb; ++i) {
-      T* dst = dst0 + (int64_t)i * x_dim;
-      const float* src = xin + ((int64_t)c * B + b0 + i) * x_dim;
-      const bool vec = (x_dim & 3) == 0 && ((reinterpret_cast<uintptr_t>(src) & 15) == 0) &&
-                       ((reinterpret_cast<uintptr_t>(dst) & (4 * sizeof(T) - 1)) == 0);
-      if (vec && x_dim <= 1024) {
-        // the row's (up to eight per lane) 16-byte loads issued before its stores
-        float4 v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int k = lane * 4 + 128 * u;
-          if (k < x_dim) v[u] = __ldg(reinterpret_cast<const float4*>(src + k));
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int k = lane * 4 + 128 * u;
-          if (k < x_dim) store4<T>(dst + k, v[u]);
-        }
-      } else if (vec) {
-        for (int k = lane * 4; k < x_dim; k += 128)
-          store4<T>(dst + k, __ldg(reinterpret_cast<const float4*>(src + k)));
-      } else {
-        for (int k = lane; k < x_dim; k += 32) dst[k] = from_f<T>(src[k]);
-      }
-    }
-  } else {
-    // rows 4q .. 4q + 3 take the four words of Philox block q
-    const U4 r = philox_block(seed, s_batch, t, (uint32_t)c, (uint32_t)q);
-    const uint32_t wd[DRAW_RPW] = {r.x, r.y, r.z, r.w};
-    const int bytes = x_dim * (int)sizeof(T);
-    const int n4 = bytes >> 4;
-    const bool vec = (bytes & 15) == 0 &&
-                     ((reinterpret_cast<uintptr_t>(pool) | reinterpret_cast<uintptr_t>(E)) & 15) == 0 &&
-                     ((e_cell * (int64_t)sizeof(T)) & 15) == 0;
-    if (vec && n4 > 128) {
-      // long rows (images): row by row, four vectors of a row in flight per lane
-      for (int i = 0; i < nb; ++i) {
-        const uint4* s4 = reinterpret_cast<const uint4*>(
-            pool + (int64_t)mulhi_u32(wd[i], (uint32_t)n_pool) * x_dim);
-        uint4* d4 = reinterpret_cast<uint4*>(dst0 + (int64_t)i * x_dim);
-#pragma unroll 4
-        for (int k = lane; k < n4; k += 32) d4[k] = __ldg(s4 + k);
-      }
-    } else if (vec) {
-      uint4 v[DRAW_RPW][4];
-#pragma unroll
-      for (int i = 0; i < DRAW_RPW; ++i) {
-        const uint4* s4 = reinterpret_cast<const uint4*>(
-            pool + (int64_t)mulhi_u32(wd[i], (uint32_t)n_pool) * x_dim);
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int k = lane + 32 * u;
-          if (i < nb && k < n4) v[i][u] = __ldg(s4 + k);
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < DRAW_RPW; ++i) {
-        uint4* d4 = reinterpret_cast<uint4*>(dst0 + (int64_t)i * x_dim);
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const int k = lane + 32 * u;
-          if (i < nb && k < n4) d4[k] = v[i][u];
-        }
-      }
-    } else {
-      for (int i = 0; i < nb; ++i) {
-        const T* src = pool + (int64_t)mulhi_u32(wd[i], (uint32_t)n_pool) * x_dim;
-        T* dst = dst0 + (int64_t)i * x_dim;
-        for (int k = lane; k < x_dim; k += 32) dst[k] = src[k];
-      }
-    }
-  }
-  if (!(parts & DRAW_NOISE)) return;
-  for (int i = 0; i < nb; ++i) {
-    const int b = b0 + i;
-    T* zr = Z + ((int64_t)c * B + b) * z_dim;
-    const uint32_t n0 = (uint32_t)b * (uint32_t)z_dim;
-    // normals n0 .. n0 + z_dim - 1; Philox block i holds normals 4i .. 4i + 3
-    if ((z_dim & 3) == 0 && ((reinterpret_cast<uintptr_t>(zr) & (4 * sizeof(T) - 1)) == 0)) {
-      // every block lies inside the row and its four normals are one aligned vector
-      for (int k = lane * 4; k < z_dim; k += 128) {
-        const U4 rn = philox_block(seed, s_noise, t, (uint32_t)c, (n0 + (uint32_t)k) >> 2);
-        const float2 g01 = box_muller(rn.x, rn.y), g23 = box_muller(rn.z, rn.w);
-        store4<T>(zr + k, make_float4(g01.x, g01.y, g23.x, g23.y));
-      }
-      continue;
-    }
-    for (uint32_t blk = (n0 >> 2) + lane; blk * 4 < n0 + (uint32_t)z_dim; blk += 32) {
-      const U4 rn = philox_block(seed, s_noise, t, (uint32_t)c, blk);
-      const float2 g01 = box_muller(rn.x, rn.y), g23 = box_muller(rn.z, rn.w);
-      const float vv[4] = {g01.x, g01.y, g23.x, g23.y};
-#pragma unroll
-      for (int qq = 0; qq < 4; ++qq) {
-        const uint32_t n = blk * 4 + qq;
-        if (n >= n0 && n < n0 + (uint32_t)z_dim) zr[n - n0] = from_f<T>(vv[qq]);
-      }
-    }
-  }
+  const int64_t bytes = (int64_t)x_dim * sizeof(T);
+  char* dst = reinterpret_cast<char*>(E + (int64_t)c * e_cell + (int64_t)b0 * x_dim);
+  const char* src = reinterpret_cast<const char*>(pool);
+  // (pool and E start on 256-byte boundaries, and a cell's part of E is 6 B whole rows)
+  if ((bytes & 15) == 0) copy_rows<uint4>(src, idx, dst, nb, bytes, lane);
+  else if ((bytes & 7) == 0) copy_rows<uint2>(src, idx, dst, nb, bytes, lane);
+  else if ((bytes & 3) == 0) copy_rows<unsigned>(src, idx, dst, nb, bytes, lane);
+  else copy_rows<unsigned short>(src, idx, dst, nb, bytes, lane);
 }
 
 template <typename T>
 void launch_draw_batch(const T* pool, int64_t n_pool, const float* xin, T* E, int64_t e_cell,
                        T* Z, int cells, int B, int x_dim, int z_dim, uint64_t seed, uint32_t t,
                        uint32_t step, int parts, bool pdl, cudaStream_t st) {
-  launch_kernel(pdl, k_draw_batch<T>, dim3((B + 8 * DRAW_RPW - 1) / (8 * DRAW_RPW), cells),
-                dim3(256), 0, st, pool, n_pool,
-                xin, E, e_cell, Z, B, x_dim, z_dim, seed, t, step, parts);
+  const int rows = xin ? 8 : 8 * DRAW_RPW;  // of a block
+  const int nr = parts & DRAW_REAL ? (B + rows - 1) / rows : 0;
+  const int nn = parts & DRAW_NOISE ? (int)(((int64_t)B * z_dim + 1023) / 1024) : 0;
+  if (nr + nn == 0) return;
+  launch_kernel(pdl, k_draw_batch<T>, dim3(nr + nn, cells), dim3(256), 0, st, pool, n_pool, xin, E,
+                e_cell, Z, B, x_dim, z_dim, seed, t, step, nr);
 }
 template void launch_draw_batch<float>(const float*, int64_t, const float*, float*, int64_t,
                                        float*, int, int, int, int, uint64_t, uint32_t, uint32_t,
@@ -534,32 +516,51 @@ __device__ float mutate(float lr, uint64_t seed, uint32_t stream, uint32_t t, ui
   return fmaxf(lr + std * n, 1e-8f);
 }
 
-// Records the choice of population `pop` (0 G, 1 D) for cell c: slot s, source individual src,
-// the new lr and the Adam coefficients (lr, 1 / (1 - beta1^t), 1 / (1 - beta2^t), t) of the
-// source's next step t.
-__device__ void write_choice(int c, int pop, int s, int src, float lr, const SelectParams& p,
-                             const SelectIO& io) {
-  const int step1 = io.step_old[pop][src] + 1;
+// The Adam coefficients (lr, 1 / (1 - beta1^t), 1 / (1 - beta2^t), t) of step t = step1.
+__device__ __forceinline__ float4 adam_coef(float lr, int step1, const SelectParams& p) {
   // 1 - beta^t = -expm1(t * log1p(-(1 - beta))): 1 - beta is exact in fp32 for beta in
   // [0.5, 1), and the expm1 form keeps full relative precision for beta^t near 1
   const float bc1 = -expm1f((float)step1 * log1pf(-(1.f - p.beta1)));
   const float bc2 = -expm1f((float)step1 * log1pf(-(1.f - p.beta2)));
-  io.coef[pop][c] = make_float4(lr, 1.f / bc1, 1.f / bc2, (float)step1);
+  return make_float4(lr, 1.f / bc1, 1.f / bc2, (float)step1);
+}
+
+// Records the choice of population `pop` (0 G, 1 D) for cell c: slot s, source individual src,
+// the new lr and the Adam coefficients of the source's next step.
+__device__ void write_choice(int c, int pop, int s, int src, float lr, const SelectParams& p,
+                             const SelectIO& io) {
+  io.coef[pop][c] = adam_coef(lr, io.step_old[pop][src] + 1, p);
   io.sel[pop][c] = s;
   io.src[pop][c] = src;
   io.lr_new[pop][c] = lr;
 }
 
 // Tournament, replacement and lr mutation of population `pop` (0 G, 1 D) of cell c, given the
-// five fitnesses f5 of the cell's neighbourhood; writes the selection, the source individual,
-// the new lr and the Adam coefficients (lr, 1 / (1 - beta1^t), 1 / (1 - beta2^t), t).
-__device__ void select_one(int c, int pop, const float* f5, const int* __restrict__ nbr,
-                           const SelectParams& p, const SelectIO& io) {
+// five fitnesses f5 of the cell's neighbourhood and the tournament's words; returns the new
+// centre's slot.
+__device__ int select_slot(const float* f5, const uint32_t* w, const SelectParams& p) {
+  const int win = tournament_slot(f5, w, p.tournament_size);
+  return p.replace_always ? win : (f5[win] < f5[0] ? win : 0);
+}
+
+// The tournament words of population `pop` of cell c.
+__device__ __forceinline__ void select_words(int c, int pop, const SelectParams& p, uint32_t (&w)[5]) {
   const U4 a = philox_block(p.seed, pop ? 6u : 5u, p.t, (uint32_t)c, 0u);
   const U4 b = philox_block(p.seed, pop ? 6u : 5u, p.t, (uint32_t)c, 1u);
-  const uint32_t w[5] = {a.x, a.y, a.z, a.w, b.x};
-  const int win = tournament_slot(f5, w, p.tournament_size);
-  const int s = p.replace_always ? win : (f5[win] < f5[0] ? win : 0);
+  w[0] = a.x;
+  w[1] = a.y;
+  w[2] = a.z;
+  w[3] = a.w;
+  w[4] = b.x;
+}
+
+// Selection of one cell and population; writes the slot, the source individual, the new lr and
+// the Adam coefficients (lr, 1 / (1 - beta1^t), 1 / (1 - beta2^t), t).
+__device__ void select_one(int c, int pop, const float* f5, const int* __restrict__ nbr,
+                           const SelectParams& p, const SelectIO& io) {
+  uint32_t w[5];
+  select_words(c, pop, p, w);
+  const int s = select_slot(f5, w, p);
   const int src = nbr[c * 5 + s];
   float lr = io.lr_old[pop][src];
   if (p.lr_mutation)
@@ -588,43 +589,53 @@ __global__ void k_select(const float* __restrict__ fG, const float* __restrict__
   select_one(c, pop, (pop ? fD : fG) + c * 5, nbr, p, io);
 }
 
+// One block per cell, a warp per mean (30), and with SELECT one more that reads what the tournaments
+// need (the words, the five slots' learning rates, steps and Adam coefficients) while the others
+// wait for the logits. LG, LD (with the non-finite flag) are optional.
+// Bound: the launch and two memory latencies (12x12 cells with selection 11.4 -> 10.3 us as a phase;
+// 2x2 cells without LG, LD and the clearing of the flag that they need 6.4 -> 5.4 us a call).
 template <bool SELECT>
-__global__ void k_fitness(const float* __restrict__ logits, int B, float* __restrict__ LG,
-                          float* __restrict__ LD, float* __restrict__ fG, float* __restrict__ fD,
-                          int* __restrict__ flag, const int* __restrict__ nbr, SelectParams sp,
-                          SelectIO io) {
-  pdl_wait();
+__global__ void __launch_bounds__(992) k_fitness(
+    const float* __restrict__ logits, int B, float* __restrict__ LG, float* __restrict__ LD,
+    float* __restrict__ fG, float* __restrict__ fD, int* __restrict__ flag,
+    const int* __restrict__ nbr, SelectParams sp, SelectIO io) {
   const int c = blockIdx.x;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   __shared__ float real_s[5], fake_d[25], fake_g[25], f_s[10];
-  const float* lc = logits + (int64_t)c * 5 * 6 * B;
-  for (int task = warp; task < 30; task += nw) {
+  __shared__ float4 coef_s[10];
+  __shared__ int src_s[10];
+  uint32_t words[5];
+  if (SELECT && warp == 30 && lane < 2) select_words(c, lane, sp, words);
+  pdl_wait();
+  if (SELECT && warp == 30) {
+    if (lane < 10) {
+      const int pop = lane / 5, src = nbr[c * 5 + lane % 5];
+      const float lr = io.lr_old[pop][src];
+      src_s[lane] = src;
+      coef_s[lane] = adam_coef(lr, io.step_old[pop][src] + 1, sp);
+    }
+  } else {
+    const float* lc = logits + (int64_t)c * 5 * 6 * B;
+    const int task = warp;
     float s1 = 0.f, s2 = 0.f;
     const bool real = task < 5;
     const int i = real ? 0 : (task - 5) / 5, j = real ? task : (task - 5) % 5;
     const float* l = lc + (int64_t)j * 6 * B + (real ? 0 : (int64_t)(1 + i) * B);
-    if (B <= 128) {
-      // a lane's (up to four) logits loaded before any is used: one memory latency per mean;
-      // the terms are still added in increasing row order
+    // four of a lane's logits loaded before any is used; the terms are still added in increasing
+    // row order
+    for (int b0 = lane; b0 < B; b0 += 128) {
       float x[4];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) x[u] = lane + 32 * u < B ? l[lane + 32 * u] : 0.f;
+      for (int u = 0; u < 4; ++u) x[u] = b0 + 32 * u < B ? l[b0 + 32 * u] : 0.f;
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
-        if (lane + 32 * u >= B) break;
+        if (b0 + 32 * u >= B) break;
         if (real) {
           s1 += softplusf(-x[u]);
         } else {
           s1 += softplusf(x[u]);
           s2 += softplusf(-x[u]);
         }
-      }
-    } else if (real) {
-      for (int b = lane; b < B; b += 32) s1 += softplusf(-l[b]);
-    } else {
-      for (int b = lane; b < B; b += 32) {
-        s1 += softplusf(l[b]);
-        s2 += softplusf(-l[b]);
       }
     }
 #pragma unroll
@@ -641,38 +652,39 @@ __global__ void k_fitness(const float* __restrict__ logits, int B, float* __rest
     }
   }
   __syncthreads();
-  if (threadIdx.x < 25) {
-    const int i = threadIdx.x / 5, j = threadIdx.x % 5;
-    const float ld = real_s[j] + fake_d[threadIdx.x];
+  if (LG && threadIdx.x < 25) {
+    const float ld = real_s[threadIdx.x % 5] + fake_d[threadIdx.x];
     const float lg = fake_g[threadIdx.x];
     LD[c * 25 + threadIdx.x] = ld;
     LG[c * 25 + threadIdx.x] = lg;
     if (!isfinite(ld) || !isfinite(lg)) atomicMin(flag, c);
-    (void)i;
   }
-  __syncthreads();
-  if (threadIdx.x < 5) {
-    const int i = threadIdx.x;
-    float sg = 0.f, sd = 0.f;
-    for (int j = 0; j < 5; ++j) {
-      sg += fake_g[i * 5 + j];
-      sd += real_s[i] + fake_d[j * 5 + i];  // f_D of slot i: mean over generator slots j
+  if (warp == (SELECT ? 30 : 1)) {
+    if (lane < 10) {
+      const int i = lane % 5;
+      float s = 0.f;
+      for (int j = 0; j < 5; ++j)  // f_D of slot i: mean over generator slots j
+        s += lane < 5 ? fake_g[i * 5 + j] : real_s[i] + fake_d[j * 5 + i];
+      (lane < 5 ? fG : fD)[c * 5 + i] = s / 5.f;
+      f_s[lane] = s / 5.f;
     }
-    fG[c * 5 + i] = sg / 5.f;
-    fD[c * 5 + i] = sd / 5.f;
-    f_s[i] = sg / 5.f;
-    f_s[5 + i] = sd / 5.f;
-  }
-  if (SELECT) {
-    // the cell's tournaments follow at once: G in thread 0, D in thread 1
-    __syncthreads();
-    if (threadIdx.x < 2) select_one(c, threadIdx.x, f_s + 5 * threadIdx.x, nbr, sp, io);
+    __syncwarp();
+    // the cell's tournaments follow at once: G in lane 0, D in lane 1
+    if (SELECT && lane < 2) {
+      const int s = select_slot(f_s + 5 * lane, words, sp), k = 5 * lane + s;
+      float4 cf = coef_s[k];
+      if (sp.lr_mutation)
+        cf.x = mutate(cf.x, sp.seed, lane ? 8u : 7u, sp.t, (uint32_t)c, sp.lr_mut_std, sp.lr_mut_thr);
+      io.coef[lane][c] = cf;
+      io.sel[lane][c] = s;
+      io.src[lane][c] = src_s[k];
+      io.lr_new[lane][c] = cf.x;
+    }
   }
 }
 
 void launch_fitness(const float* logits, int cells, int B, float* LG, float* LD, float* fG,
                     float* fD, int* flag, cudaStream_t st) {
-  // one warp per mean
   launch_pdl(k_fitness<false>, dim3(cells), dim3(960), 0, st, logits, B, LG, LD, fG, fD, flag,
              (const int*)nullptr, SelectParams{}, SelectIO{});
 }
@@ -680,7 +692,7 @@ void launch_fitness(const float* logits, int cells, int B, float* LG, float* LD,
 void launch_fitness_select(const float* logits, int cells, int B, float* LG, float* LD,
                            float* fG, float* fD, int* flag, const int* nbr,
                            const SelectParams& p, const SelectIO& io, cudaStream_t st) {
-  launch_pdl(k_fitness<true>, dim3(cells), dim3(960), 0, st, logits, B, LG, LD, fG, fD, flag, nbr,
+  launch_pdl(k_fitness<true>, dim3(cells), dim3(992), 0, st, logits, B, LG, LD, fG, fD, flag, nbr,
              p, io);
 }
 
