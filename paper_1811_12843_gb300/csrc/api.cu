@@ -125,6 +125,7 @@ struct lipz_grid {
   float *mix = nullptr, *rnorm = nullptr, *mixP = nullptr, *mixS = nullptr, *mixScore = nullptr;
   float* gram = nullptr;
   GemmSet dgram;
+  int* gemm_err = nullptr;          // status word of the tensor-core grouped GEMM
   int mix_nh = 1;
   bool mix_tc = false;
   Descs dsc[3]{}, dsc_stale[3]{};
@@ -310,12 +311,17 @@ int upload(lipz_grid* g, T** dst, const std::vector<T>& v) {
 // start are short ones).
 int make_set(lipz_grid* g, GemmSet* S, std::vector<GemmDesc> v) {
   const int es = (int)g->esz;
+  const bool tc = g->bf && !g->a.force_simt;
   auto vec = [&](const void* p, int64_t unit, int64_t other, int n_unit, const GemmDesc& d, int op) {
     return unit == 1 && other % 4 == 0 && n_unit % 4 == 0 && (uintptr_t)p % (4 * es) == 0 &&
            (!d.wsel || d.wsel_op != op || d.wsel_stride % 4 == 0);
   };
   for (GemmDesc& d : v) {
     d.vec = 0;
+    if (tc) {
+      gemm_tc_align(&d);
+      continue;
+    }
     if (d.sak == 1 ? vec(d.A, 1, d.sam, d.K, d, 1) : vec(d.A, d.sam, d.sak, d.M, d, 1))
       d.vec |= GEMM_VEC_A;
     if (d.sbk == 1 ? vec(d.B, 1, d.sbn, d.K, d, 2) : vec(d.B, d.sbn, d.sbk, d.N, d, 2))
@@ -333,7 +339,25 @@ int make_set(lipz_grid* g, GemmSet* S, std::vector<GemmDesc> v) {
   static const double weight[GEMM_N_TILES] = {1.0, 1.2, 1.3};
   static const double share[GEMM_N_TILES] = {2.5, 4, 6};
   double best = 0;
-  for (int s = 0; s < GEMM_N_TILES; ++s) {
+  if (tc) {
+    // Rounds of co-resident CTAs (two 128 x 128 or three 128 x 64 per SM), a round of the smaller
+    // weighted by its measured time. 128 x 128 against 128 x 64: 371 against 425 us for 2400 tiles
+    // of 128 x 128 (8 rounds against 11), 41 against 49 for 240 (1 against 2), 48.4 against 47.6
+    // for 270 (1 and 1), and five launches of 48 to 96 tiles (1 and 1) 74 against 54.
+    for (int s = 0; s < GEMM_TC_N_TILES; ++s) {
+      const GemmTile t = GEMM_TC_TILES[s];
+      int64_t n = 0;
+      for (const GemmDesc& d : v)
+        n += (int64_t)((d.M + t.bm - 1) / t.bm) * ((d.N + t.bn - 1) / t.bn);
+      const int64_t slots = 152 * (t.bn == 128 ? 2 : 3);
+      const double cost = (double)((n + slots - 1) / slots) * (t.bn == 128 ? 1.0 : 0.8);
+      if (s == 0 || cost < best) {
+        best = cost;
+        S->shape = s;
+      }
+    }
+  }
+  for (int s = 0; !tc && s < GEMM_N_TILES; ++s) {
     const GemmTile t = GEMM_TILES[s];
     double work = 0, last = 0;
     for (const GemmDesc& d : v) {
@@ -347,7 +371,7 @@ int make_set(lipz_grid* g, GemmSet* S, std::vector<GemmDesc> v) {
       S->shape = s;
     }
   }
-  const GemmTile t = GEMM_TILES[S->shape];
+  const GemmTile t = tc ? GEMM_TC_TILES[S->shape] : GEMM_TILES[S->shape];
   std::vector<int2> tiles;
   for (size_t i = 0; i < v.size(); ++i)
     for (int m = 0; m * t.bm < v[i].M; ++m)
@@ -587,8 +611,13 @@ int build_descs(lipz_grid* g, int p) {
   return upload(g, &D.cb, cb);
 }
 
+// Status word of the tensor-core grouped GEMM (a DCGAN's engine shares its own).
+int* gemm_error_flag(lipz_grid* g) { return g->dc ? dc_error_flag(g->dc) : g->gemm_err; }
+
 void gemm(lipz_grid* g, const GemmSet& S) {
-  if (g->bf) launch_gemm<bf16>(S.d, S.t, S.n, S.shape, g->a.leaky_slope, g->st);
+  if (g->bf && !g->a.force_simt)
+    launch_gemm_tc(S.d, S.t, S.n, S.shape, g->a.leaky_slope, gemm_error_flag(g), g->st);
+  else if (g->bf) launch_gemm<bf16>(S.d, S.t, S.n, S.shape, g->a.leaky_slope, g->st);
   else launch_gemm<float>(S.d, S.t, S.n, S.shape, g->a.leaky_slope, g->st);
 }
 
@@ -741,6 +770,9 @@ int create_impl(lipz_grid* g) {
     }
   }
   const int big = INT_MAX;
+  if (g->bf && !g->dcgan && !g->a.force_simt &&
+      ((rc = dalloc(g, &g->gemm_err, 4)) || (rc = dset(g, g->gemm_err, 0, 4))))
+    return rc;
   if ((rc = dset(g, g->gG, 0, (size_t)C * g->PGs * 4)) ||
       (rc = dset(g, g->gD, 0, (size_t)C * g->PDs * 4)) || (rc = h2d(g, g->flag, &big, 4)))
     return rc;

@@ -151,7 +151,8 @@ __device__ __forceinline__ void adam_elem(float& w, float& m, float& v, float g,
 enum Epi : int { EPI_STORE = 0, EPI_BIAS_ACT = 1, EPI_DACT = 2 };
 
 // GEMM_VEC_A / _B: the operand's unit-stride rows start on a boundary of four elements and hold a
-// multiple of four (four elements in one load).
+// multiple of four (four elements in one load). (The tensor-core GEMM keeps its operands' alignment
+// classes in the same word.)
 enum { GEMM_VEC_A = 1, GEMM_VEC_B = 2 };
 
 // A problem whose weight operand belongs to a selected individual sets wsel: the operand
@@ -176,6 +177,9 @@ struct GemmTile {
 };
 constexpr GemmTile GEMM_TILES[] = {{128, 64}, {32, 64}, {32, 32}};
 constexpr int GEMM_N_TILES = 3;
+// Those of the tensor-core one.
+constexpr GemmTile GEMM_TC_TILES[] = {{128, 128}, {128, 64}};
+constexpr int GEMM_TC_N_TILES = 2;
 
 // Column sums: out[n] = sum_{r < rows} X[r * ld + n], n < cols (bias gradients).
 struct ColSumDesc {

@@ -73,6 +73,11 @@ void launch_draw_batch(const T* pool, int64_t n_pool, const float* xin, T* E, in
 template <typename TI>
 void launch_gemm(const GemmDesc* descs, const int2* tiles, int n, int shape, float slope,
                  cudaStream_t st);
+// The bf16 GEMM on the tensor cores (shape indexes GEMM_TC_TILES); gemm_tc_align sets a problem's
+// vec. err: status word, set where a bounded wait expires.
+void gemm_tc_align(GemmDesc* d);
+void launch_gemm_tc(const GemmDesc* descs, const int2* tiles, int n, int shape, float slope,
+                    int* err, cudaStream_t st);
 template <typename T>
 void launch_gemv(const GemvDesc* descs, int n_problems, int max_rows, cudaStream_t st);
 template <typename T>
