@@ -388,6 +388,12 @@ __device__ __forceinline__ bool count_wait(const int* cnt, int need, volatile in
   }
 }
 
+// Form for warps whose lanes all poll and go on together.
+__device__ __forceinline__ bool count_wait_warp(const int* cnt, int need, volatile int* abort_flag,
+                                                int* err, int code) {
+  return __all_sync(0xffffffffu, count_wait(cnt, need, abort_flag, err, code));
+}
+
 // A cell's ranges entry: epilogue thread et takes elements et, et + 256, ... of the population's
 // ranges laid end to end. A pass's loads are issued before any is used (one memory latency per
 // row tile of partials; element by element, an entry took 14 us). A bias gradient is the sum of
@@ -505,7 +511,7 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
     for (int b = 0; b < RING; ++b) {
       mbar_init(tFull + 8 * b, 1);
-      // readers: the MMA thread, one lane of each epilogue warp, the chunk loader and storer
+      // readers: one lane of the MMA warp, of each epilogue warp, of the chunk loader and storer
       mbar_init(tEmpty + 8 * b, 1 + NUM_EPI_WARPS + 2);
     }
     *abort_flag = 0;
@@ -528,36 +534,40 @@ __global__ void __launch_bounds__(THREADS, 1)
   // are needed (programmatic dependent launch)
   pdl_wait();
 
-  // The next claimed tile for a role of one thread (the epilogue has its own, warp-wide): waits
-  // for ring slot i, returns its entry {cell, stage << 16 | tile} and releases the slot. False:
-  // the list is done or the CTA gave up.
+  // The next claimed tile for a role of a warp: waits for ring slot i, returns its entry
+  // {cell, stage << 16 | tile} and releases the slot. False: the list is done or the CTA gave up.
   auto next_tile = [&](int i, int2& e) -> bool {
     const int s = i % RING;
-    if (!mbar_wait(tFull + 8 * s, (uint32_t)((i / RING) & 1), abort_flag, err, 22)) return false;
+    if (!mbar_wait_all(tFull + 8 * s, (uint32_t)((i / RING) & 1), abort_flag, err, 22)) return false;
     e.x = ring[s].x;
     e.y = ring[s].y;
-    mbar_arrive(tEmpty + 8 * s);
+    __syncwarp();
+    if (lane == 0) mbar_arrive(tEmpty + 8 * s);
     return e.x >= 0;
   };
 
   if (warp == 0) {
-    if (lane == 0) {
+    {
+      const bool elected = elect_one();
       int issued[MAX_OPS] = {};
       bool ok = true;
       int stage = 0;
       uint32_t phase = 0;
       for (int i = 0; ok; ++i) {
-        const int idx = atomicAdd(claim, 1);
+        int idx = lane == 0 ? atomicAdd(claim, 1) : 0;
+        idx = __shfl_sync(0xffffffffu, idx, 0);
         const int2 e = idx < cp.n_list ? __ldg(&cp.list[idx]) : make_int2(-1, 0);
         const int s = i % RING;
-        if (i >= RING && !mbar_wait(tEmpty + 8 * s, (uint32_t)((i / RING - 1) & 1), abort_flag,
-                                    err, 23)) {
+        if (i >= RING && !mbar_wait_all(tEmpty + 8 * s, (uint32_t)((i / RING - 1) & 1), abort_flag,
+                                        err, 23)) {
           ok = false;
           break;
         }
-        ring[s].x = e.x;
-        ring[s].y = e.y;
-        mbar_arrive(tFull + 8 * s);
+        if (lane == 0) {
+          ring[s].x = e.x;
+          ring[s].y = e.y;
+          mbar_arrive(tFull + 8 * s);
+        }
         if (e.x < 0) break;
         const int cell = e.x, si = e.y >> 16, t = e.y & 0xFFFF;
         if (si >= RANGES_STAGE) continue;
@@ -575,7 +585,8 @@ __global__ void __launch_bounds__(THREADS, 1)
           const bool part1 = p.ksplit > 0 && kc >= p.ksplit;
           const int ka = (part1 ? kc - p.ksplit : kc) * BK + (part1 ? p.a_k_off1 : 0);
           const uint32_t sA = base + st * op_bytes, full = bFull + 8 * st;
-          if (p.a_mn) {
+          if (!elected) {
+          } else if (p.a_mn) {
             tma_load_3d(sA, mA, full, m0, ka, za);
             tma_load_3d(sA + MN_BOX_BYTES, mA, full, m0 + 64, ka, za);
           } else {
@@ -584,6 +595,8 @@ __global__ void __launch_bounds__(THREADS, 1)
         };
         auto load_b = [&](int kc, int st) {
           const uint32_t sB = base + st * op_bytes + A_BYTES, full = bFull + 8 * st;
+          issued[st]++;
+          if (!elected) return;
           mbar_expect_tx(full, bytes);
           if (p.ksplit > 0) {
             const bool part1 = kc >= p.ksplit;
@@ -594,7 +607,6 @@ __global__ void __launch_bounds__(THREADS, 1)
             for (int u = 0; u < p.BN / 64; ++u)
               tma_load_3d(sB + u * MN_BOX_BYTES, mB, full, n0 + 64 * u, kc * BK, zb);
           }
-          issued[st]++;
         };
         // a tile that reads the output of the cell's stage `dep` (its A, written by any CTA)
         // loads its first chunks' B, which does not depend on it, before it waits
@@ -602,15 +614,15 @@ __global__ void __launch_bounds__(THREADS, 1)
         const int stage0 = stage;
         for (int kc = 0; kc < p.kchunks && ok; ++kc) {
           if (kc == ahead && ahead > 0) {
-            if (!count_wait(cp.sync + (int64_t)cell * SYNC_WORDS + dep, cp.st[si].dep_need,
-                            abort_flag, err, 16)) {
+            if (!count_wait_warp(cp.sync + (int64_t)cell * SYNC_WORDS + dep, cp.st[si].dep_need,
+                                 abort_flag, err, 16)) {
               ok = false;
               break;
             }
             asm volatile("fence.proxy.async;" ::: "memory");
             for (int u = 0; u < ahead; ++u) load_a(u, (stage0 + u) % n_ops);
           }
-          if (!mbar_wait(bEmpty + 8 * stage, phase ^ 1u, abort_flag, err, 11)) {
+          if (!mbar_wait_all(bEmpty + 8 * stage, phase ^ 1u, abort_flag, err, 11)) {
             ok = false;
             break;
           }
@@ -622,8 +634,8 @@ __global__ void __launch_bounds__(THREADS, 1)
           }
         }
         if (ok && ahead == p.kchunks) {
-          if (!count_wait(cp.sync + (int64_t)cell * SYNC_WORDS + dep, cp.st[si].dep_need,
-                          abort_flag, err, 16)) {
+          if (!count_wait_warp(cp.sync + (int64_t)cell * SYNC_WORDS + dep, cp.st[si].dep_need,
+                               abort_flag, err, 16)) {
             ok = false;
             break;
           }
@@ -640,7 +652,8 @@ __global__ void __launch_bounds__(THREADS, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    {
+      const bool elected = elect_one();
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
@@ -653,7 +666,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         int m0, n0, n;
         stage_tile(p, e.y & 0xFFFF, m0, n0, n);
         const int R = lt & 1, use = lt >> 1;
-        if (use > 0 && !mbar_wait(bReg + 8 * R, (uint32_t)((use - 1) & 1), abort_flag, err, 15)) {
+        if (use > 0 && !mbar_wait_all(bReg + 8 * R, (uint32_t)((use - 1) & 1), abort_flag, err, 15)) {
           ok = false;
           break;
         }
@@ -661,7 +674,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         const uint32_t d = tmem + (uint32_t)(R * 256);
         const uint32_t idesc = idesc_bf16_major(BM, n, p.a_mn, 1);
         for (int kc = 0; kc < p.kchunks; ++kc) {
-          if (!mbar_wait(bFull + 8 * stage, phase, abort_flag, err, 12)) {
+          if (!mbar_wait_all(bFull + 8 * stage, phase, abort_flag, err, 12)) {
             ok = false;
             break;
           }
@@ -672,19 +685,19 @@ __global__ void __launch_bounds__(THREADS, 1)
             const uint64_t ad = p.a_mn ? sw128_mn_desc(sA + kk * 2048, MN_BOX_BYTES)
                                        : sw128_desc(sA + kk * 32);
             const uint64_t bd = sw128_mn_desc(sB + kk * 2048, MN_BOX_BYTES);
-            tc_mma(d, ad, bd, idesc, (kc | kk) != 0 ? 1u : 0u);
+            if (elected) tc_mma(d, ad, bd, idesc, (kc | kk) != 0 ? 1u : 0u);
           }
-          tc_commit(bEmpty + 8 * stage);
+          if (elected) tc_commit(bEmpty + 8 * stage);
           if (++stage == n_ops) {
             stage = 0;
             phase ^= 1u;
           }
         }
         if (!ok) break;
-        tc_commit(bAcc + 8 * R);
+        if (elected) tc_commit(bAcc + 8 * R);
         ++lt;
       }
-      tc_commit(bFinal);
+      if (elected) tc_commit(bFinal);
       volatile int never = 0;
       mbar_wait(bFinal, 0u, &never, err, 14);
     }
@@ -699,7 +712,8 @@ __global__ void __launch_bounds__(THREADS, 1)
     //           buffer's round trip); after a delta tile's last chunk, once its stores are
     //           written, it counts the tile for the tiles that read it. =====
     const bool storer = warp == 3 + NUM_EPI_WARPS;
-    if (lane == 0) {
+    {
+      const bool elected = elect_one();
       int buf = 0, uses[CHUNK_BUFS] = {};
       bool ok = true;
       int2 e;
@@ -721,28 +735,32 @@ __global__ void __launch_bounds__(THREADS, 1)
           const uint32_t bb = sChunk + (uint32_t)(buf * CHUNK_BYTES);
           if (storer) {
             // the (uses[buf] + 1)-th chunk of this buffer is written back
-            if (!mbar_wait(cDone + 8 * buf, (uint32_t)(uses[buf] & 1), abort_flag, err, 19)) {
+            if (!mbar_wait_all(cDone + 8 * buf, (uint32_t)(uses[buf] & 1), abort_flag, err, 19)) {
               ok = false;
               break;
             }
-            if (adam) {
+            if (!elected) {
+            } else if (adam) {
               tma_store_4d(&maps.out[si], bb, x0, y0, cell, 0);
               tma_store_3d(&maps.nb[si], bb + 3 * ADAM_ARRAY_BYTES, x0, y0, cell);
             } else {
               for (int u = 0; u < boxes; ++u)
                 tma_store_3d(&maps.out[si], bb + u * DELTA_BOX_BYTES, x0 + 64 * u, y0, cell);
             }
-            bulk_commit();
-            bulk_wait_read<0>();  // the stores have read the buffer: it may be refilled
-            mbar_arrive(cFree + 8 * buf);
+            if (elected) {
+              bulk_commit();
+              bulk_wait_read<0>();  // the stores have read the buffer: it may be refilled
+              mbar_arrive(cFree + 8 * buf);
+            }
           } else {
-            if (uses[buf] > 0 && !mbar_wait(cFree + 8 * buf, (uint32_t)((uses[buf] - 1) & 1),
+            if (uses[buf] > 0 && !mbar_wait_all(cFree + 8 * buf, (uint32_t)((uses[buf] - 1) & 1),
                                             abort_flag, err, 21)) {
               ok = false;
               break;
             }
             const uint32_t full = cFull + 8 * buf;
-            if (adam) {
+            if (!elected) {
+            } else if (adam) {
               mbar_expect_tx(full, (uint32_t)(3 * ADAM_ARRAY_BYTES));
               tma_load_4d(bb, &maps.in[si], full, x0, y0, zi, 0);
             } else {
@@ -759,7 +777,7 @@ __global__ void __launch_bounds__(THREADS, 1)
           uses[buf]++;
           if (++buf == CHUNK_BUFS) buf = 0;
         }
-        if (storer && !adam && ok) {
+        if (storer && !adam && ok && elected) {
           bulk_wait_all();
           __threadfence();
           asm volatile("red.release.gpu.global.add.s32 [%0], 1;" ::"l"(
@@ -768,7 +786,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
       }
       if (storer) {
-        bulk_wait_all();
+        if (elected) bulk_wait_all();
       } else if (*abort_flag) {
         // loads issued here land on this CTA's barriers: wait for them before it leaves
         for (int b = 0; b < CHUNK_BUFS; ++b)

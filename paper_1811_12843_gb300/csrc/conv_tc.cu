@@ -229,7 +229,8 @@ __global__ void __launch_bounds__(THREADS, conv_compact(AK) ? 2 : 1)
     // by TMA, its first (warp 2) and second (m2: warp 3) 128 rows. A tiled TMA operation holds its
     // issuing thread for 0.2 us and more, most of a chunk's time on the tensor cores, so each
     // thread issues one per chunk.
-    if (lane == 0 && (warp < 3 || p.m2)) {
+    if (warp < 3 || p.m2) {
+      const bool elected = elect_one();
       int stage = 0, issued[STAGES] = {};
       uint32_t phase = 0;
       bool ok = true;
@@ -250,7 +251,7 @@ __global__ void __launch_bounds__(THREADS, conv_compact(AK) ? 2 : 1)
             }
             // (loads may land before their bytes are announced; a pair: rank 0 expects both
             // CTAs' bytes)
-            if (warp == 0 && rank == 0)
+            if (warp == 0 && rank == 0 && elected)
               mbar_expect_tx(bFullB + 8 * stage,
                              kPair ? 2 * st_bytes
                                    : (uint32_t)(nbox * BK * 2 + (kTma ? nA * A_BYTES : 0)));
@@ -280,8 +281,13 @@ __global__ void __launch_bounds__(THREADS, conv_compact(AK) ? 2 : 1)
               }
               const int prob = transposed ? pc >> 2 : pc;
               const uint32_t dst = sS + (warp - 2) * A_BYTES;
-              if constexpr (kPair) tma_load_5d_cg2(dst, &mA, full, c0, x, ym * y0 + ya, n0, prob);
-              else tma_load_5d(dst, &mA, full, c0, x, ym * y0 + ya, n0, prob);
+              if (!elected) {
+              } else if constexpr (kPair) {
+                tma_load_5d_cg2(dst, &mA, full, c0, x, ym * y0 + ya, n0, prob);
+              } else {
+                tma_load_5d(dst, &mA, full, c0, x, ym * y0 + ya, n0, prob);
+              }
+            } else if (!elected) {
             } else if constexpr (kPair) {
               tma_load_3d_cg2(sS + nA * A_BYTES, &mW, full, kc * BK,
                               cls * p.cls_rows + j * 256 + (int)rank * (nbox / 2), indiv);
@@ -311,7 +317,8 @@ __global__ void __launch_bounds__(THREADS, conv_compact(AK) ? 2 : 1)
     }
   } else if (warp == 1) {
     // ---- MMA issue (a pair: rank 0, 256-row MMAs over both CTAs' tiles)
-    if (lane == 0 && rank == 0) {
+    if (rank == 0) {
+      const bool elected = elect_one();
       int stage = 0, uses[2] = {0, 0}, jobs = 0;
       uint32_t phase = 0;
       bool ok = true, ready = false;
@@ -335,6 +342,7 @@ __global__ void __launch_bounds__(THREADS, conv_compact(AK) ? 2 : 1)
 #pragma unroll
             for (int kk = 0; kk < BK / 16; ++kk) {
               if (kk == BK / 16 - 1) look();
+              if (!elected) continue;
               if constexpr (kPair) {
                 if (kk) tc_mma_cg2_acc(dt, dA + 2 * kk, dB + 2 * kk, idesc);
                 else tc_mma_cg2(dt, dA, dB, idesc, first ? 0u : 1u);
@@ -366,18 +374,30 @@ __global__ void __launch_bounds__(THREADS, conv_compact(AK) ? 2 : 1)
             auto look = [&] { ready = mbar_test(bFullB + 8 * next, next_phase); };
             if (p.m2) chunk(std::true_type{}, kc == 0, look);
             else chunk(std::false_type{}, kc == 0, look);
-            if constexpr (kPair) tc_commit_cg2(bEmpty + 8 * stage, 3);
-            else tc_commit(bEmpty + 8 * stage);
+            if (!elected) {
+            } else if constexpr (kPair) {
+              tc_commit_cg2(bEmpty + 8 * stage, 3);
+            } else {
+              tc_commit(bEmpty + 8 * stage);
+            }
             stage = next;
             phase = next_phase;
           }
           if (!ok) break;
-          if constexpr (kPair) tc_commit_cg2(bAccF + 8 * R, 3);
-          else tc_commit(bAccF + 8 * R);
+          if (!elected) {
+          } else if constexpr (kPair) {
+            tc_commit_cg2(bAccF + 8 * R, 3);
+          } else {
+            tc_commit(bAccF + 8 * R);
+          }
           uses[R]++;
         }
-      if constexpr (kPair) tc_commit_cg2(bFinal, 3);
-      else tc_commit(bFinal);
+      if (!elected) {
+      } else if constexpr (kPair) {
+        tc_commit_cg2(bFinal, 3);
+      } else {
+        tc_commit(bFinal);
+      }
       volatile int never = 0;
       mbar_wait(bFinal, 0u, &never, p.err, 26);
     }
@@ -869,7 +889,8 @@ __global__ void __launch_bounds__(THREADS, 2)
 
   if (warp == 0) {
     // ---- weights by TMA, one tile of 64 rows per (tile, problem)
-    if (lane == 0) {
+    {
+      const bool elected = elect_one();
       int st = 0, issued[F_B] = {};
       uint32_t phase = 0;
       bool ok = true;
@@ -881,8 +902,10 @@ __global__ void __launch_bounds__(THREADS, 2)
             ok = false;
             break;
           }
-          mbar_expect_tx(fullB + 8 * st, (uint32_t)F_B_BYTES);
-          tma_load_3d(sB + st * F_B_BYTES, &mW, fullB + 8 * st, 0, 0, indiv);
+          if (elected) {
+            mbar_expect_tx(fullB + 8 * st, (uint32_t)F_B_BYTES);
+            tma_load_3d(sB + st * F_B_BYTES, &mW, fullB + 8 * st, 0, 0, indiv);
+          }
           issued[st]++;
           if (++st == F_B) {
             st = 0;
@@ -898,7 +921,8 @@ __global__ void __launch_bounds__(THREADS, 2)
     }
   } else if (warp == 1) {
     // ---- MMA issue: three K steps of 16 (the 49th value on is zero)
-    if (lane == 0) {
+    {
+      const bool elected = elect_one();
       int sa = 0, sb = 0, job = 0;
       uint32_t pa = 0, pb = 0;
       bool ok = true;
@@ -916,24 +940,26 @@ __global__ void __launch_bounds__(THREADS, 2)
           tc_fence_after();
           const uint64_t dA = sw128_desc(base + sa * A_BYTES), dB = sw128_desc(sB + sb * F_B_BYTES);
           const uint32_t dt = tmem + (uint32_t)(R * 64);
-          tc_mma(dt, dA, dB, idesc, 0u);
-          tc_mma_acc(dt, dA + 2, dB + 2, idesc);
-          tc_mma_acc(dt, dA + 4, dB + 4, idesc);
-          tc_commit(emptyB + 8 * sb);
-          tc_commit(accF + 8 * R);
+          if (elected) {
+            tc_mma(dt, dA, dB, idesc, 0u);
+            tc_mma_acc(dt, dA + 2, dB + 2, idesc);
+            tc_mma_acc(dt, dA + 4, dB + 4, idesc);
+            tc_commit(emptyB + 8 * sb);
+            tc_commit(accF + 8 * R);
+          }
           if (++sb == F_B) {
             sb = 0;
             pb ^= 1u;
           }
         }
         if (!ok) break;
-        tc_commit(emptyA + 8 * sa);
+        if (elected) tc_commit(emptyA + 8 * sa);
         if (++sa == F_A) {
           sa = 0;
           pa ^= 1u;
         }
       }
-      tc_commit(bFinal);
+      if (elected) tc_commit(bFinal);
       volatile int never = 0;
       mbar_wait(bFinal, 0u, &never, p.err, 26);
     }
@@ -1136,7 +1162,8 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
     // a_tma: both operands by TMA, MN-major rows of 64 channels: A boxes of 64 pixels from the
     // [problem][pixel][M] map, B boxes of the chunk's 64 A pixels mapped to b's pixels (s y - p
     // + ky, s x - p + kx) by the 5-D map's traversal stride
-    if (lane == 0) {
+    {
+      const bool elected = elect_one();
       int stage = 0, issued[WG_STAGES] = {};
       uint32_t phase = 0;
       bool ok = true;
@@ -1153,10 +1180,12 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
             break;
           }
           const uint32_t full = bFull + 8 * stage;
-          mbar_expect_tx(full, (uint32_t)(BCHW ? A_BYTES : STAGE_BYTES));
           const uint32_t sA = base + stage * STAGE_BYTES, sB = sA + A_BYTES;
-          tma_load_3d(sA, &mA, full, mt * 128, (int)kb, prob);
-          tma_load_3d(sA + 8192, &mA, full, mt * 128 + 64, (int)kb, prob);
+          if (elected) {
+            mbar_expect_tx(full, (uint32_t)(BCHW ? A_BYTES : STAGE_BYTES));
+            tma_load_3d(sA, &mA, full, mt * 128, (int)kb, prob);
+            tma_load_3d(sA + 8192, &mA, full, mt * 128 + 64, (int)kb, prob);
+          }
           if constexpr (BCHW) {
             issued[stage]++;
             if (++stage == WG_STAGES) {
@@ -1171,7 +1200,8 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
           for (int atom = 0; atom < 4; ++atom) {
             const int n0 = nt * 256 + atom * 64;
             const int tap = n0 / p.Cb, c0 = n0 - tap * p.Cb;
-            tma_load_5d(sB + atom * 8192, &mB, full, c0, p.s * ax0 - p.p + (tap & 3),
+            if (elected)
+              tma_load_5d(sB + atom * 8192, &mB, full, c0, p.s * ax0 - p.p + (tap & 3),
                         p.s * ay0 - p.p + (tap >> 2), nb, prob);
           }
           issued[stage]++;
@@ -1190,7 +1220,8 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {
+    {
+      const bool elected = elect_one();
       int stage = 0, uses[2] = {0, 0}, jobs = 0;
       uint32_t phase = 0;
       bool ok = true, ready = false;
@@ -1217,24 +1248,28 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
           const uint32_t sA = base + stage * STAGE_BYTES, sB = sA + A_BYTES;
           // a 16-pixel K step is 2048 bytes: 128 in the descriptors' address field
           const uint64_t dA = sw128_mn_desc(sA, 8192), dB = sw128_mn_desc(sB, 8192);
-          tc_mma(dt, dA, dB, idesc, first ? 0u : 1u);
+          if (elected) {
+            tc_mma(dt, dA, dB, idesc, first ? 0u : 1u);
+            tc_mma_acc(dt, dA + 128, dB + 128, idesc);
+            tc_mma_acc(dt, dA + 256, dB + 256, idesc);
+          }
           first = false;
-          tc_mma_acc(dt, dA + 128, dB + 128, idesc);
-          tc_mma_acc(dt, dA + 256, dB + 256, idesc);
           // the next stage is looked at while the MMAs run (see k_conv_tc)
           const int next = stage + 1 == WG_STAGES ? 0 : stage + 1;
           const uint32_t next_phase = next ? phase : phase ^ 1u;
           ready = mbar_test(bFull + 8 * next, next_phase);
-          tc_mma_acc(dt, dA + 384, dB + 384, idesc);
-          tc_commit(bEmpty + 8 * stage);
+          if (elected) {
+            tc_mma_acc(dt, dA + 384, dB + 384, idesc);
+            tc_commit(bEmpty + 8 * stage);
+          }
           stage = next;
           phase = next_phase;
         }
         if (!ok) break;
-        tc_commit(bAccF + 8 * R);
+        if (elected) tc_commit(bAccF + 8 * R);
         uses[R]++;
       }
-      tc_commit(bFinal);
+      if (elected) tc_commit(bFinal);
       volatile int never = 0;
       mbar_wait(bFinal, 0u, &never, p.err, 33);
     }

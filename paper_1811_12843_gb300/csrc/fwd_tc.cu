@@ -254,7 +254,8 @@ __global__ void __launch_bounds__(THREADS, 1)
 
   if (warp == 0) {
     // ================================ TMA producer ================================
-    if (lane == 0) {
+    {
+      const bool elected = elect_one();
       int stage = 0;
       uint32_t phase = 0;
       int issued[STAGES] = {0, 0, 0};
@@ -275,9 +276,9 @@ __global__ void __launch_bounds__(THREADS, 1)
             const uint32_t bytes = (J.a_from_h ? 0u : (uint32_t)A_BYTES) +
                                    (uint32_t)(BK * J.box_rows * 2);
             const uint32_t full = bFull + 8 * stage;
-            mbar_expect_tx(full, bytes);
+            if (elected) mbar_expect_tx(full, bytes);
             const uint32_t sA = sStage + stage * STAGE_BYTES;
-            if (J.a_from_h) {
+            if (J.a_from_h || !elected) {
             } else if (p.part_slot) {
               const int cell = prob >> 1;
               const int slot = (prob & 1) ? 1 + __ldg(&p.part_slot[cell]) : 0;
@@ -285,7 +286,7 @@ __global__ void __launch_bounds__(THREADS, 1)
             } else {
               tma_load_3d(sA, &mA, full, kc * BK, m0, c);
             }
-            tma_load_3d(sA + A_BYTES, mb, full, kc * BK, J.brow0, k);
+            if (elected) tma_load_3d(sA + A_BYTES, mb, full, kc * BK, J.brow0, k);
             issued[stage]++;
             if (++stage == STAGES) {
               stage = 0;
@@ -305,7 +306,8 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
   } else if (warp == 1) {
     // ================================ MMA issuer ================================
-    if (lane == 0) {
+    {
+      const bool elected = elect_one();
       int stage = 0;
       uint32_t phase = 0;
       int reg_uses[2] = {0, 0};
@@ -342,24 +344,26 @@ __global__ void __launch_bounds__(THREADS, 1)
             tc_fence_after();
             const uint32_t sA = J.a_from_h ? sH + kc * H_CHUNK : sStage + stage * STAGE_BYTES;
             const uint32_t sB = sStage + stage * STAGE_BYTES + A_BYTES;
+            if (elected) {
 #pragma unroll
-            for (int kk = 0; kk < BK / 16; ++kk)
-              tc_mma(d, sw128_desc(sA + kk * 32), sw128_desc(sB + kk * 32), idesc,
-                     (kc | kk) != 0 ? 1u : 0u);
-            tc_commit(bEmpty + 8 * stage);
+              for (int kk = 0; kk < BK / 16; ++kk)
+                tc_mma(d, sw128_desc(sA + kk * 32), sw128_desc(sB + kk * 32), idesc,
+                       (kc | kk) != 0 ? 1u : 0u);
+              tc_commit(bEmpty + 8 * stage);
+            }
             if (++stage == STAGES) {
               stage = 0;
               phase ^= 1u;
             }
           }
           if (!ok) break;
-          tc_commit(bAcc + 8 * R);
+          if (elected) tc_commit(bAcc + 8 * R);
           reg_uses[R]++;
           if (J.epi == EPI_TO_H) ++h_total;
         }
       }
       // all MMAs issued by this thread complete before tensor memory is released
-      tc_commit(bFinal);
+      if (elected) tc_commit(bFinal);
       volatile int never = 0;
       mbar_wait(bFinal, 0u, &never, p.err, 5);
     }
@@ -838,7 +842,8 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
 
   if (warp == 0) {
     // ================================ TMA producer (both CTAs) ================================
-    if (lane == 0) {
+    {
+      const bool elected = elect_one();
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
@@ -870,12 +875,13 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
               break;
             }
             // rank 0 expects both CTAs' bytes; the peer's may land first
-            if (leader) mbar_expect_tx(bFull + 8 * stage, 2 * bytes);
+            if (leader && elected) mbar_expect_tx(bFull + 8 * stage, 2 * bytes);
             const uint32_t sS = sStage + stage * CF::STAGE;
             const uint32_t full = lFull + 8 * stage;
-            if (a_ring) tma_load_3d_cg2(sS, &mA, full, kc * BK, a_row, a_cell);
-            tma_load_3d_cg2(sS + (CF::A_IN ? A_BYTES : 0), mb, full, kc * BK,
-                            J.brow0 + (int)rank * (J.n / 2), k);
+            if (a_ring && elected) tma_load_3d_cg2(sS, &mA, full, kc * BK, a_row, a_cell);
+            if (elected)
+              tma_load_3d_cg2(sS + (CF::A_IN ? A_BYTES : 0), mb, full, kc * BK,
+                              J.brow0 + (int)rank * (J.n / 2), k);
             if (++stage == CF::STAGES) {
               stage = 0;
               phase ^= 1u;
@@ -893,7 +899,8 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
     }
   } else if (warp == 1) {
     // ================================ MMA issuer (rank 0) ================================
-    if (leader && lane == 0) {
+    if (leader) {
+      const bool elected = elect_one();
       int stage = 0;
       uint32_t phase = 0;
       int reg_uses[2] = {0, 0};
@@ -939,11 +946,13 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
             // a 16-element K step is 32 bytes: 2 in the descriptors' address field (a 1024-byte
             // aligned tile plus at most 96 bytes never carries out of it)
             const uint64_t dA = sw128_desc(sA), dB = sw128_desc(sB);
-            tc_mma_cg2(d, dA, dB, idesc, kc != 0 ? 1u : 0u);
+            if (elected) {
+              tc_mma_cg2(d, dA, dB, idesc, kc != 0 ? 1u : 0u);
 #pragma unroll
-            for (int kk = 1; kk < BK / 16; ++kk)
-              tc_mma_cg2_acc(d, dA + 2 * kk, dB + 2 * kk, idesc);
-            tc_commit_cg2(bEmpty + 8 * stage, 3);
+              for (int kk = 1; kk < BK / 16; ++kk)
+                tc_mma_cg2_acc(d, dA + 2 * kk, dB + 2 * kk, idesc);
+              tc_commit_cg2(bEmpty + 8 * stage, 3);
+            }
             if (++stage == CF::STAGES) {
               stage = 0;
               phase ^= 1u;
@@ -951,16 +960,16 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
           }
           if (!ok) break;
           if (KND == KIND_G && j == 0) {
-            tc_commit_cg2(bZempty, 3);
+            if (elected) tc_commit_cg2(bZempty, 3);
             ++zuse;
           }
-          tc_commit_cg2(bAcc + 8 * R, 3);
+          if (elected) tc_commit_cg2(bAcc + 8 * R, 3);
           reg_uses[R]++;
           if (J.epi == EPI_TO_H) ++h_total;
         }
       }
       // every MMA (they write both CTAs' tensor memory) completes before it is released
-      tc_commit_cg2(bFinal, 3);
+      if (elected) tc_commit_cg2(bFinal, 3);
       volatile int never = 0;
       mbar_wait(bFinal, 0u, &never, p.err, 5);
     }
