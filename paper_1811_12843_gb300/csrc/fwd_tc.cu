@@ -21,6 +21,7 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -741,6 +742,7 @@ struct PParams {
   int B, x, rows;  // rows per problem: B (generator) or 6B (discriminator)
   int kc1, n3;
   int n_pairs;
+  int split;       // generator: parts that a pair's output blocks are divided into
   // generator: {individual, first row of the pair's 256, offset into plist, rows of the
   // individual}; discriminator: {individual, problem of rank 0, problem of rank 1 (-1: none),
   // first row of rank 0's tile << 16 | first row of rank 1's tile}; problem = cell * 5 + slot
@@ -767,13 +769,26 @@ struct PParams {
   bf16* act2;
 };
 
+// A generator pair's output blocks: part i of p.split takes blocks [i n3 / split, (i + 1) n3 / split)
+// (and computes the hidden layers as the other parts do).
+struct PairPart {
+  int pair, nb0, nb;
+};
 template <int KND>
-__device__ __forceinline__ Job pair_job(const PParams& p, int j) {
+__device__ __forceinline__ PairPart pair_part(const PParams& p, int i) {
+  if (KND == KIND_D) return PairPart{i, 0, 0};
+  const int pair = i / p.split, part = i - pair * p.split;
+  const int nb0 = part * p.n3 / p.split;
+  return PairPart{pair, nb0, (part + 1) * p.n3 / p.split - nb0};
+}
+
+template <int KND>
+__device__ __forceinline__ Job pair_job(const PParams& p, const PairPart& pp, int j) {
   if (j == 0) return Job{0, p.kc1, HID, 0, 0, 0, HID, EPI_TO_H};
   if (j == 1) return Job{1, HID / BK, HID, 1, 1, 0, HID, KND == KIND_D ? EPI_LOGIT : EPI_TO_H};
-  const int nb = j - 2;
+  const int nb = pp.nb0 + j - 2;
   const int n = min(N3, p.x - nb * N3);
-  return Job{1, HID / BK, (n + 15) & ~15, (nb + p.n3) & 1, 2, nb * N3, N3, EPI_TO_E};
+  return Job{1, HID / BK, (n + 15) & ~15, (j - 2 + pp.nb) & 1, 2, nb * N3, N3, EPI_TO_E};
 }
 
 template <int KND>
@@ -844,7 +859,7 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
   // rank 0's barriers that both CTAs arrive on
   const uint32_t lFull = mapa_shared(bFull, 0), lReg = mapa_shared(bReg, 0);
   const uint32_t lH = mapa_shared(bH, 0), lZfull = mapa_shared(bZfull, 0);
-  const int nj = KND == KIND_D ? 2 : 2 + p.n3;
+  const int n_parts = KND == KIND_D ? p.n_pairs : p.n_pairs * p.split;
   const int cid = (int)cluster_id_x(), ncl = (int)nclusters_x();
   pdl_wait();
 
@@ -855,9 +870,10 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
-      for (int pi = cid; pi < p.n_pairs && ok; pi += ncl) {
+      for (int pi = cid; pi < n_parts && ok; pi += ncl) {
         const bool train = KND == KIND_D && p.train;
-        const int4 pr = train ? make_int4(0, 0, 0, 0) : __ldg(&p.pairs[pi]);
+        const PairPart pp = pair_part<KND>(p, pi);
+        const int4 pr = train ? make_int4(0, 0, 0, 0) : __ldg(&p.pairs[pp.pair]);
         const int k = train ? __ldg(&p.wsel[pi / p.mt]) : pr.x;
         int a_cell = 0, a_row = p.rows;  // no problem: rows past the end read as zero
         if (train) {
@@ -872,8 +888,8 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
             a_row = rank ? (pr.w & 0xFFFF) : (pr.w >> 16);
           }
         }
-        for (int j = 0; j < nj && ok; ++j) {
-          const Job J = pair_job<KND>(p, j);
+        for (int j = 0; j < 2 + pp.nb && ok; ++j) {
+          const Job J = pair_job<KND>(p, pp, j);
           const CUtensorMap* mb = J.bmap == 0 ? &mB1 : (J.bmap == 1 ? &mB2 : &mB3);
           const bool a_ring = CF::A_IN && !J.a_from_h;
           const uint32_t bytes = (a_ring ? (uint32_t)A_BYTES : 0u) + (uint32_t)HB_BYTES;
@@ -915,9 +931,10 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
       int h_total = 0, zuse = 0;
       int h_seen[HID / BK] = {0, 0, 0, 0};  // activation write each chunk was last waited for
       bool ok = true;
-      for (int pi = cid; pi < p.n_pairs && ok; pi += ncl) {
-        for (int j = 0; j < nj && ok; ++j) {
-          const Job J = pair_job<KND>(p, j);
+      for (int pi = cid; pi < n_parts && ok; pi += ncl) {
+        const PairPart pp = pair_part<KND>(p, pi);
+        for (int j = 0; j < 2 + pp.nb && ok; ++j) {
+          const Job J = pair_job<KND>(p, pp, j);
           const int R = J.region;
           if (reg_uses[R] > 0 &&
               !mbar_wait(bReg + 8 * R, (uint32_t)((reg_uses[R] - 1) & 1), abort_flag, p.err, 2)) {
@@ -1023,13 +1040,15 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
       }
     };
     auto tile_individual = [&](int q) {
-      return (KND == KIND_D && p.train) ? __ldg(&p.wsel[q / p.mt]) : __ldg(&p.pairs[q]).x;
+      return (KND == KIND_D && p.train) ? __ldg(&p.wsel[q / p.mt])
+                                        : __ldg(&p.pairs[pair_part<KND>(p, q).pair]).x;
     };
     float vb[NV];
-    if (cid < p.n_pairs) load_bias(tile_individual(cid), vb);
-    for (int pi = cid; pi < p.n_pairs && ok; pi += ncl, ++ltile) {
+    if (cid < n_parts) load_bias(tile_individual(cid), vb);
+    for (int pi = cid; pi < n_parts && ok; pi += ncl, ++ltile) {
       const bool train = KND == KIND_D && p.train;
-      const int4 pr = train ? make_int4(0, 0, 0, 0) : __ldg(&p.pairs[pi]);
+      const PairPart pp = pair_part<KND>(p, pi);
+      const int4 pr = train ? make_int4(0, 0, 0, 0) : __ldg(&p.pairs[pp.pair]);
       const int k = train ? __ldg(&p.wsel[pi / p.mt]) : pr.x;
       bool row_ok;
       bf16* dst = nullptr;   // generator: this row of the fakes
@@ -1062,7 +1081,7 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
           if (i < 512 + nb3) sb[i] = vb[u];
         }
         // the next tile's, in flight while this one computes
-        if (pi + ncl < p.n_pairs) load_bias(tile_individual(pi + ncl), vb);
+        if (pi + ncl < n_parts) load_bias(tile_individual(pi + ncl), vb);
         mbar_arrive(bBias + 8 * (ltile & 1));
         if (!mbar_wait_warp(bBias + 8 * (ltile & 1), (uint32_t)((ltile >> 1) & 1), abort_flag,
                             p.err, 8)) {
@@ -1070,8 +1089,8 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
           break;
         }
       }
-      for (int j = 0; j < nj && ok; ++j) {
-        const Job J = pair_job<KND>(p, j);
+      for (int j = 0; j < 2 + pp.nb && ok; ++j) {
+        const Job J = pair_job<KND>(p, pp, j);
         const int R = J.region;
         if (!mbar_wait_warp(bAcc + 8 * R, (uint32_t)(reg_uses[R] & 1), abort_flag, p.err, 6)) {
           ok = false;
@@ -1237,8 +1256,8 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
     // ================================ noise gather (generator) ================================
     // this CTA's 128 rows of the individual's z rows, 16-byte units in the 128-byte swizzle
     int zuse = 0;
-    for (int pi = cid; pi < p.n_pairs; pi += ncl, ++zuse) {
-      const int4 pr = __ldg(&p.pairs[pi]);
+    for (int pi = cid; pi < n_parts; pi += ncl, ++zuse) {
+      const int4 pr = __ldg(&p.pairs[pair_part<KND>(p, pi).pair]);
       if (zuse > 0 &&
           !mbar_wait_warp(bZempty, (uint32_t)((zuse - 1) & 1), abort_flag, p.err, 10))
         break;
@@ -1664,9 +1683,14 @@ int launch(int grid, const CUtensorMap& a, const CUtensorMap& b1, const CUtensor
 
 namespace {
 int launch_pair(int ncl, const CUtensorMap& a, const CUtensorMap& b1, const CUtensorMap& b2,
-                const CUtensorMap& b3, const tc::PParams& pp, bool gen, cudaStream_t st,
+                const CUtensorMap& b3, const tc::PParams& pq, bool gen, cudaStream_t st,
                 std::string* msg) {
-  const int clusters = pp.n_pairs < ncl ? pp.n_pairs : ncl;
+  // Small grids: a pair's output blocks in as many parts as there are idle clusters, each with the
+  // hidden layers of its own (784 outputs, four blocks; 1x1 cells, 2 pairs: 27 -> 21 us, 3x3, 18
+  // pairs: 29 -> 23). More parts than clusters would take a second round for less work each.
+  tc::PParams pp = pq;
+  pp.split = gen ? std::max(1, std::min(pp.n3, ncl / std::max(1, pp.n_pairs))) : 1;
+  const int parts = pp.n_pairs * pp.split, clusters = parts < ncl ? parts : ncl;
   if (clusters <= 0) return 0;
   cudaError_t e =
       gen ? launch_pairs(tc::k_mlp_fwd_pair<tc::KIND_G>, clusters, tc::pair_threads<tc::KIND_G>(),
