@@ -1171,9 +1171,8 @@ int train_once(lipz_grid* g, bool evaluated) {
   // forward of the selected pair
   if (g->use_tc) {
     std::string msg;
-    if (tc_run_train_g(g->tc[p], g->st, &msg) || tc_run_train_d(g->tc[p], g->st, &msg))
-      return fail(g, LIPZ_ERR_CUDA, "%s", msg.c_str());
-    n_fwd += 2;
+    if (tc_run_train(g->tc[p], g->st, &msg)) return fail(g, LIPZ_ERR_CUDA, "%s", msg.c_str());
+    n_fwd += tc_train_launches(g->tc[p]);
   } else if (!evaluated) {
     gemm(g, D.td1);
     gemm(g, D.td2);

@@ -758,15 +758,26 @@ struct PParams {
   float* logits;
   float slope;
   int* err;
-  // discriminator training forward (train != 0): pair job c * mt + t takes m-tile t of both
+  // discriminator training forward: pair job c * mt + t takes m-tile t of both
   // parts of cell c through discriminator wsel[c]: rank 0 the B real rows (slot 0 of E[c]),
   // rank 1 the selected generator's fakes (slot 1 + part_slot[c]); both hidden activations go
   // to act1 / act2 ([2c + part][B][256] bf16), the logits to logits[(2c + part) B + row]
-  int train, mt;
+  int mt;
   const int* wsel;
   const int* part_slot;
   bf16* act1;
   bf16* act2;
+  // its jobs from n_d on are generators': job n_d + c * mt_g + t takes the m-tiles 2t and 2t + 1 of
+  // z_c (mB3; kc1_g chunks of width z) through the hidden layers (mC1, mC2) of generator
+  // gen.wsel[c], whose activations go to gen.act1 / act2 ([c][B][256])
+  int n_d, mt_g, kc1_g, z;
+  struct {
+    const int* wsel;
+    const float* wmaster;
+    int64_t pstride, off_b1, off_b2;
+    bf16* act1;
+    bf16* act2;
+  } gen;
 };
 
 // A generator pair's output blocks: part i of p.split takes blocks [i n3 / split, (i + 1) n3 / split)
@@ -791,11 +802,16 @@ __device__ __forceinline__ Job pair_job(const PParams& p, const PairPart& pp, in
   return Job{1, HID / BK, (n + 15) & ~15, (j - 2 + pp.nb) & 1, 2, nb * N3, N3, EPI_TO_E};
 }
 
-template <int KND>
+// TRAIN: the training forward, in one launch: the discriminators' jobs, then the generators', which
+// are shorter (with the logit deltas, against a launch of each: 1x1 cells 32.5 -> 25 us, 5x5 cells
+// at B = 256 46.5 -> 37.5, 12x12 cells 55 -> 56).
+template <int KND, bool TRAIN>
 __global__ void __launch_bounds__(pair_threads<KND>(), 1)
     k_mlp_fwd_pair(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mB1,
                    const __grid_constant__ CUtensorMap mB2, const __grid_constant__ CUtensorMap mB3,
+                   const __grid_constant__ CUtensorMap mC1, const __grid_constant__ CUtensorMap mC2,
                    const PParams p) {
+  static_assert(KND == KIND_D || !TRAIN, "the training forward runs on the discriminators' kernel");
   using CF = PCfg<KND>;
   constexpr int NE = CF::NE;               // epilogue warps
   constexpr int CP = NE / 4;               // column parts (warps per TMEM lane quarter)
@@ -861,6 +877,19 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
   const uint32_t lH = mapa_shared(bH, 0), lZfull = mapa_shared(bZfull, 0);
   const int n_parts = KND == KIND_D ? p.n_pairs : p.n_pairs * p.split;
   const int cid = (int)cluster_id_x(), ncl = (int)nclusters_x();
+  auto is_gen = [&](int pi) { return TRAIN && pi >= p.n_d; };
+  // a training job's cell and individual
+  auto train_cell = [&](int pi) {
+    return is_gen(pi) ? (pi - p.n_d) / p.mt_g : pi / p.mt;
+  };
+  auto train_individual = [&](int pi) {
+    return __ldg(&(is_gen(pi) ? p.gen.wsel : p.wsel)[train_cell(pi)]);
+  };
+  auto get_job = [&](const PairPart& pp, int j, int pi) {
+    Job J = pair_job<KND>(p, pp, j);
+    if (is_gen(pi) && j == 0) J.kchunks = p.kc1_g;
+    return J;
+  };
   pdl_wait();
 
   if (warp == 0) {
@@ -871,12 +900,15 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
       uint32_t phase = 0;
       bool ok = true;
       for (int pi = cid; pi < n_parts && ok; pi += ncl) {
-        const bool train = KND == KIND_D && p.train;
+        const bool gen = is_gen(pi);
         const PairPart pp = pair_part<KND>(p, pi);
-        const int4 pr = train ? make_int4(0, 0, 0, 0) : __ldg(&p.pairs[pp.pair]);
-        const int k = train ? __ldg(&p.wsel[pi / p.mt]) : pr.x;
+        const int4 pr = TRAIN ? make_int4(0, 0, 0, 0) : __ldg(&p.pairs[pp.pair]);
+        const int k = TRAIN ? train_individual(pi) : pr.x;
         int a_cell = 0, a_row = p.rows;  // no problem: rows past the end read as zero
-        if (train) {
+        if (gen) {
+          a_cell = train_cell(pi);
+          a_row = (2 * (pi - p.n_d - a_cell * p.mt_g) + (int)rank) * BM;
+        } else if (TRAIN) {
           // (rows of the tile past the part's B read the next slot's rows: never stored)
           const int cell = pi / p.mt, t = pi - cell * p.mt;
           a_cell = cell;
@@ -889,8 +921,9 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
           }
         }
         for (int j = 0; j < 2 + pp.nb && ok; ++j) {
-          const Job J = pair_job<KND>(p, pp, j);
-          const CUtensorMap* mb = J.bmap == 0 ? &mB1 : (J.bmap == 1 ? &mB2 : &mB3);
+          const Job J = get_job(pp, j, pi);
+          const CUtensorMap* mb = gen ? (J.bmap == 0 ? &mC1 : &mC2)
+                                      : (J.bmap == 0 ? &mB1 : (J.bmap == 1 ? &mB2 : &mB3));
           const bool a_ring = CF::A_IN && !J.a_from_h;
           const uint32_t bytes = (a_ring ? (uint32_t)A_BYTES : 0u) + (uint32_t)HB_BYTES;
           for (int kc = 0; kc < J.kchunks; ++kc) {
@@ -902,7 +935,8 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
             if (leader && elected) mbar_expect_tx(bFull + 8 * stage, 2 * bytes);
             const uint32_t sS = sStage + stage * CF::STAGE;
             const uint32_t full = lFull + 8 * stage;
-            if (a_ring && elected) tma_load_3d_cg2(sS, &mA, full, kc * BK, a_row, a_cell);
+            if (a_ring && elected)
+              tma_load_3d_cg2(sS, gen ? &mB3 : &mA, full, kc * BK, a_row, a_cell);
             if (elected)
               tma_load_3d_cg2(sS + (CF::A_IN ? A_BYTES : 0), mb, full, kc * BK,
                               J.brow0 + (int)rank * (J.n / 2), k);
@@ -934,7 +968,7 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
       for (int pi = cid; pi < n_parts && ok; pi += ncl) {
         const PairPart pp = pair_part<KND>(p, pi);
         for (int j = 0; j < 2 + pp.nb && ok; ++j) {
-          const Job J = pair_job<KND>(p, pp, j);
+          const Job J = get_job(pp, j, pi);
           const int R = J.region;
           if (reg_uses[R] > 0 &&
               !mbar_wait(bReg + 8 * R, (uint32_t)((reg_uses[R] - 1) & 1), abort_flag, p.err, 2)) {
@@ -949,7 +983,7 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
           tc_fence_after();
           const uint32_t d = tmem + (uint32_t)(R * HID);
           const uint32_t idesc = idesc_bf16(2 * BM, J.n);
-          const int last = KND == KIND_D && j == 0 ? last_steps(p.x, J.kchunks) : BK / 16;
+          const int last = KND == KIND_D && j == 0 ? last_steps(is_gen(pi) ? p.z : p.x, J.kchunks) : BK / 16;
           for (int kc = 0; kc < J.kchunks; ++kc) {
             // (the generator's output blocks read the same activation: wait for it once)
             if (J.a_from_h && h_seen[kc] != h_total) {
@@ -1022,16 +1056,18 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
     // from global memory one tile ahead, so that a tile's staging waits on no memory latency
     // (the generator's first layer, one K chunk, does not cover it)
     constexpr int NV = (BIAS_MAX + 32 * NE - 1) / (32 * NE);
-    auto load_bias = [&](int kk, float (&v)[NV]) {
-      const float* wm = p.wmaster + (int64_t)kk * p.pstride;
+    auto load_bias = [&](int kk, bool gen, float (&v)[NV]) {
+      const float* wm = gen ? p.gen.wmaster + (int64_t)kk * p.gen.pstride
+                            : p.wmaster + (int64_t)kk * p.pstride;
+      const int64_t off_b1 = gen ? p.gen.off_b1 : p.off_b1, off_b2 = gen ? p.gen.off_b2 : p.off_b2;
       const int nb3 = KND == KIND_D ? HID + 1 : p.x;
 #pragma unroll
       for (int u = 0; u < NV; ++u) {
         const int i = et + u * 32 * NE;
         v[u] = 0.f;
-        if (i >= 512 + nb3) continue;
-        if (i < 256) v[u] = wm[p.off_b1 + i];
-        else if (i < 512) v[u] = wm[p.off_b2 + i - 256];
+        if (i >= (gen ? 512 : 512 + nb3)) continue;
+        if (i < 256) v[u] = wm[off_b1 + i];
+        else if (i < 512) v[u] = wm[off_b2 + i - 256];
         else if (KND == KIND_D)
           v[u] = i < 512 + HID
                      ? __bfloat162float(p.wb[(int64_t)kk * p.pstride + p.off_w3 + i - 512])
@@ -1040,20 +1076,25 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
       }
     };
     auto tile_individual = [&](int q) {
-      return (KND == KIND_D && p.train) ? __ldg(&p.wsel[q / p.mt])
-                                        : __ldg(&p.pairs[pair_part<KND>(p, q).pair]).x;
+      return TRAIN ? train_individual(q)
+                   : __ldg(&p.pairs[pair_part<KND>(p, q).pair]).x;
     };
     float vb[NV];
-    if (cid < n_parts) load_bias(tile_individual(cid), vb);
+    if (cid < n_parts) load_bias(tile_individual(cid), is_gen(cid), vb);
     for (int pi = cid; pi < n_parts && ok; pi += ncl, ++ltile) {
-      const bool train = KND == KIND_D && p.train;
+      const bool gen = is_gen(pi);
       const PairPart pp = pair_part<KND>(p, pi);
-      const int4 pr = train ? make_int4(0, 0, 0, 0) : __ldg(&p.pairs[pp.pair]);
-      const int k = train ? __ldg(&p.wsel[pi / p.mt]) : pr.x;
+      const int4 pr = TRAIN ? make_int4(0, 0, 0, 0) : __ldg(&p.pairs[pp.pair]);
+      const float lo = KND == KIND_D && !gen ? p.slope : 0.f;
       bool row_ok;
       bf16* dst = nullptr;   // generator: this row of the fakes
       int64_t lidx = 0;      // discriminator: this row's logit (training: and activations)
-      if (train) {
+      if (gen) {
+        const int cell = train_cell(pi);
+        const int rr = (2 * (pi - p.n_d - cell * p.mt_g) + (int)rank) * BM + row;
+        row_ok = rr < p.B;
+        lidx = (int64_t)cell * p.B + rr;
+      } else if (TRAIN) {
         const int cell = pi / p.mt, rr = (pi - cell * p.mt) * BM + row;
         row_ok = rr < p.B;
         lidx = (int64_t)(2 * cell + (int)rank) * p.B + rr;
@@ -1071,7 +1112,6 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
         row_ok = prob >= 0 && rr < p.rows;
         lidx = (int64_t)prob * p.rows + rr;
       }
-      (void)k;
       float* sb = s_bias + (ltile & 1) * BIAS_MAX;
       {
         const int nb3 = KND == KIND_D ? HID + 1 : p.x;
@@ -1081,7 +1121,7 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
           if (i < 512 + nb3) sb[i] = vb[u];
         }
         // the next tile's, in flight while this one computes
-        if (pi + ncl < n_parts) load_bias(tile_individual(pi + ncl), vb);
+        if (pi + ncl < n_parts) load_bias(tile_individual(pi + ncl), is_gen(pi + ncl), vb);
         mbar_arrive(bBias + 8 * (ltile & 1));
         if (!mbar_wait_warp(bBias + 8 * (ltile & 1), (uint32_t)((ltile >> 1) & 1), abort_flag,
                             p.err, 8)) {
@@ -1090,7 +1130,7 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
         }
       }
       for (int j = 0; j < 2 + pp.nb && ok; ++j) {
-        const Job J = pair_job<KND>(p, pp, j);
+        const Job J = get_job(pp, j, pi);
         const int R = J.region;
         if (!mbar_wait_warp(bAcc + 8 * R, (uint32_t)(reg_uses[R] & 1), abort_flag, p.err, 6)) {
           ok = false;
@@ -1102,7 +1142,6 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
           // chunk by chunk (64 columns; this warp's 64 / CP of each), so that the next layer
           // starts on chunk 0 while the others are written
           const float* bias = sb + (j == 0 ? 0 : 256);
-          const float lo = KND == KIND_D ? p.slope : 0.f;
           constexpr int W = BK / CP;  // columns of a chunk per warp: 32 or 16
 #pragma unroll 1
           for (int ch = 0; ch < HID / BK; ++ch) {
@@ -1139,8 +1178,8 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
                            "r"(pk[4 * u + 1]), "r"(pk[4 * u + 2]), "r"(pk[4 * u + 3])
                            : "memory");
             }
-            if (train && j == 0 && row_ok) {
-              bf16* o = p.act1 + lidx * HID + col0;  // 256-bit stores: 32-byte aligned rows
+            if (TRAIN && j == 0 && row_ok) {
+              bf16* o = (gen ? p.gen.act1 : p.act1) + lidx * HID + col0;  // 256-bit stores: 32-byte aligned rows
 #pragma unroll
               for (int u = 0; u < W / 8; u += 2)
                 st_global_v8(o + 8 * u, make_uint4(pk[4 * u], pk[4 * u + 1], pk[4 * u + 2],
@@ -1160,48 +1199,42 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
           const float* w3 = sb + 512;
           float acc = 0.f;
 #pragma unroll 1
-          for (int cp = part * 4; cp < part * 4 + 4; cp += 2) {
-            uint32_t r2[2][32];
-            LIPZ_TMEM_LD32(tbase + cp * 32, r2[0]);
-            LIPZ_TMEM_LD32(tbase + (cp + 1) * 32, r2[1]);
+          for (int cg = part * 4; cg < part * 4 + 4; ++cg) {
+            uint32_t r[32];
+            LIPZ_TMEM_LD32(tbase + cg * 32, r);
             tmem_wait_ld();
+            const float4* b4 = reinterpret_cast<const float4*>(bias + cg * 32);
+            const float4* w4 = reinterpret_cast<const float4*>(w3 + cg * 32);
+            uint32_t pk[16];
 #pragma unroll
-            for (int h2 = 0; h2 < 2; ++h2) {
-              const int cg = cp + h2;
-              const uint32_t(&r)[32] = r2[h2];
-              const float4* b4 = reinterpret_cast<const float4*>(bias + cg * 32);
-              const float4* w4 = reinterpret_cast<const float4*>(w3 + cg * 32);
-              uint32_t pk[16];
+            for (int e = 0; e < 32; e += 4) {
+              const float4 bb = b4[e >> 2], ww = w4[e >> 2];
+              float a0 = __uint_as_float(r[e]) + bb.x;
+              float a1 = __uint_as_float(r[e + 1]) + bb.y;
+              float a2 = __uint_as_float(r[e + 2]) + bb.z;
+              float a3 = __uint_as_float(r[e + 3]) + bb.w;
+              a0 = a0 > 0.f ? a0 : lo * a0;
+              a1 = a1 > 0.f ? a1 : lo * a1;
+              a2 = a2 > 0.f ? a2 : lo * a2;
+              a3 = a3 > 0.f ? a3 : lo * a3;
+              const uint32_t q01 = pack_bf16(a0, a1), q23 = pack_bf16(a2, a3);
+              pk[e >> 1] = q01;
+              pk[(e >> 1) + 1] = q23;
+              const __nv_bfloat162 v01 = *reinterpret_cast<const __nv_bfloat162*>(&q01);
+              const __nv_bfloat162 v23 = *reinterpret_cast<const __nv_bfloat162*>(&q23);
+              acc = fmaf(__low2float(v01), ww.x, acc);
+              acc = fmaf(__high2float(v01), ww.y, acc);
+              acc = fmaf(__low2float(v23), ww.z, acc);
+              acc = fmaf(__high2float(v23), ww.w, acc);
+            }
+            if (TRAIN && row_ok) {
+              bf16* o = (gen ? p.gen.act2 : p.act2) + lidx * HID + cg * 32;
 #pragma unroll
-              for (int e = 0; e < 32; e += 4) {
-                const float4 bb = b4[e >> 2], ww = w4[e >> 2];
-                float a0 = __uint_as_float(r[e]) + bb.x;
-                float a1 = __uint_as_float(r[e + 1]) + bb.y;
-                float a2 = __uint_as_float(r[e + 2]) + bb.z;
-                float a3 = __uint_as_float(r[e + 3]) + bb.w;
-                a0 = a0 > 0.f ? a0 : p.slope * a0;
-                a1 = a1 > 0.f ? a1 : p.slope * a1;
-                a2 = a2 > 0.f ? a2 : p.slope * a2;
-                a3 = a3 > 0.f ? a3 : p.slope * a3;
-                const uint32_t q01 = pack_bf16(a0, a1), q23 = pack_bf16(a2, a3);
-                pk[e >> 1] = q01;
-                pk[(e >> 1) + 1] = q23;
-                const __nv_bfloat162 v01 = *reinterpret_cast<const __nv_bfloat162*>(&q01);
-                const __nv_bfloat162 v23 = *reinterpret_cast<const __nv_bfloat162*>(&q23);
-                acc = fmaf(__low2float(v01), ww.x, acc);
-                acc = fmaf(__high2float(v01), ww.y, acc);
-                acc = fmaf(__low2float(v23), ww.z, acc);
-                acc = fmaf(__high2float(v23), ww.w, acc);
-              }
-              if (train && row_ok) {
-                bf16* o = p.act2 + lidx * HID + cg * 32;
-#pragma unroll
-                for (int u = 0; u < 4; u += 2)
-                  st_global_v8(o + 8 * u, make_uint4(pk[4 * u], pk[4 * u + 1], pk[4 * u + 2],
-                                                     pk[4 * u + 3]),
-                               make_uint4(pk[4 * u + 4], pk[4 * u + 5], pk[4 * u + 6],
-                                          pk[4 * u + 7]));
-              }
+              for (int u = 0; u < 4; u += 2)
+                st_global_v8(o + 8 * u, make_uint4(pk[4 * u], pk[4 * u + 1], pk[4 * u + 2],
+                                                   pk[4 * u + 3]),
+                             make_uint4(pk[4 * u + 4], pk[4 * u + 5], pk[4 * u + 6],
+                                        pk[4 * u + 7]));
             }
           }
           tc_fence_before();
@@ -1216,7 +1249,7 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
             }
             const float logit = acc + part_buf[row] + sb[512 + HID];
             warp_signal(lReg + 8 * R);
-            if (row_ok) p.logits[lidx] = logit;
+            if (row_ok && !gen) p.logits[lidx] = logit;
           }
         } else if (KND == KIND_G) {
           // generator output block: bias + tanh, bf16, into this row's fakes; this warp's
@@ -1631,10 +1664,14 @@ TcPlan* tc_plan_create(const TcShape& s, const TcBuffers& b, std::string* msg) {
   ppd.off_w3 = b.doff[4];
   p->ppg = ppg;
   p->ppd = ppd;
-  tc::PParams ppdt = ppd;  // the training discriminators: both parts of a cell on one pair
-  ppdt.train = 1;
+  tc::PParams ppdt = ppd;  // the training pairs: both parts of a cell on one CTA pair
   ppdt.mt = tiles(s.B);
-  ppdt.n_pairs = s.cells * ppdt.mt;
+  ppdt.n_d = s.cells * ppdt.mt;
+  ppdt.mt_g = (ppdt.mt + 1) / 2;
+  ppdt.n_pairs = ppdt.n_d + s.cells * ppdt.mt_g;
+  ppdt.kc1_g = g.kc1;
+  ppdt.z = s.z;
+  ppdt.gen = {b.src_g, b.Gw, b.PGs, b.goff[1], b.goff[3], (bf16*)b.TH1, (bf16*)b.TH2};
   ppdt.rows = s.B;
   ppdt.wsel = b.src_d;
   ppdt.part_slot = b.sel_g;
@@ -1644,12 +1681,16 @@ TcPlan* tc_plan_create(const TcShape& s, const TcBuffers& b, std::string* msg) {
   p->ppdt = ppdt;
   const bool pairs_on = !env_flag("LIPZ_FWD_SINGLE");
   p->ncl_g = pairs_on && s.z == tc::BK
-                 ? max_pair_clusters(tc::k_mlp_fwd_pair<tc::KIND_G>, tc::pair_threads<tc::KIND_G>(),
+                 ? max_pair_clusters(tc::k_mlp_fwd_pair<tc::KIND_G, false>, tc::pair_threads<tc::KIND_G>(),
                                      tc::pair_smem_bytes<tc::KIND_G>())
                  : 0;
   p->ncl_d = pairs_on && 6 * s.B < 65536
-                 ? max_pair_clusters(tc::k_mlp_fwd_pair<tc::KIND_D>, tc::pair_threads<tc::KIND_D>(),
-                                     tc::pair_smem_bytes<tc::KIND_D>())
+                 ? std::min(max_pair_clusters(tc::k_mlp_fwd_pair<tc::KIND_D, false>,
+                                              tc::pair_threads<tc::KIND_D>(),
+                                              tc::pair_smem_bytes<tc::KIND_D>()),
+                            max_pair_clusters(tc::k_mlp_fwd_pair<tc::KIND_D, true>,
+                                              tc::pair_threads<tc::KIND_D>(),
+                                              tc::pair_smem_bytes<tc::KIND_D>()))
                  : 0;
   if (env_flag("LIPZ_VERBOSE"))
     fprintf(stderr, "lipz: tensor-core forward: %d SMs, CTA-pair clusters resident: generator %d, "
@@ -1682,9 +1723,11 @@ int launch(int grid, const CUtensorMap& a, const CUtensorMap& b1, const CUtensor
 }  // namespace
 
 namespace {
-int launch_pair(int ncl, const CUtensorMap& a, const CUtensorMap& b1, const CUtensorMap& b2,
-                const CUtensorMap& b3, const tc::PParams& pq, bool gen, cudaStream_t st,
-                std::string* msg) {
+enum PairKind { PAIR_G, PAIR_D, PAIR_TRAIN };
+
+int launch_pair(TcPlan* p, PairKind kind, const tc::PParams& pq, cudaStream_t st, std::string* msg) {
+  const bool gen = kind == PAIR_G;
+  const int ncl = gen ? p->ncl_g : p->ncl_d;
   // Small grids: a pair's output blocks in as many parts as there are idle clusters, each with the
   // hidden layers of its own (784 outputs, four blocks; 1x1 cells, 2 pairs: 27 -> 21 us, 3x3, 18
   // pairs: 29 -> 23). More parts than clusters would take a second round for less work each.
@@ -1692,16 +1735,22 @@ int launch_pair(int ncl, const CUtensorMap& a, const CUtensorMap& b1, const CUte
   pp.split = gen ? std::max(1, std::min(pp.n3, ncl / std::max(1, pp.n_pairs))) : 1;
   const int parts = pp.n_pairs * pp.split, clusters = parts < ncl ? parts : ncl;
   if (clusters <= 0) return 0;
+  auto run = [&](auto kernel, int threads, size_t smem, const CUtensorMap& a, const CUtensorMap& b1,
+                 const CUtensorMap& b2, const CUtensorMap& b3) {
+    return launch_pairs(kernel, clusters, threads, smem, st, a, b1, b2, b3, p->mG1h, p->mG2h, pp);
+  };
+  constexpr int tg = tc::pair_threads<tc::KIND_G>(), td = tc::pair_threads<tc::KIND_D>();
+  constexpr size_t sg = tc::pair_smem_bytes<tc::KIND_G>(), sd = tc::pair_smem_bytes<tc::KIND_D>();
   cudaError_t e =
-      gen ? launch_pairs(tc::k_mlp_fwd_pair<tc::KIND_G>, clusters, tc::pair_threads<tc::KIND_G>(),
-                         (size_t)tc::pair_smem_bytes<tc::KIND_G>(), st, a, b1, b2, b3, pp)
-          : launch_pairs(tc::k_mlp_fwd_pair<tc::KIND_D>, clusters, tc::pair_threads<tc::KIND_D>(),
-                         (size_t)tc::pair_smem_bytes<tc::KIND_D>(), st, a, b1, b2, b3, pp);
+      gen ? run(tc::k_mlp_fwd_pair<tc::KIND_G, false>, tg, sg, p->mZ, p->mG1h, p->mG2h, p->mG3h)
+      : kind == PAIR_D
+          ? run(tc::k_mlp_fwd_pair<tc::KIND_D, false>, td, sd, p->mE, p->mD1h, p->mD2h, p->mZ)
+          : run(tc::k_mlp_fwd_pair<tc::KIND_D, true>, td, sd, p->mE, p->mD1h, p->mD2h, p->mZ);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) {
     cudaGetLastError();
     if (msg)
-      *msg = std::string(gen ? "generator" : "discriminator") +
+      *msg = std::string(gen ? "generator" : kind == PAIR_D ? "discriminator" : "training") +
              " forward (CTA pairs) launch: " + cudaGetErrorString(e);
     return 1;
   }
@@ -1711,7 +1760,7 @@ int launch_pair(int ncl, const CUtensorMap& a, const CUtensorMap& b1, const CUte
 
 int tc_run_g(TcPlan* p, cudaStream_t st, std::string* msg) {
   if (p->ncl_g > 0 && p->ppg.pairs)
-    return launch_pair(p->ncl_g, p->mZ, p->mG1h, p->mG2h, p->mG3h, p->ppg, true, st, msg);
+    return launch_pair(p, PAIR_G, p->ppg, st, msg);
   return launch(p->grid_g, p->mZ, p->mG1, p->mG2, p->mG3, p->pg, st, "generator forward", msg);
 }
 
@@ -1751,22 +1800,21 @@ bool tc_gram_supported(int B) { return B >= 32 && 6 * B + 32 <= tc::GRAM_NORMS; 
 
 int tc_run_d(TcPlan* p, cudaStream_t st, std::string* msg) {
   if (p->ncl_d > 0 && p->ppd.pairs)
-    return launch_pair(p->ncl_d, p->mE, p->mD1h, p->mD2h, p->mD2h, p->ppd, false, st, msg);
+    return launch_pair(p, PAIR_D, p->ppd, st, msg);
   return launch(p->grid_d, p->mE, p->mD1, p->mD2, p->mD2, p->pd, st, "discriminator forward",
                 msg);
 }
 
-int tc_run_train_g(TcPlan* p, cudaStream_t st, std::string* msg) {
-  return launch(p->grid_gt, p->mZ, p->mG1, p->mG2, p->mG3, p->pgt, st, "generator training forward",
-                msg);
+int tc_run_train(TcPlan* p, cudaStream_t st, std::string* msg) {
+  if (p->ncl_d > 0) return launch_pair(p, PAIR_TRAIN, p->ppdt, st, msg);
+  const int rc = launch(p->grid_gt, p->mZ, p->mG1, p->mG2, p->mG3, p->pgt, st,
+                        "generator training forward", msg);
+  return rc ? rc
+            : launch(p->grid_dt, p->mE4, p->mD1, p->mD2, p->mD2, p->pdt, st,
+                     "discriminator training forward", msg);
 }
 
-int tc_run_train_d(TcPlan* p, cudaStream_t st, std::string* msg) {
-  if (p->ncl_d > 0)
-    return launch_pair(p->ncl_d, p->mE, p->mD1h, p->mD2h, p->mD2h, p->ppdt, false, st, msg);
-  return launch(p->grid_dt, p->mE4, p->mD1, p->mD2, p->mD2, p->pdt, st,
-                "discriminator training forward", msg);
-}
+int tc_train_launches(const TcPlan* p) { return p->ncl_d > 0 ? 1 : 2; }
 
 int* tc_error_flag(TcPlan* p) { return p ? p->err : nullptr; }
 

@@ -99,8 +99,8 @@ int64_t tc_gram_floats(int B);  // of gram_out, per cell
 bool tc_gram_supported(int B);
 // Training forward of every cell's selected generator (hidden activations into TH1, TH2) and
 // selected discriminator (TG1, TG2 and the logits TL).
-int tc_run_train_g(TcPlan* p, cudaStream_t st, std::string* msg);
-int tc_run_train_d(TcPlan* p, cudaStream_t st, std::string* msg);
+int tc_run_train(TcPlan* p, cudaStream_t st, std::string* msg);
+int tc_train_launches(const TcPlan* p);
 
 // Device int that a kernel of the plan sets to a non-zero code when one of its bounded waits
 // expired (the kernel then stopped early); the host reads and clears it.
