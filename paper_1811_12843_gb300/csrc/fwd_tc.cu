@@ -198,6 +198,59 @@ __device__ __forceinline__ float tanh_fast(float x) {
   return copysignf(ax < 0.25f ? s : t, x);
 }
 
+// The same of two values, with the multiplications and additions of both in one instruction each:
+// 12 issue slots per element instead of 22 (two MUFU operations each either way). 2 rcp(y) is exact,
+// so one fused operation takes the place of the division and the subtraction; every one of the 2^32
+// inputs gives the same bits.
+__device__ __forceinline__ unsigned long long f2_pack(float a, float b) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ float2 f2_unpack(unsigned long long v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ unsigned long long f2_fma(unsigned long long a, unsigned long long b,
+                                                     unsigned long long c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ unsigned long long f2_mul(unsigned long long a, unsigned long long b) {
+  unsigned long long r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ unsigned long long f2_add(unsigned long long a, unsigned long long b) {
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ float rcp_approx(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float2 tanh_fast2(unsigned long long xx) {
+  const float2 x = f2_unpack(xx);
+  const float ax0 = fminf(fabsf(x.x), 16.f), ax1 = fminf(fabsf(x.y), 16.f);
+  const unsigned long long ax = f2_pack(ax0, ax1), one = f2_pack(1.f, 1.f);
+  const float2 arg = f2_unpack(f2_mul(ax, f2_pack(2.8853900817779268f, 2.8853900817779268f)));
+  const float2 y = f2_unpack(f2_add(f2_pack(ex2_approx(arg.x), ex2_approx(arg.y)), one));
+  const float2 t = f2_unpack(f2_fma(f2_pack(rcp_approx(y.x), rcp_approx(y.y)), f2_pack(-2.f, -2.f),
+                                    one));
+  const unsigned long long x2 = f2_mul(ax, ax);
+  unsigned long long q = f2_fma(x2, f2_pack(0.021869488536155203f, 0.021869488536155203f),
+                                f2_pack(-0.053968253968253971f, -0.053968253968253971f));
+  q = f2_fma(x2, q, f2_pack(0.13333333333333333f, 0.13333333333333333f));
+  q = f2_fma(x2, q, f2_pack(-0.33333333333333333f, -0.33333333333333333f));
+  const float2 s = f2_unpack(f2_mul(ax, f2_fma(x2, q, one)));
+  return make_float2(copysignf(ax0 < 0.25f ? s.x : t.x, x.x),
+                     copysignf(ax1 < 0.25f ? s.y : t.y, x.y));
+}
+
 // ---- the kernel ----------------------------------------------------------------------------
 // KND: p.kind at compile time (one variant per network kind, each with only its own paths)
 template <int KND>
@@ -710,33 +763,13 @@ __global__ void __launch_bounds__(THREADS, 1)
 //              lone tile's partner computes zeros and stores nothing).
 constexpr int HB_BYTES = (HID / 2) * BK * 2;  // 16 KB: half of a 256-row weight box
 
-template <int KND>
-struct PCfg;
-// generator: rings of weight halves only (its first layer's A is the gathered noise tile);
-// sixteen epilogue warps (its output epilogue, tanh and the fakes' stores, is the longest)
-template <>
-struct PCfg<KIND_G> {
-  static constexpr int STAGES = 8, STAGE = HB_BYTES, A_IN = 0, ZBUF = A_BYTES, NE = 16;
-};
 // discriminator: each stage holds the A chunk and the weight half; eight epilogue warps (two
 // column halves: the logit's two partial dot products are added in the one-CTA kernel's order)
-template <>
-struct PCfg<KIND_D> {
-  static constexpr int STAGES = 4, STAGE = A_BYTES + HB_BYTES, A_IN = 1, ZBUF = 0, NE = 8;
-};
-// warps: producer, MMA issuer, NE epilogue warps, noise gather
-template <int KND>
-constexpr int pair_threads() {
-  return 32 * (3 + PCfg<KND>::NE);
-}
-template <int KND>
-constexpr int pair_smem_bytes() {
-  return 1024 + PCfg<KND>::STAGES * PCfg<KND>::STAGE + PCfg<KND>::ZBUF + H_BYTES + MISC_BYTES +
-         BIAS_BYTES;
-}
-static_assert(pair_smem_bytes<KIND_G>() <= 232448, "generator pair kernel: shared memory");
-static_assert(pair_smem_bytes<KIND_D>() <= 232448, "discriminator pair kernel: shared memory");
-static_assert(2 * PCfg<KIND_G>::STAGES + 14 <= 32, "barriers must fit below the TMEM slot");
+constexpr int D_STAGES = 4, D_STAGE = A_BYTES + HB_BYTES, D_NE = 8;
+constexpr int D_THREADS = 32 * (2 + D_NE);  // producer, MMA issuer, epilogue
+constexpr int D_SMEM = 1024 + D_STAGES * D_STAGE + H_BYTES + MISC_BYTES + BIAS_BYTES;
+static_assert(D_SMEM <= 232448, "discriminator pair kernel: shared memory");
+static_assert(2 * D_STAGES + 12 <= 32, "barriers must fit below the TMEM slot");
 
 struct PParams {
   int B, x, rows;  // rows per problem: B (generator) or 6B (discriminator)
@@ -768,7 +801,7 @@ struct PParams {
   bf16* act1;
   bf16* act2;
   // its jobs from n_d on are generators': job n_d + c * mt_g + t takes the m-tiles 2t and 2t + 1 of
-  // z_c (mB3; kc1_g chunks of width z) through the hidden layers (mC1, mC2) of generator
+  // z_c (mZ; kc1_g chunks of width z) through the hidden layers (mC1, mC2) of generator
   // gen.wsel[c], whose activations go to gen.act1 / act2 ([c][B][256])
   int n_d, mt_g, kc1_g, z;
   struct {
@@ -785,56 +818,39 @@ struct PParams {
 struct PairPart {
   int pair, nb0, nb;
 };
-template <int KND>
 __device__ __forceinline__ PairPart pair_part(const PParams& p, int i) {
-  if (KND == KIND_D) return PairPart{i, 0, 0};
   const int pair = i / p.split, part = i - pair * p.split;
   const int nb0 = part * p.n3 / p.split;
   return PairPart{pair, nb0, (part + 1) * p.n3 / p.split - nb0};
 }
 
-template <int KND>
-__device__ __forceinline__ Job pair_job(const PParams& p, const PairPart& pp, int j) {
-  if (j == 0) return Job{0, p.kc1, HID, 0, 0, 0, HID, EPI_TO_H};
-  if (j == 1) return Job{1, HID / BK, HID, 1, 1, 0, HID, KND == KIND_D ? EPI_LOGIT : EPI_TO_H};
-  const int nb = pp.nb0 + j - 2;
-  const int n = min(N3, p.x - nb * N3);
-  return Job{1, HID / BK, (n + 15) & ~15, (j - 2 + pp.nb) & 1, 2, nb * N3, N3, EPI_TO_E};
-}
-
 // TRAIN: the training forward, in one launch: the discriminators' jobs, then the generators', which
 // are shorter (with the logit deltas, against a launch of each: 1x1 cells 32.5 -> 25 us, 5x5 cells
 // at B = 256 46.5 -> 37.5, 12x12 cells 55 -> 56).
-template <int KND, bool TRAIN>
-__global__ void __launch_bounds__(pair_threads<KND>(), 1)
+template <bool TRAIN>
+__global__ void __launch_bounds__(D_THREADS, 1)
     k_mlp_fwd_pair(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mB1,
-                   const __grid_constant__ CUtensorMap mB2, const __grid_constant__ CUtensorMap mB3,
+                   const __grid_constant__ CUtensorMap mB2, const __grid_constant__ CUtensorMap mZ,
                    const __grid_constant__ CUtensorMap mC1, const __grid_constant__ CUtensorMap mC2,
                    const PParams p) {
-  static_assert(KND == KIND_D || !TRAIN, "the training forward runs on the discriminators' kernel");
-  using CF = PCfg<KND>;
-  constexpr int NE = CF::NE;               // epilogue warps
-  constexpr int CP = NE / 4;               // column parts (warps per TMEM lane quarter)
+  constexpr int NE = D_NE;                 // epilogue warps
   constexpr int ARRIVALS = 2 * NE;         // one per epilogue warp of both CTAs
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   uint8_t* gbase = smem_raw + (base - raw);
-  const uint32_t sStage = base;                        // STAGES x ([A] | weight half)
-  const uint32_t sZ = base + CF::STAGES * CF::STAGE;   // generator: the gathered noise rows
-  const uint32_t sH = sZ + CF::ZBUF;                   // on-chip activation (own 128 rows)
-  uint8_t* misc = gbase + CF::STAGES * CF::STAGE + CF::ZBUF + H_BYTES;
+  const uint32_t sStage = base;                        // D_STAGES x (A | weight half)
+  const uint32_t sH = base + D_STAGES * D_STAGE;       // on-chip activation (own 128 rows)
+  uint8_t* misc = gbase + D_STAGES * D_STAGE + H_BYTES;
   uint64_t* bars = reinterpret_cast<uint64_t*>(misc);
   const uint32_t bFull = smem_u32(bars);               // [STAGES], used in rank 0
-  const uint32_t bEmpty = bFull + 8 * CF::STAGES;      // [STAGES]
-  const uint32_t bAcc = bEmpty + 8 * CF::STAGES;       // [2]
+  const uint32_t bEmpty = bFull + 8 * D_STAGES;      // [STAGES]
+  const uint32_t bAcc = bEmpty + 8 * D_STAGES;       // [2]
   const uint32_t bReg = bAcc + 16;                     // [2], rank 0
   const uint32_t bH = bReg + 16;                       // [4], rank 0
   const uint32_t bPart = bH + 32;
   const uint32_t bFinal = bPart + 8;
   const uint32_t bBias = bFinal + 8;                   // [2]
-  const uint32_t bZfull = bBias + 16;                  // rank 0
-  const uint32_t bZempty = bZfull + 8;
   float* s_bias = reinterpret_cast<float*>(misc + MISC_BYTES);
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(misc + 256);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 260);
@@ -844,7 +860,7 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
   const uint32_t rank = cluster_ctarank();
   const bool leader = rank == 0;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < CF::STAGES; ++s) {
+    for (int s = 0; s < D_STAGES; ++s) {
       mbar_init(bFull + 8 * s, 1);
       mbar_init(bEmpty + 8 * s, 1);
     }
@@ -856,8 +872,6 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
     for (int c = 0; c < HID / BK; ++c) mbar_init(bH + 8 * c, ARRIVALS);
     mbar_init(bPart, 32 * NE / 2);
     mbar_init(bFinal, 1);
-    mbar_init(bZfull, 2);
-    mbar_init(bZempty, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -874,8 +888,7 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
   const uint32_t tmem = *tmem_slot;
   // rank 0's barriers that both CTAs arrive on
   const uint32_t lFull = mapa_shared(bFull, 0), lReg = mapa_shared(bReg, 0);
-  const uint32_t lH = mapa_shared(bH, 0), lZfull = mapa_shared(bZfull, 0);
-  const int n_parts = KND == KIND_D ? p.n_pairs : p.n_pairs * p.split;
+  const uint32_t lH = mapa_shared(bH, 0);
   const int cid = (int)cluster_id_x(), ncl = (int)nclusters_x();
   auto is_gen = [&](int pi) { return TRAIN && pi >= p.n_d; };
   // a training job's cell and individual
@@ -885,11 +898,8 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
   auto train_individual = [&](int pi) {
     return __ldg(&(is_gen(pi) ? p.gen.wsel : p.wsel)[train_cell(pi)]);
   };
-  auto get_job = [&](const PairPart& pp, int j, int pi) {
-    Job J = pair_job<KND>(p, pp, j);
-    if (is_gen(pi) && j == 0) J.kchunks = p.kc1_g;
-    return J;
-  };
+  // layer j's K chunks
+  auto chunks = [&](int pi, int j) { return j ? HID / BK : is_gen(pi) ? p.kc1_g : p.kc1; };
   pdl_wait();
 
   if (warp == 0) {
@@ -899,10 +909,9 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
-      for (int pi = cid; pi < n_parts && ok; pi += ncl) {
+      for (int pi = cid; pi < p.n_pairs && ok; pi += ncl) {
         const bool gen = is_gen(pi);
-        const PairPart pp = pair_part<KND>(p, pi);
-        const int4 pr = TRAIN ? make_int4(0, 0, 0, 0) : __ldg(&p.pairs[pp.pair]);
+        const int4 pr = TRAIN ? make_int4(0, 0, 0, 0) : __ldg(&p.pairs[pi]);
         const int k = TRAIN ? train_individual(pi) : pr.x;
         int a_cell = 0, a_row = p.rows;  // no problem: rows past the end read as zero
         if (gen) {
@@ -913,34 +922,31 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
           const int cell = pi / p.mt, t = pi - cell * p.mt;
           a_cell = cell;
           a_row = (rank ? 1 + __ldg(&p.part_slot[cell]) : 0) * p.B + t * BM;
-        } else if (KND == KIND_D) {
+        } else {
           const int prob = rank ? pr.z : pr.y;
           if (prob >= 0) {
             a_cell = prob / 5;
             a_row = rank ? (pr.w & 0xFFFF) : (pr.w >> 16);
           }
         }
-        for (int j = 0; j < 2 + pp.nb && ok; ++j) {
-          const Job J = get_job(pp, j, pi);
-          const CUtensorMap* mb = gen ? (J.bmap == 0 ? &mC1 : &mC2)
-                                      : (J.bmap == 0 ? &mB1 : (J.bmap == 1 ? &mB2 : &mB3));
-          const bool a_ring = CF::A_IN && !J.a_from_h;
-          const uint32_t bytes = (a_ring ? (uint32_t)A_BYTES : 0u) + (uint32_t)HB_BYTES;
-          for (int kc = 0; kc < J.kchunks; ++kc) {
+        for (int j = 0; j < 2 && ok; ++j) {
+          const CUtensorMap* mb = gen ? (j ? &mC2 : &mC1) : (j ? &mB2 : &mB1);
+          const uint32_t bytes = (j ? 0u : (uint32_t)A_BYTES) + (uint32_t)HB_BYTES;
+          const int kchunks = chunks(pi, j);
+          for (int kc = 0; kc < kchunks; ++kc) {
             if (!mbar_wait(bEmpty + 8 * stage, phase ^ 1u, abort_flag, p.err, 1)) {
               ok = false;
               break;
             }
             // rank 0 expects both CTAs' bytes; the peer's may land first
             if (leader && elected) mbar_expect_tx(bFull + 8 * stage, 2 * bytes);
-            const uint32_t sS = sStage + stage * CF::STAGE;
+            const uint32_t sS = sStage + stage * D_STAGE;
             const uint32_t full = lFull + 8 * stage;
-            if (a_ring && elected)
-              tma_load_3d_cg2(sS, gen ? &mB3 : &mA, full, kc * BK, a_row, a_cell);
+            if (j == 0 && elected)
+              tma_load_3d_cg2(sS, gen ? &mZ : &mA, full, kc * BK, a_row, a_cell);
             if (elected)
-              tma_load_3d_cg2(sS + (CF::A_IN ? A_BYTES : 0), mb, full, kc * BK,
-                              J.brow0 + (int)rank * (J.n / 2), k);
-            if (++stage == CF::STAGES) {
+              tma_load_3d_cg2(sS + A_BYTES, mb, full, kc * BK, (int)rank * (HID / 2), k);
+            if (++stage == D_STAGES) {
               stage = 0;
               phase ^= 1u;
             }
@@ -962,47 +968,34 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
       int stage = 0;
       uint32_t phase = 0;
       int reg_uses[2] = {0, 0};
-      int h_total = 0, zuse = 0;
-      int h_seen[HID / BK] = {0, 0, 0, 0};  // activation write each chunk was last waited for
+      int tiles = 0;
       bool ok = true;
-      for (int pi = cid; pi < n_parts && ok; pi += ncl) {
-        const PairPart pp = pair_part<KND>(p, pi);
-        for (int j = 0; j < 2 + pp.nb && ok; ++j) {
-          const Job J = get_job(pp, j, pi);
-          const int R = J.region;
+      for (int pi = cid; pi < p.n_pairs && ok; pi += ncl, ++tiles) {
+        for (int j = 0; j < 2 && ok; ++j) {
+          const int R = j;  // accumulator region
           if (reg_uses[R] > 0 &&
               !mbar_wait(bReg + 8 * R, (uint32_t)((reg_uses[R] - 1) & 1), abort_flag, p.err, 2)) {
             ok = false;
             break;
           }
-          if (KND == KIND_G && j == 0 &&
-              !mbar_wait(bZfull, (uint32_t)(zuse & 1), abort_flag, p.err, 9)) {
-            ok = false;
-            break;
-          }
           tc_fence_after();
           const uint32_t d = tmem + (uint32_t)(R * HID);
-          const uint32_t idesc = idesc_bf16(2 * BM, J.n);
-          const int last = KND == KIND_D && j == 0 ? last_steps(is_gen(pi) ? p.z : p.x, J.kchunks) : BK / 16;
-          for (int kc = 0; kc < J.kchunks; ++kc) {
-            // (the generator's output blocks read the same activation: wait for it once)
-            if (J.a_from_h && h_seen[kc] != h_total) {
-              if (!mbar_wait(bH + 8 * kc, (uint32_t)((h_total - 1) & 1), abort_flag, p.err, 3)) {
-                ok = false;
-                break;
-              }
-              h_seen[kc] = h_total;
+          const uint32_t idesc = idesc_bf16(2 * BM, HID);
+          const int kchunks = chunks(pi, j);
+          const int last = j ? BK / 16 : last_steps(is_gen(pi) ? p.z : p.x, kchunks);
+          for (int kc = 0; kc < kchunks; ++kc) {
+            // (a tile's activation is write number `its tile` of every chunk)
+            if (j && !mbar_wait(bH + 8 * kc, (uint32_t)(tiles & 1), abort_flag, p.err, 3)) {
+              ok = false;
+              break;
             }
             if (!mbar_wait(bFull + 8 * stage, phase, abort_flag, p.err, 4)) {
               ok = false;
               break;
             }
             tc_fence_after();
-            const uint32_t sS = sStage + stage * CF::STAGE;
-            const uint32_t sA = (KND == KIND_G && j == 0)
-                                    ? sZ
-                                    : (J.a_from_h ? sH + kc * H_CHUNK : sS);
-            const uint32_t sB = sS + (CF::A_IN ? A_BYTES : 0);
+            const uint32_t sS = sStage + stage * D_STAGE;
+            const uint32_t sA = j ? sH + kc * H_CHUNK : sS, sB = sS + A_BYTES;
             // a 16-element K step is 32 bytes: 2 in the descriptors' address field (a 1024-byte
             // aligned tile plus at most 96 bytes never carries out of it)
             const uint64_t dA = sw128_desc(sA), dB = sw128_desc(sB);
@@ -1010,23 +1003,18 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
               tc_mma_cg2(d, dA, dB, idesc, kc != 0 ? 1u : 0u);
 #pragma unroll
               for (int kk = 1; kk < BK / 16; ++kk)
-                if (kk < last || kc + 1 < J.kchunks)
+                if (kk < last || kc + 1 < kchunks)
                   tc_mma_cg2_acc(d, dA + 2 * kk, dB + 2 * kk, idesc);
               tc_commit_cg2(bEmpty + 8 * stage, 3);
             }
-            if (++stage == CF::STAGES) {
+            if (++stage == D_STAGES) {
               stage = 0;
               phase ^= 1u;
             }
           }
           if (!ok) break;
-          if (KND == KIND_G && j == 0) {
-            if (elected) tc_commit_cg2(bZempty, 3);
-            ++zuse;
-          }
           if (elected) tc_commit_cg2(bAcc + 8 * R, 3);
           reg_uses[R]++;
-          if (J.epi == EPI_TO_H) ++h_total;
         }
       }
       // every MMA (they write both CTAs' tensor memory) completes before it is released
@@ -1038,7 +1026,7 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
     // ================================ epilogue (own 128 rows) ================================
     const int ew = warp - 2;
     const int q = warp & 3;          // TMEM lane quarter this warp may access
-    const int part = ew >> 2;        // column part: HID / CP columns of every region
+    const int part = ew >> 2;        // column half of every region
     const int row = q * 32 + lane;
     const uint32_t lane_base = (uint32_t)(q * 32) << 16;
     const int et = threadIdx.x - 64;
@@ -1054,13 +1042,12 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
     };
     // a tile's biases (and the discriminator's output weights): this thread's share, loaded
     // from global memory one tile ahead, so that a tile's staging waits on no memory latency
-    // (the generator's first layer, one K chunk, does not cover it)
-    constexpr int NV = (BIAS_MAX + 32 * NE - 1) / (32 * NE);
+    constexpr int NV = (3 * HID + 1 + 32 * NE - 1) / (32 * NE);
     auto load_bias = [&](int kk, bool gen, float (&v)[NV]) {
       const float* wm = gen ? p.gen.wmaster + (int64_t)kk * p.gen.pstride
                             : p.wmaster + (int64_t)kk * p.pstride;
       const int64_t off_b1 = gen ? p.gen.off_b1 : p.off_b1, off_b2 = gen ? p.gen.off_b2 : p.off_b2;
-      const int nb3 = KND == KIND_D ? HID + 1 : p.x;
+      constexpr int nb3 = HID + 1;
 #pragma unroll
       for (int u = 0; u < NV; ++u) {
         const int i = et + u * 32 * NE;
@@ -1068,27 +1055,24 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
         if (i >= (gen ? 512 : 512 + nb3)) continue;
         if (i < 256) v[u] = wm[off_b1 + i];
         else if (i < 512) v[u] = wm[off_b2 + i - 256];
-        else if (KND == KIND_D)
+        else
           v[u] = i < 512 + HID
                      ? __bfloat162float(p.wb[(int64_t)kk * p.pstride + p.off_w3 + i - 512])
                      : wm[p.off_b3];
-        else v[u] = wm[p.off_b3 + i - 512];
       }
     };
     auto tile_individual = [&](int q) {
       return TRAIN ? train_individual(q)
-                   : __ldg(&p.pairs[pair_part<KND>(p, q).pair]).x;
+                   : __ldg(&p.pairs[q]).x;
     };
     float vb[NV];
-    if (cid < n_parts) load_bias(tile_individual(cid), is_gen(cid), vb);
-    for (int pi = cid; pi < n_parts && ok; pi += ncl, ++ltile) {
+    if (cid < p.n_pairs) load_bias(tile_individual(cid), is_gen(cid), vb);
+    for (int pi = cid; pi < p.n_pairs && ok; pi += ncl, ++ltile) {
       const bool gen = is_gen(pi);
-      const PairPart pp = pair_part<KND>(p, pi);
-      const int4 pr = TRAIN ? make_int4(0, 0, 0, 0) : __ldg(&p.pairs[pp.pair]);
-      const float lo = KND == KIND_D && !gen ? p.slope : 0.f;
+      const int4 pr = TRAIN ? make_int4(0, 0, 0, 0) : __ldg(&p.pairs[pi]);
+      const float lo = gen ? 0.f : p.slope;
       bool row_ok;
-      bf16* dst = nullptr;   // generator: this row of the fakes
-      int64_t lidx = 0;      // discriminator: this row's logit (training: and activations)
+      int64_t lidx;  // this row's logit (training: and activations)
       if (gen) {
         const int cell = train_cell(pi);
         const int rr = (2 * (pi - p.n_d - cell * p.mt_g) + (int)rank) * BM + row;
@@ -1098,14 +1082,6 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
         const int cell = pi / p.mt, rr = (pi - cell * p.mt) * BM + row;
         row_ok = rr < p.B;
         lidx = (int64_t)(2 * cell + (int)rank) * p.B + rr;
-      } else if (KND == KIND_G) {
-        const int gr = pr.y + (int)rank * BM + row;
-        row_ok = gr < pr.w;
-        if (row_ok) {
-          const int pp = gr / p.B, b = gr - pp * p.B;
-          const int2 cs = __ldg(&p.plist[pr.z + pp]);
-          dst = p.E + (int64_t)cs.x * p.e_cell + (int64_t)((1 + cs.y) * p.B + b) * p.x;
-        }
       } else {
         const int prob = rank ? pr.z : pr.y;
         const int rr = (rank ? (pr.w & 0xFFFF) : (pr.w >> 16)) + row;
@@ -1114,14 +1090,14 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
       }
       float* sb = s_bias + (ltile & 1) * BIAS_MAX;
       {
-        const int nb3 = KND == KIND_D ? HID + 1 : p.x;
+        constexpr int nb3 = HID + 1;
 #pragma unroll
         for (int u = 0; u < NV; ++u) {
           const int i = et + u * 32 * NE;
           if (i < 512 + nb3) sb[i] = vb[u];
         }
         // the next tile's, in flight while this one computes
-        if (pi + ncl < n_parts) load_bias(tile_individual(pi + ncl), is_gen(pi + ncl), vb);
+        if (pi + ncl < p.n_pairs) load_bias(tile_individual(pi + ncl), is_gen(pi + ncl), vb);
         mbar_arrive(bBias + 8 * (ltile & 1));
         if (!mbar_wait_warp(bBias + 8 * (ltile & 1), (uint32_t)((ltile >> 1) & 1), abort_flag,
                             p.err, 8)) {
@@ -1129,29 +1105,24 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
           break;
         }
       }
-      for (int j = 0; j < 2 + pp.nb && ok; ++j) {
-        const Job J = get_job(pp, j, pi);
-        const int R = J.region;
+      for (int j = 0; j < 2 && ok; ++j) {
+        const int R = j;
         if (!mbar_wait_warp(bAcc + 8 * R, (uint32_t)(reg_uses[R] & 1), abort_flag, p.err, 6)) {
           ok = false;
           break;
         }
         tc_fence_after();
         const uint32_t tbase = tmem + lane_base + (uint32_t)(R * HID);
-        if (J.epi == EPI_TO_H) {
-          // chunk by chunk (64 columns; this warp's 64 / CP of each), so that the next layer
+        if (j == 0) {
+          // chunk by chunk (64 columns; this warp's 32 of each), so that the second layer
           // starts on chunk 0 while the others are written
-          const float* bias = sb + (j == 0 ? 0 : 256);
-          constexpr int W = BK / CP;  // columns of a chunk per warp: 32 or 16
+          const float* bias = sb;
+          constexpr int W = BK / 2;  // columns of a chunk per warp
 #pragma unroll 1
           for (int ch = 0; ch < HID / BK; ++ch) {
             const int col0 = ch * BK + part * W;
             uint32_t r[W];
-            if (W == 32) {
-              LIPZ_TMEM_LD32(tbase + col0, r);
-            } else {
-              LIPZ_TMEM_LD16(tbase + col0, r);
-            }
+            LIPZ_TMEM_LD32(tbase + col0, r);
             tmem_wait_ld();
             const float4* b4 = reinterpret_cast<const float4*>(bias + col0);
             uint32_t pk[W / 2];
@@ -1178,7 +1149,7 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
                            "r"(pk[4 * u + 1]), "r"(pk[4 * u + 2]), "r"(pk[4 * u + 3])
                            : "memory");
             }
-            if (TRAIN && j == 0 && row_ok) {
+            if (TRAIN && row_ok) {
               bf16* o = (gen ? p.gen.act1 : p.act1) + lidx * HID + col0;  // 256-bit stores: 32-byte aligned rows
 #pragma unroll
               for (int u = 0; u < W / 8; u += 2)
@@ -1192,7 +1163,7 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
           }
           tc_fence_before();
           warp_signal(lReg + 8 * R);
-        } else if (KND == KIND_D && J.epi == EPI_LOGIT) {
+        } else {
           // LeakyReLU of layer 2, rounded to bf16, dotted with the output weights: each column
           // half's partial dot product, the halves added as in the one-CTA kernel
           const float* bias = sb + 256;
@@ -1251,46 +1222,383 @@ __global__ void __launch_bounds__(pair_threads<KND>(), 1)
             warp_signal(lReg + 8 * R);
             if (row_ok && !gen) p.logits[lidx] = logit;
           }
-        } else if (KND == KIND_G) {
-          // generator output block: bias + tanh, bf16, into this row's fakes; this warp's
-          // share of the block's 16-column groups
-          const float* bias = sb + 512;
-          const int ng = J.n / 16;
-          const int per = (ng + CP - 1) / CP;
-          const int g0 = part * per, g1 = min(ng, g0 + per);
-#pragma unroll 1
-          for (int gi = g0; gi < g1; ++gi) {
-            uint32_t r[16];
-            LIPZ_TMEM_LD16(tbase + gi * 16, r);
-            tmem_wait_ld();
-            const int col0 = J.brow0 + gi * 16;
-            const float4* b4 = reinterpret_cast<const float4*>(bias + col0);
-            uint32_t pk[8];
-#pragma unroll
-            for (int qq = 0; qq < 4; ++qq) {
-              const float4 t = b4[qq];
-              pk[2 * qq] = pack_bf16(tanh_fast(__uint_as_float(r[4 * qq]) + t.x),
-                                     tanh_fast(__uint_as_float(r[4 * qq + 1]) + t.y));
-              pk[2 * qq + 1] = pack_bf16(tanh_fast(__uint_as_float(r[4 * qq + 2]) + t.z),
-                                         tanh_fast(__uint_as_float(r[4 * qq + 3]) + t.w));
-            }
-            if (row_ok && col0 < p.x)  // one 256-bit store per row and 16 columns (E's rows,
-                                       // slots and cells are 32-byte aligned: x % 16 == 0)
-              st_global_v8(dst + col0, make_uint4(pk[0], pk[1], pk[2], pk[3]),
-                           make_uint4(pk[4], pk[5], pk[6], pk[7]));
-          }
-          tc_fence_before();
-          warp_signal(lReg + 8 * R);
         }
         reg_uses[R]++;
       }
     }
-  } else if (KND == KIND_G) {
-    // ================================ noise gather (generator) ================================
+  }
+
+  __syncwarp();
+  tc_fence_before();
+  __syncthreads();
+  cluster_sync_all();  // neither CTA leaves while the peer may still arrive on its barriers
+  tc_fence_after();
+  if (warp == 1) {
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(tmem));
+  }
+}
+
+// ---- generator pairs: the next tile's hidden layers between this tile's output blocks ---------
+// The output blocks' epilogues (tanh, the fakes' stores) take most of the time; the hidden layers of
+// a tile are a chain of two MMAs and two epilogues that leaves the epilogue warps idle while each MMA
+// runs. So a cluster's jobs are ordered B0(t), L1(t + 1), B1(t), L2(t + 1), B2(t), ...: every MMA runs
+// while the epilogue of another job does. Jobs take the two tensor-memory regions in turn; the
+// activation has a buffer for even and one for odd tiles.
+// Bound: the epilogues, their MUFU operations (two per output) above all. Measured: 12x12 cells
+// 78 us with the jobs tile by tile, 74 in this order, 72 with the tanh of two outputs at a time; 5x5
+// cells at B = 256, two tiles per cluster, 45 and 43.5.
+struct GenJob {
+  int pi, t, j;  // pair part, its ordinal in this cluster, 0 or 1: hidden layer, 2 + b: output block
+  int nb0;       // first output block of the part
+};
+struct GenSeq {
+  int c, t, nb, nb0, s, ncl, n;
+  __device__ __forceinline__ GenSeq(int cid, int ncl_, int n_)
+      : c(cid - ncl_), t(-1), nb(0), nb0(0), s(0), ncl(ncl_), n(n_) {}
+  // Next job in order; false at the end.
+  __device__ __forceinline__ bool next(const PParams& p, GenJob& J) {
+    bool more = c + ncl < n;
+    if (s >= nb + (more ? 2 : 0)) {
+      if (!more) return false;
+      c += ncl;
+      ++t;
+      const PairPart pp = pair_part(p, c);
+      nb = pp.nb;
+      nb0 = pp.nb0;
+      s = 0;
+      more = c + ncl < n;
+    }
+    int layer = -1, b = s;
+    if (more) {
+      if (nb < 2) layer = s - nb;             // [B0] L1 L2
+      else if (s < 4 && (s & 1)) layer = s >> 1;
+      else b = s < 4 ? s >> 1 : s - 2;
+    }
+    J = layer >= 0 ? GenJob{c + ncl, t + 1, layer, 0} : GenJob{c, t, 2 + b, nb0};
+    ++s;
+    return true;
+  }
+};
+constexpr int G_STAGES = 4, G_NE = 16, G_CP = G_NE / 4;
+constexpr int G_THREADS = 32 * (3 + G_NE);  // producer, MMA issuer, epilogue, noise gather
+constexpr int G_B12 = 2 * HID, G_B3 = 1024;  // biases of a tile: hidden layers; output layer
+constexpr int G_SMEM = 1024 + G_STAGES * HB_BYTES + A_BYTES + 2 * H_BYTES + MISC_BYTES +
+                       (2 * G_B12 + 3 * G_B3) * 4;
+static_assert(G_SMEM <= 232448, "generator pair kernel: shared memory");
+static_assert(2 * G_STAGES + 17 <= 32, "barriers must fit below the TMEM slot");
+
+__global__ void __launch_bounds__(G_THREADS, 1)
+    k_mlp_fwd_pair_g(const __grid_constant__ CUtensorMap mB1, const __grid_constant__ CUtensorMap mB2,
+                     const __grid_constant__ CUtensorMap mB3, const PParams p) {
+  constexpr int ARRIVALS = 2 * G_NE;  // one per epilogue warp of both CTAs
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t raw = smem_u32(smem_raw);
+  const uint32_t base = (raw + 1023u) & ~1023u;
+  uint8_t* gbase = smem_raw + (base - raw);
+  const uint32_t sStage = base;                      // G_STAGES weight halves
+  const uint32_t sZ = base + G_STAGES * HB_BYTES;    // the gathered noise rows
+  const uint32_t sH = sZ + A_BYTES;                  // on-chip activation (own 128 rows), [2]
+  uint8_t* misc = gbase + G_STAGES * HB_BYTES + A_BYTES + 2 * H_BYTES;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(misc);
+  const uint32_t bFull = smem_u32(bars);             // [G_STAGES], used in rank 0
+  const uint32_t bEmpty = bFull + 8 * G_STAGES;      // [G_STAGES]
+  const uint32_t bAcc = bEmpty + 8 * G_STAGES;       // [2]
+  const uint32_t bReg = bAcc + 16;                   // [2], rank 0
+  const uint32_t bH = bReg + 16;                     // [2][4], rank 0
+  const uint32_t bFinal = bH + 64;
+  const uint32_t bBias = bFinal + 8;                 // [2]
+  const uint32_t bZfull = bBias + 16;                // rank 0
+  const uint32_t bZempty = bZfull + 8;
+  float* s_b12 = reinterpret_cast<float*>(misc + MISC_BYTES);
+  float* s_b3 = s_b12 + 2 * G_B12;
+  volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(misc + 256);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 260);
+
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = cluster_ctarank();
+  const bool leader = rank == 0;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < G_STAGES; ++s) {
+      mbar_init(bFull + 8 * s, 1);
+      mbar_init(bEmpty + 8 * s, 1);
+    }
+    for (int r = 0; r < 2; ++r) {
+      mbar_init(bAcc + 8 * r, 1);
+      mbar_init(bReg + 8 * r, ARRIVALS);
+      mbar_init(bBias + 8 * r, 32 * G_NE);
+    }
+    for (int c = 0; c < 2 * (HID / BK); ++c) mbar_init(bH + 8 * c, ARRIVALS);
+    mbar_init(bFinal, 1);
+    mbar_init(bZfull, 2);
+    mbar_init(bZempty, 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 1) {
+    // one warp of each CTA of the pair allocates together: the same columns in both
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(
+        smem_u32((const void*)tmem_slot)));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;");
+  }
+  tc_fence_before();
+  cluster_sync_all();  // no remote arrival before the peer's barriers exist
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  // rank 0's barriers that both CTAs arrive on
+  const uint32_t lFull = mapa_shared(bFull, 0), lReg = mapa_shared(bReg, 0);
+  const uint32_t lH = mapa_shared(bH, 0), lZfull = mapa_shared(bZfull, 0);
+  const int n_parts = p.n_pairs * p.split;
+  const int cid = (int)cluster_id_x(), ncl = (int)nclusters_x();
+  // MMA N of a job, and the K chunks it takes
+  auto job_n = [&](const GenJob& J) {
+    return J.j < 2 ? HID : (min(N3, p.x - (J.nb0 + J.j - 2) * N3) + 15) & ~15;
+  };
+  auto job_chunks = [](const GenJob& J) { return J.j == 0 ? 1 : HID / BK; };
+  GenJob J;
+  pdl_wait();
+
+  if (warp == 0) {
+    // ================================ TMA producer (both CTAs) ================================
+    const bool elected = elect_one();
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    GenSeq seq(cid, ncl, n_parts);
+    while (ok && seq.next(p, J)) {
+      const int k = __ldg(&p.pairs[J.pi / p.split]).x;
+      const CUtensorMap* mb = J.j == 0 ? &mB1 : (J.j == 1 ? &mB2 : &mB3);
+      const int row0 = (J.j < 2 ? 0 : (J.nb0 + J.j - 2) * N3) + (int)rank * (job_n(J) / 2);
+      const int kchunks = job_chunks(J);
+      for (int kc = 0; kc < kchunks; ++kc) {
+        if (!mbar_wait(bEmpty + 8 * stage, phase ^ 1u, abort_flag, p.err, 1)) {
+          ok = false;
+          break;
+        }
+        if (elected) {
+          // rank 0 expects both CTAs' bytes; the peer's may land first
+          if (leader) mbar_expect_tx(bFull + 8 * stage, 2 * (uint32_t)HB_BYTES);
+          tma_load_3d_cg2(sStage + stage * HB_BYTES, mb, lFull + 8 * stage, kc * BK, row0, k);
+        }
+        if (++stage == G_STAGES) {
+          stage = 0;
+          phase ^= 1u;
+        }
+      }
+    }
+    if (!ok) {
+      // loads issued here complete on rank 0's barriers: give them time to land before the CTA
+      // leaves
+      const unsigned long long t0 = globaltimer();
+      while (globaltimer() - t0 < 200000ull) {
+      }
+    }
+  } else if (warp == 1) {
+    // ================================ MMA issuer (rank 0) ================================
+    if (leader) {
+      const bool elected = elect_one();
+      int stage = 0, jobs = 0;
+      uint32_t phase = 0;
+      bool ok = true;
+      GenSeq seq(cid, ncl, n_parts);
+      for (; ok && seq.next(p, J); ++jobs) {
+        const int R = jobs & 1, use = jobs >> 1;
+        if ((use > 0 &&
+             !mbar_wait(bReg + 8 * R, (uint32_t)((use - 1) & 1), abort_flag, p.err, 2)) ||
+            (J.j == 0 && !mbar_wait(bZfull, (uint32_t)(J.t & 1), abort_flag, p.err, 9))) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        const uint32_t d = tmem + (uint32_t)(R * HID);
+        const uint32_t idesc = idesc_bf16(2 * BM, job_n(J));
+        const uint32_t hb = (uint32_t)(J.t & 1);
+        const int kchunks = job_chunks(J);
+        for (int kc = 0; kc < kchunks; ++kc) {
+          // a chunk of a buffer is written twice per tile: the first activation, which the second
+          // layer reads, and the second, which all output blocks read (the first has waited)
+          if ((J.j == 1 || J.j == 2) && !mbar_wait(bH + 8 * (4 * hb + kc), (uint32_t)(J.j - 1),
+                                                   abort_flag, p.err, 3)) {
+            ok = false;
+            break;
+          }
+          if (!mbar_wait(bFull + 8 * stage, phase, abort_flag, p.err, 4)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint32_t sA = J.j == 0 ? sZ : sH + hb * H_BYTES + kc * H_CHUNK;
+          // a 16-element K step is 32 bytes: 2 in the descriptors' address field (a 1024-byte
+          // aligned tile plus at most 96 bytes never carries out of it)
+          const uint64_t dA = sw128_desc(sA), dB = sw128_desc(sStage + stage * HB_BYTES);
+          if (elected) {
+            tc_mma_cg2(d, dA, dB, idesc, kc != 0 ? 1u : 0u);
+#pragma unroll
+            for (int kk = 1; kk < BK / 16; ++kk) tc_mma_cg2_acc(d, dA + 2 * kk, dB + 2 * kk, idesc);
+            tc_commit_cg2(bEmpty + 8 * stage, 3);
+          }
+          if (++stage == G_STAGES) {
+            stage = 0;
+            phase ^= 1u;
+          }
+        }
+        if (!ok) break;
+        if (elected) {
+          if (J.j == 0) tc_commit_cg2(bZempty, 3);
+          tc_commit_cg2(bAcc + 8 * R, 3);
+        }
+      }
+      // every MMA (they write both CTAs' tensor memory) completes before it is released
+      if (elected) tc_commit_cg2(bFinal, 3);
+      volatile int never = 0;
+      mbar_wait(bFinal, 0u, &never, p.err, 5);
+    }
+  } else if (warp < 2 + G_NE) {
+    // ================================ epilogue (own 128 rows) ================================
+    const int q = warp & 3;            // TMEM lane quarter this warp may access
+    const int part = (warp - 2) >> 2;  // column part: HID / G_CP columns of every region
+    const int row = q * 32 + lane;
+    const uint32_t lane_base = (uint32_t)(q * 32) << 16;
+    const int et = threadIdx.x - 64;
+    int jobs = 0;
+    // a warp's share is done (tensor memory read; for H chunks the rows written and made
+    // visible to the tensor cores by every lane's proxy fence): lane 0 arrives on rank 0's
+    // barrier. The H chunk is this CTA's own shared memory, read by this SM's tensor core.
+    auto warp_signal = [&](uint32_t bar_cluster) {
+      __syncwarp();
+      if (lane == 0) mbar_arrive_remote(bar_cluster);
+    };
+    // a tile's biases: this thread's share, loaded from global memory one tile ahead, so that a
+    // tile's staging waits on no memory latency
+    constexpr int NV = (G_B12 + G_B3) / (32 * G_NE);
+    float vb[NV];
+    auto load_bias = [&](int pi) {
+      const float* wm = p.wmaster + (int64_t)__ldg(&p.pairs[pi / p.split]).x * p.pstride;
+#pragma unroll
+      for (int u = 0; u < NV; ++u) {
+        const int i = et + u * 32 * G_NE;
+        vb[u] = 0.f;
+        if (i < HID) vb[u] = wm[p.off_b1 + i];
+        else if (i < G_B12) vb[u] = wm[p.off_b2 + i - HID];
+        else if (i < G_B12 + p.x) vb[u] = wm[p.off_b3 + i - G_B12];
+      }
+    };
+    if (cid < n_parts) load_bias(cid);
+    bool row_ok = false;
+    bf16* dst = nullptr;  // this row of the fakes
+    GenSeq seq(cid, ncl, n_parts);
+    for (; seq.next(p, J); ++jobs) {
+      const int R = jobs & 1;
+      if (J.j == 0) {
+        // A tile's biases are staged with its first layer. The buffers' last users (hidden layers
+        // two tiles ago, output blocks three) have finished: every thread arrives here after its
+        // last output block of the tile two ago.
+        float* b12 = s_b12 + (J.t & 1) * G_B12;
+        float* b3 = s_b3 + J.t % 3 * G_B3;
+#pragma unroll
+        for (int u = 0; u < NV; ++u) {
+          const int i = et + u * 32 * G_NE;
+          if (i < G_B12) b12[i] = vb[u];
+          else b3[i - G_B12] = vb[u];
+        }
+        if (J.pi + ncl < n_parts) load_bias(J.pi + ncl);
+        mbar_arrive(bBias + 8 * (J.t & 1));
+        if (!mbar_wait_warp(bBias + 8 * (J.t & 1), (uint32_t)((J.t >> 1) & 1), abort_flag, p.err, 8))
+          break;
+      } else if (J.j == 2) {
+        const int4 pr = __ldg(&p.pairs[J.pi / p.split]);
+        const int gr = pr.y + (int)rank * BM + row;
+        row_ok = gr < pr.w;
+        if (row_ok) {
+          const int pp = gr / p.B, b = gr - pp * p.B;
+          const int2 cs = __ldg(&p.plist[pr.z + pp]);
+          dst = p.E + (int64_t)cs.x * p.e_cell + (int64_t)((1 + cs.y) * p.B + b) * p.x;
+        }
+      }
+      if (!mbar_wait_warp(bAcc + 8 * R, (uint32_t)((jobs >> 1) & 1), abort_flag, p.err, 6)) break;
+      tc_fence_after();
+      const uint32_t tbase = tmem + lane_base + (uint32_t)(R * HID);
+      if (J.j < 2) {
+        // chunk by chunk (64 columns; this warp's 16 of each), so that the next layer starts on
+        // chunk 0 while the others are written
+        const float* bias = s_b12 + (J.t & 1) * G_B12 + J.j * HID;
+        const uint32_t hb = (uint32_t)(J.t & 1);
+        constexpr int W = BK / G_CP;
+#pragma unroll 1
+        for (int ch = 0; ch < HID / BK; ++ch) {
+          const int col0 = ch * BK + part * W;
+          uint32_t r[W];
+          LIPZ_TMEM_LD16(tbase + col0, r);
+          tmem_wait_ld();
+          const float4* b4 = reinterpret_cast<const float4*>(bias + col0);
+          uint32_t pk[W / 2];
+#pragma unroll
+          for (int e = 0; e < W; e += 4) {
+            const float4 bb = b4[e >> 2];
+            float a0 = __uint_as_float(r[e]) + bb.x;
+            float a1 = __uint_as_float(r[e + 1]) + bb.y;
+            float a2 = __uint_as_float(r[e + 2]) + bb.z;
+            float a3 = __uint_as_float(r[e + 3]) + bb.w;
+            a0 = a0 > 0.f ? a0 : 0.f * a0;
+            a1 = a1 > 0.f ? a1 : 0.f * a1;
+            a2 = a2 > 0.f ? a2 : 0.f * a2;
+            a3 = a3 > 0.f ? a3 : 0.f * a3;
+            pk[e >> 1] = pack_bf16(a0, a1);
+            pk[(e >> 1) + 1] = pack_bf16(a2, a3);
+          }
+          const uint32_t chunk = sH + hb * H_BYTES + (uint32_t)(ch * H_CHUNK) + (uint32_t)row * 128u;
+#pragma unroll
+          for (int u = 0; u < W / 8; ++u) {
+            const uint32_t unit = (uint32_t)(part * (W / 8) + u);
+            const uint32_t addr = chunk + ((unit ^ (uint32_t)(row & 7)) << 4);
+            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(pk[4 * u]),
+                         "r"(pk[4 * u + 1]), "r"(pk[4 * u + 2]), "r"(pk[4 * u + 3])
+                         : "memory");
+          }
+          asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+          warp_signal(lH + 8 * (4 * hb + ch));
+        }
+      } else {
+        // output block: bias + tanh, bf16, into this row's fakes; this warp's share of the block's
+        // 16-column groups
+        const int brow0 = (J.nb0 + J.j - 2) * N3;
+        const float* bias = s_b3 + J.t % 3 * G_B3;
+        const int ng = job_n(J) / 16;
+        const int per = (ng + G_CP - 1) / G_CP;
+        const int g0 = part * per, g1 = min(ng, g0 + per);
+#pragma unroll 1
+        for (int gi = g0; gi < g1; ++gi) {
+          uint32_t r[16];
+          LIPZ_TMEM_LD16(tbase + gi * 16, r);
+          tmem_wait_ld();
+          const int col0 = brow0 + gi * 16;
+          const ulonglong2* b4 = reinterpret_cast<const ulonglong2*>(bias + col0);
+          uint32_t pk[8];
+#pragma unroll
+          for (int qq = 0; qq < 4; ++qq) {
+            const ulonglong2 t = b4[qq];
+            const float2 u = tanh_fast2(f2_add(
+                f2_pack(__uint_as_float(r[4 * qq]), __uint_as_float(r[4 * qq + 1])), t.x));
+            const float2 v = tanh_fast2(f2_add(
+                f2_pack(__uint_as_float(r[4 * qq + 2]), __uint_as_float(r[4 * qq + 3])), t.y));
+            pk[2 * qq] = pack_bf16(u.x, u.y);
+            pk[2 * qq + 1] = pack_bf16(v.x, v.y);
+          }
+          if (row_ok && col0 < p.x)  // one 256-bit store per row and 16 columns (E's rows,
+                                     // slots and cells are 32-byte aligned: x % 16 == 0)
+            st_global_v8(dst + col0, make_uint4(pk[0], pk[1], pk[2], pk[3]),
+                         make_uint4(pk[4], pk[5], pk[6], pk[7]));
+        }
+      }
+      tc_fence_before();
+      warp_signal(lReg + 8 * R);
+    }
+  } else {
+    // ================================ noise gather ================================
     // this CTA's 128 rows of the individual's z rows, 16-byte units in the 128-byte swizzle
     int zuse = 0;
     for (int pi = cid; pi < n_parts; pi += ncl, ++zuse) {
-      const int4 pr = __ldg(&p.pairs[pair_part<KND>(p, pi).pair]);
+      const int4 pr = __ldg(&p.pairs[pi / p.split]);
       if (zuse > 0 &&
           !mbar_wait_warp(bZempty, (uint32_t)((zuse - 1) & 1), abort_flag, p.err, 10))
         break;
@@ -1681,16 +1989,11 @@ TcPlan* tc_plan_create(const TcShape& s, const TcBuffers& b, std::string* msg) {
   p->ppdt = ppdt;
   const bool pairs_on = !env_flag("LIPZ_FWD_SINGLE");
   p->ncl_g = pairs_on && s.z == tc::BK
-                 ? max_pair_clusters(tc::k_mlp_fwd_pair<tc::KIND_G, false>, tc::pair_threads<tc::KIND_G>(),
-                                     tc::pair_smem_bytes<tc::KIND_G>())
+                 ? max_pair_clusters(tc::k_mlp_fwd_pair_g, tc::G_THREADS, tc::G_SMEM)
                  : 0;
   p->ncl_d = pairs_on && 6 * s.B < 65536
-                 ? std::min(max_pair_clusters(tc::k_mlp_fwd_pair<tc::KIND_D, false>,
-                                              tc::pair_threads<tc::KIND_D>(),
-                                              tc::pair_smem_bytes<tc::KIND_D>()),
-                            max_pair_clusters(tc::k_mlp_fwd_pair<tc::KIND_D, true>,
-                                              tc::pair_threads<tc::KIND_D>(),
-                                              tc::pair_smem_bytes<tc::KIND_D>()))
+                 ? std::min(max_pair_clusters(tc::k_mlp_fwd_pair<false>, tc::D_THREADS, tc::D_SMEM),
+                            max_pair_clusters(tc::k_mlp_fwd_pair<true>, tc::D_THREADS, tc::D_SMEM))
                  : 0;
   if (env_flag("LIPZ_VERBOSE"))
     fprintf(stderr, "lipz: tensor-core forward: %d SMs, CTA-pair clusters resident: generator %d, "
@@ -1729,23 +2032,20 @@ int launch_pair(TcPlan* p, PairKind kind, const tc::PParams& pq, cudaStream_t st
   const bool gen = kind == PAIR_G;
   const int ncl = gen ? p->ncl_g : p->ncl_d;
   // Small grids: a pair's output blocks in as many parts as there are idle clusters, each with the
-  // hidden layers of its own (784 outputs, four blocks; 1x1 cells, 2 pairs: 27 -> 21 us, 3x3, 18
-  // pairs: 29 -> 23). More parts than clusters would take a second round for less work each.
+  // hidden layers of its own (784 outputs, four blocks; 1x1 cells, 2 pairs: 27 -> 20 us, 3x3, 18
+  // pairs: 29 -> 22). More parts than clusters would take a second round for less work each.
   tc::PParams pp = pq;
   pp.split = gen ? std::max(1, std::min(pp.n3, ncl / std::max(1, pp.n_pairs))) : 1;
   const int parts = pp.n_pairs * pp.split, clusters = parts < ncl ? parts : ncl;
   if (clusters <= 0) return 0;
-  auto run = [&](auto kernel, int threads, size_t smem, const CUtensorMap& a, const CUtensorMap& b1,
-                 const CUtensorMap& b2, const CUtensorMap& b3) {
-    return launch_pairs(kernel, clusters, threads, smem, st, a, b1, b2, b3, p->mG1h, p->mG2h, pp);
+  auto run_d = [&](auto kernel) {
+    return launch_pairs(kernel, clusters, tc::D_THREADS, (size_t)tc::D_SMEM, st, p->mE, p->mD1h,
+                        p->mD2h, p->mZ, p->mG1h, p->mG2h, pp);
   };
-  constexpr int tg = tc::pair_threads<tc::KIND_G>(), td = tc::pair_threads<tc::KIND_D>();
-  constexpr size_t sg = tc::pair_smem_bytes<tc::KIND_G>(), sd = tc::pair_smem_bytes<tc::KIND_D>();
-  cudaError_t e =
-      gen ? run(tc::k_mlp_fwd_pair<tc::KIND_G, false>, tg, sg, p->mZ, p->mG1h, p->mG2h, p->mG3h)
-      : kind == PAIR_D
-          ? run(tc::k_mlp_fwd_pair<tc::KIND_D, false>, td, sd, p->mE, p->mD1h, p->mD2h, p->mZ)
-          : run(tc::k_mlp_fwd_pair<tc::KIND_D, true>, td, sd, p->mE, p->mD1h, p->mD2h, p->mZ);
+  cudaError_t e = gen ? launch_pairs(tc::k_mlp_fwd_pair_g, clusters, tc::G_THREADS,
+                                     (size_t)tc::G_SMEM, st, p->mG1h, p->mG2h, p->mG3h, pp)
+                  : kind == PAIR_D ? run_d(tc::k_mlp_fwd_pair<false>)
+                                   : run_d(tc::k_mlp_fwd_pair<true>);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) {
     cudaGetLastError();
