@@ -71,7 +71,10 @@ struct lipz_grid {
   cudaEvent_t ev_x2 = nullptr;
   const float* pre_host = nullptr;
   int pre_buf = -1;
-  int* hstat = nullptr;            // pinned host copies of the device error flags
+  // results and status words on their way to the host in one copy: [fG | fD | LG | LD | 8 words] at
+  // most, on the device and in pinned host memory
+  float* rstage = nullptr;
+  float* hres = nullptr;
   // lipz_iterate_batch_async: per call slot (alternating) a pinned copy of its iteration's
   // fitnesses and device status words (gathered on the device into `astage` first: one copy)
   // with the caller's result pointers, and an event at its end; per staging buffer an event
@@ -711,7 +714,9 @@ int create_impl(lipz_grid* g) {
   g->st = g->own_st;
   CK(g, cudaStreamCreateWithFlags(&g->copy_st, cudaStreamNonBlocking));
   CK(g, cudaEventCreateWithFlags(&g->ev_x, cudaEventDisableTiming));
-  CK(g, cudaMallocHost(&g->hstat, 8 * sizeof(int)));
+  const size_t res_words = (size_t)C * 60 + 8;
+  CK(g, cudaMallocHost(&g->hres, res_words * 4));
+  if ((rc = dalloc(g, &g->rstage, res_words * 4))) return rc;
   g->dcgan = g->a.kind == LIPZ_DCGAN64;
   make_layouts(g);
   g->e_cell = (int64_t)6 * B * x;
@@ -1316,18 +1321,56 @@ int deliver_pending(lipz_grid* g) {
   return LIPZ_OK;
 }
 
-int check_flag(lipz_grid* g) {
+// Waits for the stream and reports its status, with up to four device arrays (n 0: none) brought
+// along: one kernel gathers them and the status words, and one copy brings them to the host (a copy
+// of each, two arrays and seven flags, took about 20 us more).
+struct HostResult {
+  float* host;
+  const float* dev;
+  size_t n;
+};
+int finish(lipz_grid* g, const HostResult (&r)[4]) {
   // a pending pipelined call completes first; the flags read here cover its iteration too
-  int rc0 = deliver_pending(g);
-  if (rc0) return rc0;
+  int rc = deliver_pending(g);
+  if (rc) return rc;
   int* dev[8];
   flag_ptrs(g, dev);
-  for (int i = 0; i < 8; ++i) {
-    g->hstat[i] = i < 7 ? 0 : INT_MAX;
-    if (dev[i]) CK(g, cudaMemcpyAsync(&g->hstat[i], dev[i], 4, cudaMemcpyDeviceToHost, g->st));
+  StatusFlags fl;
+  for (int i = 0; i < 8; ++i) fl.p[i] = dev[i];
+  ResultArrays o{};
+  size_t n = 0;
+  for (int a = 0; a < 4; ++a) {
+    if (!r[a].host) continue;
+    // (a destination that is no host memory is left to the copy, which accepts or refuses it)
+    cudaPointerAttributes at;
+    if (cudaPointerGetAttributes(&at, r[a].host) != cudaSuccess) {
+      cudaGetLastError();
+    } else if (at.type == cudaMemoryTypeDevice) {
+      CK(g, cudaMemcpyAsync(r[a].host, r[a].dev, r[a].n * 4, cudaMemcpyDeviceToHost, g->st));
+      continue;
+    }
+    o.p[a] = r[a].dev;
+    o.n[a] = (int)r[a].n;
+    n += r[a].n;
   }
+  launch_gather_results(o, fl, g->rstage, true, g->st);
+  CKL(g);
+  CK(g, cudaMemcpyAsync(g->hres, g->rstage, (n + 8) * 4, cudaMemcpyDeviceToHost, g->st));
   CK(g, cudaStreamSynchronize(g->st));
-  return flag_status(g, dev, g->hstat);
+  const float* h = g->hres;
+  for (int a = 0; a < 4; ++a) {
+    if (o.n[a]) memcpy(r[a].host, h, o.n[a] * sizeof(float));
+    h += o.n[a];
+  }
+  return flag_status(g, dev, reinterpret_cast<const int*>(h));
+}
+
+int check_flag(lipz_grid* g) { return finish(g, {}); }
+
+// The fitnesses [cells][5] of the last evaluation, with its status.
+int finish_fitness(lipz_grid* g, float* fit_g, float* fit_d) {
+  const size_t n = (size_t)g->cells * 5;
+  return finish(g, {{fit_g, g->fG, n}, {fit_d, g->fD, n}, {}, {}});
 }
 
 float bf16_bits_to_float(uint16_t b) {
@@ -1440,7 +1483,7 @@ int lipz_grid_destroy(lipz_grid* g) {
   }
   if (g->ev_x) cudaEventDestroy(g->ev_x);
   if (g->ev_x2) cudaEventDestroy(g->ev_x2);
-  if (g->hstat) cudaFreeHost(g->hstat);
+  if (g->hres) cudaFreeHost(g->hres);
   if (g->hstat_a) cudaFreeHost(g->hstat_a);
   for (int i = 0; i < 2; ++i) {
     if (g->ev_it[i]) cudaEventDestroy(g->ev_it[i]);
@@ -1509,12 +1552,8 @@ int lipz_eval_neighborhoods(lipz_grid* g, float* fit_g, float* fit_d, float* pai
   if (rc) return rc;
   if (fit_g || fit_d || pair_lg || pair_ld) {
     const size_t C = g->cells;
-    if (fit_g) CK(g, cudaMemcpyAsync(fit_g, g->fG, C * 20, cudaMemcpyDeviceToHost, g->st));
-    if (fit_d) CK(g, cudaMemcpyAsync(fit_d, g->fD, C * 20, cudaMemcpyDeviceToHost, g->st));
-    if (pair_lg) CK(g, cudaMemcpyAsync(pair_lg, g->LG, C * 100, cudaMemcpyDeviceToHost, g->st));
-    if (pair_ld) CK(g, cudaMemcpyAsync(pair_ld, g->LD, C * 100, cudaMemcpyDeviceToHost, g->st));
-    CK(g, cudaStreamSynchronize(g->st));
-    return check_flag(g);
+    return finish(g, {{fit_g, g->fG, C * 5}, {fit_d, g->fD, C * 5}, {pair_lg, g->LG, C * 25},
+                      {pair_ld, g->LD, C * 25}});
   }
   return LIPZ_OK;
 }
@@ -1560,10 +1599,7 @@ int lipz_iterate_batch(lipz_grid* g, const float* x_host, float* fit_g, float* f
   CK(g, cudaEventRecord(g->ev_x, g->copy_st));
   int rc;
   if ((rc = eval_impl(g, g->xin, true, g->ev_x)) || (rc = train_impl(g))) return rc;
-  const size_t C = g->cells;
-  if (fit_g) CK(g, cudaMemcpyAsync(fit_g, g->fG, C * 20, cudaMemcpyDeviceToHost, g->st));
-  if (fit_d) CK(g, cudaMemcpyAsync(fit_d, g->fD, C * 20, cudaMemcpyDeviceToHost, g->st));
-  return check_flag(g);  // one stream synchronisation for the results and the flags
+  return finish_fitness(g, fit_g, fit_d);
 }
 
 int lipz_iterate_batch_next(lipz_grid* g, const float* x_host, const float* x_next,
@@ -1607,10 +1643,7 @@ int lipz_iterate_batch_next(lipz_grid* g, const float* x_host, const float* x_ne
     g->pre_host = nullptr;
     return rc;
   }
-  const size_t C = g->cells;
-  if (fit_g) CK(g, cudaMemcpyAsync(fit_g, g->fG, C * 20, cudaMemcpyDeviceToHost, g->st));
-  if (fit_d) CK(g, cudaMemcpyAsync(fit_d, g->fD, C * 20, cudaMemcpyDeviceToHost, g->st));
-  return check_flag(g);
+  return finish_fitness(g, fit_g, fit_d);
 }
 
 int lipz_iterate_batch_async(lipz_grid* g, const float* x_host, const float* x_next,
@@ -1668,7 +1701,7 @@ int lipz_iterate_batch_async(lipz_grid* g, const float* x_host, const float* x_n
   flag_ptrs(g, dev);
   StatusFlags fl;
   for (int i = 0; i < 8; ++i) fl.p[i] = dev[i];
-  launch_gather_status(g->fG, g->fD, (int)n5, fl, g->astage, true, g->st);
+  launch_gather_results({{g->fG, g->fD}, {(int)n5, (int)n5}}, fl, g->astage, true, g->st);
   CKL(g);
   float* hs = g->hstat_a + slot * stage_words;
   CK(g, cudaMemcpyAsync(hs, g->astage, stage_words * 4, cudaMemcpyDeviceToHost, g->st));

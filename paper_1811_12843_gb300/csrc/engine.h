@@ -88,8 +88,13 @@ void launch_colsum(const ColSumDesc* descs, int n_problems, int max_cols, cudaSt
 struct StatusFlags {
   const int* p[8];
 };
-void launch_gather_status(const float* fG, const float* fD, int n, const StatusFlags& fl,
-                          float* out, bool pdl, cudaStream_t st);
+// Up to four result arrays (n 0: none) that go to the host together.
+struct ResultArrays {
+  const float* p[4];
+  int n[4];
+};
+void launch_gather_results(const ResultArrays& o, const StatusFlags& fl, float* out, bool pdl,
+                           cudaStream_t st);
 // LG, LD and flag may be null together.
 void launch_fitness(const float* logits, int cells, int B, float* LG, float* LD, float* fG,
                     float* fD, int* flag, cudaStream_t st);

@@ -1156,24 +1156,30 @@ void launch_mix_es(const float* part, int nh, bool tri, int cells, int rows, int
              B, mix, S, score, seed, t, sigma);
 }
 
-// The iteration's results for one host copy: out[0, n) = fG, out[n, 2n) = fD (n = cells * 5),
-// then the eight status words (a null flag reads as its all-clear value: 0 for the first
-// seven, INT_MAX for the last).
-__global__ void k_gather_status(const float* __restrict__ fG, const float* __restrict__ fD, int n,
-                                StatusFlags fl, float* __restrict__ out) {
+// Results for one host copy: the arrays of o one after the other, then the eight status words (a
+// null flag reads as its all-clear value: 0 for the first seven, INT_MAX for the last).
+__global__ void __launch_bounds__(256) k_gather_results(ResultArrays o, StatusFlags fl,
+                                                        float* __restrict__ out) {
   pdl_wait();
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < 2 * n; i += gridDim.x * blockDim.x)
-    out[i] = i < n ? fG[i] : fD[i - n];
+  int base = 0;
+  for (int a = 0; a < 4; ++a) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < o.n[a]; i += gridDim.x * blockDim.x)
+      out[base + i] = o.p[a][i];
+    base += o.n[a];
+  }
   if (blockIdx.x == 0 && threadIdx.x < 8) {
     const int* f = fl.p[threadIdx.x];
-    reinterpret_cast<int*>(out + 2 * n)[threadIdx.x] =
+    reinterpret_cast<int*>(out + base)[threadIdx.x] =
         f ? *f : (threadIdx.x < 7 ? 0 : 0x7FFFFFFF);
   }
 }
 
-void launch_gather_status(const float* fG, const float* fD, int n, const StatusFlags& fl,
-                          float* out, bool pdl, cudaStream_t st) {
-  launch_kernel(pdl, k_gather_status, dim3(2), dim3(256), 0, st, fG, fD, n, fl, out);
+void launch_gather_results(const ResultArrays& o, const StatusFlags& fl, float* out, bool pdl,
+                           cudaStream_t st) {
+  int n = 1;
+  for (int a = 0; a < 4; ++a) n = o.n[a] > n ? o.n[a] : n;
+  const int blocks = (n + 255) / 256;
+  launch_kernel(pdl, k_gather_results, dim3(blocks < 32 ? blocks : 32), dim3(256), 0, st, o, fl, out);
 }
 
 }  // namespace lipz
