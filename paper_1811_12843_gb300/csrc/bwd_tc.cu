@@ -51,7 +51,7 @@ constexpr int CHUNK_BYTES = 3 * ADAM_ARRAY_BYTES + ADAM_WB_BYTES;      // 28 KB
 // barriers, the ring of claimed tiles and the TMEM slot
 constexpr int MISC_BYTES = 512;
 // Claimed tiles a CTA holds: the one in its epilogue and the next, whose operands load meanwhile.
-// (Four: the tiles claimed early by busy CTAs lengthen the tail, 386 against 382 us at 12x12.)
+// (Four: the tiles claimed early by busy CTAs lengthen the tail, 1 % at 12x12.)
 constexpr int RING = 2;
 constexpr int CHUNK_BUFS = 4;
 // Operand ring: 96 KB in stages of 16 KB of A and BN x 128 bytes of B, BN the grid's tile width
@@ -112,10 +112,10 @@ struct GParams {
 // its stores are written; the producer of a tile that reads it acquires the count before its loads.
 //
 // Bound: HBM on large grids (26 B per parameter through the chunk stream; 2.36 GB of DRAM traffic
-// at 12x12, B = 100: 382 us, 0.91 of the measured copy rate), the chain of five dependent tiles
-// on small ones (about 8 us each). One CTA per cell walking its own tiles took 422 us at 12x12
+// at 12x12, B = 100: 373 us, 0.93 of the measured copy rate), the chain of five dependent tiles
+// on small ones (about 7 us each). One CTA per cell walking its own tiles took 422 us at 12x12
 // (its delta tiles stopped its stream), and left most SMs idle on small grids: 307 us at 1x1
-// (now 41), 421 at 5x5, B = 256 (102). Cells 4 to 40 apart per level instead of all of them (a
+// (now 38), 421 at 5x5, B = 256 (99). Cells 4 to 40 apart per level instead of all of them (a
 // smaller window of activations) were slower: 400 to 535 us at 12x12.
 // ---------------------------------------------------------------------------------------------
 constexpr int MAX_STAGES = 10;
@@ -704,7 +704,8 @@ __global__ void __launch_bounds__(THREADS, 1)
   } else if (warp >= 2 + NUM_EPI_WARPS) {
     // ===== chunk stream: the epilogue's inputs of every chunk of every EPI_ADAM and EPI_DACT
     // tile, in tile order, into the four buffers in turn, and its results back out. A tiled TMA
-    // operation holds its issuing thread for about 0.2 us, so two warps share the work:
+    // operation holds its issuing warp for a time (0.2 us in a loop of one lane; all lanes and an
+    // elected issuer: 381 -> 373 us at 12x12), so two warps share the work:
     //   loader: a chunk's load, once the storer has released the chunk's buffer;
     //   storer: a chunk's stores once its epilogue half is done, then, when the stores have read
     //           the buffer, its release to the loader (releasing it one chunk later, to keep a
@@ -1008,9 +1009,9 @@ TcbPlan* tcb_plan_create(const TcbShape& s, const TcbBuffers& b, std::string* ms
   const bf16* Gw = b.Gwb;
   const bf16* Dw = b.Dwb;
   // Tiles of 128 columns: their operands leave three ring stages (256: two, and coarser tiles at
-  // the end of the list; 382 against 387 us at 12x12, 87 against 93 at 5x5). Where a cell's 42 or
-  // so weight tiles of 128 columns would leave SMs idle, 64 (41 against 45 us at 1x1; 447 against
-  // 382 at 12x12, four loads of A's 128 rows where 128 columns need two).
+  // the end of the list; 1 % slower at 12x12, 6 % at 5x5). Where a cell's 42 or
+  // so weight tiles of 128 columns would leave SMs idle, 64 (10 % faster at 1x1; 17 %
+  // slower at 12x12, four loads of A's 128 rows where 128 columns need two).
   const int bn = C * ((h / 128) * (2 * (h / 128) + (x + 127) / 128 + 1) + (x + 127) / 128 * 2) < sms
                      ? 64
                      : 128;

@@ -87,9 +87,10 @@ enum { AK_CONV = 0, AK_TRANS = 1, AK_SCATTER = 2, AK_NCHW = 3, AK_GATHER = 4,
 // tile's rows; rank 0 issues MMAs of 256 rows (two per chunk with m2) that read both halves, so
 // that a CTA's tensor core gets a 128 x 256 (m2: 256 x 128) chunk product from 32 (40) KB of
 // operands instead of 48. Bound: the tensor cores at nbox 256 (a 256 x 256 x 64 chunk in 640 to
-// 690 clocks, cuBLAS's rate; 850 before the MMA thread looked at the next stage early), shared
-// memory at nbox 128 (1,046: each MMA reads as many bytes of B as of A). Discriminator
-// evaluation of the 3x3 configuration 7.17 -> 6.55 ms; without pairs 6.65.
+// 690 clocks, cuBLAS's rate; 850 before the MMA warp looked at the next stage early), shared
+// memory at nbox 128 (each MMA reads as many bytes of B as of A). Discriminator evaluation of the
+// 3x3 configuration 7.17 -> 6.55 ms; without pairs 6.65; 4.81 with the first layer's own kernel,
+// every cell in one launch and converged issuing warps.
 constexpr bool conv_pair(int ak, int om) {
   return ak == AK_CONV ||
          (ak == AK_TRANS && (om == CTC_F32_HWC || om == CTC_DLRELU_HWC));
@@ -227,8 +228,8 @@ __global__ void __launch_bounds__(THREADS, conv_compact(AK) ? 2 : 1)
   if (warp == 0 || (kTma && (warp == 2 || warp == 3))) {
     // ---- TMA: the weights (warp 0, which also announces the stage's bytes) and, where A comes
     // by TMA, its first (warp 2) and second (m2: warp 3) 128 rows. A tiled TMA operation holds its
-    // issuing thread for 0.2 us and more, most of a chunk's time on the tensor cores, so each
-    // thread issues one per chunk.
+    // issuer for up to 0.2 us, most of a chunk's time on the tensor cores, so each warp issues one
+    // per chunk.
     if (warp < 3 || p.m2) {
       const bool elected = elect_one();
       int stage = 0, issued[STAGES] = {};
@@ -1158,10 +1159,12 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
     k1 = k0 + p.kc < Kp ? k0 + p.kc : Kp;
   };
   const bool tma = p.a_tma;
-  if (warp == 0 && tma) {
+  if (tma && (warp == 0 || (!BCHW && warp >= 2 && warp < 6))) {
     // a_tma: both operands by TMA, MN-major rows of 64 channels: A boxes of 64 pixels from the
-    // [problem][pixel][M] map, B boxes of the chunk's 64 A pixels mapped to b's pixels (s y - p
-    // + ky, s x - p + kx) by the 5-D map's traversal stride
+    // [problem][pixel][M] map (warp 0, which also announces the stage's bytes), B boxes of the
+    // chunk's 64 A pixels mapped to b's pixels (s y - p + ky, s x - p + kx) by the 5-D map's
+    // traversal stride (warps 2 to 5, 64 of the 256 columns each: one warp's six boxes a chunk took
+    // longer than its MMAs; the 3x3 configuration's D2-D4 and G2-G4 858 -> 569 us)
     {
       const bool elected = elect_one();
       int stage = 0, issued[WG_STAGES] = {};
@@ -1181,28 +1184,19 @@ __global__ void __launch_bounds__(WG_THREADS, 1)
           }
           const uint32_t full = bFull + 8 * stage;
           const uint32_t sA = base + stage * STAGE_BYTES, sB = sA + A_BYTES;
-          if (elected) {
+          if (elected && warp == 0) {
             mbar_expect_tx(full, (uint32_t)(BCHW ? A_BYTES : STAGE_BYTES));
             tma_load_3d(sA, &mA, full, mt * 128, (int)kb, prob);
             tma_load_3d(sA + 8192, &mA, full, mt * 128 + 64, (int)kb, prob);
           }
-          if constexpr (BCHW) {
-            issued[stage]++;
-            if (++stage == WG_STAGES) {
-              stage = 0;
-              phase ^= 1u;
-            }
-            continue;
-          }
-          const int nb = (int)(kb >> (2 * la));
-          const int ay0 = (int)((kb >> la) & (Ha - 1)), ax0 = (int)(kb & (Wa - 1));
-#pragma unroll
-          for (int atom = 0; atom < 4; ++atom) {
-            const int n0 = nt * 256 + atom * 64;
+          if (!BCHW && warp != 0) {
+            const int nb = (int)(kb >> (2 * la));
+            const int ay0 = (int)((kb >> la) & (Ha - 1)), ax0 = (int)(kb & (Wa - 1));
+            const int atom = warp - 2, n0 = nt * 256 + atom * 64;
             const int tap = n0 / p.Cb, c0 = n0 - tap * p.Cb;
             if (elected)
               tma_load_5d(sB + atom * 8192, &mB, full, c0, p.s * ax0 - p.p + (tap & 3),
-                        p.s * ay0 - p.p + (tap >> 2), nb, prob);
+                          p.s * ay0 - p.p + (tap >> 2), nb, prob);
           }
           issued[stage]++;
           if (++stage == WG_STAGES) {
