@@ -80,8 +80,9 @@ enum { LIPZ_STEP_STREAM_STRIDE = 256 };
  * product rounded to bfloat16 (nearest even), products accumulate in fp32; biases, logits,
  * losses, gradients and the Adam state (fp32 master weights, m, v) stay fp32.
  * LIPZ_FP32: everything fp32. Constraints: z_dim, hidden, x_dim, batch >= 1; hidden <= 1024;
- * tournament_size in 1..5; the tensor-core path additionally needs hidden == 256 and z_dim,
- * x_dim multiples of 16 (other shapes run on the CUDA-core kernels).
+ * tournament_size in 1..5. bf16 runs on the tensor cores: in chained kernels where hidden == 256
+ * and z_dim, x_dim are multiples of 16, in one grouped product per layer elsewhere; fp32 on the
+ * CUDA cores.
  */
 typedef struct lipz_arch {
   uint32_t struct_size;
@@ -102,7 +103,7 @@ typedef struct lipz_arch {
   float lr_mut_prob;       /* 0.5 */
   float leaky_slope;       /* 0.2 */
   int32_t keep_grads;      /* 1: keep the last train step's gradients for lipz_get_gradients */
-  int32_t force_simt;      /* 1: run the forward on the CUDA-core kernels even where the
+  int32_t force_simt;      /* 1: run an MLP on the CUDA-core kernels even where the
                               tensor-core kernels apply (for comparisons) */
   int32_t train_steps;     /* K >= 1 (default 1): Adam steps of each cell's new centre pair per
                               iteration. Step 0 uses the evaluation minibatch; step k >= 1
@@ -291,9 +292,9 @@ LIPZ_API int lipz_get_gradients(lipz_grid* g, float* grad_g, float* grad_d);
  * Per-phase device timing (tracing). Phases: LIPZ_PHASE_BATCH (minibatch draw), _G_FWD and
  * _D_FWD (evaluation forward of all generator / discriminator slots), _FITNESS (BCE losses and
  * fitness), _SELECT, _TRAIN_FWD (forward of the selected pairs and the logit deltas),
- * _TRAIN_BWD (their backward; on the tensor-core path one kernel, which also applies Adam to
- * the weight matrices unless arch.keep_grads is set), _ADAM (bias gradients, then the rest of
- * the update and replacement), _MIXTURE (with arch.mixture: the mixture step at the end of
+ * _TRAIN_BWD (their backward; in the chained tensor-core kernels one launch, which also applies
+ * Adam unless arch.keep_grads is set), _ADAM (where the backward does not: the update and
+ * replacement), _MIXTURE (with arch.mixture: the mixture step at the end of
  * an evaluation). While enabled, every phase is bracketed by CUDA events on
  * the grid's stream. lipz_profile_read waits for the stream and writes, per phase, the summed
  * device milliseconds (ms[n]), the number of phase executions (count[n]) and of kernel launches

@@ -111,8 +111,8 @@ struct GParams {
 // however few CTAs are resident. A delta tile that others read is counted in global memory once
 // its stores are written; the producer of a tile that reads it acquires the count before its loads.
 //
-// Bound: HBM on large grids (26 B per parameter through the chunk stream; 2.36 GB of DRAM traffic
-// at 12x12, B = 100: 373 us, 0.93 of the measured copy rate), the chain of five dependent tiles
+// Bound: HBM on large grids (26 B per parameter through the chunk stream; 2.32 GB in all at 12x12,
+// B = 100: 373 us, 0.92 of the measured copy rate), the chain of five dependent tiles
 // on small ones (about 7 us each). One CTA per cell walking its own tiles took 422 us at 12x12
 // (its delta tiles stopped its stream), and left most SMs idle on small grids: 307 us at 1x1
 // (now 38), 421 at 5x5, B = 256 (99). Cells 4 to 40 apart per level instead of all of them (a
