@@ -343,17 +343,16 @@ int make_set(lipz_grid* g, GemmSet* S, std::vector<GemmDesc> v) {
   static const double share[GEMM_N_TILES] = {2.5, 4, 6};
   double best = 0;
   if (tc) {
-    // Rounds of co-resident CTAs (two 128 x 128 or three 128 x 64 per SM), a round of the smaller
-    // weighted by its measured time. 128 x 128 against 128 x 64: 371 against 425 us for 2400 tiles
-    // of 128 x 128 (8 rounds against 11), 41 against 49 for 240 (1 against 2), 48.4 against 47.6
-    // for 270 (1 and 1), and five launches of 48 to 96 tiles (1 and 1) 74 against 54.
+    // Rounds of co-resident CTAs (two per SM), a round of the narrower tiles weighted by its measured
+    // time. 128 x 128 against 128 x 64: 475 against 633 us for 2400 tiles of 128 x 128 (8 rounds
+    // against 16), 47 against 56 for 240 (1 against 2), 58 against 66 for 270 (1 against 2), and five
+    // launches of 48 to 96 tiles (1 and 1) 77 against 55.
     for (int s = 0; s < GEMM_TC_N_TILES; ++s) {
       const GemmTile t = GEMM_TC_TILES[s];
       int64_t n = 0;
       for (const GemmDesc& d : v)
         n += (int64_t)((d.M + t.bm - 1) / t.bm) * ((d.N + t.bn - 1) / t.bn);
-      const int64_t slots = 152 * (t.bn == 128 ? 2 : 3);
-      const double cost = (double)((n + slots - 1) / slots) * (t.bn == 128 ? 1.0 : 0.8);
+      const double cost = (double)((n + 303) / 304) * (t.bn == 128 ? 1.0 : 0.8);
       if (s == 0 || cost < best) {
         best = cost;
         S->shape = s;

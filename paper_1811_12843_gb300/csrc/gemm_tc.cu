@@ -8,9 +8,9 @@
 // transposed products need no transposition. Three chunks of 64 k: two in flight while one is
 // multiplied.
 // Bound: the launch and the latency of a tile's chunks on small grids (11 us a launch), the staging's
-// L2 reads and instructions on large ones (320 TFLOP/s at 100 problems of 768 x 512 x 1000).
+// L2 reads and instructions on large ones (250 TFLOP/s at 100 problems of 768 x 512 x 1000).
 // Measured per phase against the CUDA-core kernel, 3x4 cells, 37 rows, 50 -> 200 -> 200 -> 500:
-// generators 82 -> 30 us, discriminators 210 -> 41, backward 157 -> 53.
+// generators 82 -> 34 us, discriminators 210 -> 46, backward 157 -> 55.
 #include "common.cuh"
 #include "engine.h"
 #include "tc_ptx.cuh"
@@ -128,7 +128,7 @@ struct TileLoader {
 };
 
 template <int BN>
-__global__ void __launch_bounds__(NT)
+__global__ void __launch_bounds__(NT, 2)
     k_gemm_tc(const GemmDesc* __restrict__ descs, const int2* __restrict__ tiles, float slope,
               int* err) {
   constexpr int STAGE = (BM + BN) * BK * 2;
@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(NT)
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32((const void*)tmem_slot)),
-                 "n"(BN));
+                 "n"(2 * BN));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   tc_fence_before();
@@ -189,7 +189,28 @@ __global__ void __launch_bounds__(NT)
   load(1);
   const int n = (min(BN, N - n0) + 63) & ~63;
   const uint32_t idesc = idesc_bf16_major(BM, n, la.kmaj ? 0 : 1, lb.kmaj ? 0 : 1);
+  // A chunk's sums stand in tensor memory (even and odd chunks apart) and are added to fp32 sums in
+  // registers, rounded to nearest: the tensor cores' own additions truncate, and over 784 k that is
+  // 12.3 x 2^-24 of the result (root mean square, normal operands) where one fp32 chain loses 3.5 and
+  // these sums 1.6 (64 k: 1.1, and the chain 0.9). It costs 7 to 20 % of the kernel's time.
+  constexpr int CW = BN / 2;  // columns of a thread: half of the tile's
+  const int q = warp & 3, half = warp >> 2;
   bool ok = true;
+  float acc[CW];
+#pragma unroll
+  for (int e = 0; e < CW; ++e) acc[e] = 0.f;
+  auto add_chunk = [&](int kc) {
+    tc_fence_after();
+    const uint32_t t = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)((kc & 1) * BN + half * CW);
+#pragma unroll
+    for (int c = 0; c < CW; c += 32) {
+      uint32_t r[32];
+      LIPZ_TMEM_LD32(t + c, r);
+      tmem_wait_ld();
+#pragma unroll
+      for (int e = 0; e < 32; ++e) acc[c + e] += __uint_as_float(r[e]);
+    }
+  };
   for (int kc = 0; kc < nk; ++kc) {
     asm volatile("cp.async.wait_group 1;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -200,53 +221,52 @@ __global__ void __launch_bounds__(NT)
       const uint32_t sA = base + (uint32_t)(kc % STAGES) * STAGE, sB = sA + BM * BK * 2;
       const int steps = min(BK / 16, (K - kc * BK + 15) / 16);
       for (int kk = 0; kk < steps; ++kk)
-        tc_mma(tmem, la.kmaj ? sw128_desc(sA + kk * 32) : sw128_mn_desc(sA + kk * 2048, BOX),
+        tc_mma(tmem + (uint32_t)(kc & 1) * BN,
+               la.kmaj ? sw128_desc(sA + kk * 32) : sw128_mn_desc(sA + kk * 2048, BOX),
                lb.kmaj ? sw128_desc(sB + kk * 32) : sw128_mn_desc(sB + kk * 2048, BOX), idesc,
-               (kc | kk) != 0 ? 1u : 0u);
+               kk != 0 ? 1u : 0u);
       tc_commit(bar + 8 * (kc % STAGES));
     }
-    // chunk kc + 2 goes where chunk kc - 1 was, once its MMAs have read it
-    if (kc > 0 && kc + 2 < nk)
-      ok = mbar_wait(bar + 8 * ((kc - 1) % STAGES), (uint32_t)(((kc - 1) / STAGES) & 1), abort_flag,
-                     err, 1) && ok;
     __syncwarp();
+    // chunk kc + 2 goes where chunk kc - 1 was, once its MMAs have read it
+    if (kc > 0)
+      ok = mbar_wait_warp(bar + 8 * ((kc - 1) % STAGES), (uint32_t)(((kc - 1) / STAGES) & 1),
+                          abort_flag, err, 1) && ok;
     load(kc + 2);
+    if (kc > 0) add_chunk(kc - 1);
   }
   // the last commit covers every MMA of the tile
-  ok = mbar_wait(bar + 8 * ((nk - 1) % STAGES), (uint32_t)(((nk - 1) / STAGES) & 1), abort_flag, err,
-                 2) && ok;
+  ok = mbar_wait_warp(bar + 8 * ((nk - 1) % STAGES), (uint32_t)(((nk - 1) / STAGES) & 1), abort_flag,
+                      err, 2) && ok;
+  add_chunk(nk - 1);
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   ok = __syncthreads_and(ok);
-  tc_fence_after();
   // 32 x 32 blocks of a warp's lane quarter, turned in shared memory so that a warp's global
   // accesses run along the rows
-  const int q = warp & 3;
   float* st = reinterpret_cast<float*>(gbase) + warp * 32 * EPI_LD;
   const int rows = min(32, M - m0 - q * 32);
-  for (int blk = warp >> 2; blk < BN / 32 && ok; blk += 2) {
-    const int col = n0 + blk * 32 + lane;
-    if (rows <= 0 || n0 + blk * 32 >= N) break;
-    uint32_t r[32];
-    LIPZ_TMEM_LD32(tmem + ((uint32_t)(q * 32) << 16) + blk * 32, r);
-    tmem_wait_ld();
 #pragma unroll
-    for (int e = 0; e < 32; ++e) st[lane * EPI_LD + e] = __uint_as_float(r[e]);
+  for (int c = 0; c < CW; c += 32) {
+    const int c0 = n0 + half * CW + c, col = c0 + lane;
+    if (!ok || rows <= 0 || c0 >= N) break;
+#pragma unroll
+    for (int e = 0; e < 32; ++e) st[lane * EPI_LD + e] = acc[c + e];
     __syncwarp();
     if (col < N) {
       const int64_t row0 = m0 + q * 32;
-      const int64_t c0 = row0 * d.scm + (int64_t)col * d.scn;
+      const int64_t o0 = row0 * d.scm + (int64_t)col * d.scn;
       if (d.epi == EPI_STORE) {
-        float* out = (float*)d.C + c0;
+        float* out = (float*)d.C + o0;
 #pragma unroll 8
         for (int i = 0; i < rows; ++i) out[i * d.scm] = st[i * EPI_LD + lane];
       } else if (d.epi == EPI_BIAS_ACT) {
-        bf16* out = (bf16*)d.C + c0;
+        bf16* out = (bf16*)d.C + o0;
         const float b = bias ? bias[col] : 0.f;
 #pragma unroll 4
         for (int i = 0; i < rows; ++i)
           out[i * d.scm] = __float2bfloat16(act_fwd(d.act, st[i * EPI_LD + lane] + b, slope));
       } else {
-        bf16* out = (bf16*)d.C + c0;
+        bf16* out = (bf16*)d.C + o0;
         const bf16* aux = (const bf16*)d.aux + row0 * d.sxm + (int64_t)col * d.sxn;
         for (int i0 = 0; i0 < rows; i0 += 8) {
           float a[8];
@@ -267,7 +287,8 @@ __global__ void __launch_bounds__(NT)
   __syncthreads();
   tc_fence_after();
   if (warp == 1)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(BN));
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
+                 "n"(2 * BN));
 }
 
 template <int BN>
