@@ -8,9 +8,9 @@
 // transposed products need no transposition. Three chunks of 64 k: two in flight while one is
 // multiplied.
 // Bound: the launch and the latency of a tile's chunks on small grids (11 us a launch), the staging's
-// L2 reads and instructions on large ones (250 TFLOP/s at 100 problems of 768 x 512 x 1000).
+// L2 reads and instructions on large ones (270 TFLOP/s at 100 problems of 768 x 512 x 1000).
 // Measured per phase against the CUDA-core kernel, 3x4 cells, 37 rows, 50 -> 200 -> 200 -> 500:
-// generators 82 -> 34 us, discriminators 210 -> 46, backward 157 -> 55.
+// generators 82 -> 33 us, discriminators 210 -> 45, backward 157 -> 52.
 #include "common.cuh"
 #include "engine.h"
 #include "tc_ptx.cuh"
@@ -195,6 +195,7 @@ __global__ void __launch_bounds__(NT, 2)
   // these sums 1.6 (64 k: 1.1, and the chain 0.9). It costs 7 to 20 % of the kernel's time.
   constexpr int CW = BN / 2;  // columns of a thread: half of the tile's
   const int q = warp & 3, half = warp >> 2;
+  const bool elected = elect_one();
   bool ok = true;
   float acc[CW];
 #pragma unroll
@@ -216,16 +217,22 @@ __global__ void __launch_bounds__(NT, 2)
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     tc_fence_before();
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (warp == 0) {
       tc_fence_after();
       const uint32_t sA = base + (uint32_t)(kc % STAGES) * STAGE, sB = sA + BM * BK * 2;
       const int steps = min(BK / 16, (K - kc * BK + 15) / 16);
-      for (int kk = 0; kk < steps; ++kk)
-        tc_mma(tmem + (uint32_t)(kc & 1) * BN,
-               la.kmaj ? sw128_desc(sA + kk * 32) : sw128_mn_desc(sA + kk * 2048, BOX),
-               lb.kmaj ? sw128_desc(sB + kk * 32) : sw128_mn_desc(sB + kk * 2048, BOX), idesc,
-               kk != 0 ? 1u : 0u);
-      tc_commit(bar + 8 * (kc % STAGES));
+      // (a step of 16 k further on: 32 bytes K-major, 2048 MN-major; 16-byte units)
+      const uint64_t dA = la.kmaj ? sw128_desc(sA) : sw128_mn_desc(sA, BOX);
+      const uint64_t dB = lb.kmaj ? sw128_desc(sB) : sw128_mn_desc(sB, BOX);
+      const uint32_t iA = la.kmaj ? 2 : 128, iB = lb.kmaj ? 2 : 128;
+      const uint32_t dt = tmem + (uint32_t)(kc & 1) * BN;
+      if (elected) {
+        tc_mma(dt, dA, dB, idesc, 0u);
+#pragma unroll
+        for (int kk = 1; kk < BK / 16; ++kk)
+          if (kk < steps) tc_mma_acc(dt, dA + kk * iA, dB + kk * iB, idesc);
+        tc_commit(bar + 8 * (kc % STAGES));
+      }
     }
     __syncwarp();
     // chunk kc + 2 goes where chunk kc - 1 was, once its MMAs have read it
