@@ -89,10 +89,11 @@ struct GParams {
   // x_slot (non-null) a 4-D map {n, rows, slots, cells}, slot 1 + x_slot[cell]
   int x_row0;
   const int* x_slot;
-  // split K (ksplit > 0): chunks [0, ksplit) read K rows kc * 64 of A and of B's slot 0;
-  // chunks [ksplit, kchunks) read K rows (kc - ksplit) * 64 of A shifted by a_k_off1 and of B's
-  // slot 1 + b_slot_sel[cell]; B is then a 4-D map {n, K rows, slots, cells}
-  int ksplit, a_k_off1;
+  // split K (ksplit > 0): chunks [0, ksplit) read K rows kc * 64 of A's part 0 and of B's slot 0;
+  // chunks [ksplit, kchunks) read K rows (kc - ksplit) * 64 of A's part 1 and of B's slot
+  // 1 + b_slot_sel[cell]. Both maps are 4-D, {m or n, K rows, parts or slots, cells}, so that rows
+  // past a part read as zero in both (A's next part belongs to a stage that may still be writing)
+  int ksplit;
   const int* b_slot_sel;
   // EPI_DACT: column sums of the fp32 deltas over the 32 rows q of row tile i go to
   // bias_part[cell * bias_cell + (4 i + q) * N + n] (together a bias gradient); null = none
@@ -582,10 +583,13 @@ __global__ void __launch_bounds__(THREADS, 1)
         int m0, n0, n;
         stage_tile(p, t, m0, n0, n);
         auto load_a = [&](int kc, int st) {
-          const bool part1 = p.ksplit > 0 && kc >= p.ksplit;
-          const int ka = (part1 ? kc - p.ksplit : kc) * BK + (part1 ? p.a_k_off1 : 0);
+          const int ka = kc * BK;
           const uint32_t sA = base + st * op_bytes, full = bFull + 8 * st;
           if (!elected) {
+          } else if (p.ksplit > 0) {
+            const int part = kc >= p.ksplit, kp = ka - part * p.ksplit * BK;
+            tma_load_4d(sA, mA, full, m0, kp, part, za);
+            tma_load_4d(sA + MN_BOX_BYTES, mA, full, m0 + 64, kp, part, za);
           } else if (p.a_mn) {
             tma_load_3d(sA, mA, full, m0, ka, za);
             tma_load_3d(sA + MN_BOX_BYTES, mA, full, m0 + 64, ka, za);
@@ -923,7 +927,8 @@ bool map3b_rows(CUtensorMap* m, const bf16* base, uint64_t inner, uint64_t rows,
   return true;
 }
 
-// bf16 4-D map {inner, rows, slots, depth} (E seen as [cells][6][B][x]); box {64, 64, 1, 1},
+// bf16 4-D map {inner, rows, slots, depth} (E seen as [cells][6][B][x], the D-loss rows of D1 as
+// [cells][2][B][h]); box {64, 64, 1, 1},
 // 128-byte swizzle: rows past `rows` within a slot read as zero.
 bool map4(CUtensorMap* m, const void* base, uint64_t inner, uint64_t rows, uint64_t slots,
           uint64_t depth, uint64_t slot_elems, uint64_t depth_elems, std::string* msg) {
@@ -1083,7 +1088,8 @@ TcbPlan* tcb_plan_create(const TcbShape& s, const TcbBuffers& b, std::string* ms
     ok = ok && map3(&P->maps.in[si], X, P->cells.st[si].p.N, rows, C, cell, 64, msg);
   };
   // weight gradient dW[o][i] = sum_r A[r][o] Bm[r][i] (both read MN-major) of the tensor at `off`
-  // of a population: the Adam step in the epilogue, or the gradient stored
+  // of a population: the Adam step in the epilogue, or the gradient stored. A's rows: a_rows per
+  // cell, with split K a_rows per part
   auto weight = [&](int si, const void* A, int a_rows, int64_t a_cell, const TcbBuffers::AdamPop& ap,
                     const int* src, int64_t off, int64_t Ps, float* grad) {
     tcb::GParams& q = P->cells.st[si].p;
@@ -1091,7 +1097,9 @@ TcbPlan* tcb_plan_create(const TcbShape& s, const TcbBuffers& b, std::string* ms
     q.epi = tcb::EPI_F32;
     q.C = grad + off;
     q.c_cell = Ps;
-    ok = ok && map3(&P->maps.a[si], A, q.M, a_rows, C, a_cell, 64, msg);
+    ok = ok && (q.ksplit > 0 ? map4(&P->maps.a[si], A, q.M, a_rows, 2, C, (int64_t)a_rows * q.M,
+                                    a_cell, msg)
+                             : map3(&P->maps.a[si], A, q.M, a_rows, C, a_cell, 64, msg));
     if (!b.fuse_adam) return;
     // w, m, v are one allocation in three equal parts: the part size is the 4th dimension's
     // stride, the same for the old and the new snapshot
@@ -1143,8 +1151,7 @@ TcbPlan* tcb_plan_create(const TcbShape& s, const TcbBuffers& b, std::string* ms
         b.goff[1]);
   aux3(S_A1, b.TH1, B, Bh, 0);
   // dW2d = J2^T TG1 and dW1d = D1^T X over the 2B D-loss rows. X = [E[c] rows 0..B-1 (real); E[c]
-  // fake rows of slot sel_g[c]] is read in place: K splits into the two B-row parts (rows past B
-  // in a part read as zero), D1 rows shifted by B in the second part
+  // fake rows of slot sel_g[c]] is read in place: K splits into the two B-row parts of X and of D1
   stage(S_DW2D, h, h, 2 * B, bn);
   weight(S_DW2D, b.J2, 3 * B, 3 * Bh, b.adam_d, b.src_d, b.doff[2], b.PDs, b.gD);
   act3(S_DW2D, b.TG1, 2 * B, 2 * Bh);
@@ -1152,10 +1159,9 @@ TcbPlan* tcb_plan_create(const TcbShape& s, const TcbBuffers& b, std::string* ms
     tcb::GParams& q = stage(S_DW1D, h, x, 2 * B, bn);
     q.ksplit = (B + 63) / 64;
     q.kchunks = 2 * q.ksplit;
-    q.a_k_off1 = B;
     q.b_slot_sel = b.sel_g;
   }
-  weight(S_DW1D, b.D1, 3 * B, 3 * Bh, b.adam_d, b.src_d, b.doff[0], b.PDs, b.gD);
+  weight(S_DW1D, b.D1, B, 3 * Bh, b.adam_d, b.src_d, b.doff[0], b.PDs, b.gD);
   ok = ok && map4(&P->maps.b[S_DW1D], b.E, x, B, 6, C, Bx, b.e_cell, msg);
   // dW3g = A3^T TH2, dW2g = A2^T TH1, dW1g = A1^T Z
   stage(S_DW3G, x, h, B, bn);

@@ -1,6 +1,7 @@
 """The tensor-core backward's tile list: batches at the edges of its 128-row tiles and 64-row K
 chunks, output widths that end inside a tile or a 64-column box, grids on both sides of its tile
-width rule (64 columns up to three cells, 128 beyond) and one with more cells than SMs."""
+width rule (64 columns up to three cells, 128 beyond) and one with more cells than SMs; and a first
+step on memory that holds NaN."""
 
 import numpy as np
 import pytest
@@ -35,3 +36,25 @@ def test_fused_adam_equals_stored_gradients_and_repeats(L, rows, cols, batch, x)
         sa = np.frombuffer(a.export_state(), np.uint8)
         assert np.array_equal(sa, np.frombuffer(b.export_state(), np.uint8)), it
         assert np.array_equal(sa, np.frombuffer(c.export_state(), np.uint8)), it
+
+
+@pytest.mark.parametrize("rows,cols,batch", [(1, 1, 1), (1, 1, 31), (1, 1, 100), (3, 3, 100),
+                                             (5, 5, 65), (12, 12, 100)])
+def test_first_step_reads_nothing_unwritten(L, rows, cols, batch):  # noqa: F811
+    """The first step of a grid whose buffers come from memory full of NaN equals that of a grid on
+    memory full of zeros: no tile reads a row that its own dependencies have not written, not even
+    against the zeros past a batch that is no multiple of the 64-row K chunk."""
+    import torch
+    pool = _pool(9, 500, 784)
+    states = []
+    for byte in (0xFF, 0x00):
+        junk = [torch.full((1 << 28,), byte, dtype=torch.uint8, device="cuda") for _ in range(16)]
+        torch.cuda.synchronize()
+        del junk
+        torch.cuda.empty_cache()
+        g = _grid(L, rows, cols, 3, pool, precision="bf16", batch=batch)
+        g.iterate(1)
+        states.append(np.frombuffer(g.export_state(), np.uint8))
+        g.close()
+    assert np.all(np.isfinite(states[0][64:].view(np.float32)))
+    assert np.array_equal(states[0], states[1])
