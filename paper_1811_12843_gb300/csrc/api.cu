@@ -613,8 +613,11 @@ int build_descs(lipz_grid* g, int p) {
   return upload(g, &D.cb, cb);
 }
 
-// Status word of the tensor-core grouped GEMM (a DCGAN's engine shares its own).
-int* gemm_error_flag(lipz_grid* g) { return g->dc ? dc_error_flag(g->dc) : g->gemm_err; }
+// Status word of the tensor-core grouped GEMM: a DCGAN's tensor-core engine shares its own.
+int* gemm_error_flag(const lipz_grid* g) {
+  int* dc = g->dc ? dc_error_flag(g->dc) : nullptr;
+  return dc ? dc : g->gemm_err;
+}
 
 void gemm(lipz_grid* g, const GemmSet& S) {
   if (g->bf && !g->a.force_simt)
@@ -774,7 +777,8 @@ int create_impl(lipz_grid* g) {
     }
   }
   const int big = INT_MAX;
-  if (g->bf && !g->dcgan && !g->a.force_simt &&
+  // (a DCGAN runs the grouped GEMM too, for the mixture)
+  if (g->bf && !g->a.force_simt &&
       ((rc = dalloc(g, &g->gemm_err, 4)) || (rc = dset(g, g->gemm_err, 0, 4))))
     return rc;
   if ((rc = dset(g, g->gG, 0, (size_t)C * g->PGs * 4)) ||
@@ -1281,7 +1285,7 @@ void flag_ptrs(lipz_grid* g, int* (&dev)[8]) {
                g->tcb[0] ? tcb_error_flag(g->tcb[0]) : nullptr,
                g->tcb[1] ? tcb_error_flag(g->tcb[1]) : nullptr,
                g->tcb[2] ? tcb_error_flag(g->tcb[2]) : nullptr,
-               g->dc ? dc_error_flag(g->dc) : nullptr, g->flag};
+               gemm_error_flag(g), g->flag};
   for (int i = 0; i < 8; ++i) dev[i] = d[i];
 }
 
