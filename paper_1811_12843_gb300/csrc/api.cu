@@ -35,6 +35,7 @@ struct GemmSet {
   GemmDesc* d = nullptr;
   int2* t = nullptr;
   int n = 0, shape = 0;
+  bool tc = false;  // k_gemm_tc, else k_gemm
 };
 
 struct Descs {
@@ -43,8 +44,9 @@ struct Descs {
   GemmSet g1, g2, g3, d1, d2;
   GemvDesc* d3;
   // training (per parity): the discriminator's forward of later minibatch steps, and the backward
-  // in launches of independent products: {dW2d, D1}, {dW1d, A3}, {dW3g, A2}, {dW2g, A1}, {dW1g}
-  GemmSet td1, td2, bw[5];
+  // in launches of independent products: {dW2d, D1}, {dW1d, A3}, {dW3g, A2}, {dW2g, A1}, then
+  // {dW1g} and the gradients that another kernel forms than the deltas of their launch
+  GemmSet td1, td2, bw[6];
   GemvDesc* tgv;
   ColSumDesc* cb;  // bias gradients of every cell (D's b2 comes from k_dlogit)
 };
@@ -310,11 +312,17 @@ int upload(lipz_grid* g, T** dst, const std::vector<T>& v) {
   return h2d(g, *dst, v.data(), v.size() * sizeof(T));
 }
 
-// One grouped-GEMM launch of the problems v (the longest sums first, so that the last blocks to
-// start are short ones).
+// Whether a product runs on the tensor cores.
+bool gemm_on_tc(const lipz_grid* g, const GemmDesc& d) {
+  return g->bf && !g->a.force_simt &&
+         d.K >= (d.epi == EPI_STORE ? GEMM_TC_MIN_K_STORE : GEMM_TC_MIN_K);
+}
+
+// One grouped-GEMM launch of the problems v, all of one kernel (the longest sums first, so that the
+// last blocks to start are short ones).
 int make_set(lipz_grid* g, GemmSet* S, std::vector<GemmDesc> v) {
   const int es = (int)g->esz;
-  const bool tc = g->bf && !g->a.force_simt;
+  const bool tc = S->tc = !v.empty() && gemm_on_tc(g, v[0]);
   auto vec = [&](const void* p, int64_t unit, int64_t other, int n_unit, const GemmDesc& d, int op) {
     return unit == 1 && other % 4 == 0 && n_unit % 4 == 0 && (uintptr_t)p % (4 * es) == 0 &&
            (!d.wsel || d.wsel_op != op || d.wsel_stride % 4 == 0);
@@ -498,7 +506,7 @@ int build_descs(lipz_grid* g, int p) {
   int rc;
 
   // ---- training descriptors: weights of the selected individual (wsel = src_g / src_d)
-  std::vector<GemmDesc> td1, td2, bw[5];
+  std::vector<GemmDesc> td1, td2, bw[5];  // bw: as Descs::bw, dW1g in the last
   std::vector<GemvDesc> tgv;
   std::vector<ColSumDesc> cb;
   auto selg = [&](GemmDesc d, int c) {
@@ -608,8 +616,17 @@ int build_descs(lipz_grid* g, int p) {
       ((rc = make_set(g, &D.td1, td1)) || (rc = make_set(g, &D.td2, td2)) ||
        (rc = upload(g, &D.tgv, tgv))))
     return rc;
-  for (int k = 0; k < 5; ++k)
-    if ((rc = make_set(g, &D.bw[k], bw[k]))) return rc;
+  std::vector<GemmDesc> last[2];  // by kernel
+  for (int k = 0; k < 5; ++k) {
+    // (a cell's delta products come last in bw[0 .. 3]; the last launches hold gradients only)
+    const bool tc = gemm_on_tc(g, bw[k].back());
+    std::vector<GemmDesc> v;
+    for (const GemmDesc& d : bw[k])
+      (k < 4 && gemm_on_tc(g, d) == tc ? v : last[gemm_on_tc(g, d)]).push_back(d);
+    if (k < 4 && (rc = make_set(g, &D.bw[k], v))) return rc;
+  }
+  for (int k = 0; k < 2; ++k)
+    if (!last[k].empty() && (rc = make_set(g, &D.bw[4 + k], last[k]))) return rc;
   return upload(g, &D.cb, cb);
 }
 
@@ -620,7 +637,7 @@ int* gemm_error_flag(const lipz_grid* g) {
 }
 
 void gemm(lipz_grid* g, const GemmSet& S) {
-  if (g->bf && !g->a.force_simt)
+  if (S.tc)
     launch_gemm_tc(S.d, S.t, S.n, S.shape, g->a.leaky_slope, gemm_error_flag(g), g->st);
   else if (g->bf) launch_gemm<bf16>(S.d, S.t, S.n, S.shape, g->a.leaky_slope, g->st);
   else launch_gemm<float>(S.d, S.t, S.n, S.shape, g->a.leaky_slope, g->st);
@@ -1217,7 +1234,9 @@ int train_once(lipz_grid* g, bool evaluated) {
     for (const GemmSet& S : D.bw) gemm(g, S);
     colsum(g, D.cb, 4 * C, h > x ? h : x);
     CKL(g);
-    phase_end(g, LIPZ_PHASE_TRAIN_BWD, 6);
+    int n_bwd = 1;
+    for (const GemmSet& S : D.bw) n_bwd += S.n > 0;
+    phase_end(g, LIPZ_PHASE_TRAIN_BWD, n_bwd);
     phase_begin(g, LIPZ_PHASE_ADAM);
   }
   // Adam + replacement into the other snapshot (after the bias sums on the tensor-core path)

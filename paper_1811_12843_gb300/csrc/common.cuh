@@ -180,6 +180,10 @@ constexpr int GEMM_N_TILES = 3;
 // Those of the tensor-core one.
 constexpr GemmTile GEMM_TC_TILES[] = {{128, 128}, {128, 64}};
 constexpr int GEMM_TC_N_TILES = 2;
+// The shortest sums that it takes, in a forward or delta product and in a weight gradient (EPI_STORE),
+// and the shortest that it forms in whole chunks of 64 k: below, its error would be larger than that of
+// k_gemm's fp32 chain (the figures stand in k_gemm_tc).
+constexpr int GEMM_TC_MIN_K = 48, GEMM_TC_MIN_K_STORE = 64, GEMM_TC_CHUNK_K = 160;
 
 // Column sums: out[n] = sum_{r < rows} X[r * ld + n], n < cols (bias gradients).
 struct ColSumDesc {

@@ -10,7 +10,10 @@
 // Bound: the launch and the latency of a tile's chunks on small grids (11 us a launch), the staging's
 // L2 reads and instructions on large ones (270 TFLOP/s at 100 problems of 768 x 512 x 1000).
 // Measured per phase against the CUDA-core kernel, 3x4 cells, 37 rows, 50 -> 200 -> 200 -> 500:
-// generators 82 -> 33 us, discriminators 210 -> 45, backward 157 -> 52.
+// generators 82 -> 35 us, discriminators 210 -> 45, backward 157 -> 67 (52 with the generator's weight
+// gradients, over 37 rows, here too).
+#include <type_traits>
+
 #include "common.cuh"
 #include "engine.h"
 #include "tc_ptx.cuh"
@@ -135,13 +138,14 @@ __global__ void __launch_bounds__(NT, 2)
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw), base = (raw + 1023u) & ~1023u;
   uint8_t* gbase = smem_raw + (base - raw);
-  uint64_t* bars = reinterpret_cast<uint64_t*>(gbase + STAGES * STAGE);  // [STAGES]: stage read
+  uint64_t* bars = reinterpret_cast<uint64_t*>(gbase + STAGES * STAGE);  // [2]: a sum's MMAs done
   const uint32_t bar = smem_u32(bars);
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(gbase + STAGES * STAGE + 64);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(gbase + STAGES * STAGE + 68);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) mbar_init(bar + 8 * s, 1);
+    mbar_init(bar, 1);
+    mbar_init(bar + 8, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -189,10 +193,16 @@ __global__ void __launch_bounds__(NT, 2)
   load(1);
   const int n = (min(BN, N - n0) + 63) & ~63;
   const uint32_t idesc = idesc_bf16_major(BM, n, la.kmaj ? 0 : 1, lb.kmaj ? 0 : 1);
-  // A chunk's sums stand in tensor memory (even and odd chunks apart) and are added to fp32 sums in
-  // registers, rounded to nearest: the tensor cores' own additions truncate, and over 784 k that is
-  // 12.3 x 2^-24 of the result (root mean square, normal operands) where one fp32 chain loses 3.5 and
-  // these sums 1.6 (64 k: 1.1, and the chain 0.9). It costs 7 to 20 % of the kernel's time.
+  // A chunk's sums stand in tensor memory (even and odd ones apart) and are added to fp32 sums in
+  // registers, rounded to nearest: the tensor cores' own additions truncate. That costs 7 to 20 % of
+  // the kernel's time with chunks of 64 k; where fewer additions follow, K below GEMM_TC_CHUNK_K, every
+  // MMA step of 16 k is a sum of its own. Error against 64 bits, in 2^-24 of the result's root mean
+  // square, as one sum in tensor memory, by chunks of 64, of 16, and of an fp32 FMA chain (in brackets
+  // for operands that are half zeros, as a weight gradient's are): 784 k 12.3, 1.56, 2.11 and 3.19;
+  // 160 k by 64 1.19 (0.657), chain 1.37 (0.667); 144 k by 16 1.00 (0.595), chain 1.28 (0.638); 64 k
+  // 0.97, 0.97, 0.74 (0.396) and 0.87 (0.398). 48 k by 16 0.66 (0.332), chain 0.73 (0.324): weight
+  // gradients over fewer than GEMM_TC_MIN_K_STORE rows go to k_gemm, and so do other products over
+  // fewer than GEMM_TC_MIN_K (16 k 0.43 and 0.38).
   constexpr int CW = BN / 2;  // columns of a thread: half of the tile's
   const int q = warp & 3, half = warp >> 2;
   const bool elected = elect_one();
@@ -200,9 +210,9 @@ __global__ void __launch_bounds__(NT, 2)
   float acc[CW];
 #pragma unroll
   for (int e = 0; e < CW; ++e) acc[e] = 0.f;
-  auto add_chunk = [&](int kc) {
+  auto add_sum = [&](int i) {
     tc_fence_after();
-    const uint32_t t = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)((kc & 1) * BN + half * CW);
+    const uint32_t t = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)((i & 1) * BN + half * CW);
 #pragma unroll
     for (int c = 0; c < CW; c += 32) {
       uint32_t r[32];
@@ -212,40 +222,51 @@ __global__ void __launch_bounds__(NT, 2)
       for (int e = 0; e < 32; ++e) acc[c + e] += __uint_as_float(r[e]);
     }
   };
-  for (int kc = 0; kc < nk; ++kc) {
-    asm volatile("cp.async.wait_group 1;" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 0) {
-      tc_fence_after();
-      const uint32_t sA = base + (uint32_t)(kc % STAGES) * STAGE, sB = sA + BM * BK * 2;
-      const int steps = min(BK / 16, (K - kc * BK + 15) / 16);
-      // (a step of 16 k further on: 32 bytes K-major, 2048 MN-major; 16-byte units)
-      const uint64_t dA = la.kmaj ? sw128_desc(sA) : sw128_mn_desc(sA, BOX);
-      const uint64_t dB = lb.kmaj ? sw128_desc(sB) : sw128_mn_desc(sB, BOX);
-      const uint32_t iA = la.kmaj ? 2 : 128, iB = lb.kmaj ? 2 : 128;
-      const uint32_t dt = tmem + (uint32_t)(kc & 1) * BN;
-      if (elected) {
-        tc_mma(dt, dA, dB, idesc, 0u);
-#pragma unroll
-        for (int kk = 1; kk < BK / 16; ++kk)
-          if (kk < steps) tc_mma_acc(dt, dA + kk * iA, dB + kk * iB, idesc);
-        tc_commit(bar + 8 * (kc % STAGES));
+  // the sums of `per` MMA steps
+  auto product = [&](auto per_c) {
+    constexpr int per = decltype(per_c)::value;
+    const int steps = (K + 15) / 16, sums = (steps + per - 1) / per;
+    for (int i = 0; i < sums; ++i) {
+      const int s0 = i * per, kc = s0 / (BK / 16), k0 = s0 % (BK / 16);  // first step; in its chunk
+      if (k0 == 0) {
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       }
+      // (and every warp has read the sum before the last, whose place this one takes)
+      tc_fence_before();
+      __syncthreads();
+      if (warp == 0) {
+        tc_fence_after();
+        const uint32_t sA = base + (uint32_t)(kc % STAGES) * STAGE, sB = sA + BM * BK * 2;
+        // (a step of 16 k further on: 32 bytes K-major, 2048 MN-major; 16-byte units)
+        const uint32_t iA = la.kmaj ? 2 : 128, iB = lb.kmaj ? 2 : 128;
+        const uint64_t dA = (la.kmaj ? sw128_desc(sA) : sw128_mn_desc(sA, BOX)) + k0 * iA;
+        const uint64_t dB = (lb.kmaj ? sw128_desc(sB) : sw128_mn_desc(sB, BOX)) + k0 * iB;
+        const uint32_t dt = tmem + (uint32_t)(i & 1) * BN;
+        const int n_mma = min(per, steps - s0);
+        if (elected) {
+          tc_mma(dt, dA, dB, idesc, 0u);
+#pragma unroll
+          for (int kk = 1; kk < BK / 16; ++kk)
+            if (kk < n_mma) tc_mma_acc(dt, dA + kk * iA, dB + kk * iB, idesc);
+          tc_commit(bar + 8 * (i & 1));
+        }
+      }
+      __syncwarp();
+      if (i > 0)
+        ok = mbar_wait_warp(bar + 8 * ((i - 1) & 1), (uint32_t)(((i - 1) >> 1) & 1), abort_flag, err,
+                            1) && ok;
+      // chunk kc + 2 goes where chunk kc - 1 was, whose MMAs have read it
+      if (k0 == 0) load(kc + 2);
+      if (i > 0) add_sum(i - 1);
     }
-    __syncwarp();
-    // chunk kc + 2 goes where chunk kc - 1 was, once its MMAs have read it
-    if (kc > 0)
-      ok = mbar_wait_warp(bar + 8 * ((kc - 1) % STAGES), (uint32_t)(((kc - 1) / STAGES) & 1),
-                          abort_flag, err, 1) && ok;
-    load(kc + 2);
-    if (kc > 0) add_chunk(kc - 1);
-  }
-  // the last commit covers every MMA of the tile
-  ok = mbar_wait_warp(bar + 8 * ((nk - 1) % STAGES), (uint32_t)(((nk - 1) / STAGES) & 1), abort_flag,
-                      err, 2) && ok;
-  add_chunk(nk - 1);
+    // the last commit covers every MMA of the tile
+    ok = mbar_wait_warp(bar + 8 * ((sums - 1) & 1), (uint32_t)(((sums - 1) >> 1) & 1), abort_flag, err,
+                        2) && ok;
+    add_sum(sums - 1);
+  };
+  if (K < GEMM_TC_CHUNK_K) product(std::integral_constant<int, 1>{});
+  else product(std::integral_constant<int, BK / 16>{});
   asm volatile("cp.async.wait_group 0;" ::: "memory");
   ok = __syncthreads_and(ok);
   // 32 x 32 blocks of a warp's lane quarter, turned in shared memory so that a warp's global

@@ -130,3 +130,29 @@ def gradient_parity(label, a, gg, gd, refG, refD, tol, pair_inputs):
         label, len(worst), worst.max(), np.median(worst),
         ", ".join("%s: %.1e" % (n, v) for n, v in zip(names, err.max(axis=0)))))
     return refG, refD, worst
+
+
+def native_program(tmp_path_factory, name, source, replaces=()):
+    """Compiles a CUDA program that includes library sources (``replaces``) to reach their internals
+    and links it with the library's other objects. Returns the executable's path."""
+    import os
+    import subprocess
+    from paper_1811_12843_gb300 import _build
+    obj = os.path.join(_build.OUT_DIR, "obj")
+    others = [os.path.join(obj, s.replace(".cu", ".o")) for s in _build.SOURCES
+              if s not in replaces]
+    _build.build(force=not all(map(os.path.exists, others)))
+    d = tmp_path_factory.mktemp(name)
+    src, exe = str(d / (name + ".cu")), str(d / name)
+    with open(src, "w") as f:
+        f.write(source)
+    subprocess.run([_build._nvcc()] + _build.ARCH + _build.FLAGS + [src] + others + ["-o", exe],
+                   check=True, capture_output=True, text=True)
+    return exe
+
+
+def run_program(*cmd):
+    import subprocess
+    r = subprocess.run(cmd, capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0, r.stdout + r.stderr
+    return r.stdout

@@ -2,10 +2,9 @@
 those that a check reads and resets. The test program is the engine's host side with its internals in
 reach, linked with the library's other objects."""
 
-import os
-import subprocess
-
 import pytest
+
+from helpers import native_program, run_program
 
 PROGRAM = r"""
 #include "api.cu"
@@ -72,26 +71,11 @@ int main(int argc, char**) { return argc > 1 ? device() : host(); }
 
 @pytest.fixture(scope="module")
 def program(tmp_path_factory):
-    from paper_1811_12843_gb300 import _build
-    obj = os.path.join(_build.OUT_DIR, "obj")
-    others = [os.path.join(obj, s.replace(".cu", ".o")) for s in _build.SOURCES if s != "api.cu"]
-    _build.build(force=not all(map(os.path.exists, others)))
-    d = tmp_path_factory.mktemp("status")
-    src, exe = str(d / "status.cu"), str(d / "status")
-    with open(src, "w") as f:
-        f.write(PROGRAM)
-    subprocess.run([_build._nvcc()] + _build.ARCH + _build.FLAGS + [src] + others + ["-o", exe],
-                   check=True, capture_output=True, text=True)
-    return exe
-
-
-def _run(*cmd):
-    r = subprocess.run(cmd, capture_output=True, text=True, timeout=120)
-    assert r.returncode == 0, r.stdout + r.stderr
+    return native_program(tmp_path_factory, "status", PROGRAM, replaces=("api.cu",))
 
 
 def test_every_status_word_is_listed(program):
-    _run(program)
+    run_program(program)
 
 
 @pytest.mark.gpu
@@ -99,4 +83,4 @@ def test_a_raised_word_is_reported_and_reset(program):
     torch = pytest.importorskip("torch")
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
-    _run(program, "device")
+    run_program(program, "device")
