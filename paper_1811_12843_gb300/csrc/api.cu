@@ -776,8 +776,8 @@ int create_impl(lipz_grid* g) {
   }
   if (g->a.mixture) {
     const size_t R = (size_t)6 * B;
-    g->mix_tc = g->bf && !g->a.force_simt && tc_supported(z, h, x, B) && tc_gram_supported(B);
-    g->mix_nh = g->mix_tc ? tc_gram_halves(B) : 1;
+    g->mix_tc = g->bf && !g->a.force_simt && tc_supported(z, h, x, B) && tc_gram_supported(B, x);
+    g->mix_nh = g->mix_tc ? tc_gram_parts(B) : 1;
     if ((rc = dalloc(g, &g->rnorm, C * R * 4)) ||
         (rc = dalloc(g, &g->mixP, (g->mix_tc ? C * tc_gram_floats(B) : C * R * 6) * 4)) ||
         (rc = dalloc(g, &g->mixS, C * 36 * 4)) || (rc = dalloc(g, &g->mixScore, C * 4)) ||

@@ -45,17 +45,32 @@ constexpr int H_CHUNK = BM * BK * 2;         // one 64-column chunk of the on-ch
 constexpr int H_BYTES = BM * HID * 2;        // 64 KB
 constexpr int N3 = 256;                      // generator output columns per MMA block
 constexpr int NUM_EPI_WARPS = 8;
-constexpr int THREADS = 64 + 32 * NUM_EPI_WARPS;
 constexpr int MISC_BYTES = 2048;
 constexpr int BIAS_MAX = 256 + 256 + 1024;  // floats per tile: b1, b2, then b3 (G) or w3, b3 (D)
 constexpr int BIAS_BYTES = 2 * BIAS_MAX * 4;  // double-buffered by tile
 // floats of one buffer of row norms (Gram kind, which has no on-chip activation: its region holds
 // two)
 constexpr int GRAM_NORMS = H_BYTES / 8;
+constexpr int GRAM_WIDE = 384;  // row width from which tensor memory sums 128 k at a time
 constexpr int SMEM_BYTES = 1024 + STAGES * STAGE_BYTES + H_BYTES + MISC_BYTES + BIAS_BYTES;
 
-enum { KIND_G = 0, KIND_D = 1, KIND_GRAM = 2 };
-enum { EPI_TO_H = 0, EPI_LOGIT = 1, EPI_TO_E = 2, EPI_ACT_OUT = 3, EPI_GRAM = 4 };
+enum { KIND_G = 0, KIND_D = 1, KIND_GRAM = 2, KIND_GRAM_SUMS = 3 };
+constexpr bool is_gram(int kind) { return kind >= KIND_GRAM; }
+// Gram kinds: parts that the columns of a block are divided into, the epilogue warps per lane quarter
+// (sums leave a thread 64 products in registers)
+template <int KND>
+constexpr int gram_parts() {
+  return KND == KIND_GRAM_SUMS ? 4 : 2;
+}
+template <int KND>
+constexpr int epi_warps() {
+  return is_gram(KND) ? 4 * gram_parts<KND>() : NUM_EPI_WARPS;
+}
+template <int KND>
+constexpr int threads() {
+  return 64 + 32 * epi_warps<KND>();
+}
+enum { EPI_TO_H = 0, EPI_LOGIT = 1, EPI_TO_E = 2, EPI_ACT_OUT = 3, EPI_GRAM = 4 };  // last: gram_block
 
 struct KParams {
   int kind;
@@ -93,10 +108,11 @@ struct KParams {
   // upper triangle only (the column blocks from the row tile's on; elements left of the diagonal
   // count zero, those on it a half), reduced in the epilogue to sums of exp(-||e_r - e_s||^2 / x)
   // over the 32 rows r of a warp in each of the (at most two) blocks of B rows they meet and the
-  // columns s of each block. rnorm [cells][rows] holds ||e_r||^2; the sums go to
-  // gram_out[cell][row tile][row quarter][half][2][6], half = 2 * column block + column half.
+  // columns s of each block (of the warp's part of every 256 columns). rnorm [cells][rows] holds
+  // ||e_r||^2; the sums go to gram_out[cell][row tile][row quarter][column part][2][6].
   const float* rnorm;
   float* gram_out;
+  int sum_chunks;  // KIND_GRAM_SUMS: K chunks that tensor memory sums at a time (1 or 2)
 };
 
 struct Job {
@@ -113,7 +129,7 @@ struct Job {
 template <int KND>
 __device__ __forceinline__ Job get_job(const KParams& p, int j) {
   Job J;
-  if (KND == KIND_GRAM) {
+  if (is_gram(KND)) {
     // column block j of the Gram matrix: MMA N rounded up to 16 (rows past 6B read as zero)
     const int n = min(HID, p.rows - j * HID);
     J = Job{0, p.kc1, (n + 15) & ~15, j & 1, 0, j * HID, HID, EPI_GRAM};
@@ -134,7 +150,7 @@ __device__ __forceinline__ Job get_job(const KParams& p, int j) {
 
 template <int KND>
 __device__ __forceinline__ int n_jobs(const KParams& p) {
-  if (KND == KIND_GRAM) return (p.rows + HID - 1) / HID;
+  if (is_gram(KND)) return (p.rows + HID - 1) / HID;
   return (KND == KIND_D || p.train) ? 2 : 2 + p.n3;
 }
 
@@ -147,14 +163,14 @@ __device__ __forceinline__ int last_steps(int K, int kchunks) {
 // First job of a tile: the Gram kind starts at the column block that holds its diagonal.
 template <int KND>
 __device__ __forceinline__ int first_job(int m0) {
-  return KND == KIND_GRAM ? m0 / HID : 0;
+  return is_gram(KND) ? m0 / HID : 0;
 }
 
 // A tile's problem and first row. The Gram kind's tiles go from the longest (row tile 0 of every
 // cell) to the shortest, every other round of the CTAs backwards, so that their sums balance.
 template <int KND>
 __device__ __forceinline__ void tile_place(const KParams& p, int tile, int& prob, int& m0) {
-  if (KND == KIND_GRAM) {
+  if (is_gram(KND)) {
     const int g = (int)gridDim.x, round = tile / g;
     if (round & 1) {
       const int last = min(g, p.n_tiles - round * g) - 1;
@@ -172,12 +188,12 @@ __device__ __forceinline__ void tile_place(const KParams& p, int tile, int& prob
 // Problem -> (cell whose activations are the A operand, individual whose weights are B).
 template <int KND>
 __device__ __forceinline__ int prob_cell(const KParams& p, int prob) {
-  return (p.train || p.centre || KND == KIND_GRAM) ? prob : prob / 5;
+  return (p.train || p.centre || is_gram(KND)) ? prob : prob / 5;
 }
 template <int KND>
 __device__ __forceinline__ int prob_individual(const KParams& p, int prob) {
   if (p.train) return __ldg(&p.wsel[p.part_slot ? prob >> 1 : prob]);
-  if (KND == KIND_GRAM) return prob;
+  if (is_gram(KND)) return prob;
   return p.centre ? p.indiv_off + prob : __ldg(&p.nbr[prob]);
 }
 
@@ -251,13 +267,166 @@ __device__ __forceinline__ float2 tanh_fast2(unsigned long long xx) {
                      copysignf(ax1 < 0.25f ? s.y : t.y, x.y));
 }
 
+// Gaussian kernel exp((2 e_r.e_s - |e_r|^2 - |e_s|^2) / x) of row rr against 32 columns s from col0 on,
+// added per block of B >= 32 columns (col0 lies in block blk) to acc: columns s > r in full, s = r half.
+// The group meets at most one block boundary (at column sp of it, the same for every lane), columns past
+// the last row count zero; two interleaved partial sums per side, combined in a fixed order. sb holds
+// -|e_s|^2 / x, nr that of row rr.
+__device__ __forceinline__ void gram_group(const KParams& p, const float (&dot)[32], int col0, int blk,
+                                           int m0, int rr, float nr, float two_ix, const float* sb,
+                                           float (&acc)[6]) {
+  const int sp = (blk + 1) * p.B - col0;
+  const int nv = p.rows - col0;
+  const bool diag = col0 < m0 + BM;  // the tile's diagonal may cross the group
+  const int dg = rr - col0;          // this row's diagonal column in the group
+  const float4* s4 = reinterpret_cast<const float4*>(sb + col0);
+  float lo0 = 0.f, lo1 = 0.f, hi0 = 0.f, hi1 = 0.f;
+  if (!diag && sp >= 32 && nv >= 32) {
+    // (most groups: every column counts, in one block)
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const float4 ns = s4[q];
+      lo0 += __expf(fmaf(dot[4 * q], two_ix, nr + ns.x));
+      lo1 += __expf(fmaf(dot[4 * q + 1], two_ix, nr + ns.y));
+      lo0 += __expf(fmaf(dot[4 * q + 2], two_ix, nr + ns.z));
+      lo1 += __expf(fmaf(dot[4 * q + 3], two_ix, nr + ns.w));
+    }
+  } else {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const float4 ns = s4[q];
+      const float nsv[4] = {ns.x, ns.y, ns.z, ns.w};
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int e = 4 * q + u;
+        float v = __expf(fmaf(dot[e], two_ix, nr + nsv[u]));
+        v = e < nv ? v : 0.f;
+        if (diag) v = e > dg ? v : (e == dg ? 0.5f * v : 0.f);
+        const float vl = e < sp ? v : 0.f, vh = e < sp ? 0.f : v;
+        if (e & 1) {
+          lo1 += vl;
+          hi1 += vh;
+        } else {
+          lo0 += vl;
+          hi0 += vh;
+        }
+      }
+    }
+  }
+  const float lo = lo0 + lo1, hi = hi0 + hi1;
+#pragma unroll
+  for (int t = 0; t < 6; ++t) acc[t] += t == blk ? lo : (t == blk + 1 ? hi : 0.f);
+}
+
+// Gram kinds' epilogue of one column block: the groups of this warp's part of its columns. `sums` sums
+// of earlier blocks went through tensor memory's two regions. Returns false on a timeout.
+//   KIND_GRAM: a block's products stand in tensor memory whole. Its additions truncate: the block means
+//   of 784-wide rows are off by 1.1e-7 (root mean square; 1024-wide 1.7e-7, all of it bias).
+//   KIND_GRAM_SUMS: tensor memory sums p.sum_chunks chunks at a time, and these sums are added in
+//   registers: 784-wide 5e-8, 1024-wide 6e-8, as with a stored fp32 Gram matrix (which batches above
+//   250, that take this kind, would otherwise have).
+// Bound: the exponentials beside the MMAs; for sums their handshakes, and that a block's exponentials
+// overlap with the next block's first two sums only. Mixture phase, 784-wide rows: 12x12 cells, B = 100
+// 111 us whole (117 with a reduction over the lanes after every block and no path of their own for full
+// groups), 138 as sums; 5x5 cells, B = 256 66 whole, 78 as sums, 5025 with the stored matrix on the CUDA
+// cores.
+template <int KND>
+__device__ __forceinline__ bool gram_block(const KParams& p, const Job& J, int m0, int part, int rr,
+                                           uint32_t tmem_row, const float* sb, float (&acc)[6],
+                                           int& sums, uint32_t bAcc, uint32_t bReg,
+                                           volatile int* abort_flag) {
+  constexpr int COLS = HID / gram_parts<KND>(), NG = COLS / 32;  // columns of the warp; groups
+  const int cb = J.brow0 + part * COLS;
+  // groups that hold anything: up to the last row, from the tile's first row on
+  auto live = [&](int g) { return cb + 32 * g < p.rows && cb + 32 * g + 32 > m0; };
+  const float nr = rr < p.rows ? sb[rr] : 0.f, two_ix = 2.f / (float)p.x;
+  int blk = cb / p.B;
+  auto group = [&](int g, const float (&dot)[32]) {
+    const int col0 = cb + 32 * g;
+    if (col0 >= (blk + 1) * p.B) ++blk;
+    if (live(g)) gram_group(p, dot, col0, blk, m0, rr, nr, two_ix, sb, acc);
+  };
+  auto wait_sum = [&] {
+    const bool ok = mbar_wait_warp(bAcc + 8 * (sums & 1), (uint32_t)((sums >> 1) & 1), abort_flag,
+                                   p.err, 6);
+    tc_fence_after();
+    return ok;
+  };
+  auto release_sum = [&] {
+    tc_fence_before();
+    mbar_arrive(bReg + 8 * (sums & 1));
+    ++sums;
+  };
+  if constexpr (KND == KIND_GRAM) {
+    if (!wait_sum()) return false;
+#pragma unroll 1
+    for (int g = 0; g < NG; ++g) {
+      uint32_t r[32];
+      LIPZ_TMEM_LD32(tmem_row + (uint32_t)((sums & 1) * HID + part * COLS + g * 32), r);
+      tmem_wait_ld();
+      float dot[32];
+#pragma unroll
+      for (int e = 0; e < 32; ++e) dot[e] = __uint_as_float(r[e]);
+      group(g, dot);
+    }
+    release_sum();
+  } else {
+    float dot[NG][32];
+#pragma unroll
+    for (int g = 0; g < NG; ++g)
+#pragma unroll
+      for (int e = 0; e < 32; ++e) dot[g][e] = 0.f;
+    for (int kc = 0; kc < J.kchunks; kc += p.sum_chunks) {
+      if (!wait_sum()) return false;
+#pragma unroll
+      for (int g = 0; g < 2 * NG; ++g) {
+        if (!live(g / 2)) continue;
+        uint32_t r[16];
+        LIPZ_TMEM_LD16(tmem_row + (uint32_t)((sums & 1) * HID + part * COLS + g * 16), r);
+        tmem_wait_ld();
+#pragma unroll
+        for (int e = 0; e < 16; ++e) dot[g / 2][(g & 1) * 16 + e] += __uint_as_float(r[e]);
+      }
+      release_sum();
+    }
+#pragma unroll
+    for (int g = 0; g < NG; ++g) group(g, dot[g]);
+  }
+  return true;
+}
+
+// The sums of a warp's 32 rows (of the tile at m0, quarter q of it) over its columns of every block of
+// the tile: those of its rows in the block of the first one, then those in the next.
+template <int KND>
+__device__ __forceinline__ void gram_out(const KParams& p, int c, int m0, int q, int part, int lane,
+                                         const float (&acc)[6]) {
+  const int w0 = m0 + q * 32, rr = w0 + lane;
+  const bool ok = rr < p.rows, first = rr < (w0 / p.B + 1) * p.B;
+  float out = 0.f;
+#pragma unroll
+  for (int t = 0; t < 6; ++t) {
+    float a0 = ok && first ? acc[t] : 0.f, a1 = ok && !first ? acc[t] : 0.f;
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+      a0 += __shfl_xor_sync(0xffffffffu, a0, o);
+      a1 += __shfl_xor_sync(0xffffffffu, a1, o);
+    }
+    if (lane == t) out = a0;
+    if (lane == 6 + t) out = a1;
+  }
+  if (lane < 12 && w0 < p.rows)
+    p.gram_out[((((int64_t)c * p.mtiles + m0 / BM) * 4 + q) * gram_parts<KND>() + part) * 12 + lane] =
+        out;
+}
+
 // ---- the kernel ----------------------------------------------------------------------------
 // KND: p.kind at compile time (one variant per network kind, each with only its own paths)
 template <int KND>
-__global__ void __launch_bounds__(THREADS, 1)
+__global__ void __launch_bounds__(threads<KND>(), 1)
     k_mlp_fwd(const __grid_constant__ CUtensorMap mA, const __grid_constant__ CUtensorMap mB1,
               const __grid_constant__ CUtensorMap mB2, const __grid_constant__ CUtensorMap mB3,
               const KParams p) {
+  constexpr int NE = epi_warps<KND>();
   extern __shared__ uint8_t smem_raw[];
   // 1024-byte alignment for the swizzled tiles
   const uint32_t raw = smem_u32(smem_raw);
@@ -287,13 +456,13 @@ __global__ void __launch_bounds__(THREADS, 1)
     }
     mbar_init(bAcc, 1);
     mbar_init(bAcc + 8, 1);
-    mbar_init(bReg, 32 * NUM_EPI_WARPS);
-    mbar_init(bReg + 8, 32 * NUM_EPI_WARPS);
-    for (int c = 0; c < HID / BK; ++c) mbar_init(bH + 8 * c, 32 * NUM_EPI_WARPS);
-    mbar_init(bPart, 32 * NUM_EPI_WARPS / 2);
+    mbar_init(bReg, 32 * NE);
+    mbar_init(bReg + 8, 32 * NE);
+    for (int c = 0; c < HID / BK; ++c) mbar_init(bH + 8 * c, 32 * NE);
+    mbar_init(bPart, 32 * NE / 2);
     mbar_init(bFinal, 1);
-    mbar_init(bBias, 32 * NUM_EPI_WARPS);
-    mbar_init(bBias + 8, 32 * NUM_EPI_WARPS);
+    mbar_init(bBias, 32 * NE);
+    mbar_init(bBias + 8, 32 * NE);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -373,24 +542,30 @@ __global__ void __launch_bounds__(THREADS, 1)
       int reg_uses[2] = {0, 0};
       int h_total = 0;  // activations written to H so far (each chunk barrier: one phase each)
       bool ok = true;
-      int jobs_done = 0;
+      int sums = 0;                            // Gram kind: sums so far
+      const int sum_mask = KND == KIND_GRAM_SUMS ? p.sum_chunks - 1 : -1;
       for (int tile = blockIdx.x; tile < p.n_tiles && ok; tile += gridDim.x) {
         int prob, m0;
         tile_place<KND>(p, tile, prob, m0);
-        for (int j = first_job<KND>(m0); j < nj && ok; ++j, ++jobs_done) {
+        for (int j = first_job<KND>(m0); j < nj && ok; ++j) {
           const Job J = get_job<KND>(p, j);
-          // the Gram kind alternates the two accumulators over all its jobs (3 per tile)
-          const int R = KND == KIND_GRAM ? (jobs_done & 1) : J.region;
-          if (reg_uses[R] > 0 &&
-              !mbar_wait(bReg + 8 * R, (uint32_t)((reg_uses[R] - 1) & 1), abort_flag, p.err, 2)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t d = tmem + (uint32_t)(R * HID);
           const uint32_t idesc = idesc_bf16(BM, J.n);
           const int last = J.a_from_h ? BK / 16 : last_steps(KND == KIND_G ? p.z : p.x, J.kchunks);
+          int R = J.region;
           for (int kc = 0; kc < J.kchunks; ++kc) {
+            const bool first = kc == 0 || (KND == KIND_GRAM_SUMS && (kc & sum_mask) == 0);
+            if (first) {
+              // the Gram kinds' sums take the two accumulators in turn
+              if (is_gram(KND)) R = sums++ & 1;
+              if (reg_uses[R] > 0 &&
+                  !mbar_wait(bReg + 8 * R, (uint32_t)((reg_uses[R] - 1) & 1), abort_flag, p.err, 2)) {
+                ok = false;
+                break;
+              }
+              reg_uses[R]++;
+              tc_fence_after();
+            }
+            const uint32_t d = tmem + (uint32_t)(R * HID);
             // a layer reading the on-chip activation starts on chunk kc as soon as the epilogue
             // has written that chunk (write number h_total - 1)
             if (J.a_from_h &&
@@ -410,17 +585,16 @@ __global__ void __launch_bounds__(THREADS, 1)
               for (int kk = 0; kk < BK / 16; ++kk)
                 if (kk < last || kc + 1 < J.kchunks)
                   tc_mma(d, sw128_desc(sA + kk * 32), sw128_desc(sB + kk * 32), idesc,
-                         (kc | kk) != 0 ? 1u : 0u);
+                         first && kk == 0 ? 0u : 1u);
               tc_commit(bEmpty + 8 * stage);
+              if (kc + 1 == J.kchunks || (KND == KIND_GRAM_SUMS && (kc & sum_mask) == sum_mask))
+                tc_commit(bAcc + 8 * R);
             }
             if (++stage == STAGES) {
               stage = 0;
               phase ^= 1u;
             }
           }
-          if (!ok) break;
-          if (elected) tc_commit(bAcc + 8 * R);
-          reg_uses[R]++;
           if (J.epi == EPI_TO_H) ++h_total;
         }
       }
@@ -433,13 +607,13 @@ __global__ void __launch_bounds__(THREADS, 1)
     // ================================ epilogue ================================
     const int ew = warp - 2;
     const int q = warp & 3;        // TMEM lane quarter this warp may access
-    const int hf = ew >> 2;        // column half
+    const int hf = ew >> 2;        // column half (Gram kind: part)
     const int row = q * 32 + lane; // row of the tile
     const uint32_t lane_base = (uint32_t)(q * 32) << 16;
     int reg_uses[2] = {0, 0};
     bool ok = true;
-    int ltile = 0, jobs_done = 0;
-    const int et = threadIdx.x - 64;  // epilogue thread 0..255
+    int ltile = 0, sums = 0;
+    const int et = threadIdx.x - 64;  // epilogue thread
     for (int tile = blockIdx.x; tile < p.n_tiles && ok; tile += gridDim.x, ++ltile) {
       int prob, m0;
       tile_place<KND>(p, tile, prob, m0);
@@ -452,14 +626,14 @@ __global__ void __launch_bounds__(THREADS, 1)
       // The tile's biases (and D's output weights) go to shared memory once, while the MMAs
       // run, so that no epilogue waits on a global load. Buffer ltile & 1; a thread cannot
       // reach tile ltile + 2 before every thread has passed this tile's arrival.
-      float* sb = KND == KIND_GRAM ? reinterpret_cast<float*>(gbase + STAGES * STAGE_BYTES) +
+      float* sb = is_gram(KND) ? reinterpret_cast<float*>(gbase + STAGES * STAGE_BYTES) +
                                          (ltile & 1) * GRAM_NORMS
                                    : s_bias + (ltile & 1) * BIAS_MAX;
-      if (KND == KIND_GRAM) {
+      if (is_gram(KND)) {
         // the squared norms of the cell's rows (the Gram tile's row and column terms)
         // -|e_s|^2 / x for the cell's rows s, zero for the 32 entries past the last row
         const float ix = 1.f / (float)p.x;
-        for (int i = et; i < p.rows + 32; i += 32 * NUM_EPI_WARPS)
+        for (int i = et; i < p.rows + 32; i += 32 * NE)
           sb[i] = i < p.rows ? -__ldg(&p.rnorm[(int64_t)c * p.rows + i]) * ix : 0.f;
         mbar_arrive(bBias + 8 * (ltile & 1));
         if (!mbar_wait_warp(bBias + 8 * (ltile & 1), (uint32_t)((ltile >> 1) & 1), abort_flag,
@@ -470,11 +644,11 @@ __global__ void __launch_bounds__(THREADS, 1)
       } else {
         // every load is issued before the first is stored, so their latencies overlap
         const int nb3 = KND == KIND_D ? HID + 1 : p.x;
-        constexpr int NV = (BIAS_MAX + 32 * NUM_EPI_WARPS - 1) / (32 * NUM_EPI_WARPS);
+        constexpr int NV = (BIAS_MAX + 32 * NE - 1) / (32 * NE);
         float v[NV];
 #pragma unroll
         for (int u = 0; u < NV; ++u) {
-          const int i = et + u * 32 * NUM_EPI_WARPS;
+          const int i = et + u * 32 * NE;
           v[u] = 0.f;
           if (i >= 512 + nb3) continue;
           if (i < 256) v[u] = wm[p.off_b1 + i];
@@ -487,7 +661,7 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
 #pragma unroll
         for (int u = 0; u < NV; ++u) {
-          const int i = et + u * 32 * NUM_EPI_WARPS;
+          const int i = et + u * 32 * NE;
           if (i < 512 + nb3) sb[i] = v[u];
         }
         mbar_arrive(bBias + 8 * (ltile & 1));
@@ -497,9 +671,16 @@ __global__ void __launch_bounds__(THREADS, 1)
           break;
         }
       }
-      for (int j = first_job<KND>(m0); j < nj && ok; ++j, ++jobs_done) {
+      float acc[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};  // Gram kind: this row's sums by block
+      for (int j = first_job<KND>(m0); j < nj && ok; ++j) {
         const Job J = get_job<KND>(p, j);
-        const int R = KND == KIND_GRAM ? (jobs_done & 1) : J.region;
+        if constexpr (is_gram(KND)) {
+          ok = gram_block<KND>(p, J, m0, hf, rr, tmem + lane_base, sb, acc, sums, bAcc, bReg,
+                               abort_flag);
+          if (ok && j + 1 == nj) gram_out<KND>(p, c, m0, q, hf, lane, acc);
+          continue;
+        }
+        const int R = J.region;
         if (!mbar_wait_warp(bAcc + 8 * R, (uint32_t)(reg_uses[R] & 1), abort_flag, p.err, 6)) {
           ok = false;
           break;
@@ -629,76 +810,6 @@ __global__ void __launch_bounds__(THREADS, 1)
             mbar_arrive(bReg + 8 * R);
             if (row_ok) p.logits[(int64_t)prob * p.rows + rr] = logit;
           }
-        } else if (J.epi == EPI_GRAM) {
-          // Gaussian kernel exp((2 e_r.e_s - |e_r|^2 - |e_s|^2) / x) of this thread's row r
-          // against the warp's 128 columns s >= r, summed per column block of B >= 32 rows: a group
-          // of 32 columns meets at most one block boundary (at column sp of the group, the same
-          // for every lane), columns past the last row count zero; two interleaved partial sums
-          // per side, combined in a fixed order. (Bound: the exponentials beside the MMAs. Mixture
-          // phase at 5x5, B = 256: 74 us, 5025 with the stored Gram matrix of the CUDA-core path,
-          // which batches above 250 took; the triangle halves the work of the full square.)
-          const float nr = row_ok ? sb[rr] : 0.f;
-          const float two_ix = 2.f / (float)p.x;
-          float acc[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-#pragma unroll 1
-          for (int cg = hf * 4; cg < hf * 4 + 4; ++cg) {
-            const int col0 = J.brow0 + cg * 32;
-            if (col0 >= p.rows) break;
-            if (col0 + 32 <= m0) continue;  // left of the tile's first row
-            uint32_t r[32];
-            LIPZ_TMEM_LD32(tbase + cg * 32, r);
-            tmem_wait_ld();
-            const int blk = col0 / p.B;
-            const int sp = (blk + 1) * p.B - col0;
-            const int nv = p.rows - col0;
-            const bool diag = col0 < m0 + BM;  // the tile's diagonal may cross the group
-            const int dg = rr - col0;          // this row's diagonal column in the group
-            const float4* s4 = reinterpret_cast<const float4*>(sb + col0);
-            float lo0 = 0.f, lo1 = 0.f, hi0 = 0.f, hi1 = 0.f;
-#pragma unroll
-            for (int q = 0; q < 8; ++q) {
-              const float4 ns = s4[q];
-              const float nsv[4] = {ns.x, ns.y, ns.z, ns.w};
-#pragma unroll
-              for (int u = 0; u < 4; ++u) {
-                const int e = 4 * q + u;
-                float v = __expf(fmaf(__uint_as_float(r[e]), two_ix, nr + nsv[u]));
-                v = e < nv ? v : 0.f;
-                if (diag) v = e > dg ? v : (e == dg ? 0.5f * v : 0.f);
-                const float vl = e < sp ? v : 0.f, vh = e < sp ? 0.f : v;
-                if (e & 1) {
-                  lo1 += vl;
-                  hi1 += vh;
-                } else {
-                  lo0 += vl;
-                  hi0 += vh;
-                }
-              }
-            }
-            const float lo = lo0 + lo1, hi = hi0 + hi1;
-#pragma unroll
-            for (int t = 0; t < 6; ++t) acc[t] += t == blk ? lo : (t == blk + 1 ? hi : 0.f);
-          }
-          tc_fence_before();
-          mbar_arrive(bReg + 8 * R);
-          // the warp's rows in the block of its first row, and those in the next one
-          const int w0 = m0 + q * 32;
-          const bool first = rr < (w0 / p.B + 1) * p.B;
-          float out = 0.f;
-#pragma unroll
-          for (int t = 0; t < 6; ++t) {
-            float a0 = row_ok && first ? acc[t] : 0.f, a1 = row_ok && !first ? acc[t] : 0.f;
-#pragma unroll
-            for (int o = 16; o; o >>= 1) {
-              a0 += __shfl_xor_sync(0xffffffffu, a0, o);
-              a1 += __shfl_xor_sync(0xffffffffu, a1, o);
-            }
-            if (lane == t) out = a0;
-            if (lane == 6 + t) out = a1;
-          }
-          if (lane < 12 && w0 < p.rows)
-            p.gram_out[((((int64_t)c * p.mtiles + m0 / BM) * 4 + q) * (2 * nj) + 2 * j + hf) * 12 +
-                       lane] = out;
         } else {
           // generator output block: bias + tanh, bf16, into the fake rows of E[c]
           const float* bias = sb + 512;
@@ -1849,6 +1960,9 @@ TcPlan* tc_plan_create(const TcShape& s, const TcBuffers& b, std::string* msg) {
                            tc::SMEM_BYTES) != cudaSuccess ||
       cudaFuncSetAttribute(tc::k_mlp_fwd<tc::KIND_D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                            tc::SMEM_BYTES) != cudaSuccess ||
+      cudaFuncSetAttribute(tc::k_mlp_fwd<tc::KIND_GRAM_SUMS>,
+                           cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           tc::SMEM_BYTES) != cudaSuccess ||
       cudaFuncSetAttribute(tc::k_mlp_fwd<tc::KIND_GRAM>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize,
                            tc::SMEM_BYTES) != cudaSuccess) {
@@ -1918,7 +2032,7 @@ TcPlan* tc_plan_create(const TcShape& s, const TcBuffers& b, std::string* msg) {
   dt.act2 = (bf16*)b.TG2;
   dt.logits = b.TL;
   tc::KParams gm{};  // Gram matrix of every cell's evaluation rows (mixture score)
-  gm.kind = tc::KIND_GRAM;
+  gm.kind = s.B <= 250 ? tc::KIND_GRAM : tc::KIND_GRAM_SUMS;
   gm.cells = s.cells;
   gm.B = s.B;
   gm.z = s.z;
@@ -1932,6 +2046,7 @@ TcPlan* tc_plan_create(const TcShape& s, const TcBuffers& b, std::string* msg) {
   gm.err = p->err;
   gm.rnorm = b.rnorm;
   gm.gram_out = b.gram_out;
+  gm.sum_chunks = s.x >= tc::GRAM_WIDE ? 2 : 1;
   p->pg = g;
   p->pgc = gc;
   p->pgram = gm;
@@ -2012,10 +2127,13 @@ namespace {
 int launch(int grid, const CUtensorMap& a, const CUtensorMap& b1, const CUtensorMap& b2,
            const CUtensorMap& b3, const tc::KParams& kp, cudaStream_t st, const char* what,
            std::string* msg) {
-  auto k = kp.kind == tc::KIND_GRAM ? tc::k_mlp_fwd<tc::KIND_GRAM>
-           : kp.kind == tc::KIND_D  ? tc::k_mlp_fwd<tc::KIND_D>
-                                    : tc::k_mlp_fwd<tc::KIND_G>;
-  launch_pdl(k, dim3(grid), dim3(tc::THREADS), tc::SMEM_BYTES, st, a, b1, b2, b3, kp);
+  const bool sums = kp.kind == tc::KIND_GRAM_SUMS;
+  auto k = sums                       ? tc::k_mlp_fwd<tc::KIND_GRAM_SUMS>
+           : kp.kind == tc::KIND_GRAM ? tc::k_mlp_fwd<tc::KIND_GRAM>
+           : kp.kind == tc::KIND_D    ? tc::k_mlp_fwd<tc::KIND_D>
+                                      : tc::k_mlp_fwd<tc::KIND_G>;
+  const int threads = sums ? tc::threads<tc::KIND_GRAM_SUMS>() : tc::threads<tc::KIND_G>();
+  launch_pdl(k, dim3(grid), dim3(threads), tc::SMEM_BYTES, st, a, b1, b2, b3, kp);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     if (msg) *msg = std::string(what) + " launch: " + cudaGetErrorString(e);
@@ -2081,22 +2199,27 @@ int tc_run_g_centre(TcPlan* p, cudaStream_t st, std::string* msg) {
 }
 
 int tc_run_gram(TcPlan* p, cudaStream_t st, std::string* msg) {
-  if (!p->pgram.rnorm || !p->pgram.gram_out || !tc_gram_supported(p->s.B)) {
+  if (!p->pgram.rnorm || !p->pgram.gram_out || !tc_gram_supported(p->s.B, p->s.x)) {
     if (msg) *msg = "tensor-core Gram kernel: no buffers, or batch outside 32..1360";
     return 1;
   }
   return launch(p->grid_gram, p->mE, p->mEB, p->mEB, p->mEB, p->pgram, st, "mixture Gram", msg);
 }
 
-int tc_gram_halves(int B) { return 2 * ((6 * B + tc::HID - 1) / tc::HID); }
+int tc_gram_parts(int B) {
+  return B <= 250 ? tc::gram_parts<tc::KIND_GRAM>() : tc::gram_parts<tc::KIND_GRAM_SUMS>();
+}
 
 int64_t tc_gram_floats(int B) {
-  return (int64_t)((6 * B + tc::BM - 1) / tc::BM) * 4 * tc_gram_halves(B) * 12;
+  return (int64_t)((6 * B + tc::BM - 1) / tc::BM) * 4 * tc_gram_parts(B) * 12;
 }
 
 // B >= 32: a 32-column group meets at most one block boundary; the norms and 32 zero entries
-// past them fit one norm buffer (B <= 1360)
-bool tc_gram_supported(int B) { return B >= 32 && 6 * B + 32 <= tc::GRAM_NORMS; }
+// past them fit one norm buffer (B <= 1360). Sums over fewer than GEMM_TC_CHUNK_K are less exact by
+// chunks of 64 than in the stored fp32 matrix, which batches above 250 keep for them.
+bool tc_gram_supported(int B, int x) {
+  return B >= 32 && 6 * B + 32 <= tc::GRAM_NORMS && (B <= 250 || x >= GEMM_TC_CHUNK_K);
+}
 
 int tc_run_d(TcPlan* p, cudaStream_t st, std::string* msg) {
   if (p->ncl_d > 0 && p->ppd.pairs)

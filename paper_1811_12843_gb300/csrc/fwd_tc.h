@@ -90,13 +90,13 @@ int tc_run_d(TcPlan* p, cudaStream_t st, std::string* msg);
 // Mixture score: for every cell c and each 32 rows of E[c], the sums of
 // exp(-||E[c][r] - E[c][s]||^2 / x) over its rows r in the block of the first and in the next block
 // of B rows, and over the columns s > r (s = r counting a half) of each block, into
-// gram_out[c][row tile of 128][4][h][2][6], split over the tc_gram_halves(B) column ranges h of
-// 128 (ranges before the 256 columns that hold the tile's diagonal are not written).
-// 32 <= B <= 1360, i.e. tc_gram_supported.
+// gram_out[c][row tile of 128][4][tc_gram_parts(B)][2][6], divided among equal parts of every 256
+// columns.
+// 32 <= B <= 1360 (250 for narrow rows), i.e. tc_gram_supported.
 int tc_run_gram(TcPlan* p, cudaStream_t st, std::string* msg);
-int tc_gram_halves(int B);
+int tc_gram_parts(int B);
 int64_t tc_gram_floats(int B);  // of gram_out, per cell
-bool tc_gram_supported(int B);
+bool tc_gram_supported(int B, int x);
 // Training forward of every cell's selected generator (hidden activations into TH1, TH2) and
 // selected discriminator (TG1, TG2 and the logits TL).
 int tc_run_train(TcPlan* p, cudaStream_t st, std::string* msg);

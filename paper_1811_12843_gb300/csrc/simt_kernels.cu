@@ -1075,7 +1075,7 @@ __device__ __forceinline__ float mix_mmd2(const float* w, const float* S) {
 //   TRI = false: S[a][b] = (sum over the rows r of block a of part[c][r][b]) / B^2;
 //   TRI = true (tensor-core Gram kernel): part[c][row tile][quarter][h][2][6] holds the upper
 //   triangle's sums, so S[a][b] = S[b][a] for a < b, and S[a][a] counts each element twice (the
-//   diagonal was counted half). nh = column ranges h of 128.
+//   diagonal was counted half). nh = column parts h.
 template <bool TRI>
 __global__ void __launch_bounds__(192) k_mix_es(const float* __restrict__ part, int nh, int rows,
                                                 int B, float* mix, float* __restrict__ S_out,
@@ -1092,7 +1092,7 @@ __global__ void __launch_bounds__(192) k_mix_es(const float* __restrict__ part, 
     const float* p = part + (int64_t)c * ((rows + 127) / 128 * 4) * nh * 12;
     for (int i = lane; i < (last - first + 1) * nh; i += 32) {
       const int g = first + i / nh, h = i % nh;
-      if (g >= groups || h / 2 < g * 32 / 128 * 128 / 256) continue;
+      if (g >= groups) continue;
       const int slot = a - g * 32 / B;  // the group's first block, or the next
       const float* q = p + ((int64_t)g * nh + h) * 12 + slot * 6;
 #pragma unroll

@@ -1,6 +1,6 @@
 """The tensor-core Gram kernel's tiles: batches at the edges of its 32-row groups, 128-row tiles,
 256-column blocks and of its range (32 to 1360), against the oracle, and at the largest batch
-against the CUDA-core path."""
+against the CUDA-core path; and its sums' own error."""
 
 import numpy as np
 import pytest
@@ -32,3 +32,25 @@ def test_largest_batches_against_the_cuda_core_path(L, batch):  # noqa: F811
         g.eval()
         means.append(g.mixture(blocks=True)[1])
     assert np.max(np.abs(means[0] - means[1])) < 2e-2 * np.max(np.abs(means[1]))
+
+
+@pytest.mark.parametrize("x,batch", [(784, 256), (1024, 256), (1024, 300)])
+def test_products_are_as_exact_as_a_stored_fp32_matrix(L, x, batch):  # noqa: F811
+    """The block mean of the real rows with themselves, known exactly, for batches above 250: the mean
+    of its error over 24 cells. A result's own rounding is at most 2^-24 and the exponentials' mean error
+    (1 / x and the argument rounded) about as much; tensor memory's truncation, if all of a product's
+    terms were summed there, would add 1e-7 (784) to 1.7e-7 (1024)."""
+    pool = _pool(6, 3000, x)
+    errs = []
+    for seed in range(6):
+        g = L.Grid(2, 2, seed=seed, precision="bf16", batch=batch, x_dim=x, mixture=1)
+        g.set_data(pool)
+        g.eval()
+        X = g.batch()[0].astype(np.float64)
+        S = g.mixture(blocks=True)[1]
+        for c in range(4):
+            n = (X[c] ** 2).sum(1)
+            ref = np.exp(-(n[:, None] + n - 2.0 * X[c] @ X[c].T) / x).mean()
+            errs.append((S[c][0, 0] - ref) / ref)
+        g.close()
+    assert abs(np.mean(errs)) < 1.5 * 2.0 ** -24, np.mean(errs)
