@@ -212,10 +212,18 @@ int wgrad_splits(const ConvDesc& d) {
   return (int)std::max<int64_t>(1, std::min<int64_t>(64, K / 4096));
 }
 
-}  // namespace
+// Whether the tensor-core discriminator evaluation takes the shape.
+bool tc_disc(const DcShape& s) { return s.bf && s.ndf % 64 == 0 && 8 * s.ndf <= 512; }
 
-DcPlan* dc_plan_create(const DcShape& s, const DcBuffers& b, std::string* msg) {
+// Bytes of the discriminator evaluation's activations of one cell (layers 1 and 2).
+int64_t eval_cell_bytes(const DcShape& s) {
+  return (int64_t)5 * 6 * s.B * (32 * 32 + 16 * 16 * 2) * s.ndf * (s.bf ? 2 : 4);
+}
+
+// The plan with `ecells` cells per launch of the discriminator evaluation.
+DcPlan* create_plan(const DcShape& s, const DcBuffers& b, int ecells, std::string* msg) {
   DcPlan* p = new DcPlan();
+  p->ecells = ecells;
   p->s = s;
   p->b = b;
   const int C = s.cells, B = s.B, g = s.ngf, d = s.ndf, z = s.z;
@@ -246,7 +254,7 @@ DcPlan* dc_plan_create(const DcShape& s, const DcBuffers& b, std::string* msg) {
   }
   const int PE = C * 5;
   p->tcg = s.bf && g % 64 == 0;
-  const bool tcd = s.bf && d % 64 == 0 && 8 * d <= 512;
+  const bool tcd = tc_disc(s);
   // tensor-core training forward (both networks' widths multiples of 64): channel-last
   // activations, read by the CUDA-core backward kernels in that layout
   const bool tct = tcd && p->tcg;
@@ -262,27 +270,12 @@ DcPlan* dc_plan_create(const DcShape& s, const DcBuffers& b, std::string* msg) {
   float *ec, *emean, *einv, *tc, *tmean, *tinv, *dh;
   void *eh, *ex, *ey, *th, *ta, *P, *Q, *P2, *Q2, *dcb, *d5;
   int64_t stats = 15 * (int64_t)g;  // channels of the four batch-normalised layers
-  // The discriminator evaluation's activations, for the cells that share a launch: the
-  // tensor-core path takes as many as 8 GB hold (one cell per launch leaves the last wave of 480
-  // tiles on 152 SMs a sixth full: 5.1 against 4.6 ms for the 3x3 configuration's layers 2-4),
-  // and one where that much is not free
-  const int64_t per_cell = (int64_t)5 * 6 * B * (dmax + dsz[2]) * es;
-  p->ecells = tcd ? (int)std::min<int64_t>(C, std::max<int64_t>(1, (int64_t)8000000000 / per_cell))
-                  : 1;
-  auto alloc_chunk = [&]() -> int {
-    for (;;) {
-      if (!dev_alloc(p, &ex, (size_t)p->ecells * 5 * 6 * B * dmax * es, msg) &&
-          !dev_alloc(p, &ey, (size_t)p->ecells * 5 * 6 * B * dsz[2] * es, msg))
-        return 0;
-      if (p->ecells == 1) return 1;
-      p->ecells = 1;
-    }
-  };
   if (dev_alloc(p, &ec, (size_t)PE * B * gmax * 4, msg) ||
       dev_alloc(p, &eh, (size_t)PE * B * gmax * es, msg) ||
       dev_alloc(p, &emean, (size_t)PE * stats * 4, msg) ||
       dev_alloc(p, &einv, (size_t)PE * stats * 4, msg) ||
-      alloc_chunk() ||
+      dev_alloc(p, &ex, (size_t)ecells * 5 * 6 * B * dmax * es, msg) ||
+      dev_alloc(p, &ey, (size_t)ecells * 5 * 6 * B * dsz[2] * es, msg) ||
       dev_alloc(p, &tc, (size_t)C * B * gall * 4, msg) ||
       dev_alloc(p, &th, (size_t)C * B * gall * es, msg) ||
       dev_alloc(p, &tmean, (size_t)C * stats * 4, msg) ||
@@ -1071,6 +1064,28 @@ DcPlan* dc_plan_create(const DcShape& s, const DcBuffers& b, std::string* msg) {
   p->eval_launches = 9 + 5 * C;
   p->train_launches = tct ? 60 + (p->scg ? 1 : 0) + (p->scd ? 2 : 0) : 50;
   return p;
+}
+
+}  // namespace
+
+// The tensor-core discriminator evaluation takes as many cells per launch as 8 GB of activations hold
+// (one cell per launch leaves the last wave of 480 tiles on 152 SMs a sixth full: 5.1 against 4.6 ms
+// for the 3x3 configuration's layers 2-4), but no more than leave free what they take beyond one cell's:
+// a grid that fits with one cell per launch is created, and the caller's pool keeps its room.
+DcPlan* dc_plan_create(const DcShape& s, const DcBuffers& b, std::string* msg) {
+  const int64_t cell = eval_cell_bytes(s);
+  int n = 1;
+  if (tc_disc(s))
+    n = (int)std::min<int64_t>(s.cells, std::max<int64_t>(1, (int64_t)8000000000 / cell));
+  for (;; n = (n + 1) / 2) {
+    DcPlan* p = create_plan(s, b, n, msg);
+    if (n == 1) return p;
+    size_t free_b = 0, total_b = 0;
+    if (p && cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && (int64_t)free_b >= (n - 1) * cell)
+      return p;
+    cudaGetLastError();
+    dc_plan_destroy(p);
+  }
 }
 
 void dc_plan_destroy(DcPlan* p) {

@@ -2,7 +2,7 @@
 CTA pair or a 256-row tile, one and several cells per launch, and widths with 128- and 256-column
 weight tiles. One iteration through the TMA kernels (CTA pairs, 256-row tiles, the shared first
 layer) must end in the state of the one-CTA kernels that gather their A rows, bit for bit, and the
-evaluation must meet the oracle."""
+evaluation must meet the oracle. And a grid for whose cells' shared launches the memory is not there."""
 
 import numpy as np
 import pytest
@@ -37,3 +37,41 @@ def test_evaluation_against_the_oracle(L, batch):  # noqa: F811
     ref = O.eval_neighborhoods(s, O.batches(s, pool))
     g.eval()
     assert max_rel(g.logits(), ref["logits"]) < 2e-2
+
+
+def test_little_memory_means_fewer_cells_per_launch(L):  # noqa: F811
+    """Where only one cell's evaluation buffers fit beside what a grid cannot do without, the grid is
+    created and computes the same."""
+    import torch
+    cells, batch = 4, 64
+    kw = dict(precision="bf16", batch=batch, ngf=64, ndf=64)
+    pool = _field_pool(4, 40)
+
+    def run():
+        g = _grid(L, 1, cells, 13, pool, **kw)
+        g.iterate(1)
+        state = np.frombuffer(g.export_state(), np.uint8)
+        g.close()
+        return state
+
+    def free():
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        return torch.cuda.mem_get_info()[0]
+
+    run()
+    before = free()
+    g = _grid(L, 1, cells, 13, pool, **kw)
+    used = before - free()
+    g.close()
+    ref = run()
+    cell = 30 * batch * (64 * 32 * 32 + 128 * 16 * 16) * 2
+    assert used > cells * cell
+    # all but one cell's buffers less than the grid took, and some allocations' rounding more
+    room = used - (cells - 1) * cell + (256 << 20)
+    hold = torch.empty(free() - room, dtype=torch.uint8, device="cuda")
+    try:
+        assert np.array_equal(run(), ref)
+    finally:
+        del hold
+        torch.cuda.empty_cache()
