@@ -19,6 +19,7 @@
 #include <stdint.h>
 
 #include <algorithm>
+#include <cstdlib>
 #include <string>
 #include <type_traits>
 
@@ -2604,6 +2605,12 @@ bool ctc_make_weight_maps(ConvWeightMaps* m, const void* base, uint64_t K, uint6
          ctc_make_map(&m->half, base, K, rows, depth, depth_elems, nbox / 2, msg);
 }
 
+// LIPZ_CONV_SINGLE=1: no CTA pairs and no first-layer kernel of its own (for comparisons).
+static bool conv_single() {
+  const char* v = getenv("LIPZ_CONV_SINGLE");
+  return v && v[0] == '1';
+}
+
 bool ctc_make_out_map(CUtensorMap* m, CtcParams* q, const ConvTcDesc* descs, int n_probs,
                       std::string* msg) {
   q->tma_out = 0;
@@ -2612,14 +2619,16 @@ bool ctc_make_out_map(CUtensorMap* m, CtcParams* q, const ConvTcDesc* descs, int
   const int64_t per = M * q->co;
   int64_t pstride = per;
   if (n_probs > 1) pstride = (int64_t)(descs[1].out - descs[0].out);
-  bool fits = pstride >= per && pstride % 8 == 0 && ((uintptr_t)descs[0].out & 15) == 0 &&
-              q->share >= 1 && n_probs % q->share == 0;
+  bool fits = !conv_single() && pstride >= per && pstride % 8 == 0 &&
+              ((uintptr_t)descs[0].out & 15) == 0 && q->share >= 1 && n_probs % q->share == 0;
   for (int i = 1; i < n_probs && fits; ++i)
     fits = (int64_t)(descs[i].out - descs[0].out) == i * pstride &&
            descs[i].in == descs[i - i % q->share].in;
   if (!fits) {
-    if (msg) *msg = "first convolution: outputs not at one stride, or a group's inputs differ";
-    return false;
+    // (k_conv_tc builds the tile for every problem and stores its outputs itself)
+    q->n_tiles *= q->share;
+    q->share = 1;
+    return true;
   }
   if (!ensure_encode(msg)) return false;
   cuuint64_t dims[3] = {(cuuint64_t)q->co, (cuuint64_t)M, (cuuint64_t)n_probs};
@@ -2672,7 +2681,7 @@ const ConvVariant kConvVariants[] = {
 int conv_ak(const CtcParams& p) {
   return p.scatter   ? ctc::AK_SCATTER
          : p.tma_out ? ctc::AK_FIRST
-         : p.nchw_in ? (p.nbox <= 64 ? ctc::AK_NCHW : ctc::AK_NCHW_WIDE)
+         : p.nchw_in ? (p.nbox <= 64 && p.out_mode == CTC_F32_HWC ? ctc::AK_NCHW : ctc::AK_NCHW_WIDE)
          : p.a_tma   ? (p.transposed ? (p.m2 && p.nbox <= 64 ? ctc::AK_TRANS_C : ctc::AK_TRANS)
                                      : ctc::AK_CONV)
                      : ctc::AK_GATHER;
@@ -2691,6 +2700,7 @@ bool ctc_make_act_map(CUtensorMap* m, CtcParams* q, const ConvTcDesc* descs, int
   q->a_tma = 0;
   q->m2 = 0;
   q->mt1 = q->mtiles;
+  const int mtiles1 = q->mtiles, n_tiles1 = q->n_tiles;
   if (!use_tma || q->nchw_in || q->ci % 64 != 0 || n_probs < 1) return true;
   const int lq = q->scatter ? q->lhi : q->lho - q->transposed;
   if (lq > 7) return true;
@@ -2745,12 +2755,16 @@ bool ctc_make_act_map(CUtensorMap* m, CtcParams* q, const ConvTcDesc* descs, int
     a.val.clusterDim.z = 1;
     cfg.attrs = &a;
     cfg.numAttrs = 1;
-    if (cudaOccupancyMaxActiveClusters(&q->clusters, (const void*)conv_kernel(*q), &cfg) !=
+    if (conv_single() ||
+        cudaOccupancyMaxActiveClusters(&q->clusters, (const void*)conv_kernel(*q), &cfg) !=
             cudaSuccess ||
         q->clusters < 1) {
+      // no pair can be resident: single CTAs whose gather warps load A
       cudaGetLastError();
-      if (msg) *msg = "no CTA pair of the tensor-core convolution can be resident";
-      return false;
+      q->a_tma = q->m2 = 0;
+      q->mtiles = q->mt1 = mtiles1;
+      q->n_tiles = n_tiles1;
+      return true;
     }
     const int mtp = (q->mt1 + 1) / 2;
     q->n_tiles = q->n_tiles / q->mtiles * mtp;

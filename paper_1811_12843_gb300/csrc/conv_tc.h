@@ -143,15 +143,16 @@ int ctc_bn_slots(const CtcParams& q, int n_probs);
 // the input pixels of 128 output pixels (traversal stride 2 for the convolution, 1 for the
 // parity classes). Sets q->a_tma = 1 when it applies (else 0, and the gather warps load A;
 // use_tma = false forces that), and then q->m2, the 256-row tile and CTA pair counts where they
-// apply (ctc_prepare comes first);
+// apply (ctc_prepare comes first; where no pair can be resident, a_tma stays 0);
 // q->mtiles and q->n_tiles must count 128-row tiles on entry. False only when the driver
 // refuses the map.
 bool ctc_make_act_map(CUtensorMap* m, CtcParams* q, const ConvTcDesc* descs, int n_probs,
                       std::string* msg, bool use_tma = true);
 // Output map of a first-layer launch (nchw_in, CTC_LRELU_HWC, co 64; else nothing is done) whose
-// problems' outputs sit at a uniform stride from descs[0].out: dims (64 channels, output pixels,
-// problems), boxes of 32 pixels in the 128-byte swizzle. Sets q->tma_out = 1; false when the
-// outputs or the groups' shared inputs do not fit, or the driver refuses the map.
+// problems' outputs sit at a uniform stride from descs[0].out and whose groups of q->share problems
+// read the same inputs: dims (64 channels, output pixels, problems), boxes of 32 pixels in the 128-byte
+// swizzle. Sets q->tma_out = 1 when it applies (else 0, and q->share = 1 with n_tiles to match); false
+// only when the driver refuses the map.
 bool ctc_make_out_map(CUtensorMap* m, CtcParams* q, const ConvTcDesc* descs, int n_probs,
                       std::string* msg);
 bool ctc_prepare(std::string* msg);

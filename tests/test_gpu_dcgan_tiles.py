@@ -1,8 +1,9 @@
 """The tensor-core convolutions' tiles: batches whose output pixels end inside a 128-row tile, a
 CTA pair or a 256-row tile, one and several cells per launch, and widths with 128- and 256-column
 weight tiles. One iteration through the TMA kernels (CTA pairs, 256-row tiles, the shared first
-layer) must end in the state of the one-CTA kernels that gather their A rows, bit for bit, and the
-evaluation must meet the oracle. And a grid for whose cells' shared launches the memory is not there."""
+layer) must end in the state of the one-CTA kernels that gather their A rows, and in that of a device
+where no pair can be resident and no output map applies, bit for bit, and the evaluation must meet the
+oracle. And a grid for whose cells' shared launches the memory is not there."""
 
 import numpy as np
 import pytest
@@ -21,12 +22,14 @@ pytestmark = pytest.mark.gpu
 def test_tma_pairs_equal_gathered_tiles(L, monkeypatch, rows, cols, batch, ngf, ndf):  # noqa: F811
     pool = _field_pool(6, 64)
     out = []
-    for gather in ("0", "1"):
+    for gather, single in (("0", "0"), ("1", "0"), ("0", "1")):
         monkeypatch.setenv("LIPZ_CONV_GATHER", gather)
+        monkeypatch.setenv("LIPZ_CONV_SINGLE", single)
         g = _grid(L, rows, cols, 3, pool, precision="bf16", batch=batch, ngf=ngf, ndf=ndf)
         g.iterate(2)
         out.append(np.frombuffer(g.export_state(), np.uint8))
     assert np.array_equal(out[0], out[1])
+    assert np.array_equal(out[0], out[2])
 
 
 @pytest.mark.parametrize("batch", [1, 9])
