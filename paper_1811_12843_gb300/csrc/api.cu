@@ -89,7 +89,7 @@ struct lipz_grid {
   bool buf_read[2] = {false, false};
   int a_last = 1;                  // slot of the newest call
   bool a_pending = false;          // the newest call's status is still to be reported
-  int device = 0;
+  int device = 0, sms = 1;
   // population snapshots: ping-pong pair, or three in rotation with stale neighbours (the
   // snapshot being written must not be the one the stale neighbours are read from)
   PopView G[3]{}, D[3]{};
@@ -341,7 +341,7 @@ int make_set(lipz_grid* g, GemmSet* S, std::vector<GemmDesc> v) {
   std::stable_sort(v.begin(), v.end(),
                    [](const GemmDesc& a, const GemmDesc& b) { return a.K > b.K; });
   // The tile shape with the least estimated time, in multiply-adds of one SM: the padded tiles'
-  // work over 152 SMs, a multiply-add weighted by what it costs in the shape (outputs per value
+  // work over the SMs, a multiply-add weighted by what it costs in the shape (outputs per value
   // read from shared memory), and a quarter of the longest tile's time, which has an SM's `share`th
   // part. Measured, fp32: 128 x 64 against 32 x 32 takes 367 against 525 us for the
   // discriminators of a 3x3 grid (900 against 6840 tiles), 215 against 173 for its backward (36 to
@@ -354,13 +354,13 @@ int make_set(lipz_grid* g, GemmSet* S, std::vector<GemmDesc> v) {
     // Rounds of co-resident CTAs (two per SM), a round of the narrower tiles weighted by its measured
     // time. 128 x 128 against 128 x 64: 475 against 633 us for 2400 tiles of 128 x 128 (8 rounds
     // against 16), 47 against 56 for 240 (1 against 2), 58 against 66 for 270 (1 against 2), and five
-    // launches of 48 to 96 tiles (1 and 1) 77 against 55.
+    // launches of 48 to 96 tiles (1 and 1) 77 against 55 (152 SMs).
     for (int s = 0; s < GEMM_TC_N_TILES; ++s) {
       const GemmTile t = GEMM_TC_TILES[s];
       int64_t n = 0;
       for (const GemmDesc& d : v)
         n += (int64_t)((d.M + t.bm - 1) / t.bm) * ((d.N + t.bn - 1) / t.bn);
-      const double cost = (double)((n + 303) / 304) * (t.bn == 128 ? 1.0 : 0.8);
+      const double cost = (double)((n + 2 * g->sms - 1) / (2 * g->sms)) * (t.bn == 128 ? 1.0 : 0.8);
       if (s == 0 || cost < best) {
         best = cost;
         S->shape = s;
@@ -375,7 +375,7 @@ int make_set(lipz_grid* g, GemmSet* S, std::vector<GemmDesc> v) {
       work += tile * ((d.M + t.bm - 1) / t.bm) * ((d.N + t.bn - 1) / t.bn);
       last = std::max(last, tile * share[s]);
     }
-    const double cost = work / 152 + 0.25 * last;
+    const double cost = work / g->sms + 0.25 * last;
     if (s == 0 || cost < best) {
       best = cost;
       S->shape = s;
@@ -728,6 +728,7 @@ int create_impl(lipz_grid* g) {
   const size_t es = g->esz;
   int rc;
   CK(g, cudaGetDevice(&g->device));
+  CK(g, cudaDeviceGetAttribute(&g->sms, cudaDevAttrMultiProcessorCount, g->device));
   // the grid's own stream (lipz_set_stream may replace it)
   CK(g, cudaStreamCreateWithFlags(&g->own_st, cudaStreamNonBlocking));
   g->st = g->own_st;
