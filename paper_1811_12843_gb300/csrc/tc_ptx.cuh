@@ -116,18 +116,8 @@ __device__ __forceinline__ void tma_store_4d(const CUtensorMap* map, uint32_t sr
       "r"(x), "r"(y), "r"(z), "r"(w), "r"(src)
       : "memory");
 }
-// 256-bit global accesses (32-byte aligned): one per 16 bf16 of a row, half the L1 wavefronts
-// of two 16-byte accesses when the lanes of a warp touch 32 different rows
-struct U8 {
-  uint4 a, b;
-};
-__device__ __forceinline__ U8 ld_global_v8(const void* p) {
-  uint32_t r0, r1, r2, r3, r4, r5, r6, r7;
-  asm("ld.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-               : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3), "=r"(r4), "=r"(r5), "=r"(r6), "=r"(r7)
-               : "l"(p));
-  return U8{make_uint4(r0, r1, r2, r3), make_uint4(r4, r5, r6, r7)};
-}
+// 256-bit global store (32-byte aligned): one per 16 bf16 of a row, half the L1 wavefronts of two
+// 16-byte stores when the lanes of a warp touch 32 different rows
 __device__ __forceinline__ void st_global_v8(void* p, uint4 a, uint4 b) {
   asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "r"(a.x),
                "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)
@@ -299,12 +289,6 @@ __device__ __forceinline__ uint32_t mapa_shared(uint32_t addr, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
 }
-// Arrive (release at cluster scope) on an mbarrier given by its shared::cluster address: the
-// peer's waiter (acquire at cluster scope) then sees this thread's earlier writes.
-__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar_cluster) {
-  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar_cluster)
-               : "memory");
-}
 // Arrive on an mbarrier given by its shared::cluster address with the default (CTA-scope)
 // semantics: for signals that order no memory (a tensor-memory region has been read).
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t bar_cluster) {
@@ -315,40 +299,6 @@ __device__ __forceinline__ float ex2_approx(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
-}
-__device__ __forceinline__ bool mbar_try_cluster(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n"
-      " selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// Bounded wait (acquire at cluster scope: the barrier's arrivals may come from the peer CTA).
-__device__ __forceinline__ bool mbar_wait_cl(uint32_t bar, uint32_t parity, volatile int* abort_flag,
-                                             int* err, int code) {
-  if (mbar_try_cluster(bar, parity)) return true;
-  const unsigned long long t0 = globaltimer();
-  for (uint32_t it = 1;; ++it) {
-    if (mbar_try_cluster(bar, parity)) return true;
-    if ((it & 255u) == 0) {
-      if (*abort_flag) return false;
-      if (globaltimer() - t0 > WAIT_NS) {
-        *abort_flag = 1;
-        atomicExch(err, code);
-        return false;
-      }
-    }
-  }
-}
-__device__ __forceinline__ bool mbar_wait_cl_warp(uint32_t bar, uint32_t parity,
-                                                  volatile int* abort_flag, int* err, int code) {
-  int ok = 0;
-  if ((threadIdx.x & 31) == 0) ok = mbar_wait_cl(bar, parity, abort_flag, err, code) ? 1 : 0;
-  ok = __shfl_sync(0xffffffffu, ok, 0);
-  return ok != 0;
 }
 // Every thread of both CTAs; orders the set-up (barrier initialisation, TMEM allocation) before
 // any access from the peer, and at the end every access from the peer before exit.
