@@ -1,6 +1,7 @@
 """The CUDA-core grouped GEMM and the gathered training inputs: sizes at the edges of the output
 tiles (32, 64, 128) and of the 16-wide k-slices, rows that allow and forbid four-element loads, in
-both precisions, and grids on both sides of the tile-shape rule; one iteration against the oracle.
+both precisions (bf16 with force_simt, which keeps it off the tensor cores), and grids on both sides of
+the tile-shape rule; one iteration against the oracle.
 """
 
 import pytest
@@ -19,6 +20,6 @@ def test_one_iteration_against_the_oracle(L, precision, rows, cols, batch, z, hi
     """Evaluation, gradients, Adam and weights by the rules of the one-iteration checks."""
     pool = _pool(5, 500, x)
     g = _grid(L, rows, cols, 23, pool, precision=precision, batch=batch, z_dim=z, hidden=hidden,
-              x_dim=x, keep_grads=1)
+              x_dim=x, keep_grads=1, force_simt=int(precision == "bf16"))
     _one_iteration_check(L, g, pool, 1e-4 if precision == "fp32" else 2e-2,
                          label="CUDA-core %s h=%d" % (precision, hidden))
