@@ -81,8 +81,9 @@ enum { LIPZ_STEP_STREAM_STRIDE = 256 };
  * losses, gradients and the Adam state (fp32 master weights, m, v) stay fp32.
  * LIPZ_FP32: everything fp32. Constraints: z_dim, hidden, x_dim, batch >= 1; hidden <= 1024;
  * tournament_size in 1..5. bf16 runs on the tensor cores: in chained kernels where hidden == 256
- * and z_dim, x_dim are multiples of 16, in one grouped product per layer elsewhere; fp32 on the
- * CUDA cores.
+ * and z_dim, x_dim are multiples of 16, in one grouped product per layer elsewhere (there, sums over
+ * fewer than 48 terms and weight gradients over fewer than 64 rows run on the CUDA cores, which form
+ * them more exactly); fp32 on the CUDA cores.
  */
 typedef struct lipz_arch {
   uint32_t struct_size;

@@ -42,9 +42,10 @@ struct TcbBuffers {
   int64_t PGs, PDs;
   const int64_t *goff, *doff;
   const int *src_g, *src_d;
-  // fuse_adam != 0: the weight-gradient tiles apply Adam instead of storing the gradient (the
-  // biases and D's output layer stay in gG / gD). Per population: the old snapshot (read at
-  // src[cell]), the new one (written at the cell) and the per-cell coefficients.
+  // fuse_adam != 0: the launch applies Adam instead of storing the gradients, the weight matrices'
+  // in their gradients' tiles, the biases and D's output layer (whose gradient it reads from gD) in
+  // the cells' ranges entries. Per population: the old snapshot (read at src[cell]), the new one
+  // (written at the cell) and the per-cell coefficients.
   int fuse_adam;
   struct AdamPop {
     const float *w, *m, *v;
@@ -66,8 +67,9 @@ struct TcbPlan;
 // hidden == 256, z == 64, x a multiple of 16, 1 <= batch <= 256.
 bool tcb_supported(int z, int h, int x, int B);
 TcbPlan* tcb_plan_create(const TcbShape& s, const TcbBuffers& b, std::string* msg);
-// All nine products of every cell in one launch, as the tiles of the stages 0 D1, 1 dW2(D), 2 A3,
-// 3 dW1(D), 4 A2, 5 dW3(G), 6 A1, 7 dW2(G), 8 dW1(G), claimed by persistent CTAs.
+// Every product of every cell in one launch, as the tiles of ten stages (D1's rows of G's loss, D1's
+// rows of D's loss, A3, A2, A1, then dW2(D), dW1(D), dW3(G), dW2(G), dW1(G)) and two entries per cell
+// for the remaining ranges, claimed by persistent CTAs.
 int tcb_run(TcbPlan* p, cudaStream_t st, std::string* msg);
 int* tcb_error_flag(TcbPlan* p);
 void tcb_plan_destroy(TcbPlan* p);

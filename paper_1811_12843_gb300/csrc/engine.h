@@ -180,7 +180,7 @@ void launch_row_norms(const T* E, int64_t e_cell, int cells, int rows, int x, fl
                       cudaStream_t st);
 void launch_mix_partials(const float* gram, const float* rnorm, int cells, int rows, int B, int x,
                          float* out, cudaStream_t st);
-// tri: part is the tensor-core Gram kernel's (upper triangle), nh its column ranges.
+// tri: part is the tensor-core Gram kernel's (upper triangle), nh its column parts.
 void launch_mix_es(const float* part, int nh, bool tri, int cells, int rows, int B, float* mix,
                    float* S, float* score, uint64_t seed, uint32_t t, float sigma, cudaStream_t st);
 // Choice of every cell's own centre (slot 0), for the later minibatch steps of an iteration.
