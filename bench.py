@@ -86,7 +86,7 @@ _derive()
 # dram__bytes_write.sum) of these same kernels, each with the summary it comes from. A phase
 # whose kernels changed after its capture has no entry (null traffic).
 PHASE_TRAFFIC = {
-    "train_bwd": (2131.1e6, "profiles/k_bwd_fused_adam_12x12_bf16.md"),
+    "train_bwd": (2131.9e6, "profiles/k_bwd_fused_adam_12x12_bf16.md"),
     "d_fwd": (236.6e6, "profiles/k_mlp_fwd_pair_eval_12x12_bf16.md"),
     "g_fwd": (145.6e6, "profiles/k_mlp_fwd_pair_eval_12x12_bf16.md"),
     "batch": (21.2e6, "profiles/launches_12x12_bf16_iteration.md"),
